@@ -110,8 +110,9 @@ __global__ void props_grad_kernel(Phys ph, int64_t n_int, const int64_t *nbr_ptr
 // Gradient sums of one row by its W-lane group (a row-tile round): entries
 // beg + sub + j W, j < nmax (nmax warp-uniform; see row_dot_n), each adding
 // (E_j - E_i) g_ij to the three components.  Slots past the row's end add
-// fma(0, 0, g) = g.
-template <int W, int U>
+// fma(0, 0, g) = g.  D3: three dimensions (below, the z weights are zero and are
+// neither stored nor read: 3 of 4 FP64 operations and 20 of 28 bytes a pair).
+template <int W, int U, bool D3>
 __device__ __forceinline__ Sum3 grad_row_n(int64_t beg, int64_t end, const int32_t *__restrict__ gcol,
                                            const double *__restrict__ gvx,
                                            const double *__restrict__ gvy,
@@ -131,7 +132,7 @@ __device__ __forceinline__ Sum3 grad_row_n(int64_t beg, int64_t end, const int32
       c[u] = ok ? __ldg(gcol + kk) : -1;
       ax[u] = ok ? __ldg(gvx + kk) : 0.0;
       ay[u] = ok ? __ldg(gvy + kk) : 0.0;
-      az[u] = ok ? __ldg(gvz + kk) : 0.0;
+      az[u] = D3 && ok ? __ldg(gvz + kk) : 0.0;
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -139,7 +140,7 @@ __device__ __forceinline__ Sum3 grad_row_n(int64_t beg, int64_t end, const int32
       const double dE = __ldg(E + c[u]) - Ei;
       gx = fmadd(dE, ax[u], gx);
       gy = fmadd(dE, ay[u], gy);
-      gz = fmadd(dE, az[u], gz);
+      if (D3) gz = fmadd(dE, az[u], gz);
     }
   }
   const int rem = nmax - j;  // warp-uniform, < U
@@ -152,14 +153,14 @@ __device__ __forceinline__ Sum3 grad_row_n(int64_t beg, int64_t end, const int32
       const int32_t c = ok ? __ldg(gcol + kk) : -1;
       ax[u] = ok ? __ldg(gvx + kk) : 0.0;
       ay[u] = ok ? __ldg(gvy + kk) : 0.0;
-      az[u] = ok ? __ldg(gvz + kk) : 0.0;
+      az[u] = D3 && ok ? __ldg(gvz + kk) : 0.0;
       dE[u] = c >= 0 ? __ldg(E + c) - Ei : 0.0;
     }
 #pragma unroll 1
     for (int u = 0; u < rem; ++u) {
       gx = fmadd(dE[0], ax[0], gx);
       gy = fmadd(dE[0], ay[0], gy);
-      gz = fmadd(dE[0], az[0], gz);
+      if (D3) gz = fmadd(dE[0], az[0], gz);
 #pragma unroll
       for (int q = 0; q + 1 < U; ++q) {
         dE[q] = dE[q + 1];
@@ -181,7 +182,7 @@ __device__ __forceinline__ Sum3 grad_row_n(int64_t beg, int64_t end, const int32
 // a row, up to U slots of pair data).
 constexpr int kPairMinBlocks = 3;
 
-template <int W, int U>
+template <int W, int U, bool D3>
 __global__ void __launch_bounds__(kBlock, kPairMinBlocks)
     props_grad_pre_kernel(Phys ph, int64_t n_int, const int64_t *nbr_ptr, const int32_t *gcol,
                           const double *gvx, const double *gvy, const double *gvz,
@@ -205,7 +206,7 @@ __global__ void __launch_bounds__(kBlock, kPairMinBlocks)
       const int64_t rb = __shfl_sync(0xffffffffu, b, t, W);
       const int64_t re = __shfl_sync(0xffffffffu, e, t, W);
       const double Ei = __shfl_sync(0xffffffffu, Eo, t, W);
-      return grad_row_n<W, U>(rb, re, gcol, gvx, gvy, gvz, E, Ei, sub,
+      return grad_row_n<W, U, D3>(rb, re, gcol, gvx, gvy, gvz, E, Ei, sub,
                               tile_nmax<W>(rb, re, sub));
     });
     if (active) {
@@ -222,22 +223,28 @@ __global__ void __launch_bounds__(kBlock, kPairMinBlocks)
   }
 }
 
-// pair geometry for the gradient (once per particle set)
+// pair geometry for the gradient (once per particle set); gvz == nullptr below
+// three dimensions.  A warp per row, so that the list reads and the writes are
+// coalesced: a thread per row took 26.7 ms for 1.44e8 pairs (1.3e6 rows), this
+// takes 2.8 ms.
 __global__ void grad_geom_kernel(int64_t n_int, const int64_t *nbr_ptr, const int32_t *nbr_col,
                                  const double *nbr_F, const double *px, const double *py,
                                  const double *pz, const double *V, const int32_t *kind,
                                  const int32_t *copysrc, int32_t *gcol, double *gvx, double *gvy,
                                  double *gvz) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_int;
-       i += (int64_t)gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t i = warp; i < n_int; i += nwarps) {
     const double xi = px[i], yi = py[i], zi = pz[i];
-    for (int64_t k = nbr_ptr[i]; k < nbr_ptr[i + 1]; ++k) {
+    const int64_t e = nbr_ptr[i + 1];
+    for (int64_t k = nbr_ptr[i] + lane; k < e; k += 32) {
       const int32_t j = nbr_col[k];
       gcol[k] = kind[j] == SPH_RT_COPY ? copysrc[j] : j;
       const double vf = V[j] * nbr_F[k];
       gvx[k] = vf * (xi - px[j]);
       gvy[k] = vf * (yi - py[j]);
-      gvz[k] = vf * (zi - pz[j]);
+      if (gvz) gvz[k] = vf * (zi - pz[j]);
     }
   }
 }
@@ -685,14 +692,15 @@ sph_rt_status launch_properties(sph_rt *s, double dt) {
   SPH_LAUNCHED(s);
   if (s->cfg.limiter != SPH_RT_LIMITER_NONE) {
     // pair geometry once per particle set, if it fits a modest share of memory
+    const bool d3 = s->dim == 3;
     const double geom_bytes = 28.0 * (double)s->nnz_nbr;
     if (!s->gvx && geom_bytes < 24e9) {
       s->gcol = dalloc<int32_t>(s, s->nnz_nbr);
       s->gvx = dalloc<double>(s, s->nnz_nbr);
       s->gvy = dalloc<double>(s, s->nnz_nbr);
-      s->gvz = dalloc<double>(s, s->nnz_nbr);
-      if (!s->gcol || !s->gvx || !s->gvy || !s->gvz) return SPH_RT_ENOMEM;
-      grad_geom_kernel<<<grid_items(s, s->n_int, kBlock), kBlock, 0, s->stream>>>(
+      s->gvz = d3 ? dalloc<double>(s, s->nnz_nbr) : nullptr;
+      if (!s->gcol || !s->gvx || !s->gvy || (d3 && !s->gvz)) return SPH_RT_ENOMEM;
+      grad_geom_kernel<<<grid_items(s, s->n_int, kWarpsPerBlock), kBlock, 0, s->stream>>>(
           s->n_int, s->nbr_ptr, s->nbr_col, s->nbr_F, s->px, s->py, s->pz, s->V, s->kind,
           s->copysrc, s->gcol, s->gvx, s->gvy, s->gvz);
       SPH_LAUNCHED(s);
@@ -700,10 +708,16 @@ sph_rt_status launch_properties(sph_rt *s, double dt) {
     if (s->gvx) {
       RowShape sh = shape_for_mean(s->n_int ? (double)s->nnz_nbr / (double)s->n_int : 0.0);
       int gr = row_grid_blocks(s->num_sms, s->n_int, sh.W, kPairMinBlocks);
-      SPH_DISPATCH_SHAPE(sh.W, sh.U,
-                         (props_grad_pre_kernel<W, U><<<gr, kBlock, 0, s->stream>>>(
-                             ph, s->n_int, s->nbr_ptr, s->gcol, s->gvx, s->gvy, s->gvz, s->E,
-                             s->sigma, s->R, s->lambda, s->D)));
+      if (d3)
+        SPH_DISPATCH_SHAPE(sh.W, sh.U,
+                           (props_grad_pre_kernel<W, U, true><<<gr, kBlock, 0, s->stream>>>(
+                               ph, s->n_int, s->nbr_ptr, s->gcol, s->gvx, s->gvy, s->gvz, s->E,
+                               s->sigma, s->R, s->lambda, s->D)));
+      else
+        SPH_DISPATCH_SHAPE(sh.W, sh.U,
+                           (props_grad_pre_kernel<W, U, false><<<gr, kBlock, 0, s->stream>>>(
+                               ph, s->n_int, s->nbr_ptr, s->gcol, s->gvx, s->gvy, nullptr, s->E,
+                               s->sigma, s->R, s->lambda, s->D)));
       SPH_LAUNCHED(s);
     } else {
       int W = row_width(s->nnz_nbr, s->n_int);

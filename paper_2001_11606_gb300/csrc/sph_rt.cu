@@ -171,6 +171,21 @@ void *dalloc_bytes(sph_rt *s, size_t bytes) {
   return p;
 }
 
+// A buffer that outlives free_all(): taken from the handle's free list (or the
+// cache, or CUDA) without joining the particle set's buffers, and handed back
+// with hold_give once the stream has finished with it.
+static void *hold_take(sph_rt *s, size_t bytes, size_t *got) {
+  void *p = dalloc_bytes(s, bytes > 0 ? bytes : 1);
+  if (!p) return nullptr;
+  *got = s->alloc_size[p];
+  s->alloc_size.erase(p);
+  s->allocs.pop_back();  // dalloc_bytes appended it
+  return p;
+}
+static void hold_give(sph_rt *s, void *p, size_t got) {
+  if (p) s->pool.emplace(got, p);
+}
+
 void free_all(sph_rt *s) {
   if (s->gate_host) *s->gate_host = s->gate_epoch;  // release a held timing gate
   if (s->cuda_ready) cudaStreamSynchronize(s->stream);
@@ -612,17 +627,16 @@ __global__ void caller_layout_kernel(int64_t n, int dim, const int64_t *slot2cal
 static sph_rt_status rebuild_particles(sph_rt *s, const double *new_pos) {
   const int64_t n = s->n;
   const int dim = s->dim;
-  double *pos_c = nullptr, *arr = nullptr;
-  int32_t *kind_c = nullptr;
-  int64_t *copy_c = nullptr;
+  // held apart from the particle set's buffers, which set_particles_common
+  // releases before it has read these
+  size_t b_pos = 0, b_arr = 0, b_kind = 0, b_copy = 0;
+  double *pos_c = (double *)hold_take(s, sizeof(double) * n * dim, &b_pos);
+  double *arr = (double *)hold_take(s, sizeof(double) * n * 6, &b_arr);
+  int32_t *kind_c = (int32_t *)hold_take(s, sizeof(int32_t) * n, &b_kind);
+  int64_t *copy_c = (int64_t *)hold_take(s, sizeof(int64_t) * n, &b_copy);
   sph_rt_status rc = SPH_RT_OK;
-  if (cudaMalloc(&pos_c, sizeof(double) * n * dim) != cudaSuccess ||
-      cudaMalloc(&arr, sizeof(double) * n * 6) != cudaSuccess ||
-      cudaMalloc(&kind_c, sizeof(int32_t) * n) != cudaSuccess ||
-      cudaMalloc(&copy_c, sizeof(int64_t) * n) != cudaSuccess) {
-    cudaGetLastError();
+  if (!pos_c || !arr || !kind_c || !copy_c)
     rc = set_error(s, SPH_RT_ENOMEM, "no device memory for the particle rebuild");
-  }
   if (!rc) {
     const int g = (int)((n + kBlock - 1) / kBlock < (int64_t)s->num_sms * 8
                             ? (n + kBlock - 1) / kBlock
@@ -643,10 +657,11 @@ static sph_rt_status rebuild_particles(sph_rt *s, const double *new_pos) {
   if (!rc)
     rc = set_particles_common(s, n, pos_c, arr, arr + n, arr + 2 * n, arr + 3 * n, kind_c, copy_c,
                               arr + 4 * n, arr + 5 * n, true);
-  cudaFree(pos_c);
-  cudaFree(arr);
-  cudaFree(kind_c);
-  cudaFree(copy_c);
+  if (rc) cudaStreamSynchronize(s->stream);  // a failed rebuild may have work queued
+  hold_give(s, pos_c, b_pos);
+  hold_give(s, arr, b_arr);
+  hold_give(s, kind_c, b_kind);
+  hold_give(s, copy_c, b_copy);
   return rc;
 }
 
