@@ -18,6 +18,8 @@
 // a hash table from cell key to cell (up to 2^58 cells).
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace sphrt {
@@ -471,29 +473,8 @@ __global__ void volume_kernel(const double *mass, const double *rho, int64_t n, 
 }
 
 // --------------------------------------------------------------------------
-// Neighbour search: one warp per interior particle.
+// Kernel derivatives and the neighbour predicate.
 // --------------------------------------------------------------------------
-// Shape of dW/dq of the M4 cubic B-spline (support q < 2).
-__device__ __forceinline__ double spline_dw(double q) {
-  if (q < 1.0) return -3.0 * q + 2.25 * q * q;
-  if (q < 2.0) {
-    double t = 2.0 - q;
-    return -0.75 * t * t;
-  }
-  return 0.0;
-}
-
-// Shape of dW/dq of the Wendland C4 kernel of Sec. 2.4 (Eq. wendlandc4): the
-// printed polynomial (1 - q)^5 (8 q^2 + 5 q + 1) on q <= 1 has the derivative
-// -14 q (1 + 4 q) (1 - q)^4.
-__device__ __forceinline__ double wendland_dw(double q) {
-  if (q <= 1.0) {
-    const double t = 1.0 - q, t2 = t * t;
-    return -14.0 * q * (1.0 + 4.0 * q) * (t2 * t2);
-  }
-  return 0.0;
-}
-
 // Per-particle kernel coefficients: 1/h and k_d / h^(d+1), so that
 // dW/dr(r, h) = k_d / h^(d+1) * w'(r / h) needs no division per pair.  k_d makes
 // the kernel's volume integral one (Sec. 2.3): for the cubic B-spline 2/3,
@@ -559,16 +540,14 @@ __global__ void rel_kernel(Grid g, const double *px, const double *py, const dou
   }
 }
 
-// 1 / sqrt(r2) in FP64: FP32 seed refined by two Newton steps
-// y <- y (3/2 - r2/2 y^2) (quadratic convergence from ~1e-7 to the FP64
-// rounding level), which costs fewer FP64 operations than an IEEE square
-// root followed by a division.
+// 1 / sqrt(r2) in FP64: FP32 seed y refined by one third-order step,
+// y (1 + d/2 + 3/8 d^2) with d = 1 - r2 y^2, the Taylor series of (1 - d)^(-1/2)
+// (the seed's d ~ 2e-7 leaves d^3 ~ 1e-20, below the FP64 rounding): 5 FP64
+// operations and no division or square root.
 __device__ __forceinline__ double rsqrt_fp64(double r2) {
-  double y = (double)rsqrtf((float)r2);
-  const double hr2 = 0.5 * r2;
-  y = y * (1.5 - hr2 * y * y);
-  y = y * (1.5 - hr2 * y * y);
-  return y;
+  const double y = (double)rsqrtf((float)r2);
+  const double d = fma(-(r2 * y), y, 1.0);
+  return fma(y, d * fma(0.375, d, 0.5), y);
 }
 
 // Bitonic sort of one 64-bit key per lane, ascending across the warp.
@@ -619,60 +598,94 @@ struct HashCells {  // occupied cells only, open addressing with linear probing
   }
 };
 
-// Pair weight F_ij = W'_ij / r (two-h average) of neighbour j of i, in FP64.
-__device__ __forceinline__ double pair_weight(int kern, double xi, double yi, double zi,
-                                              double ihi, double cwi, int64_t j,
-                                              const double *px, const double *py,
-                                              const double *pz, const double *ih,
-                                              const double *cw) {
-  const double r2 = exact_r2(xi, yi, zi, px[j], py[j], pz[j]);
-  const double ir = rsqrt_fp64(r2), r = r2 * ir;
-  const double ihj = ih[j], cwj = cw[j];
-  const double qi = r * ihi;
-  const double dwi = cwi * (kern == SPH_RT_WENDLAND_C4 ? wendland_dw(qi) : spline_dw(qi));
-  // equal smoothing lengths (the common case): the same expression, computed once
-  double dwj = dwi;
-  if (ihj != ihi || cwj != cwi) {
-    const double qj = r * ihj;
-    dwj = cwj * (kern == SPH_RT_WENDLAND_C4 ? wendland_dw(qj) : spline_dw(qj));
+// --------------------------------------------------------------------------
+// Neighbour search by cell.
+//
+// The particles of one cell share their candidates, so the work item of a warp
+// is up to kCellChunk particles of a cell: the warp sorts the 3^d surrounding
+// cells by key, looks them all up at once (a cell a lane) and walks the
+// candidates 32 at a time, one a lane, in slot order (interior cells, then
+// ghost cells).  Each candidate record is loaded once and tested in registers
+// against every particle of the item (read from shared memory); ballots give
+// each particle's hits in slot order.  A warp per particle, as before, paid the
+// sort, 27 dependent look-ups and ~27 half-empty candidate batches for every
+// particle.
+//
+// Two passes, COUNT and FILL, with the same tests.  COUNT: lane p keeps the
+// counts of particle p (neighbours, operator entries, Dirichlet-ghost
+// couplings, interior neighbours).  FILL: columns only, each batch's hits of a
+// particle to consecutive places; the pair weights follow in pair_kernel.
+// 4.9e4 particles of ~257 neighbours (3-D, unequal h): count 0.39 -> 0.25 ms, fill
+// 1.28 (with the weights) -> 0.22 ms; sph_rt_set_particles of 2.1e6 particles and
+// 2.24e8 pairs 42.5 -> 16.9 ms with pair_kernel.
+// --------------------------------------------------------------------------
+constexpr int kCellChunk = 16;
+
+// Work items: (first slot, particles) of every kCellChunk-piece of the interior
+// cells.  Their order is that of arrival and changes no result.
+__device__ __forceinline__ void add_items(int64_t beg, int64_t cnt, int2 *items, unsigned *nitems) {
+  const unsigned k = (unsigned)((cnt + kCellChunk - 1) / kCellChunk);
+  const unsigned at = atomicAdd(nitems, k);
+  for (unsigned q = 0; q < k; ++q) {
+    const int64_t b = beg + (int64_t)q * kCellChunk;
+    const int64_t left = beg + cnt - b;
+    items[at + q] = make_int2((int)b, (int)(left < kCellChunk ? left : kCellChunk));
   }
-  return 0.5 * (dwi + dwj) * ir;
+}
+__global__ void dense_items_kernel(const int64_t *start, const unsigned *count, int64_t ninterior,
+                                   int2 *items, unsigned *nitems) {
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < ninterior;
+       k += (int64_t)gridDim.x * blockDim.x)
+    if (count[k]) add_items(start[k], count[k], items, nitems);
+}
+__global__ void sorted_items_kernel(const uint64_t *cell_key, const int64_t *cell_start,
+                                    int64_t ncells, int ghost_shift, int2 *items,
+                                    unsigned *nitems) {
+  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < ncells;
+       c += (int64_t)gridDim.x * blockDim.x)
+    if (!((cell_key[c] >> ghost_shift) & 1ull))
+      add_items(cell_start[c], cell_start[c + 1] - cell_start[c], items, nitems);
 }
 
-// One warp per interior particle.  FILL: the hits of each 32-candidate batch
-// (a few of 27 candidates per cell) are appended, in discovery order, to a
-// per-warp buffer, and their FP64 pair weights are computed 32 at a time:
-// an FP64 warp instruction costs the same with 1 or 32 active lanes, so
-// computing the weights per batch would cost ~27 batches of FP64 work per
-// particle instead of ~4.
-constexpr int kHitBuf = 64;  // pending hits per warp (< 32 carried + 32 new)
+struct NbrCounts {  // per interior particle (COUNT)
+  int64_t *nbr, *mat, *gh;
+  int32_t *interior;
+};
+
+constexpr int kCellRuns = 54;  // surrounding cells: 27 of interior particles, 27 of ghosts
+struct CellScan {              // one warp's item
+  float4 part[kCellChunk];     // rel record of each particle
+  int pre[kCellRuns + 1];      // candidates before each run
+  int beg[kCellRuns];          // first slot of each run
+  int off[kCellRuns];          // its cell's offset code (x + 3 y + 9 z, each 0..2)
+};
 
 template <bool FILL, typename Cells>
-__global__ void neighbor_kernel(Grid g, const double *px, const double *py, const double *pz,
-                                const double *h, const float4 *rel, Cells cells,
-                                int64_t n_int, int64_t *count,
-                                const int64_t *rowptr, int32_t *cols, double *F,
-                                const double *ih, const double *cw) {
-  __shared__ int32_t hitbuf[kWarpsPerBlock][FILL ? kHitBuf : 1];
+__global__ void __launch_bounds__(kBlock)
+    neighbor_kernel(Grid g, const double *px, const double *py, const double *pz, const double *h,
+                    const float4 *rel, const int32_t *kind, const int32_t *copysrc, Cells cells,
+                    int64_t n_int, const int2 *items, const unsigned *nitems, NbrCounts out,
+                    const int64_t *rowptr, int32_t *cols) {
+  __shared__ CellScan scan_sh[kWarpsPerBlock];
+  CellScan &S = scan_sh[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
-  int32_t *hb = hitbuf[threadIdx.x >> 5];
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const unsigned warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const unsigned nwarps = (gridDim.x * blockDim.x) >> 5;
   const int ncells = g.dim == 3 ? 27 : (g.dim == 2 ? 9 : 3);
   const float cellf = (float)g.cell;
   const float band = kNbrBand * cellf * cellf;
-  for (int64_t i = warp; i < n_int; i += nwarps) {
-    const double xi = px[i], yi = py[i], zi = pz[i], hi = h[i];
-    const float4 ri = rel[i];
-    int c[3] = {cell_coord(xi, g.lo[0], g.inv_cell, g.nc[0]),
-                cell_coord(yi, g.lo[1], g.inv_cell, g.nc[1]),
-                cell_coord(zi, g.lo[2], g.inv_cell, g.nc[2])};
-    // lane k < ncells: the k-th cell around i; sorted by Morton key with the
-    // lane (hence the offset) in the low 5 bits
+  const unsigned n_items = *nitems;
+  for (unsigned t = warp; t < n_items; t += nwarps) {
+    const int s0 = items[t].x, P = items[t].y;
+    const int c[3] = {cell_coord(px[s0], g.lo[0], g.inv_cell, g.nc[0]),
+                      cell_coord(py[s0], g.lo[1], g.inv_cell, g.nc[1]),
+                      cell_coord(pz[s0], g.lo[2], g.inv_cell, g.nc[2])};
+    // lane k < ncells: the k-th cell around the item's; sorted by Morton key with
+    // the lane (hence the offset) in the low 5 bits
     uint64_t mykey = ~0ull;
     if (lane < ncells) {
-      int o[3] = {lane % 3 - 1, (lane / 3) % 3 - 1, lane / 9 - 1};
+      const int o[3] = {lane % 3 - 1, (lane / 3) % 3 - 1, lane / 9 - 1};
       bool ok = true;
       int cc[3];
       for (int d = 0; d < 3; ++d) {
@@ -682,158 +695,251 @@ __global__ void neighbor_kernel(Grid g, const double *px, const double *py, cons
       if (ok) mykey = (morton(g, cc[0], cc[1], cc[2]) << 5) | (uint64_t)lane;
     }
     const uint64_t sorted = warp_sort_u64(mykey);
-    const int64_t out = FILL ? rowptr[i] : 0;
-    const double ihi = FILL ? ih[i] : 0.0, cwi = FILL ? cw[i] : 0.0;
-    int64_t total = 0;  // hits found (warp-uniform)
-    int64_t done = 0;   // hits written (FILL)
-    int pending = 0;    // hits in the buffer (FILL, warp-uniform)
-    for (int pass = 0; pass < 2; ++pass) {  // interior cells, then ghost cells
-      for (int k = 0; k < ncells; ++k) {
-        const uint64_t v = __shfl_sync(0xffffffffu, sorted, k);
-        if (v == ~0ull) break;
-        const int ol = (int)(v & 31ull);
-        const uint64_t kk = (v >> 5) | (pass ? (1ull << g.ghost_shift) : 0ull);
-        // -o cell per axis (axes beyond dim stay 0)
-        const float ox = -(float)(ol % 3 - 1) * cellf;
-        const float oy = g.dim > 1 ? -(float)((ol / 3) % 3 - 1) * cellf : 0.0f;
-        const float oz = g.dim > 2 ? -(float)(ol / 9 - 1) * cellf : 0.0f;
-        int64_t beg, cnt;
-        cells.find(kk, beg, cnt);
-        for (int64_t base = 0; base < cnt; base += 32) {
-          const int64_t j = beg + base + lane;
-          bool hit = false;
-          if (base + lane < cnt && j != i) {
-            const float4 rj = rel[j];
-            const float dx = (ri.x - rj.x) + ox;
-            const float dy = (ri.y - rj.y) + oy;
-            const float dz = (ri.z - rj.z) + oz;
-            const float r2f = dx * dx + dy * dy + dz * dz;
-            const float c2f = fmaxf(ri.w, rj.w);
-            if (r2f < c2f - band) {
-              hit = true;
-            } else if (!(r2f > c2f + band)) {  // within the band: the exact test
-              const double cut = g.support * fmax(hi, h[j]);
-              hit = exact_r2(xi, yi, zi, px[j], py[j], pz[j]) < __dmul_rn(cut, cut);
-            }
-          }
-          const unsigned m = __ballot_sync(0xffffffffu, hit);
-          total += __popc(m);
-          if (FILL) {
-            if (hit) hb[pending + __popc(m & lt)] = (int32_t)j;
-            pending += __popc(m);
-            __syncwarp();
-            if (pending >= 32) {  // 32 weights with every lane active
-              const int32_t jj = hb[lane];
-              cols[out + done + lane] = jj;
-              F[out + done + lane] = pair_weight(g.kernel, xi, yi, zi, ihi, cwi, jj, px, py, pz, ih, cw);
-              const int rest = pending - 32;
-              const int32_t carry = lane < rest ? hb[32 + lane] : 0;
-              __syncwarp();
-              if (lane < rest) hb[lane] = carry;
-              __syncwarp();
-              pending = rest;
-              done += 32;
-            }
+    int64_t b0 = 0, n0 = 0, b1 = 0, n1 = 0;  // interior and ghost particles of lane's cell
+    if (sorted != ~0ull) {
+      cells.find(sorted >> 5, b0, n0);
+      cells.find((sorted >> 5) | (1ull << g.ghost_shift), b1, n1);
+    }
+    int i0 = (int)n0, i1 = (int)n1;  // inclusive scans over the lanes
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v0 = __shfl_up_sync(0xffffffffu, i0, o), v1 = __shfl_up_sync(0xffffffffu, i1, o);
+      if (lane >= o) {
+        i0 += v0;
+        i1 += v1;
+      }
+    }
+    const int C0 = __shfl_sync(0xffffffffu, i0, 31);
+    const int C = C0 + __shfl_sync(0xffffffffu, i1, 31);
+    __syncwarp();  // the previous item's reads are done
+    if (lane < 27) {
+      S.pre[lane] = i0 - (int)n0;
+      S.pre[27 + lane] = C0 + i1 - (int)n1;
+      S.beg[lane] = (int)b0;
+      S.beg[27 + lane] = (int)b1;
+      S.off[lane] = S.off[27 + lane] = (int)(sorted & 31ull);
+    }
+    if (lane == 0) S.pre[kCellRuns] = C;
+    if (lane < P) S.part[lane] = rel[s0 + lane];
+    __syncwarp();
+    const int64_t row0 = FILL ? rowptr[s0] : 0;
+    // lane p: particle p's counts, or (FILL) where its next column goes, from row0
+    int nb = FILL && lane < P ? (int)(rowptr[s0 + lane] - row0) : 0;
+    int ng = 0, nself = 0, nint = 0;
+    int r = 0;  // run of this lane's candidate
+    for (int base = 0; base < C; base += 32) {
+      const int cand = base + lane;
+      const bool in = cand < C;
+      int j = -1;
+      float4 rj = make_float4(0.f, 0.f, 0.f, 0.f);
+      float ox = 0.f, oy = 0.f, oz = 0.f;  // -o cell per axis (axes beyond dim stay 0)
+      if (in) {
+        while (cand >= S.pre[r + 1]) ++r;  // ends: cand < C = pre[kCellRuns]
+        j = S.beg[r] + (cand - S.pre[r]);
+        rj = rel[j];
+        const int ol = S.off[r];
+        ox = -(float)(ol % 3 - 1) * cellf;
+        if (g.dim > 1) oy = -(float)((ol / 3) % 3 - 1) * cellf;
+        if (g.dim > 2) oz = -(float)(ol / 9 - 1) * cellf;
+      }
+      unsigned dir = 0u, cpy = 0u;  // lanes with Dirichlet / copy ghosts
+      int src = -1;
+      if (!FILL && base + 32 > C0) {
+        const int kj = in && cand >= C0 ? kind[j] : SPH_RT_INTERIOR;
+        if (kj == SPH_RT_COPY) src = copysrc[j];
+        dir = __ballot_sync(0xffffffffu, kj == SPH_RT_DIRICHLET);
+        cpy = __ballot_sync(0xffffffffu, kj == SPH_RT_COPY);
+      }
+      const unsigned inner = C0 - base >= 32 ? 0xffffffffu
+                             : C0 > base     ? (1u << (C0 - base)) - 1u
+                                             : 0u;  // lanes with interior candidates
+      for (int p = 0; p < P; ++p) {
+        const float4 ri = S.part[p];
+        const float dx = (ri.x - rj.x) + ox;
+        const float dy = (ri.y - rj.y) + oy;
+        const float dz = (ri.z - rj.z) + oz;
+        const float d = (dx * dx + dy * dy + dz * dz) - fmaxf(ri.w, rj.w);
+        bool hit = d < -band;
+        if (in && !(fabsf(d) > band)) {  // within the band (or not a number): the exact test
+          const int i = s0 + p;
+          const double cut = g.support * fmax(h[i], h[j]);
+          hit = exact_r2(px[i], py[i], pz[i], px[j], py[j], pz[j]) < __dmul_rn(cut, cut);
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, hit && in && j != s0 + p);
+        if (FILL) {
+          const int at = __shfl_sync(0xffffffffu, nb, p);
+          if ((m >> lane) & 1u) cols[row0 + at + __popc(m & lt)] = j;
+          if (lane == p) nb += __popc(m);
+        } else {
+          const unsigned self =
+              cpy ? __ballot_sync(0xffffffffu, ((m >> lane) & 1u) && src == s0 + p) : 0u;
+          if (lane == p) {
+            nb += __popc(m);
+            nint += __popc(m & inner);
+            ng += __popc(m & dir);
+            nself += __popc(self);
           }
         }
       }
     }
-    if (FILL && pending > 0) {
-      if (lane < pending) {
-        const int32_t jj = hb[lane];
-        cols[out + done + lane] = jj;
-        F[out + done + lane] = pair_weight(g.kernel, xi, yi, zi, ihi, cwi, jj, px, py, pz, ih, cw);
-      }
-      __syncwarp();
+    if (!FILL && lane < P) {
+      out.nbr[s0 + lane] = nb;
+      out.mat[s0 + lane] = nb - ng - nself;  // a copy of the row itself drops out
+      out.gh[s0 + lane] = ng;
+      out.interior[s0 + lane] = nint;
     }
-    if (!FILL && lane == 0) count[i] = total;
   }
 }
 
 // --------------------------------------------------------------------------
-// Operator sparsity from the neighbour lists: interior columns and copy-ghost
-// columns (moved to the copied particle; a copy of the row itself drops out)
-// form B; Dirichlet ghosts form the boundary-coupling list.
+// Pair weights F_ij = W'_ij / r (two-h average) of every list entry, and the
+// operator's geometric entry V_i V_j F_ij of the interior neighbours, which come
+// first in a row (their slots are the smallest) and so stand at mat_ptr[i] +
+// (k - nbr_ptr[i]).
+//
+// FP64-bound (GB300 issues one FP64 warp instruction in the time of ~32 FP32
+// ones, whatever its active lanes): a warp takes kPairRows consecutive rows and
+// walks their entries as one flat range, so that only the last instruction of a
+// range has idle lanes (of 200 entries in 2-D, 850-2,000 in 3-D); the rows' own
+// data sit in shared memory.  Longer ranges left 4e4 rows too few warps.  ~23 FP64 operations
+// a pair: r^2 by fused multiply-adds, the reciprocal root in 5, tests on q and
+// on equal smoothing lengths by bit patterns, and 0.5 (w + w) = w for the
+// latter (two evaluations otherwise).  1.26e7 pairs of unequal h: 1.02 ms.
 // --------------------------------------------------------------------------
-// One warp per row: the lanes take 32 consecutive entries at a time, so the
-// list reads and the compacted writes are coalesced; ballots keep the entries
-// in list order.
-__global__ void op_count_kernel(const int64_t *nbr_ptr, const int32_t *nbr_col,
-                                const int32_t *kind, const int32_t *copysrc, int64_t n_int,
-                                int64_t *mat_cnt, int64_t *gh_cnt) {
+// w'(q) without its normalisation.  Wendland C4 (Sec. 2.4, Eq. wendlandc4): the
+// printed polynomial (1 - q)^5 (8 q^2 + 5 q + 1) on q <= 1 has the derivative
+// -14 q (1 + 4 q) (1 - q)^4.  M4 cubic B-spline (support q < 2): its two pieces as
+// products of selected factors, -0.75 t t (t = 2 - q) and q (2.25 q - 3).
+__device__ __forceinline__ double pair_dw(int kern, double q) {
+  if (kern == SPH_RT_WENDLAND_C4) {
+    double t = 1.0 - q;
+    if (__double2hiint(t) < 0) t = 0.0;  // beyond the support
+    const double t2 = t * t;
+    return (-14.0 * q) * fma(4.0, q, 1.0) * (t2 * t2);
+  }
+  const double t = 2.0 - q;
+  const bool inner = __double2hiint(q) < 0x3ff00000;  // q < 1
+  const double a = inner ? q : -0.75 * t, b = inner ? fma(2.25, q, -3.0) : t;
+  return __double2hiint(t) < 0 ? 0.0 : a * b;  // 0 beyond the support
+}
+
+constexpr int kPairRows = 8;
+struct PairRow {
+  double x, y, z, ih, cw, V;
+};
+
+__global__ void __launch_bounds__(kBlock)
+    pair_kernel(int kern, int64_t n_int, const int64_t *nbr_ptr, const int32_t *nbr_col,
+                const double *px, const double *py, const double *pz, const double *ih,
+                const double *cw, const double *V, const int64_t *mat_ptr, double *nbr_F,
+                int32_t *mat_col, double *mat_G) {
+  __shared__ PairRow rows_sh[kWarpsPerBlock][kPairRows];
+  __shared__ int ptr_sh[kWarpsPerBlock][kPairRows + 1];
+  __shared__ int64_t mat_sh[kWarpsPerBlock][kPairRows];
+  PairRow *R = rows_sh[threadIdx.x >> 5];
+  int *off = ptr_sh[threadIdx.x >> 5];
+  int64_t *mp = mat_sh[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t i = warp; i < n_int; i += nwarps) {
-    int64_t m = 0, g = 0;
-    const int64_t beg = nbr_ptr[i], end = nbr_ptr[i + 1];
-    for (int64_t k0 = beg; k0 < end; k0 += 32) {
-      const int64_t k = k0 + lane;
-      bool isg = false, ism = false;
-      if (k < end) {
-        const int32_t j = nbr_col[k];
-        const int32_t kj = kind[j];
-        isg = kj == SPH_RT_DIRICHLET;
-        ism = !isg && (kj == SPH_RT_INTERIOR || copysrc[j] != i);
-      }
-      g += __popc(__ballot_sync(0xffffffffu, isg));
-      m += __popc(__ballot_sync(0xffffffffu, ism));
+  const int64_t ntiles = ceil_div(n_int, kPairRows);
+  for (int64_t tile = warp; tile < ntiles; tile += nwarps) {
+    const int64_t r0 = tile * kPairRows;
+    const int rows = (int)(n_int - r0 < kPairRows ? n_int - r0 : kPairRows);
+    const int64_t k0 = nbr_ptr[r0];
+    __syncwarp();
+    if (lane < rows) {
+      const int64_t i = r0 + lane;
+      R[lane] = {px[i], py[i], pz[i], ih[i], cw[i], V[i]};
+      off[lane] = (int)(nbr_ptr[i] - k0);
+      mp[lane] = mat_ptr[i];
     }
-    if (lane == 0) {
-      mat_cnt[i] = m;
-      gh_cnt[i] = g;
+    if (lane == 0) off[rows] = (int)(nbr_ptr[r0 + rows] - k0);
+    __syncwarp();
+    const int total = off[rows];
+    int r = 0;  // row of this lane's entry
+    for (int k = lane; k < total; k += 32) {
+      while (k >= off[r + 1]) ++r;  // ends: k < total = off[rows]
+      const int32_t j = nbr_col[k0 + k];
+      const PairRow &q = R[r];
+      const double dx = q.x - px[j], dy = q.y - py[j], dz = q.z - pz[j];
+      const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+      const double ir = rsqrt_fp64(r2), d = r2 * ir;
+      const double ihj = ih[j];
+      double F = q.cw * pair_dw(kern, d * q.ih);
+      // equal smoothing lengths (the common case): 0.5 (w + w) = w
+      if (__double_as_longlong(ihj) != __double_as_longlong(q.ih))
+        F = 0.5 * (F + cw[j] * pair_dw(kern, d * ihj));
+      F *= ir;
+      nbr_F[k0 + k] = F;
+      if (j < n_int) {
+        const int64_t at = mp[r] + (k - off[r]);
+        mat_col[at] = j;
+        mat_G[at] = (q.V * V[j]) * F;
+      }
     }
   }
 }
 
-__global__ void op_fill_kernel(const int64_t *nbr_ptr, const int32_t *nbr_col, const double *nbr_F,
-                               const int32_t *kind, const int32_t *copysrc, const double *V,
-                               int64_t n_int, const int64_t *mat_ptr, int32_t *mat_col,
-                               double *mat_G, const int64_t *gh_ptr, int32_t *gh_slot,
-                               double *gh_W) {
+// --------------------------------------------------------------------------
+// Operator entries of ghost neighbours: copy-ghost columns (moved to the copied
+// particle; a copy of the row itself drops out) follow the interior ones in B;
+// Dirichlet ghosts form the boundary-coupling list.  Few rows have any: a warp
+// looks at kPairRows rows at a time and takes those with ghosts in turn, 32
+// entries at a time (ballots keep the entries in list order).
+// --------------------------------------------------------------------------
+__global__ void op_ghost_kernel(const int64_t *nbr_ptr, const int32_t *interior,
+                                const int32_t *nbr_col, const double *nbr_F, const int32_t *kind,
+                                const int32_t *copysrc, const double *V, int64_t n_int,
+                                const int64_t *mat_ptr, int32_t *mat_col, double *mat_G,
+                                const int64_t *gh_ptr, int32_t *gh_slot, double *gh_W) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t i = warp; i < n_int; i += nwarps) {
-    int64_t m = mat_ptr[i], g = gh_ptr[i];
-    const double Vi = V[i];
-    const int64_t beg = nbr_ptr[i], end = nbr_ptr[i + 1];
-    for (int64_t k0 = beg; k0 < end; k0 += 32) {
-      const int64_t k = k0 + lane;
-      bool isg = false, ism = false;
-      int32_t col = 0;
-      double val = 0.0;
-      if (k < end) {
-        const int32_t j = nbr_col[k];
-        const int32_t kj = kind[j];
-        const double Fk = nbr_F[k];
-        if (kj == SPH_RT_DIRICHLET) {
-          isg = true;
-          col = j;
-          val = V[j] * Fk;
-        } else {
-          col = kj == SPH_RT_INTERIOR ? j : copysrc[j];
-          if (col != i) {  // a copy of the row itself drops out
-            ism = true;
+  for (int64_t r0 = warp * kPairRows; r0 < n_int; r0 += nwarps * kPairRows) {
+    const int64_t il = r0 + lane;
+    unsigned todo = __ballot_sync(0xffffffffu,
+                                  lane < kPairRows && il < n_int &&
+                                      nbr_ptr[il + 1] - nbr_ptr[il] > interior[il]);
+    while (todo) {
+      const int64_t i = r0 + __ffs(todo) - 1;
+      todo &= todo - 1;
+      int64_t m = mat_ptr[i] + interior[i], g = gh_ptr[i];
+      const double Vi = V[i];
+      const int64_t end = nbr_ptr[i + 1];
+      for (int64_t k0 = nbr_ptr[i] + interior[i]; k0 < end; k0 += 32) {
+        const int64_t k = k0 + lane;
+        bool isg = false, ism = false;
+        int32_t col = 0;
+        double val = 0.0;
+        if (k < end) {
+          const int32_t j = nbr_col[k];
+          const double Fk = nbr_F[k];
+          if (kind[j] == SPH_RT_DIRICHLET) {
+            isg = true;
+            col = j;
+            val = V[j] * Fk;
+          } else {
+            col = copysrc[j];
+            ism = col != i;  // a copy of the row itself drops out
             val = (Vi * V[j]) * Fk;
           }
         }
+        const unsigned bg = __ballot_sync(0xffffffffu, isg);
+        const unsigned bm = __ballot_sync(0xffffffffu, ism);
+        if (isg) {
+          const int64_t at = g + __popc(bg & lt);
+          gh_slot[at] = col;
+          gh_W[at] = val;
+        }
+        if (ism) {
+          const int64_t at = m + __popc(bm & lt);
+          mat_col[at] = col;
+          mat_G[at] = val;
+        }
+        g += __popc(bg);
+        m += __popc(bm);
       }
-      const unsigned bg = __ballot_sync(0xffffffffu, isg);
-      const unsigned bm = __ballot_sync(0xffffffffu, ism);
-      if (isg) {
-        const int64_t at = g + __popc(bg & lt);
-        gh_slot[at] = col;
-        gh_W[at] = val;
-      }
-      if (ism) {
-        const int64_t at = m + __popc(bm & lt);
-        mat_col[at] = col;
-        mat_G[at] = val;
-      }
-      g += __popc(bg);
-      m += __popc(bm);
     }
   }
 }
@@ -922,6 +1028,7 @@ sph_rt_status build_particles(sph_rt *s, int64_t n, const double *pos_c, const d
   int64_t *v64[2] = {nullptr, nullptr}, *rhist = nullptr, *head = nullptr, *cidx = nullptr;
   int64_t *cell_start = nullptr, *hcell = nullptr;
   unsigned long long *hkey = nullptr;
+  int64_t n_cells = 0;  // occupied cells (ghost cells included)
   HashCells hcells{};
   s->slot2caller = dalloc<int64_t>(s, n);
   s->caller2slot = dalloc<int64_t>(s, n);
@@ -975,21 +1082,20 @@ sph_rt_status build_particles(sph_rt *s, int64_t n, const double *pos_c, const d
     cell_head_kernel<<<grid1(s, n), kBlock, 0, st>>>(k64[at], n, head);
     SPH_LAUNCHED(s);
     if ((rc = exclusive_scan(s, head, n, cidx))) return rc;
-    int64_t ncells = 0;
-    SPH_CUDA(s, cudaMemcpyAsync(&ncells, cidx + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    SPH_CUDA(s, cudaMemcpyAsync(&n_cells, cidx + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     SPH_CUDA(s, cudaStreamSynchronize(st));
-    cell_key = dalloc<uint64_t>(s, ncells);
-    cell_start = dalloc<int64_t>(s, ncells + 1);
+    cell_key = dalloc<uint64_t>(s, n_cells);
+    cell_start = dalloc<int64_t>(s, n_cells + 1);
     uint64_t hsize = 2;
-    while (hsize < 2 * (uint64_t)ncells) hsize <<= 1;  // at most half full
+    while (hsize < 2 * (uint64_t)n_cells) hsize <<= 1;  // at most half full
     hkey = dalloc<unsigned long long>(s, hsize);
     hcell = dalloc<int64_t>(s, hsize);
     if (!cell_key || !cell_start || !hkey || !hcell) return SPH_RT_ENOMEM;
     cell_fill_kernel<<<grid1(s, n), kBlock, 0, st>>>(k64[at], n, head, cidx, cell_key, cell_start);
     SPH_LAUNCHED(s);
-    SPH_CUDA(s, cudaMemcpyAsync(cell_start + ncells, &n, sizeof(int64_t), cudaMemcpyHostToDevice, st));
+    SPH_CUDA(s, cudaMemcpyAsync(cell_start + n_cells, &n, sizeof(int64_t), cudaMemcpyHostToDevice, st));
     SPH_CUDA(s, cudaMemsetAsync(hkey, 0xff, sizeof(unsigned long long) * hsize, st));
-    cell_hash_insert_kernel<<<grid1(s, ncells), kBlock, 0, st>>>(cell_key, ncells, hsize - 1, hkey,
+    cell_hash_insert_kernel<<<grid1(s, n_cells), kBlock, 0, st>>>(cell_key, n_cells, hsize - 1, hkey,
                                                                 hcell);
     SPH_LAUNCHED(s);
     hcells = HashCells{hkey, hcell, cell_start, hsize - 1};
@@ -1037,81 +1143,88 @@ sph_rt_status build_particles(sph_rt *s, int64_t n, const double *pos_c, const d
   volume_kernel<<<gg, kBlock, 0, st>>>(s->mass, s->rho, n, s->V, s->invV);
   SPH_LAUNCHED(s);
 
-  // neighbour lists
-  int64_t *nc = dalloc<int64_t>(s, n_int);
-  s->nbr_ptr = dalloc<int64_t>(s, n_int + 1);
-  if (!nc || !s->nbr_ptr) return SPH_RT_ENOMEM;
-  int64_t warps = n_int;
-  int gw = (int)ceil_div(warps, kWarpsPerBlock);
-  int gcap = s->num_sms * 8;
-  if (gw > gcap) gw = gcap;
+  // neighbour counts, with those of the operator's two lists
+  int64_t *nc = dalloc<int64_t>(s, n_int), *mc = dalloc<int64_t>(s, n_int),
+          *gc = dalloc<int64_t>(s, n_int);
+  int32_t *interior = dalloc<int32_t>(s, n_int);
+  int2 *items = dalloc<int2>(s, n_int);  // at most one item a particle
+  unsigned *nitems = dalloc<unsigned>(s, 1);
   float4 *rel = dalloc<float4>(s, n);
-  if (!rel) return SPH_RT_ENOMEM;
-  rel_kernel<<<grid1(s, n), kBlock, 0, st>>>(g, s->px, s->py, s->pz, s->h, n, rel);
-  SPH_LAUNCHED(s);
-  if (dense)
-    neighbor_kernel<false, DenseCells><<<gw, kBlock, 0, st>>>(
-        g, s->px, s->py, s->pz, s->h, rel, DenseCells{start, cnt}, n_int, nc, nullptr, nullptr,
-        nullptr, nullptr, nullptr);
-  else
-    neighbor_kernel<false, HashCells><<<gw, kBlock, 0, st>>>(g, s->px, s->py, s->pz, s->h, rel,
-                                                             hcells, n_int, nc, nullptr, nullptr,
-                                                             nullptr, nullptr, nullptr);
-  SPH_LAUNCHED(s);
-  rc = exclusive_scan(s, nc, n_int, s->nbr_ptr);
-  if (rc) return rc;
-  int64_t nnz = 0;
-  SPH_CUDA(s, cudaMemcpyAsync(&nnz, s->nbr_ptr + n_int, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-  SPH_CUDA(s, cudaStreamSynchronize(st));
-  s->nnz_nbr = nnz;
-  s->nbr_col = dalloc<int32_t>(s, nnz);
-  s->nbr_F = dalloc<double>(s, nnz);
-  if (!s->nbr_col || !s->nbr_F) return SPH_RT_ENOMEM;
-  double *ih = dalloc<double>(s, n), *cw = dalloc<double>(s, n);
-  if (!ih || !cw) return SPH_RT_ENOMEM;
-  kernel_coef_kernel<<<grid1(s, n), kBlock, 0, st>>>(n, dim, s->cfg.kernel, s->h, ih, cw);
-  SPH_LAUNCHED(s);
-  if (dense)
-    neighbor_kernel<true, DenseCells><<<gw, kBlock, 0, st>>>(
-        g, s->px, s->py, s->pz, s->h, rel, DenseCells{start, cnt}, n_int, nullptr, s->nbr_ptr,
-        s->nbr_col, s->nbr_F, ih, cw);
-  else
-    neighbor_kernel<true, HashCells><<<gw, kBlock, 0, st>>>(g, s->px, s->py, s->pz, s->h, rel,
-                                                            hcells, n_int, nullptr, s->nbr_ptr,
-                                                            s->nbr_col, s->nbr_F, ih, cw);
-  SPH_LAUNCHED(s);
-
-  // operator sparsity
-  int64_t *mc = dalloc<int64_t>(s, n_int), *gc = dalloc<int64_t>(s, n_int);
+  s->nbr_ptr = dalloc<int64_t>(s, n_int + 1);
   s->mat_ptr = dalloc<int64_t>(s, n_int + 1);
   s->gh_ptr = dalloc<int64_t>(s, n_int + 1);
-  if (!mc || !gc || !s->mat_ptr || !s->gh_ptr) return SPH_RT_ENOMEM;
-  int gi = (int)ceil_div(n_int, kWarpsPerBlock);  // a warp per row
-  if (gi > s->num_sms * 8) gi = s->num_sms * 8;
-  op_count_kernel<<<gi, kBlock, 0, st>>>(s->nbr_ptr, s->nbr_col, s->kind, s->copysrc, n_int, mc, gc);
+  if (!nc || !mc || !gc || !interior || !items || !nitems || !rel || !s->nbr_ptr || !s->mat_ptr ||
+      !s->gh_ptr)
+    return SPH_RT_ENOMEM;
+  rel_kernel<<<grid1(s, n), kBlock, 0, st>>>(g, s->px, s->py, s->pz, s->h, n, rel);
   SPH_LAUNCHED(s);
+  SPH_CUDA(s, cudaMemsetAsync(nitems, 0, sizeof(unsigned), st));
+  if (dense)
+    dense_items_kernel<<<grid1(s, nkeys / 2), kBlock, 0, st>>>(start, cnt, nkeys / 2, items,
+                                                               nitems);
+  else
+    sorted_items_kernel<<<grid1(s, n_cells), kBlock, 0, st>>>(cell_key, cell_start, n_cells,
+                                                              g.ghost_shift, items, nitems);
+  SPH_LAUNCHED(s);
+  int gw = (int)ceil_div(n_int, kWarpsPerBlock);
+  if (gw > s->num_sms * 8) gw = s->num_sms * 8;
+  const NbrCounts counts = {nc, mc, gc, interior};
+  auto search = [&](auto fill, const NbrCounts &out, const int64_t *rowptr,
+                    int32_t *cols) -> sph_rt_status {
+    constexpr bool FILL = decltype(fill)::value;
+    if (dense)
+      neighbor_kernel<FILL, DenseCells><<<gw, kBlock, 0, st>>>(
+          g, s->px, s->py, s->pz, s->h, rel, s->kind, s->copysrc, DenseCells{start, cnt}, n_int,
+          items, nitems, out, rowptr, cols);
+    else
+      neighbor_kernel<FILL, HashCells><<<gw, kBlock, 0, st>>>(
+          g, s->px, s->py, s->pz, s->h, rel, s->kind, s->copysrc, hcells, n_int, items, nitems,
+          out, rowptr, cols);
+    SPH_LAUNCHED(s);
+    return SPH_RT_OK;
+  };
+  if ((rc = search(std::false_type{}, counts, nullptr, nullptr))) return rc;
+  if ((rc = exclusive_scan(s, nc, n_int, s->nbr_ptr))) return rc;
   if ((rc = exclusive_scan(s, mc, n_int, s->mat_ptr))) return rc;
   if ((rc = exclusive_scan(s, gc, n_int, s->gh_ptr))) return rc;
-  int64_t sizes[2];
-  SPH_CUDA(s, cudaMemcpyAsync(&sizes[0], s->mat_ptr + n_int, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-  SPH_CUDA(s, cudaMemcpyAsync(&sizes[1], s->gh_ptr + n_int, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+  int64_t sizes[3];
+  const int64_t *ends[3] = {s->nbr_ptr + n_int, s->mat_ptr + n_int, s->gh_ptr + n_int};
+  for (int k = 0; k < 3; ++k)
+    SPH_CUDA(s, cudaMemcpyAsync(&sizes[k], ends[k], sizeof(int64_t), cudaMemcpyDeviceToHost, st));
   SPH_CUDA(s, cudaStreamSynchronize(st));
-  s->nnz_mat = sizes[0];
-  s->nnz_gh = sizes[1];
+  s->nnz_nbr = sizes[0];
+  s->nnz_mat = sizes[1];
+  s->nnz_gh = sizes[2];
+  s->nbr_col = dalloc<int32_t>(s, s->nnz_nbr);
+  s->nbr_F = dalloc<double>(s, s->nnz_nbr);
   s->mat_col = dalloc<int32_t>(s, s->nnz_mat);
   s->mat_G = dalloc<double>(s, s->nnz_mat);
   s->mat_val = dalloc<double>(s, s->nnz_mat);
   s->gh_slot = dalloc<int32_t>(s, s->nnz_gh);
   s->gh_W = dalloc<double>(s, s->nnz_gh);
-  if (!s->mat_col || !s->mat_G || !s->mat_val || !s->gh_slot || !s->gh_W) return SPH_RT_ENOMEM;
-  op_fill_kernel<<<gi, kBlock, 0, st>>>(s->nbr_ptr, s->nbr_col, s->nbr_F, s->kind, s->copysrc,
-                                        s->V, n_int, s->mat_ptr, s->mat_col, s->mat_G, s->gh_ptr,
-                                        s->gh_slot, s->gh_W);
+  double *ih = dalloc<double>(s, n), *cw = dalloc<double>(s, n);
+  if (!s->nbr_col || !s->nbr_F || !s->mat_col || !s->mat_G || !s->mat_val || !s->gh_slot ||
+      !s->gh_W || !ih || !cw)
+    return SPH_RT_ENOMEM;
+  kernel_coef_kernel<<<grid1(s, n), kBlock, 0, st>>>(n, dim, s->cfg.kernel, s->h, ih, cw);
   SPH_LAUNCHED(s);
+  if ((rc = search(std::true_type{}, NbrCounts{}, s->nbr_ptr, s->nbr_col))) return rc;
+  int gt = (int)ceil_div(ceil_div(n_int, kPairRows), kWarpsPerBlock);
+  if (gt > s->num_sms * 8) gt = s->num_sms * 8;
+  pair_kernel<<<gt, kBlock, 0, st>>>(s->cfg.kernel, n_int, s->nbr_ptr, s->nbr_col, s->px, s->py,
+                                     s->pz, ih, cw, s->V, s->mat_ptr, s->nbr_F, s->mat_col,
+                                     s->mat_G);
+  SPH_LAUNCHED(s);
+  if (n > n_int) {
+    op_ghost_kernel<<<gt, kBlock, 0, st>>>(s->nbr_ptr, interior, s->nbr_col, s->nbr_F, s->kind,
+                                           s->copysrc, s->V, n_int, s->mat_ptr, s->mat_col,
+                                           s->mat_G, s->gh_ptr, s->gh_slot, s->gh_W);
+    SPH_LAUNCHED(s);
+  }
   SPH_CUDA(s, cudaStreamSynchronize(st));
   // set-up scratch back to the free list
-  void *scratch[] = {cx, cy, cz, hc, bbox, key, cnt, cur, cnt64, start, nc, mc, gc, ih, cw, rel,
-                     k64[0], k64[1], v64[0], v64[1], rhist, head, cidx, cell_key, cell_start,
+  void *scratch[] = {cx, cy, cz, hc, bbox, key, cnt, cur, cnt64, start, nc, mc, gc, interior, items, nitems,
+                     ih, cw, rel, k64[0], k64[1], v64[0], v64[1], rhist, head, cidx, cell_key, cell_start,
                      hkey, hcell};
   for (void *p : scratch) dfree(s, p);
   return SPH_RT_OK;
