@@ -337,7 +337,8 @@ sph_rt_status sph_rt_get_properties(sph_rt *s, double *T, double *sigma, double 
 
 /* Kernel timing (config.kernel_timing = 1): number of SpMV launches on the
  * fine operator since the last reset, their summed CUDA-event time in ms, and
- * their algorithmic bytes (12 per stored nonzero + 8 per row for rowptr,
+ * their algorithmic bytes (12 per stored nonzero, 10 where a large
+ * particle set's columns are kept as 2-byte dictionary places, + 8 per row for rowptr,
  * x and y).  reset != 0 clears the counters after reading. */
 sph_rt_status sph_rt_kernel_stats(sph_rt *s, int64_t *launches, double *total_ms,
                                   double *bytes, int reset);

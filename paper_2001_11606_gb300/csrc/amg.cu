@@ -31,6 +31,7 @@
 #include <cooperative_groups.h>
 
 #include "common.cuh"
+#include "sliced.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -48,10 +49,6 @@ constexpr int kUndecided = 1, kRoot = 2, kNonroot = 0, kIsolated = 3;
 constexpr int kHash = 4096;        // shared hash-table slots per coarse row
 constexpr int kCoarseTarget = 512;  // stop coarsening at or below this many rows
 constexpr int kMaxLevels = 12;
-// Levels at or below this many stored entries (~7 MB in FP64, L2-resident)
-// may run in the cluster-resident tail (which must hold at least two levels);
-// the larger levels post-smooth through A P.
-constexpr int64_t kTailMaxNnz = 600000;
 static_assert(1 + kMaxLevels <= kChebSlots, "one Chebyshev slot per AMG level");
 
 }  // namespace sphrt
@@ -90,8 +87,13 @@ struct SphLevel {
   SrcList ap_seg_src;             // source: k < nnz (off-diagonal entry) or nnz + i (diagonal)
   int64_t *apg_ptr = nullptr;     // [nnz_c + nc + 1] next level's Galerkin sums over A P entries
   int32_t *apg_src = nullptr;     // (P^T (A P): each A P entry (i, K) adds to (agg[i], K))
-  double *ap_val = nullptr;     // [nnz_ap]
+  double *ap_val = nullptr;     // [nnz_ap], or in slice order [ap_sl.padded]
   float *ap_val32 = nullptr;
+  // A P in slices, where the operator is (ap_ptr and ap_col then only describe its
+  // rows): ap_pos is each operator entry's place within its row's A P entries
+  SlicedRowsData ap_sl;
+  uint16_t *ap_pos = nullptr;
+  int ap_most = 0;              // most A P entries of a row
   // finest level, mixed form with the V-cycle's CG product (fine_post_smooth = 0):
   // the CG's FP32 search direction p, its product q = B p and w = B z
   float *p32 = nullptr, *q32 = nullptr, *w32 = nullptr;
@@ -585,17 +587,13 @@ __global__ void convert_kernel(int64_t n, const S *in, D *out) {
 // ---------------------------------------------------------------------------
 // V-cycle kernels
 // ---------------------------------------------------------------------------
-// PRE: load the row operands before the row sums (coarse levels) or after
-// them (finest level), as in cheb_step_body.
-template <int W, int U, typename MT, typename VT, bool PRE>
-__device__ __forceinline__ void resid_level_body(const CsrView<MT> &A, const VT *r, const VT *z,
-                                                 VT *res, const Scalars *sc, int *wflag) {
+// One sweep, two names (finest level vs coarse levels in profiles); the coarse one
+// loads its row operands before the row sums, as in cheb_step_kernel.
+template <int W, int U, typename MT, typename VT>
+__global__ void __launch_bounds__(kBlock, kCoarseMinBlocks)
+    resid_level_kernel(CsrView<MT> A, const VT *r, const VT *z, VT *res, const Scalars *sc) {
   pdl_wait();
-  if (sc && sc->done) {
-    mark_work(wflag, 0);
-    return;
-  }
-  mark_work(wflag, 1);
+  if (sc && sc->done) return;
   const int own = tile_own_row<W>(threadIdx.x & 31);
   int64_t r0, r1;
   warp_rows<W>(A.n, r0, r1);
@@ -604,29 +602,28 @@ __device__ __forceinline__ void resid_level_body(const CsrView<MT> &A, const VT 
     const int64_t i = base + own;
     const bool active = own < rows;
     VT ri = VT(0), dg = VT(0), zi = VT(0);
-    auto operands = [&]() {
+    if (active) {
       ri = r[i];
       dg = (VT)A.diag[i];
       zi = z[i];
-    };
-    if (PRE && active) operands();
-    const VT s = tile_row_sums<W, U, MT, VT>(base, rows, A.ptr, A.col, A.val, z);
-    if (active) {
-      if (!PRE) operands();
-      res[i] = ri - fmadd(dg, zi, s);
     }
+    const VT s = tile_row_sums<W, U, MT, VT>(base, rows, A.ptr, A.col, A.val, z);
+    if (active) res[i] = ri - fmadd(dg, zi, s);
   }
 }
-// one body, two names: finest level vs coarse levels in profiles
-template <int W, int U, typename MT, typename VT>
-__global__ void __launch_bounds__(kBlock, kCoarseMinBlocks) resid_level_kernel(CsrView<MT> A, const VT *r, const VT *z, VT *res,
-                                   const Scalars *sc, int *wflag) {
-  resid_level_body<W, U, MT, VT, true>(A, r, z, res, sc, wflag);
-}
-template <int W, int U, typename MT, typename VT>
-__global__ void __launch_bounds__(kBlock, sweep_min_blocks(U)) fine_resid_level_kernel(CsrView<MT> A, const VT *r, const VT *z, VT *res,
-                                        const Scalars *sc, int *wflag) {
-  resid_level_body<W, U, MT, VT, false>(A, r, z, res, sc, wflag);
+template <typename Rows, typename VT>
+__global__ void __launch_bounds__(kBlock, Rows::kMinBlocks)
+    fine_resid_level_kernel(Rows A, const VT *r, const VT *z, VT *res, const Scalars *sc,
+                            int *wflag) {
+  pdl_wait();
+  if (sc && sc->done) {
+    mark_work(wflag, 0);
+    return;
+  }
+  mark_work(wflag, 1);
+  A.each(
+      z, [&](int64_t i) { return Ops3<VT>{r[i], (VT)A.A.diag[i], z[i]}; },
+      [&](int64_t i, VT s, const Ops3<VT> &o) { res[i] = o.a - fmadd(o.b, o.c, s); });
 }
 
 // Sum of res over the members [m0, m1) of an aggregate, in member order.
@@ -942,18 +939,49 @@ __global__ void ap_galerkin_target_kernel(int64_t n, const int64_t *ap_ptr, cons
   }
 }
 
+// The same targets for A P in slices: tgt is in slice order (padding stays -1).
+__global__ void ap_sliced_target_kernel(int64_t n, const int64_t *ap_ptr, const int32_t *ap_col,
+                                        SlicedRowsData ap, const int32_t *agg, int64_t nnz_c,
+                                        const int64_t *cptr, const int32_t *ccol, int32_t *tgt,
+                                        int *missing) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t I = agg[i];
+    if (I < 0) continue;
+    const int q0 = ap.place[i];
+    const int64_t k0 = ap.ptr[i / kBlock * kWarpsPerBlock + q0 / 32] + q0 % 32;
+    const int64_t b = ap_ptr[i], c0 = cptr[I], c1 = cptr[I + 1];
+    for (int64_t q = b; q < ap_ptr[i + 1]; ++q) {
+      const int32_t K = ap_col[q];
+      int64_t t = nnz_c + I;
+      if (K != I) {  // binary search in the sorted coarse row I
+        int64_t lo = c0, hi = c1;
+        while (lo < hi) {
+          const int64_t mid = (lo + hi) / 2;
+          if (ccol[mid] < K) lo = mid + 1; else hi = mid;
+        }
+        t = lo;
+        if (lo >= c1 || ccol[lo] != K) {
+          *missing = 1;
+          t = -1;
+        }
+      }
+      tgt[k0 + (q - b) * 32] = (int32_t)t;
+    }
+  }
+}
+
 // First post-smoothing step of a level with the prolongation folded in:
 // z = z_pre + P e_c, res2 = res - (A P) e_c (= r - A z), d = c2 D^{-1} res2
 // (step 0 from a nonzero guess), z_out = z + d.  z_out may be z_pre.
 // DOT (finest level, smoother degree 1, where this is the V-cycle's last
 // sweep): also the preconditioned inner product of DotFuse over the new z.
-template <int W, int U, typename MT, typename VT, bool PRE, bool DOT>
-__device__ __forceinline__ void post_ap_body(int64_t n, const int64_t *ap_ptr,
-                                             const int32_t *ap_col, const MT *ap_val,
-                                             const int32_t *agg, const VT *ec, const VT *z_pre,
-                                             const VT *res, const MT *invdiag, const ChebCoef *cf,
-                                             VT *d, VT *z_out, const Scalars *sc, int *wflag,
-                                             const DotFuse &df) {
+// Finest level (Rows over A P):
+template <typename Rows, typename VT, bool DOT>
+__global__ void __launch_bounds__(kBlock, Rows::kMinBlocks)
+    fine_post_ap_kernel(Rows A, const int32_t *agg, const VT *ec, const VT *z_pre, const VT *res,
+                        const VT *invdiag, const ChebCoef *cf, VT *d, VT *z_out,
+                        const Scalars *sc, int *wflag, const DotFuse df) {
   pdl_wait();
   if (sc && sc->done) {
     mark_work(wflag, 0);
@@ -961,41 +989,27 @@ __device__ __forceinline__ void post_ap_body(int64_t n, const int64_t *ap_ptr,
   }
   mark_work(wflag, 1);
   const VT c2 = (VT)cf->inv_theta;
-  const int own = tile_own_row<W>(threadIdx.x & 31);
-  int64_t r0, r1;
-  warp_rows<W>(n, r0, r1);
   double da = 0.0, db = 0.0;  // (r, z) and (r, z_old) partials (DOT)
-  for (int64_t base = r0; base < r1; base += 32) {
-    const int rows = (int)(r1 - base < 32 ? r1 - base : 32);
-    const int64_t i = base + own;
-    const bool active = own < rows;
-    VT zp = VT(0), rs = VT(0), idg = VT(0), pe = VT(0);
-    auto operands = [&]() {
-      zp = z_pre[i];
-      rs = res[i];
-      idg = (VT)invdiag[i];
-      const int32_t a = agg[i];
-      pe = a >= 0 ? ec[a] : VT(0);
-    };
-    if (PRE && active) operands();
-    const VT s = tile_row_sums<W, U, MT, VT>(base, rows, ap_ptr, ap_col, ap_val, ec);
-    if (active) {
-      if (!PRE) operands();
-      const VT zi = zp + pe;
-      const VT di = (c2 * idg) * (rs - s);
-      const VT zo = zi + di;
-      d[i] = di;
-      z_out[i] = zo;
-      if (DOT) {
-        const double ri = df.r[i], zn = (double)zo;
-        if (df.flex) {
-          if (!df.first) db += ri * df.z64[i];
-          df.z64[i] = zn;
+  A.each(
+      ec,
+      [&](int64_t i) {
+        const int32_t a = agg[i];
+        return Ops3<VT>{z_pre[i] + (a >= 0 ? ec[a] : VT(0)), c2 * invdiag[i], res[i]};
+      },
+      [&](int64_t i, VT s, const Ops3<VT> &o) {
+        const VT di = o.b * (o.c - s);
+        const VT zo = o.a + di;
+        d[i] = di;
+        z_out[i] = zo;
+        if (DOT) {
+          const double ri = df.r[i], zn = widen(zo);
+          if (df.flex) {
+            if (!df.first) db += ri * df.z64[i];
+            df.z64[i] = zn;
+          }
+          da += ri * zn;
         }
-        da += ri * zn;
-      }
-    }
-  }
+      });
   if (DOT) {
     __shared__ double sh[32];
     da = block_sum(da, sh);
@@ -1010,33 +1024,38 @@ __device__ __forceinline__ void post_ap_body(int64_t n, const int64_t *ap_ptr,
     }
   }
 }
-// the same sweep under two names: finest level / coarser levels in profiles
-template <int W, int U, typename MT, typename VT>
-__global__ void __launch_bounds__(kBlock, sweep_min_blocks(U))
-    fine_post_ap_kernel(int64_t n, const int64_t *ap_ptr, const int32_t *ap_col,
-                        const MT *ap_val, const int32_t *agg, const VT *ec, const VT *z_pre,
-                        const VT *res, const MT *invdiag, const ChebCoef *cf, VT *d, VT *z_out,
-                        const Scalars *sc, int *wflag) {
-  post_ap_body<W, U, MT, VT, false, false>(n, ap_ptr, ap_col, ap_val, agg, ec, z_pre, res,
-                                           invdiag, cf, d, z_out, sc, wflag, DotFuse{});
-}
-template <int W, int U, typename MT, typename VT>
-__global__ void __launch_bounds__(kBlock, sweep_min_blocks(U))
-    fine_post_ap_dot_kernel(int64_t n, const int64_t *ap_ptr, const int32_t *ap_col,
-                            const MT *ap_val, const int32_t *agg, const VT *ec, const VT *z_pre,
-                            const VT *res, const MT *invdiag, const ChebCoef *cf, VT *d,
-                            VT *z_out, const Scalars *sc, int *wflag, const DotFuse df) {
-  post_ap_body<W, U, MT, VT, false, true>(n, ap_ptr, ap_col, ap_val, agg, ec, z_pre, res, invdiag,
-                                          cf, d, z_out, sc, wflag, df);
-}
+// coarser levels (row operands before the row sums)
 template <int W, int U, typename MT, typename VT>
 __global__ void __launch_bounds__(kBlock, kCoarseMinBlocks)
     post_ap_kernel(int64_t n, const int64_t *ap_ptr, const int32_t *ap_col, const MT *ap_val,
                    const int32_t *agg, const VT *ec, const VT *z_pre, const VT *res,
-                   const MT *invdiag, const ChebCoef *cf, VT *d, VT *z_out, const Scalars *sc,
-                   int *wflag) {
-  post_ap_body<W, U, MT, VT, true, false>(n, ap_ptr, ap_col, ap_val, agg, ec, z_pre, res, invdiag,
-                                          cf, d, z_out, sc, wflag, DotFuse{});
+                   const MT *invdiag, const ChebCoef *cf, VT *d, VT *z_out, const Scalars *sc) {
+  pdl_wait();
+  if (sc && sc->done) return;
+  const VT c2 = (VT)cf->inv_theta;
+  const int own = tile_own_row<W>(threadIdx.x & 31);
+  int64_t r0, r1;
+  warp_rows<W>(n, r0, r1);
+  for (int64_t base = r0; base < r1; base += 32) {
+    const int rows = (int)(r1 - base < 32 ? r1 - base : 32);
+    const int64_t i = base + own;
+    const bool active = own < rows;
+    VT zp = VT(0), rs = VT(0), idg = VT(0), pe = VT(0);
+    if (active) {
+      zp = z_pre[i];
+      rs = res[i];
+      idg = (VT)invdiag[i];
+      const int32_t a = agg[i];
+      pe = a >= 0 ? ec[a] : VT(0);
+    }
+    const VT s = tile_row_sums<W, U, MT, VT>(base, rows, ap_ptr, ap_col, ap_val, ec);
+    if (active) {
+      const VT zi = zp + pe;
+      const VT di = (c2 * idg) * (rs - s);
+      d[i] = di;
+      z_out[i] = zi + di;
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1077,17 +1096,17 @@ __device__ __forceinline__ void fcg_scalars(const double (&o)[5], int first, Sca
 }
 
 // Row epilogue shared by the two forms of the last sweep: z and B z of row i
-// and the five inner-product partials.
+// and the five inner-product partials (zo, qo, po: the previous z, q, p).
 template <typename VT>
-__device__ __forceinline__ void fcg_row(int64_t i, VT zn, VT wn, const VT *r, VT *z, VT *w,
-                                        const VT *p, const VT *q, int first, double (&acc)[5]) {
-  const double ri = (double)r[i], zd = (double)zn, wd = (double)wn;
+__device__ __forceinline__ void fcg_row(int64_t i, VT zn, VT wn, VT r, VT zo, VT qo, VT po, VT *z,
+                                        VT *w, int first, double (&acc)[5]) {
+  const double ri = widen(r), zd = widen(zn), wd = widen(wn);
   acc[0] += ri * zd;
   acc[2] += zd * wd;
   if (!first) {
-    acc[1] += ri * (double)z[i];
-    acc[3] += zd * (double)q[i];
-    acc[4] += (double)p[i] * wd;
+    acc[1] += ri * widen(zo);
+    acc[3] += zd * widen(qo);
+    acc[4] += widen(po) * wd;
   }
   z[i] = zn;
   w[i] = wn;
@@ -1115,10 +1134,9 @@ template <typename VT>
 __host__ __device__ constexpr int fcg_min_blocks() {
   return sizeof(VT) == sizeof(float) ? 4 : 3;
 }
-template <int W, int U, typename MT, typename VT>
+template <typename Rows, typename VT>
 __global__ void __launch_bounds__(kBlock, fcg_min_blocks<VT>())
-    fine_ap_cg_kernel(int64_t n, const int64_t *ap_ptr, const int32_t *ap_col, const MT *ap_val,
-                      const int32_t *agg, const VT *ec, const VT *z_pre, const VT *res,
+    fine_ap_cg_kernel(Rows A, const int32_t *agg, const VT *ec, const VT *z_pre, const VT *res,
                       const VT *r, VT *z, VT *w, const VT *p, const VT *q, int first, Scalars *sc,
                       double *partials, int *wflag) {
   pdl_wait();
@@ -1127,22 +1145,19 @@ __global__ void __launch_bounds__(kBlock, fcg_min_blocks<VT>())
     return;
   }
   mark_work(wflag, 1);
-  const int own = tile_own_row<W>(threadIdx.x & 31);
-  int64_t r0, r1;
-  warp_rows<W>(n, r0, r1);
   double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  for (int64_t base = r0; base < r1; base += 32) {
-    const int rows = (int)(r1 - base < 32 ? r1 - base : 32);
-    const int64_t i = base + own;
-    const VT s = tile_row_sums<W, U, MT, VT>(base, rows, ap_ptr, ap_col, ap_val, ec);
-    if (own < rows) {
-      const int32_t a = agg[i];
-      const VT pe = a >= 0 ? ec[a] : VT(0);
-      const VT zn = z_pre[i] + pe;
-      const VT res2 = res[i] - s;
-      fcg_row<VT>(i, zn, r[i] - res2, r, z, w, p, q, first, acc);
-    }
-  }
+  A.each(
+      ec,
+      [&](int64_t i) {
+        const int32_t a = agg[i];
+        const VT pe = a >= 0 ? ec[a] : VT(0);
+        return Ops7<VT>{z_pre[i] + pe, res[i], r[i], first ? VT(0) : z[i],
+                        first ? VT(0) : q[i], first ? VT(0) : p[i]};
+      },
+      [&](int64_t i, VT s, const Ops7<VT> &o) {
+        const VT res2 = o.b - s;
+        fcg_row<VT>(i, o.a, o.c - res2, o.c, o.d, o.e, o.f, z, w, first, acc);
+      });
   fcg_reduce<VT>(acc, first, sc, partials);
 }
 
@@ -1179,7 +1194,8 @@ __global__ void __launch_bounds__(kBlock, fcg_min_blocks<VT>())
     const VT s = tile_row_sums<W, U, MT, VT>(base, rows, A.ptr, A.col, A.val, t);
     if (own < rows) {
       const VT ti = t[i];
-      fcg_row<VT>(i, ti, fmadd((VT)A.diag[i], ti, s), r, z, w, p, q, first, acc);
+      fcg_row<VT>(i, ti, fmadd((VT)A.diag[i], ti, s), r[i], first ? VT(0) : z[i],
+                  first ? VT(0) : q[i], first ? VT(0) : p[i], z, w, first, acc);
     }
   }
   fcg_reduce<VT>(acc, first, sc, partials);
@@ -1574,6 +1590,50 @@ static sph_rt_status level_vectors_fine(sph_rt *s, SphLevel *L) {
   return SPH_RT_OK;
 }
 
+__global__ void max_len_kernel(int64_t n, const int32_t *len, int *most) {
+  int m = 0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x)
+    m = max(m, len[i]);
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(most, m);
+}
+
+// Slices of the finest level's A P from its CSR rows.  *again: they have no
+// dictionary within the caps, and the fine operator is back in CSR rows; A P is
+// then to be built like a coarser level's.
+static void *take_level(sph_rt *s, void *L, size_t bytes) {
+  return lvl_alloc(s, static_cast<SphLevel *>(L), bytes);
+}
+static sph_rt_status build_ap_slices(sph_rt *s, SphLevel *L, bool *again) {
+  bool ok = false;
+  sph_rt_status rc = sliced_build(s, L->n, L->ap_ptr, L->ap_col, nullptr, take_level, L, &L->ap_sl,
+                                  nullptr, &ok);
+  if (rc) return rc;
+  int *most = scratch<int>(s, 1);
+  if (!most) return SPH_RT_ENOMEM;
+  SPH_CUDA(s, cudaMemsetAsync(most, 0, sizeof(int), s->stream));
+  if (ok) {
+    max_len_kernel<<<gcap(s, L->n, kBlock), kBlock, 0, s->stream>>>(L->n, L->ap_sl.len, most);
+    SPH_LAUNCHED(s);
+  }
+  SPH_CUDA(s, cudaMemcpyAsync(&L->ap_most, most, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+  SPH_CUDA(s, cudaStreamSynchronize(s->stream));
+  dfree(s, most);
+  if (!ok || L->ap_most >= kNoPlace) {
+    L->ap_sl = SlicedRowsData{};
+    L->ap_pos = nullptr;
+    *again = true;
+    return sliced_undo(s);
+  }
+  const size_t size = (size_t)L->ap_sl.padded + 1;
+  if (s->cfg.precision == SPH_RT_MIXED)
+    L->ap_val32 = lalloc<float>(s, L, size);
+  else
+    L->ap_val = lalloc<double>(s, L, size);
+  return L->ap_val || L->ap_val32 ? SPH_RT_OK : SPH_RT_ENOMEM;
+}
+
 // structure of A P on the finest level (see ap_structure_kernel)
 static sph_rt_status build_ap(sph_rt *s, size_t l) {
   SphLevel *L = s->levels[l];
@@ -1600,8 +1660,14 @@ static sph_rt_status build_ap(sph_rt *s, size_t l) {
                                                                       tmp, cnt, map, dmap);
     SPH_LAUNCHED(s);
   }
-  sph_rt_status rc = exclusive_scan(s, cnt, n, L->ap_ptr);
-  if (rc) return rc;
+  sph_rt_status rc;
+  const bool sliced = l == 0 && s->sl.ptr != nullptr;
+  if (sliced) {  // the relative places, before they are made absolute
+    L->ap_pos = lalloc<uint16_t>(s, L, (size_t)s->sl.padded + 1);
+    if (!L->ap_pos) return SPH_RT_ENOMEM;
+    if ((rc = sliced_places(s, map, L->ap_pos))) return rc;
+  }
+  if ((rc = exclusive_scan(s, cnt, n, L->ap_ptr))) return rc;
   int64_t total = 0;
   SPH_CUDA(s, cudaMemcpyAsync(&total, L->ap_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost,
                               s->stream));
@@ -1609,26 +1675,40 @@ static sph_rt_status build_ap(sph_rt *s, size_t l) {
   if (total >= ((int64_t)1 << 31)) return set_error(s, SPH_RT_EINVAL, "A P too large");
   L->nnz_ap = total;
   L->ap_col = lalloc<int32_t>(s, L, (size_t)total);
-  L->ap_val = lalloc<double>(s, L, (size_t)total);
-  if (!L->ap_col || !L->ap_val) return SPH_RT_ENOMEM;
-  if (s->cfg.precision == SPH_RT_MIXED && !(L->ap_val32 = lalloc<float>(s, L, (size_t)total)))
-    return SPH_RT_ENOMEM;
+  if (!L->ap_col) return SPH_RT_ENOMEM;
   ap_compact_kernel<<<gcap(s, n, kBlock), kBlock, 0, s->stream>>>(n, L->ptr, tmp, L->ap_ptr,
                                                                   L->ap_col, map, dmap);
   SPH_LAUNCHED(s);
-  // sources of each A P entry in increasing source order
-  if ((rc = source_sort(s, L, L->nnz + n, map, total, &L->ap_seg_ptr, &L->ap_seg_src)))
-    return rc;
-  // next level's Galerkin sources: the A P entries of its members' rows
+  bool again = false;
+  if (sliced && (rc = build_ap_slices(s, L, &again))) return rc;
+  if (!sliced || again) {
+    L->ap_val = lalloc<double>(s, L, (size_t)total);
+    if (!L->ap_val) return SPH_RT_ENOMEM;
+    if (s->cfg.precision == SPH_RT_MIXED && !(L->ap_val32 = lalloc<float>(s, L, (size_t)total)))
+      return SPH_RT_ENOMEM;
+    // sources of each A P entry in increasing source order
+    if ((rc = source_sort(s, L, L->nnz + n, map, total, &L->ap_seg_ptr, &L->ap_seg_src)))
+      return rc;
+  }
+  // next level's Galerkin sources: the A P entries of its members' rows, numbered
+  // as they are stored
   SphLevel *C = s->levels[l + 1];
-  int32_t *tgt = scratch<int32_t>(s, (size_t)total);
+  const int64_t stored = L->ap_sl.ptr ? L->ap_sl.padded : total;
+  int32_t *tgt = scratch<int32_t>(s, (size_t)stored + 1);
   int *missing = scratch<int>(s, 1);
   if (!tgt || !missing) return SPH_RT_ENOMEM;
   SPH_CUDA(s, cudaMemsetAsync(missing, 0, sizeof(int), s->stream));
-  ap_galerkin_target_kernel<<<gcap(s, n, kBlock), kBlock, 0, s->stream>>>(
-      n, L->ap_ptr, L->ap_col, L->agg, C->nnz, C->ptr, C->col, tgt, missing);
+  if (L->ap_sl.ptr) {
+    fill_i32_kernel<<<gcap(s, stored, kBlock), kBlock, 0, s->stream>>>(stored, -1, tgt);
+    SPH_LAUNCHED(s);
+    ap_sliced_target_kernel<<<gcap(s, n, kBlock), kBlock, 0, s->stream>>>(
+        n, L->ap_ptr, L->ap_col, L->ap_sl, L->agg, C->nnz, C->ptr, C->col, tgt, missing);
+  } else {
+    ap_galerkin_target_kernel<<<gcap(s, n, kBlock), kBlock, 0, s->stream>>>(
+        n, L->ap_ptr, L->ap_col, L->agg, C->nnz, C->ptr, C->col, tgt, missing);
+  }
   SPH_LAUNCHED(s);
-  if ((rc = bucket_sort<int32_t>(s, L, total, tgt, C->nnz + C->n, &L->apg_ptr, &L->apg_src,
+  if ((rc = bucket_sort<int32_t>(s, L, stored, tgt, C->nnz + C->n, &L->apg_ptr, &L->apg_src,
                                  nullptr)))
     return rc;
   int miss = 0;
@@ -1644,7 +1724,7 @@ static sph_rt_status build_ap(sph_rt *s, size_t l) {
   return SPH_RT_OK;
 }
 
-static sph_rt_status build_structure(sph_rt *s) {
+static sph_rt_status build_structure(sph_rt *s, double *csr) {
   amg_release(s);
   SphLevel *L0 = new SphLevel();
   CsrView<double> A = fine_view(s);
@@ -1652,7 +1732,7 @@ static sph_rt_status build_structure(sph_rt *s) {
   L0->nnz = A.nnz;
   L0->ptr = const_cast<int64_t *>(A.ptr);
   L0->col = const_cast<int32_t *>(A.col);
-  L0->val = const_cast<double *>(A.val);
+  L0->val = csr ? csr : const_cast<double *>(A.val);
   L0->diag = const_cast<double *>(A.diag);
   L0->invdiag = const_cast<double *>(A.invdiag);
   L0->W = A.W;
@@ -1749,7 +1829,7 @@ static sph_rt_status level_fp32(sph_rt *s, size_t l) {
   SphLevel *L = s->levels[l];
   if (L->r32) return SPH_RT_OK;
   if (l == 0) {
-    L->val32 = s->mat_val32;
+    L->val32 = s->mat_val32;  // none where the operator is in slices
     L->diag32 = s->diag32;
     L->invdiag32 = s->invdiag32;
   } else {
@@ -1762,7 +1842,7 @@ static sph_rt_status level_fp32(sph_rt *s, size_t l) {
   L->res32 = lalloc<float>(s, L, L->n);
   L->d32 = lalloc<float>(s, L, L->n);
   L->t32 = lalloc<float>(s, L, L->n);
-  if (!L->val32 || !L->diag32 || !L->invdiag32 || !L->r32 || !L->z32 || !L->res32 || !L->d32 ||
+  if ((!L->val32 && !(l == 0 && s->sl.ptr)) || !L->diag32 || !L->invdiag32 || !L->r32 || !L->z32 || !L->res32 || !L->d32 ||
       !L->t32)
     return SPH_RT_ENOMEM;
   return SPH_RT_OK;
@@ -1777,7 +1857,12 @@ static sph_rt_status galerkin_levels(sph_rt *s) {
   for (size_t l = 0; l + 1 < s->levels.size(); ++l) {
     SphLevel *L = s->levels[l], *C = s->levels[l + 1];
     const CsrView<T> Lv = LV::view(L), Cv = LV::view(C);
-    if (L->ap_ptr) {  // A P of this level (its values are final: level l is done)
+    if (L->ap_sl.ptr) {
+      const SlicedView<T> F = fine_sliced<T>(s);
+      sph_rt_status rc = sliced_ap_values<T>(s, L->ap_pos, L->agg, L->ap_sl, L->ap_most, F.val,
+                                             F.diag, const_cast<T *>(LV::ap(L)));
+      if (rc) return rc;
+    } else if (L->ap_ptr) {  // A P of this level (its values are final: level l is done)
       sph_rt_status rc = launch_galerkin<T>(s, L->nnz_ap, 0, L->ap_seg_ptr, L->ap_seg_src,
                                             L->nnz, Lv.val, Lv.diag, const_cast<T *>(LV::ap(L)),
                                             nullptr, nullptr);
@@ -1788,7 +1873,8 @@ static sph_rt_status galerkin_levels(sph_rt *s) {
     // P^T (A P): its sources are A P entries (fewer than 2^31)
     sph_rt_status rc =
         L->apg_ptr ? launch_galerkin<T>(s, C->nnz, C->n, L->apg_ptr, SrcList{L->apg_src, nullptr},
-                                        L->nnz_ap, LV::ap(L), nullptr, cval, cdiag, cinv)
+                                        L->ap_sl.ptr ? L->ap_sl.padded : L->nnz_ap, LV::ap(L),
+                                        nullptr, cval, cdiag, cinv)
                    : launch_galerkin<T>(s, C->nnz, C->n, L->seg_ptr, L->seg_src, L->nnz, Lv.val,
                                         Lv.diag, cval, cdiag, cinv);
     if (rc) return rc;
@@ -1852,7 +1938,10 @@ static void tail_setup(sph_rt *s);
 sph_rt_status amg_setup(sph_rt *s) {
   sph_rt_status rc;
   if (!s->amg_ready || s->cfg.amg_rebuild) {
-    if ((rc = build_structure(s))) return rc;
+    // the set-up reads the finest level's values in CSR order
+    double *csr = nullptr;
+    if (s->sl.ptr && (rc = sliced_to_csr(s, &csr))) return rc;
+    if ((rc = build_structure(s, csr))) return rc;
     if (s->cfg.precision == SPH_RT_MIXED)
       tail_setup<float>(s);
     else
@@ -1862,6 +1951,11 @@ sph_rt_status amg_setup(sph_rt *s) {
     // bitwise the same V-cycle
     for (size_t l = 0; l + 1 < s->levels.size() && s->levels[l]->nnz > kTailMaxNnz; ++l)
       if ((rc = build_ap(s, l))) return rc;
+    if (csr) {
+      SPH_CUDA(s, cudaStreamSynchronize(s->stream));
+      dfree(s, csr);
+      s->levels[0]->val = s->mat_val;  // none, unless A P took the slices back
+    }
   }
   return numeric(s);
 }
@@ -1869,6 +1963,35 @@ sph_rt_status amg_setup(sph_rt *s) {
 // ---------------------------------------------------------------------------
 // V-cycle
 // ---------------------------------------------------------------------------
+// Launch CALL over the rows of the finest level's A P, sliced or in CSR row tiles
+// of shape `sh` and CSR_BLOCKS_ blocks per SM (as SPH_FINE_ROWS).
+#define SPH_AP_ROWS(s_, L_, T_, CSR_BLOCKS_, CALL)                                         \
+  do {                                                                                     \
+    if ((L_)->ap_sl.ptr) {                                                                 \
+      using Rows = SlicedRows<T_>;                                                         \
+      const Rows rows{sliced_view<T_>((L_)->ap_sl, (L_)->n, (L_)->nnz_ap, LV::ap(L_),      \
+                                      nullptr, nullptr)};                                  \
+      const int grid = sliced_grid(                                                        \
+          s_, (L_)->n, (CSR_BLOCKS_) < Rows::kMinBlocks ? (CSR_BLOCKS_) : Rows::kMinBlocks); \
+      const size_t smem = (size_t)(L_)->ap_sl.dict_max * sizeof(T_);                       \
+      CALL;                                                                                \
+    } else {                                                                               \
+      CsrView<T_> apv;                                                                     \
+      apv.n = (L_)->n;                                                                     \
+      apv.ptr = (L_)->ap_ptr;                                                              \
+      apv.col = (L_)->ap_col;                                                              \
+      apv.val = LV::ap(L_);                                                                \
+      const size_t smem = 0;                                                               \
+      SPH_DISPATCH_SHAPE(sh.W, sh.U, ({                                                    \
+                           using Rows = CsrRows<W, U, T_>;                                 \
+                           const Rows rows{apv};                                           \
+                           const int grid =                                                \
+                               row_grid_blocks((s_)->num_sms, apv.n, W, CSR_BLOCKS_);      \
+                           CALL;                                                           \
+                         }));                                                              \
+    }                                                                                      \
+  } while (0)
+
 template <typename T>
 static sph_rt_status launch_tail(sph_rt *s, size_t l0, const T *r, T *z, const Scalars *sc) {
   using LV = LevelVecs<T>;
@@ -2004,23 +2127,22 @@ static sph_rt_status vcycle(sph_rt *s, size_t l, const T *r, T *z, const Scalars
   // when init_done)
   if ((rc = cheb_apply<T, T>(s, A, r, z, LV::d(L), LV::t(L), deg, cf, true, sc, init_done)))
     return rc;
-  const int gw = l == 0 ? row_grid(s->num_sms, L->n, A.W, A.U)
-                        : row_grid_blocks(s->num_sms, L->n, A.W, kCoarseMinBlocks);
+  const int gw = row_grid_blocks(s->num_sms, L->n, A.W, kCoarseMinBlocks);
   T *res = LV::res(L);
   // fine-level residual sweeps are timed with the other fine SpMV-class kernels;
   // per row: rowptr, diag, r, z, res
   int *wf = l == 0 ? timing_begin(s) : nullptr;
   if (l == 0)
-    SPH_DISPATCH_SHAPE(A.W, A.U,
-                       (pdl_launch(s, fine_resid_level_kernel<W, U, T, T>, gw, kBlock, 0,
-                           A, r, z, res, sc, wf)));
+    SPH_FINE_ROWS(s, T, A, sizeof(T),
+                  (pdl_launch(s, fine_resid_level_kernel<Rows, T>, grid, kBlock, smem, rows, r, z,
+                              res, sc, wf)));
   else
     SPH_DISPATCH_SHAPE(A.W, A.U,
                        (pdl_launch(s, resid_level_kernel<W, U, T, T>, gw, kBlock, 0, A, r, z, res,
-                                                                                      sc, wf)));
+                                   sc)));
   SPH_LAUNCHED(s);
   if (l == 0)
-    timing_end(s, (4.0 + sizeof(T)) * (double)A.nnz + (8.0 + 4.0 * sizeof(T)) * (double)A.n,
+    timing_end(s, ((s->sl.ptr ? 2.0 : 4.0) + sizeof(T)) * (double)A.nnz + (8.0 + 4.0 * sizeof(T)) * (double)A.n,
                kTimedResid);
   SphLevel *C = s->levels[l + 1];
   // a launched, non-coarsest next level takes its smoother start from the restriction
@@ -2043,34 +2165,35 @@ static sph_rt_status vcycle(sph_rt *s, size_t l, const T *r, T *z, const Scalars
     T *bufs[2] = {z, LV::t(L)};
     const int w0 = (deg - 1) % 2;
     const RowShape sh = shape_for_mean(L->n ? (double)L->nnz_ap / (double)L->n : 0.0);
-    const int gp = l == 0 ? row_grid(s->num_sms, L->n, sh.W, sh.U)
-                          : row_grid_blocks(s->num_sms, L->n, sh.W, kCoarseMinBlocks);
     int *wf = l == 0 ? timing_begin(s) : nullptr;
     // with degree 1 this sweep is the V-cycle's last: the inner product rides along
     const bool dot = l == 0 && df && dot_done && deg == 1;
     if (dot) {
-      SPH_DISPATCH_SHAPE(sh.W, sh.U,
-                         (pdl_launch(s, fine_post_ap_dot_kernel<W, U, T, T>, gp, kBlock, 0,
-                             L->n, L->ap_ptr, L->ap_col, LV::ap(L), L->agg, LV::z(C), z, res,
-                             A.invdiag, cf, LV::d(L), bufs[w0], sc, wf, *df)));
+      SPH_AP_ROWS(s, L, T, sweep_min_blocks(sh.U),
+                  (pdl_launch(s, fine_post_ap_kernel<Rows, T, true>, grid, kBlock, smem, rows,
+                              (const int32_t *)L->agg, (const T *)LV::z(C), (const T *)z,
+                              (const T *)res, A.invdiag, cf, LV::d(L), bufs[w0], sc, wf, *df)));
       *dot_done = true;
-    } else if (l == 0)
-      SPH_DISPATCH_SHAPE(sh.W, sh.U,
-                         (pdl_launch(s, fine_post_ap_kernel<W, U, T, T>, gp, kBlock, 0,
-                             L->n, L->ap_ptr, L->ap_col, LV::ap(L), L->agg, LV::z(C), z, res,
-                             A.invdiag, cf, LV::d(L), bufs[w0], sc, wf)));
-    else
+    } else if (l == 0) {
+      SPH_AP_ROWS(s, L, T, sweep_min_blocks(sh.U),
+                  (pdl_launch(s, fine_post_ap_kernel<Rows, T, false>, grid, kBlock, smem, rows,
+                              (const int32_t *)L->agg, (const T *)LV::z(C), (const T *)z,
+                              (const T *)res, A.invdiag, cf, LV::d(L), bufs[w0], sc, wf,
+                              DotFuse{})));
+    } else {
+      const int gp = row_grid_blocks(s->num_sms, L->n, sh.W, kCoarseMinBlocks);
       SPH_DISPATCH_SHAPE(sh.W, sh.U,
                          (pdl_launch(s, post_ap_kernel<W, U, T, T>, gp, kBlock, 0,
                              L->n, L->ap_ptr, L->ap_col, LV::ap(L), L->agg, LV::z(C), z, res,
-                             A.invdiag, cf, LV::d(L), bufs[w0], sc, nullptr)));
+                             A.invdiag, cf, LV::d(L), bufs[w0], sc)));
+    }
     SPH_LAUNCHED(s);
     // A P entry: column + value; per row: ap_ptr, agg, the coarse entry of P e_c,
     // z_pre, res, 1/diag, d, z_out; with the inner product also r (and, flexible,
     // the FP64 z read and written)
     if (l == 0)
       timing_end(s,
-                 (4.0 + sizeof(T)) * (double)L->nnz_ap +
+                 ((L->ap_sl.ptr ? 2.0 : 4.0) + sizeof(T)) * (double)L->nnz_ap +
                      (12.0 + 6.0 * sizeof(T) + (dot ? (df->flex ? 24.0 : 8.0) : 0.0)) *
                          (double)L->n,
                  kTimedPost);
@@ -2172,13 +2295,12 @@ static sph_rt_status fcg_cycle_t(sph_rt *s, const FcgSet<T> &v, int first) {
   CsrView<T> A = LV::view(L);
   const Scalars *sc = s->sc;
   T *res = LV::res(L);
-  const int gw = row_grid(s->num_sms, L->n, A.W, A.U);
   int *wf = timing_begin(s);
-  SPH_DISPATCH_SHAPE(A.W, A.U,
-                     (pdl_launch(s, fine_resid_level_kernel<W, U, T, T>, gw, kBlock, 0, A, v.r,
-                                 v.zpre, res, sc, wf)));
+  SPH_FINE_ROWS(s, T, A, sizeof(T),
+                (pdl_launch(s, fine_resid_level_kernel<Rows, T>, grid, kBlock, smem, rows,
+                            (const T *)v.r, (const T *)v.zpre, res, sc, wf)));
   SPH_LAUNCHED(s);
-  timing_end(s, (4.0 + sizeof(T)) * (double)A.nnz + (8.0 + 4.0 * sizeof(T)) * (double)A.n,
+  timing_end(s, ((s->sl.ptr ? 2.0 : 4.0) + sizeof(T)) * (double)A.nnz + (8.0 + 4.0 * sizeof(T)) * (double)A.n,
              kTimedResid);
   SphLevel *C = s->levels[1];
   const int deg = s->cfg.cheb_degree;
@@ -2198,18 +2320,17 @@ static sph_rt_status fcg_cycle_t(sph_rt *s, const FcgSet<T> &v, int first) {
   if (rc) return rc;
   if (L->ap_ptr && LV::ap(L)) {
     const RowShape sh = shape_for_mean(L->n ? (double)L->nnz_ap / (double)L->n : 0.0);
-    const int gp = row_grid_blocks(s->num_sms, L->n, sh.W, fcg_min_blocks<T>());
     wf = timing_begin(s);
-    SPH_DISPATCH_SHAPE(sh.W, sh.U,
-                       (pdl_launch(s, fine_ap_cg_kernel<W, U, T, T>, gp, kBlock, 0, L->n,
-                                   L->ap_ptr, L->ap_col, LV::ap(L), L->agg, (const T *)LV::z(C),
-                                   (const T *)v.zpre, (const T *)res, (const T *)v.r, v.z, v.w,
-                                   (const T *)v.p, (const T *)v.q, first, s->sc, s->partials,
-                                   wf)));
+    SPH_AP_ROWS(s, L, T, fcg_min_blocks<T>(),
+                (pdl_launch(s, fine_ap_cg_kernel<Rows, T>, grid, kBlock, smem, rows,
+                            (const int32_t *)L->agg, (const T *)LV::z(C), (const T *)v.zpre,
+                            (const T *)res, (const T *)v.r, v.z, v.w, (const T *)v.p,
+                            (const T *)v.q, first, s->sc, s->partials, wf)));
     SPH_LAUNCHED(s);
     // A P entry: column + value; per row: ap_ptr, agg, P e_c, z_pre, res, r, z r/w, w,
     // p, q
-    timing_end(s, (4.0 + sizeof(T)) * (double)L->nnz_ap + (12.0 + 10.0 * sizeof(T)) * (double)L->n,
+    timing_end(s, ((L->ap_sl.ptr ? 2.0 : 4.0) + sizeof(T)) * (double)L->nnz_ap +
+                      (12.0 + 10.0 * sizeof(T)) * (double)L->n,
                kTimedPost);
     return SPH_RT_OK;
   }
@@ -2269,7 +2390,13 @@ void amg_signature(const sph_rt *s, std::vector<uint64_t> &sig) {
                           (uint64_t)(uintptr_t)L->ap_ptr,
                           (uint64_t)(uintptr_t)L->ap_col,
                           (uint64_t)(uintptr_t)L->ap_val,
-                          (uint64_t)(uintptr_t)L->ap_val32};
+                          (uint64_t)(uintptr_t)L->ap_val32,
+                          (uint64_t)(uintptr_t)L->ap_sl.ptr,
+                          (uint64_t)(uintptr_t)L->ap_sl.idx,
+                          (uint64_t)(uintptr_t)L->ap_sl.dict,
+                          (uint64_t)(uintptr_t)L->ap_sl.dptr,
+                          (uint64_t)(uintptr_t)L->ap_sl.len,
+                          (uint64_t)L->ap_sl.dict_max};
     sig.insert(sig.end(), v, v + sizeof v / sizeof v[0]);
   }
 }

@@ -201,6 +201,40 @@ __host__ __device__ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + 
 __device__ __forceinline__ double fmadd(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float fmadd(float a, float b, float c) { return fmaf(a, b, c); }
 
+// FP32 <-> FP64 conversions on the integer pipe, with the results of the
+// conversion instructions (round to nearest even when narrowing).  On GB300 the
+// instructions run on the FP64 pipe, which issues one warp instruction in ~16
+// cycles per SM; the ~6-9 integer instructions take a third of that.  Zeros,
+// subnormals, infinities, NaN and narrowed values outside FP32's normal range take
+// the instruction.
+__device__ __forceinline__ double widen(float v) {
+  const uint32_t u = __float_as_uint(v), e = (u >> 23) & 0xffu;
+  if (e - 1u < 254u)  // normal: rebias the exponent by 1023 - 127, shift the fraction
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)),
+                            (int)(u << 29));
+  return (double)v;
+}
+__device__ __forceinline__ double widen(double v) { return v; }
+// narrow_ok: 2^-126 <= |v| < 2^127, where narrow_fast is exact.
+__device__ __forceinline__ bool narrow_ok(double v) {
+  return (((uint32_t)__double2hiint(v) >> 20) & 0x7ffu) - 897u < 253u;
+}
+__device__ __forceinline__ float narrow_fast(double v) {
+  // round the fraction to 23 bits, ties to even (a carry into the exponent is the
+  // right result), then rebias
+  const unsigned long long x = (unsigned long long)__double_as_longlong(v);
+  const unsigned long long r = x + 0x0fffffffull + ((x >> 29) & 1ull);
+  return __uint_as_float(((uint32_t)(x >> 32) & 0x80000000u) | ((uint32_t)(r >> 29) - 0xc0000000u));
+}
+template <typename T>
+__device__ __forceinline__ T narrow(double v);
+template <>
+__device__ __forceinline__ double narrow<double>(double v) { return v; }
+template <>
+__device__ __forceinline__ float narrow<float>(double v) {
+  return narrow_ok(v) ? narrow_fast(v) : (float)v;
+}
+
 template <int W, int U, typename MT, typename VT>
 __device__ __forceinline__ VT row_dot(int64_t beg, int64_t end, const int32_t *__restrict__ col,
                                       const MT *__restrict__ val, const VT *__restrict__ x,
@@ -574,12 +608,157 @@ struct CsrView {
   int U = 4;
 };
 
+// ---------------------------------------------------------------------------
+// Sliced operators: the layout of the finest level's sweeps on large particle
+// sets (sliced.cu builds it from the CSR rows; sliced_wanted says when).
+//
+// Rows are cut into groups of kBlock (one thread block's), sorted by length
+// within the group (order: the row of each place) and cut into slices of 32
+// (one warp's).  Entry t of the row of lane l of slice s stands at ptr[s] + 32 t
+// + l, so a warp's loads are whole lines and a thread sums one row in list order,
+// with no reduction across lanes; the sorting (by eighths of the length, so that
+// most neighbouring rows stay together) keeps a warp's rows of nearly one length
+// (unsorted, the longest of 32 rows is 13 % over the mean at 64^3, and an FP64
+// instruction costs all 32 lanes).  Columns are 16-bit places in the group's
+// dictionary, the sorted list of its distinct columns (neighbours of Morton-
+// consecutive particles are few: ~7 per row for a group of 256 rows of ~104
+// entries): a group stages x at its dictionary's columns in shared memory, one
+// coalesced pass, and gathers from there.
+//
+// What it buys over the CSR row tiles: 2 instead of 4 bytes of column per entry
+// (6 instead of 8 bytes in FP32, 10 instead of 12 in FP64), one line per warp
+// load instead of 8 sectors, and gathers that do not go through the L1 tags,
+// which bound the FP32 sweeps.  V-cycle residual at 128^3 in FP32: 0.38 -> 0.24 ms
+// (5.9 TB/s of the bytes it must move); FP64 sweeps stay FP64-bound (one
+// multiply-add per entry): 0.21 -> 0.18 ms at 97 x 96 x 91.
+// ---------------------------------------------------------------------------
+template <typename T>
+struct SlicedView {
+  int64_t n = 0;
+  const int64_t *ptr = nullptr;    // [slices + 1] first entry of each slice (multiples of 32)
+  const uint16_t *idx = nullptr;   // place in the group's dictionary
+  const T *val = nullptr;
+  const int32_t *len = nullptr;    // [n] entries of the row of each place
+  const uint8_t *order = nullptr;  // [n] row within the group of each place
+  const int64_t *dptr = nullptr;   // [groups + 1]
+  const int32_t *dict = nullptr;   // columns, ascending within a group
+  const T *diag = nullptr;
+  const T *invdiag = nullptr;
+  int64_t nnz = 0;     // entries without the padding
+  int dict_max = 0;    // largest dictionary
+};
+
+// Row sources of the finest level's sweeps: each(x, pre, f) calls f(i, s, o) for
+// every row i with s its off-diagonal sum over x and o = pre(i) its operands;
+// every thread of the block takes part.  Sliced rows load the operands before the
+// sums, so that their latency passes behind the staging of x; the row tiles after
+// them (fewer registers, more warps).
+template <int W_, int U_, typename MT>
+struct CsrRows {
+  static constexpr int W = W_, U = U_, kMinBlocks = sweep_min_blocks(U_);
+  CsrView<MT> A;
+  template <typename VT, typename P, typename F>
+  __device__ __forceinline__ void each(const VT *x, const P &pre, const F &f) const {
+    const int own = tile_own_row<W>(threadIdx.x & 31);
+    int64_t r0, r1;
+    warp_rows<W>(A.n, r0, r1);
+    for (int64_t base = r0; base < r1; base += 32) {
+      const int rows = (int)(r1 - base < 32 ? r1 - base : 32);
+      const VT s = tile_row_sums<W, U, MT, VT>(base, rows, A.ptr, A.col, A.val, x);
+      if (own < rows) f(base + own, s, pre(base + own));
+    }
+  }
+};
+
+constexpr int kSliceU = 8;  // entries in flight per thread
+// operands of a row
+template <typename T>
+struct Ops1 { T a; };
+template <typename T>
+struct Ops2 { T a, b; };
+template <typename T>
+struct Ops3 { T a, b, c; };
+template <typename T>
+struct Ops4 { T a, b, c, d; };
+template <typename T>
+struct Ops7 { T a, b, c, d, e, f, g; };
+template <typename MT>
+struct SlicedRows {
+  // FP32 sweeps are bound by HBM and load latency (more warps), FP64 ones by the
+  // FP64 pipe (registers for the operands)
+  static constexpr int kMinBlocks = sizeof(MT) == sizeof(float) ? 5 : 4;
+  SlicedView<MT> A;
+  // dictionary places and values of one batch, then their products in order
+  template <typename VT>
+  __device__ __forceinline__ VT row_sum(int64_t slice, int len, const VT *xs) const {
+    const int64_t k0 = A.ptr[slice] + (threadIdx.x & 31);
+    const int width = __reduce_max_sync(0xffffffffu, len);
+    VT s = VT(0);
+    int c[kSliceU];
+    MT v[kSliceU];
+    auto load = [&](int t) {
+#pragma unroll
+      for (int u = 0; u < kSliceU; ++u) {
+        const int64_t k = k0 + (int64_t)(t + u) * 32;
+        const bool in = t + u < len;
+        c[u] = in ? (int)__ldg(A.idx + k) : 0;
+        v[u] = in ? __ldg(A.val + k) : MT(0);
+      }
+    };
+    int t = 0;
+    for (; t + kSliceU <= width; t += kSliceU) {
+      load(t);
+#pragma unroll
+      for (int u = 0; u < kSliceU; ++u) s = fmadd((VT)v[u], xs[c[u]], s);
+    }
+    if (t < width) {  // as many products as the longest row has left
+      load(t);
+#pragma unroll
+      for (int u = 0; u < kSliceU - 1; ++u)
+        if (t + u < width) s = fmadd((VT)v[u], xs[c[u]], s);
+    }
+    return s;
+  }
+  template <typename VT, typename P, typename F>
+  __device__ __forceinline__ void each(const VT *x, const P &pre, const F &f) const {
+    extern __shared__ __align__(16) unsigned char slice_smem[];
+    VT *xs = reinterpret_cast<VT *>(slice_smem);
+    __shared__ VT sums[kBlock];  // the rows' sums in row order, for the epilogue
+    const int64_t groups = (A.n + kBlock - 1) / kBlock;
+    for (int64_t g = blockIdx.x; g < groups; g += gridDim.x) {
+      const int64_t d0 = A.dptr[g];
+      const int nd = (int)(A.dptr[g + 1] - d0);
+      const int64_t i = g * kBlock + threadIdx.x;
+      const auto ops = pre(i < A.n ? i : A.n - 1);
+      for (int t = threadIdx.x; t < nd; t += kBlock) xs[t] = __ldg(x + __ldg(A.dict + d0 + t));
+      __syncthreads();
+      const int64_t slice = i >> 5;
+      if (slice * 32 < A.n) {  // warp-uniform
+        const VT s = row_sum<VT>(slice, i < A.n ? A.len[i] : 0, xs);
+        if (i < A.n) sums[A.order[i]] = s;
+      }
+      __syncthreads();  // also: xs may be staged again
+      if (i < A.n) f(i, sums[threadIdx.x], ops);
+    }
+  }
+};
+
 }  // namespace sphrt
 
 // --------------------------------------------------------------------------
 // Internal handle.
 // --------------------------------------------------------------------------
 struct SphLevel;  // AMG level (amg.cu)
+
+// Buffers of a sliced operator's structure (see SlicedView).
+struct SlicedRowsData {
+  int64_t *ptr = nullptr, *dptr = nullptr;
+  uint16_t *idx = nullptr;
+  int32_t *len = nullptr, *dict = nullptr;
+  uint8_t *order = nullptr, *place = nullptr;  // row of each place, place of each row
+  int64_t padded = 0;  // entries with the padding
+  int dict_max = 0;
+};
 
 struct sph_rt {
   sph_rt_config cfg;
@@ -627,6 +806,12 @@ struct sph_rt {
   float *mat_val32 = nullptr;  // FP32 copy for the mixed form (written by the assembly)
   float *diag32 = nullptr, *invdiag32 = nullptr;
   double *diag = nullptr, *invdiag = nullptr;
+  // the same operator in slices (sl.ptr == nullptr: not built, the CSR values above
+  // are in use; otherwise mat_G, mat_val and mat_val32 are not)
+  SlicedRowsData sl;
+  double *sl_G = nullptr, *sl_val = nullptr;
+  float *sl_val32 = nullptr;
+  bool sl_refused = false;  // a group's dictionary was too large for this particle set
   int64_t *gh_ptr = nullptr;   // Dirichlet-ghost couplings
   int32_t *gh_slot = nullptr;
   double *gh_W = nullptr;      // V_j F_ij

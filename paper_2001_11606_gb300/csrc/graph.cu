@@ -172,7 +172,9 @@ static std::vector<uint64_t> loop_signature(const sph_rt *s, double dt) {
   const void *bufs[] = {s->b,     s->x,     s->r,    s->z,     s->z_old, s->p,      s->q,
                         s->w,     s->tmp_n2, s->invV, s->sc,   s->partials, s->e_l, s->e_new,
                         s->E_l,   s->E_old, s->e_old, s->rho, s->sigma, s->f,       s->Qe,
-                        s->QE,    s->gb,    s->V,     s->cheb_slots};
+                        s->QE,    s->gb,    s->V,     s->cheb_slots, s->sl.ptr, s->sl.idx,
+                        s->sl.len, s->sl.order, s->sl.dptr, s->sl.dict, s->sl_val, s->sl_val32, s->diag,
+                        s->invdiag, s->diag32, s->invdiag32};
   sig_u64(v, bufs, sizeof bufs);
   CsrView<double> A = fine_view(s);
   sig_u64(v, &A, sizeof A);

@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "sliced.cuh"
 
 namespace sphrt {
 
@@ -38,28 +39,21 @@ __device__ __forceinline__ T ld(const T *p) {
 // ---------------------------------------------------------------------------
 // r = b - B x;  rnorm2 = ||r / V||^2;  done = rnorm2 <= thresh2.
 // ---------------------------------------------------------------------------
-template <int W, int U>
-__global__ void __launch_bounds__(kBlock, sweep_min_blocks(U)) resid_kernel(CsrView<double> A, const double *b, const double *x, double *r,
-                             const double *invV, Scalars *sc, double *partials, int *wflag) {
+template <typename Rows>
+__global__ void __launch_bounds__(kBlock, Rows::kMinBlocks)
+    resid_kernel(Rows A, const double *b, const double *x, double *r, const double *invV,
+                 Scalars *sc, double *partials, int *wflag) {
   pdl_wait();
   mark_work(wflag, 1);
-  const int own = tile_own_row<W>(threadIdx.x & 31);
-  int64_t r0, r1;
-  warp_rows<W>(A.n, r0, r1);
   double acc = 0.0;
-  for (int64_t base = r0; base < r1; base += 32) {
-    const int rows = (int)(r1 - base < 32 ? r1 - base : 32);
-    const int64_t i = base + own;
-    const bool active = own < rows;
-    const double s = tile_row_sums<W, U, double, double>(base, rows, A.ptr, A.col, A.val, x);
-    if (active) {
-      const double bi = b[i], dg = A.diag[i], xi = x[i], iv = invV[i];
-      double ri = bi - fmadd(dg, xi, s);
-      r[i] = ri;
-      double ru = ri * iv;
-      acc += ru * ru;
-    }
-  }
+  A.each(
+      x, [&](int64_t i) { return Ops4<double>{b[i], A.A.diag[i], x[i], invV[i]}; },
+      [&](int64_t i, double s, const Ops4<double> &o) {
+        const double ri = o.a - fmadd(o.b, o.c, s);
+        r[i] = ri;
+        const double ru = ri * o.d;
+        acc += ru * ru;
+      });
   __shared__ double sh[32];
   acc = block_sum(acc, sh);
   double part[1] = {acc}, out[1];
@@ -76,9 +70,10 @@ __global__ void __launch_bounds__(kBlock, sweep_min_blocks(U)) resid_kernel(CsrV
 // w = B z;  q = w + beta q;  p = z + beta p;  pq = (p, q);  alpha = rho / pq.
 // (q = B p without a second SpMV: B p = B z + beta B p_old.)
 // ---------------------------------------------------------------------------
-template <int W, int U>
-__global__ void __launch_bounds__(kBlock, sweep_min_blocks(U)) spmv_pq_kernel(CsrView<double> A, const double *z, double *q, double *p, int first,
-                               Scalars *sc, double *partials, int *wflag) {
+template <typename Rows>
+__global__ void __launch_bounds__(kBlock, Rows::kMinBlocks)
+    spmv_pq_kernel(Rows A, const double *z, double *q, double *p, int first, Scalars *sc,
+                   double *partials, int *wflag) {
   pdl_wait();
   if (sc->done) {
     mark_work(wflag, 0);
@@ -86,26 +81,20 @@ __global__ void __launch_bounds__(kBlock, sweep_min_blocks(U)) spmv_pq_kernel(Cs
   }
   mark_work(wflag, 1);
   const double beta = first ? 0.0 : sc->beta;
-  const int own = tile_own_row<W>(threadIdx.x & 31);
-  int64_t r0, r1;
-  warp_rows<W>(A.n, r0, r1);
   double acc = 0.0;
-  for (int64_t base = r0; base < r1; base += 32) {
-    const int rows = (int)(r1 - base < 32 ? r1 - base : 32);
-    const int64_t i = base + own;
-    const bool active = own < rows;
-    const double s = tile_row_sums<W, U, double, double>(base, rows, A.ptr, A.col, A.val, z);
-    if (active) {
-      const double zi = z[i], dg = A.diag[i];
-      const double qo = first ? 0.0 : q[i], po = first ? 0.0 : p[i];
-      double wi = fmadd(dg, zi, s);
-      double qi = first ? wi : fmadd(beta, qo, wi);
-      double pi = first ? zi : fmadd(beta, po, zi);
-      q[i] = qi;
-      p[i] = pi;
-      acc += pi * qi;
-    }
-  }
+  A.each(
+      z,
+      [&](int64_t i) {
+        return Ops4<double>{z[i], A.A.diag[i], first ? 0.0 : q[i], first ? 0.0 : p[i]};
+      },
+      [&](int64_t i, double s, const Ops4<double> &o) {
+        const double wi = fmadd(o.b, o.a, s);
+        const double qi = first ? wi : fmadd(beta, o.c, wi);
+        const double pi = first ? o.a : fmadd(beta, o.d, o.a);
+        q[i] = qi;
+        p[i] = pi;
+        acc += pi * qi;
+      });
   __shared__ double sh[32];
   acc = block_sum(acc, sh);
   double part[1] = {acc}, out[1];
@@ -283,18 +272,16 @@ __global__ void cheb_init_zero_kernel(int64_t n, const VT *r, const MT *invdiag,
 }
 
 
-// PRE: load the row operands before the row sums (coarse levels: shorter
-// dependent chain) or after them (finest level: fewer registers, more warps).
-template <int W, int U, typename MT, typename VT, bool PRE>
-__device__ __forceinline__ void cheb_step_body(const CsrView<MT> &A, const VT *r, const VT *z_in,
-                                               VT *z_out, VT *d, const ChebCoef *cf, int k,
-                                               const Scalars *sc, int *wflag) {
+// The same sweep under two names, so that profiles separate the finest level
+// (HBM-streamed operator) from the coarse levels (L2-resident).  The coarse one
+// loads its row operands before the row sums (a shorter dependent chain), the
+// fine one after them (fewer registers, more warps).
+template <int W, int U, typename MT, typename VT>
+__global__ void __launch_bounds__(kBlock, kCoarseMinBlocks)
+    cheb_step_kernel(CsrView<MT> A, const VT *r, const VT *z_in, VT *z_out, VT *d,
+                     const ChebCoef *cf, int k, const Scalars *sc) {
   pdl_wait();
-  if (sc && sc->done) {
-    mark_work(wflag, 0);
-    return;
-  }
-  mark_work(wflag, 1);
+  if (sc && sc->done) return;
   // step k of the recurrence; k = 0 is the first step from a nonzero guess
   const double c1 = k > 0 ? cf->c1[k] : 0.0, c2 = k > 0 ? cf->c2[k] : cf->inv_theta;
   const VT vc1 = (VT)c1, vc2 = (VT)c2;
@@ -306,18 +293,16 @@ __device__ __forceinline__ void cheb_step_body(const CsrView<MT> &A, const VT *r
     const int64_t i = base + own;
     const bool active = own < rows;
     VT ri = VT(0), zi = VT(0), dg = VT(0), idg = VT(0), dold = VT(0);
-    auto operands = [&]() {
+    if (active) {
       ri = r[i];
       zi = z_in[i];
       dg = (VT)A.diag[i];
       idg = (VT)A.invdiag[i];
       if (k > 0) dold = d[i];  // the first step must not read d
-    };
-    if (PRE && active) operands();
+    }
     const VT s = tile_row_sums<W, U, MT, VT>(base, rows, A.ptr, A.col, A.val, z_in);
     if (active) {
-      if (!PRE) operands();
-      VT res = ri - fmadd(dg, zi, s);
+      const VT res = ri - fmadd(dg, zi, s);
       VT di = (vc2 * idg) * res;
       if (k > 0) di = fmadd(vc1, dold, di);
       d[i] = di;
@@ -325,18 +310,32 @@ __device__ __forceinline__ void cheb_step_body(const CsrView<MT> &A, const VT *r
     }
   }
 }
-// The same sweep under two names, so that profiles separate the finest
-// level (HBM-streamed operator) from the coarse levels (L2-resident).
-template <int W, int U, typename MT, typename VT>
-__global__ void __launch_bounds__(kBlock, kCoarseMinBlocks) cheb_step_kernel(CsrView<MT> A, const VT *r, const VT *z_in, VT *z_out, VT *d,
-                                 const ChebCoef *cf, int k, const Scalars *sc, int *wflag) {
-  cheb_step_body<W, U, MT, VT, true>(A, r, z_in, z_out, d, cf, k, sc, wflag);
-}
-template <int W, int U, typename MT, typename VT>
-__global__ void __launch_bounds__(kBlock, sweep_min_blocks(U)) fine_cheb_step_kernel(CsrView<MT> A, const VT *r, const VT *z_in, VT *z_out,
-                                      VT *d, const ChebCoef *cf, int k, const Scalars *sc,
-                                      int *wflag) {
-  cheb_step_body<W, U, MT, VT, false>(A, r, z_in, z_out, d, cf, k, sc, wflag);
+template <typename Rows, typename VT>
+__global__ void __launch_bounds__(kBlock, Rows::kMinBlocks)
+    fine_cheb_step_kernel(Rows A, const VT *r, const VT *z_in, VT *z_out, VT *d,
+                          const ChebCoef *cf, int k, const Scalars *sc, int *wflag) {
+  pdl_wait();
+  if (sc && sc->done) {
+    mark_work(wflag, 0);
+    return;
+  }
+  mark_work(wflag, 1);
+  const double c1 = k > 0 ? cf->c1[k] : 0.0, c2 = k > 0 ? cf->c2[k] : cf->inv_theta;
+  const VT vc1 = (VT)c1, vc2 = (VT)c2;
+  A.each(
+      z_in,
+      [&](int64_t i) {
+        // the first step must not read d
+        return Ops7<VT>{z_in[i], r[i], (VT)A.A.diag[i], (VT)A.A.invdiag[i],
+                        k > 0 ? d[i] : VT(0)};
+      },
+      [&](int64_t i, VT s, const Ops7<VT> &o) {
+        const VT res = o.b - fmadd(o.c, o.a, s);
+        VT di = (vc2 * o.d) * res;
+        if (k > 0) di = fmadd(vc1, o.e, di);
+        d[i] = di;
+        z_out[i] = o.a + di;
+      });
 }
 
 // ---------------------------------------------------------------------------
@@ -415,12 +414,12 @@ void timing_end(sph_rt *s, double bytes, int kind) {
   cudaEventRecord(s->ev_pool[s->ev_used++], s->stream);
 }
 
-// Algorithmic bytes of the SpMV-class kernels: column index and value per
-// stored nonzero (the gathered vector entry counted once, per row) plus the
-// per-row vectors each kernel reads and writes.
+// Algorithmic bytes of the fine SpMV-class kernels: column (4 bytes, or a 2-byte
+// dictionary place) and value per stored nonzero (the gathered vector entry
+// counted once, per row) plus the per-row vectors each kernel reads and writes.
 template <typename MT>
-double spmv_class_bytes(const CsrView<MT> &A, int row_bytes) {
-  return (4.0 + sizeof(MT)) * (double)A.nnz + (double)row_bytes * (double)A.n;
+double spmv_class_bytes(const sph_rt *s, const CsrView<MT> &A, int row_bytes) {
+  return ((s->sl.ptr ? 2.0 : 4.0) + sizeof(MT)) * (double)A.nnz + (double)row_bytes * (double)A.n;
 }
 // resid: rowptr, diag, b, x, r, 1/V        spmv_pq: rowptr, diag, z, q r/w, p r/w
 constexpr int kRowBytesResid = 48, kRowBytesSpmvPQ = 56;
@@ -439,19 +438,18 @@ sph_rt_status cheb_apply(sph_rt *s, const CsrView<MT> &A, const VT *r, VT *z, VT
   // fine-level sweeps are timed with the other fine SpMV-class kernels; per row:
   // rowptr, diag, 1/diag, r, z_in, z_out, d r/w (vectors of type VT)
   const bool fine = A.ptr == s->mat_ptr;
-  const int gw = fine ? row_grid(s->num_sms, A.n, A.W, A.U)
-                      : row_grid_blocks(s->num_sms, A.n, A.W, kCoarseMinBlocks);
-  const double bytes = spmv_class_bytes(A, 8 + 2 * (int)sizeof(MT) + 5 * (int)sizeof(VT));
+  const int gw = row_grid_blocks(s->num_sms, A.n, A.W, kCoarseMinBlocks);
+  const double bytes = spmv_class_bytes(s, A, 8 + 2 * (int)sizeof(MT) + 5 * (int)sizeof(VT));
   auto step = [&](const VT *zin, VT *zout, int k) -> sph_rt_status {
     int *wf = fine ? timing_begin(s) : nullptr;
     if (fine)
-      SPH_DISPATCH_SHAPE(A.W, A.U,
-                         (pdl_launch(s, fine_cheb_step_kernel<W, U, MT, VT>, gw, kBlock, 0,
-                             A, r, zin, zout, d, cf, k, sc, wf)));
+      SPH_FINE_ROWS(s, MT, A, sizeof(VT),
+                    (pdl_launch(s, fine_cheb_step_kernel<Rows, VT>, grid, kBlock, smem, rows, r,
+                                zin, zout, d, cf, k, sc, wf)));
     else
       SPH_DISPATCH_SHAPE(A.W, A.U,
                          (pdl_launch(s, cheb_step_kernel<W, U, MT, VT>, gw, kBlock, 0,
-                             A, r, zin, zout, d, cf, k, sc, wf)));
+                             A, r, zin, zout, d, cf, k, sc)));
     SPH_LAUNCHED(s);
     if (fine) timing_end(s, bytes, kTimedCheb);
     return SPH_RT_OK;
@@ -642,11 +640,11 @@ sph_rt_status fcg_cycle(sph_rt *s, const FcgVecs &v, int first);
 // form), valid for the next solve's start if this replacement ends the solve.
 // Else the start of a solve, skipped when that B x is valid (fcg_start_y_kernel
 // starts from it instead).
-template <int W, int U, typename T>
-__global__ void __launch_bounds__(kBlock, sweep_min_blocks(U))
-    fcg_resid_kernel(CsrView<double> A, const double *b, const double *x, T *r, T *zpre,
-                     const T *invdiag, const ChebCoef *cf, const double *invV, int gated,
-                     double *y, Scalars *sc, double *partials, int *wflag) {
+template <typename Rows, typename T>
+__global__ void __launch_bounds__(kBlock, Rows::kMinBlocks)
+    fcg_resid_kernel(Rows A, const double *b, const double *x, T *r, T *zpre, const T *invdiag,
+                     const ChebCoef *cf, const double *invV, int gated, double *y, Scalars *sc,
+                     double *partials, int *wflag) {
   pdl_wait();
   if (gated ? (sc->done || !sc->ru) : sc->yvalid) {
     mark_work(wflag, 0);
@@ -654,25 +652,22 @@ __global__ void __launch_bounds__(kBlock, sweep_min_blocks(U))
   }
   mark_work(wflag, 1);
   const double c0 = cf->inv_theta;
-  const int own = tile_own_row<W>(threadIdx.x & 31);
-  int64_t r0, r1;
-  warp_rows<W>(A.n, r0, r1);
   double acc = 0.0;
-  for (int64_t base = r0; base < r1; base += 32) {
-    const int rows = (int)(r1 - base < 32 ? r1 - base : 32);
-    const int64_t i = base + own;
-    const double s = tile_row_sums<W, U, double, double>(base, rows, A.ptr, A.col, A.val, x);
-    if (own < rows) {
-      const double bx = fmadd(A.diag[i], x[i], s);
-      const double ri = b[i] - bx;
-      const T rt = (T)ri;
-      r[i] = rt;
-      zpre[i] = (T)(c0 * (double)invdiag[i] * (double)rt);
-      if (y) y[i] = bx;
-      const double ru = ri * invV[i];
-      acc += ru * ru;
-    }
-  }
+  A.each(
+      x,
+      [&](int64_t i) {
+        return Ops7<double>{A.A.diag[i], x[i], b[i], invV[i], widen(invdiag[i])};
+      },
+      [&](int64_t i, double s, const Ops7<double> &o) {
+        const double bx = fmadd(o.a, o.b, s);
+        const double ri = o.c - bx;
+        const T rt = narrow<T>(ri);
+        r[i] = rt;
+        zpre[i] = narrow<T>(c0 * o.e * widen(rt));
+        if (y) y[i] = bx;
+        const double ru = ri * o.d;
+        acc += ru * ru;
+      });
   __shared__ double sh[32];
   acc = block_sum(acc, sh);
   double part[1] = {acc}, out[1];
@@ -702,9 +697,9 @@ __global__ void fcg_start_y_kernel(int64_t n, const double *b, const double *y, 
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     const double ri = b[i] - y[i];
-    const T rt = (T)ri;
+    const T rt = narrow<T>(ri);
     r[i] = rt;
-    zpre[i] = (T)(c0 * (double)invdiag[i] * (double)rt);
+    zpre[i] = narrow<T>(c0 * widen(invdiag[i]) * widen(rt));
     const double ru = ri * invV[i];
     acc += ru * ru;
   }
@@ -746,11 +741,12 @@ __global__ void fcg_update_kernel(int64_t n, double *x, T *r, T *p, T *q, const 
     const T qi = first ? wi : fmadd(beta, q[i], wi);
     p[i] = pi;
     q[i] = qi;
-    x[i] += alpha * (double)pi;
+    x[i] += alpha * widen(pi);
     const T ri = r[i] - ta * qi;
     r[i] = ri;
-    zpre[i] = (T)(c0 * (double)invdiag[i] * (double)ri);
-    const double ru = (double)ri * invV[i];
+    const double rd = widen(ri);
+    zpre[i] = narrow<T>(c0 * widen(invdiag[i]) * rd);
+    const double ru = rd * invV[i];
     acc += ru * ru;
   }
   __shared__ double sh[32];
@@ -782,25 +778,24 @@ __global__ void fcg_update_kernel(int64_t n, double *x, T *r, T *p, T *q, const 
 
 static sph_rt_status fcg_resid_launch(sph_rt *s, const FcgVecs &v, int gated) {
   CsrView<double> A = fine_view(s);
-  const int gw = row_grid(s->num_sms, A.n, A.W, A.U);
   const bool mixed = s->cfg.precision == SPH_RT_MIXED;
   // the mixed form keeps B x of its replacements in w (its CG vectors are FP32)
   double *y = mixed && gated ? s->w : nullptr;
   int *wf = timing_begin(s);
   if (mixed)
-    SPH_DISPATCH_SHAPE(A.W, A.U,
-                       (pdl_launch(s, fcg_resid_kernel<W, U, float>, gw, kBlock, 0, A, s->b,
+    SPH_FINE_ROWS(s, double, A, sizeof(double),
+                       (pdl_launch(s, fcg_resid_kernel<Rows, float>, grid, kBlock, smem, rows, s->b,
                                    s->x, v.f32.r, v.f32.zpre, v.f32.invdiag, v.cf, s->invV, gated,
                                    y, s->sc, s->partials, wf)));
   else
-    SPH_DISPATCH_SHAPE(A.W, A.U,
-                       (pdl_launch(s, fcg_resid_kernel<W, U, double>, gw, kBlock, 0, A, s->b,
+    SPH_FINE_ROWS(s, double, A, sizeof(double),
+                       (pdl_launch(s, fcg_resid_kernel<Rows, double>, grid, kBlock, smem, rows, s->b,
                                    s->x, v.f64.r, v.f64.zpre, v.f64.invdiag, v.cf, s->invV, gated,
                                    y, s->sc, s->partials, wf)));
   SPH_LAUNCHED(s);
   // rowptr, diag, b, x, 1/V, r, zpre, 1/diag (+ y)
   const double tb = mixed ? 4.0 : 8.0;
-  timing_end(s, spmv_class_bytes(A, 40 + (int)(3 * tb) + (y ? 8 : 0)), kTimedTrueResid);
+  timing_end(s, spmv_class_bytes(s, A, 40 + (int)(3 * tb) + (y ? 8 : 0)), kTimedTrueResid);
   if (mixed && !gated) {
     pdl_launch(s, fcg_start_y_kernel<float>, grid_cap(s, A.n, kBlock), kBlock, 0, A.n, s->b,
                (const double *)s->w, v.f32.r, v.f32.zpre, v.f32.invdiag, v.cf, s->invV, s->sc,
@@ -848,22 +843,20 @@ static sph_rt_status fcg_iteration(sph_rt *s) {
 sph_rt_status pcg_prologue(sph_rt *s) {
   if (fcg_active(s)) return fcg_prologue(s);
   CsrView<double> A = fine_view(s);
-  const int gw = row_grid(s->num_sms, A.n, A.W, A.U);
   sph_rt_status rc;
   int *wf = timing_begin(s);
-  SPH_DISPATCH_SHAPE(A.W, A.U,
-                     (pdl_launch(s, resid_kernel<W, U>, gw, kBlock, 0, A, s->b, s->x, s->r,
-                                                                       s->invV, s->sc,
-                                                                       s->partials, wf)));
+  SPH_FINE_ROWS(s, double, A, sizeof(double),
+                (pdl_launch(s, resid_kernel<Rows>, grid, kBlock, smem, rows, s->b, s->x, s->r,
+                            s->invV, s->sc, s->partials, wf)));
   SPH_LAUNCHED(s);
-  timing_end(s, spmv_class_bytes(A, kRowBytesResid), kTimedResid);
+  timing_end(s, spmv_class_bytes(s, A, kRowBytesResid), kTimedResid);
   if ((rc = precondition(s, A, 1))) return rc;
   wf = timing_begin(s);
-  SPH_DISPATCH_SHAPE(A.W, A.U,
-                     (pdl_launch(s, spmv_pq_kernel<W, U>, gw, kBlock, 0, A, s->z, s->q, s->p, 1,
-                                                                         s->sc, s->partials, wf)));
+  SPH_FINE_ROWS(s, double, A, sizeof(double),
+                (pdl_launch(s, spmv_pq_kernel<Rows>, grid, kBlock, smem, rows, s->z, s->q, s->p, 1,
+                            s->sc, s->partials, wf)));
   SPH_LAUNCHED(s);
-  timing_end(s, spmv_class_bytes(A, kRowBytesSpmvPQ), kTimedSpmvPQ);
+  timing_end(s, spmv_class_bytes(s, A, kRowBytesSpmvPQ), kTimedSpmvPQ);
   return SPH_RT_OK;
 }
 
@@ -882,7 +875,6 @@ __global__ void copy_vec_kernel(int64_t n, const double *src, double *dst, const
 sph_rt_status pcg_iteration(sph_rt *s) {
   if (fcg_active(s)) return fcg_iteration(s);
   CsrView<double> A = fine_view(s);
-  const int gw = row_grid(s->num_sms, A.n, A.W, A.U);
   const int g = grid_cap(s, A.n, kBlock);
   sph_rt_status rc;
   FineInit<double> f64 = {};
@@ -901,11 +893,11 @@ sph_rt_status pcg_iteration(sph_rt *s) {
   }
   if ((rc = precondition(s, A, 0, init))) return rc;
   int *wf = timing_begin(s);
-  SPH_DISPATCH_SHAPE(A.W, A.U,
-                     (pdl_launch(s, spmv_pq_kernel<W, U>, gw, kBlock, 0, A, s->z, s->q, s->p, 0,
-                                                                         s->sc, s->partials, wf)));
+  SPH_FINE_ROWS(s, double, A, sizeof(double),
+                (pdl_launch(s, spmv_pq_kernel<Rows>, grid, kBlock, smem, rows, s->z, s->q, s->p, 0,
+                            s->sc, s->partials, wf)));
   SPH_LAUNCHED(s);
-  timing_end(s, spmv_class_bytes(A, kRowBytesSpmvPQ), kTimedSpmvPQ);
+  timing_end(s, spmv_class_bytes(s, A, kRowBytesSpmvPQ), kTimedSpmvPQ);
   return SPH_RT_OK;
 }
 

@@ -17,6 +17,7 @@
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "sliced.cuh"
 
 namespace sphrt {
 
@@ -402,6 +403,117 @@ __global__ void __launch_bounds__(kBlock, kPairMinBlocks)
     *gersh_out = out[0];
 }
 
+// a4 on a sliced operator: a thread per row, D at the row group's dictionary in
+// shared memory (see SlicedView).  Reads 10 bytes (place, G) and writes 8 (12 with
+// the FP32 copy) per entry, but the FP64 pipe bounds it (three operations an entry,
+// 80 % busy): the FP32 copy is narrowed with integer instructions, and the values
+// of a batch are formed without a branch between them, so that their chains
+// overlap.  2.18e8 entries: 2.10 -> 1.61 ms with the FP32 copy.
+template <bool F32>
+__global__ void __launch_bounds__(kBlock, 4)
+    assemble_sliced_kernel(Phys ph, SlicedView<double> A, double *__restrict__ val,
+                           float *__restrict__ val32, const int64_t *gh_ptr,
+                           const int32_t *gh_slot, const double *gh_W, const double *V,
+                           const double *sigma, const double *f, const double *D, const double *E,
+                           double *diag, double *invdiag, double *gb, double *partials,
+                           unsigned *counter, double *gersh_out, float *diag32,
+                           float *invdiag32) {
+  extern __shared__ __align__(16) unsigned char asm_smem[];
+  double *Ds = reinterpret_cast<double *>(asm_smem);
+  __shared__ double sums[3][kBlock];
+  const int64_t groups = (A.n + kBlock - 1) / kBlock;
+  double gmax = 0.0;
+  for (int64_t g = blockIdx.x; g < groups; g += gridDim.x) {
+    const int64_t d0 = A.dptr[g];
+    const int nd = (int)(A.dptr[g + 1] - d0);
+    for (int t = threadIdx.x; t < nd; t += kBlock) Ds[t] = D[A.dict[d0 + t]];
+    __syncthreads();
+    const int64_t i = g * kBlock + threadIdx.x;  // place in the slices, then row
+    if (i < A.n) {
+      const int len = A.len[i], row = A.order[i];
+      const int64_t k0 = A.ptr[i >> 5] + (threadIdx.x & 31);
+      const double Di = D[g * kBlock + row];
+      double offsum = 0.0;
+      const int width = __reduce_max_sync(__activemask(), len);  // rows of one warp
+      for (int t = 0; t < width; t += kSliceU) {
+        int c[kSliceU];
+        double v[kSliceU];
+        const int64_t k1 = k0 + (int64_t)t * 32;
+#pragma unroll
+        for (int u = 0; u < kSliceU; ++u) {
+          const bool in = t + u < len;
+          c[u] = in ? (int)__ldg(A.idx + k1 + u * 32) : 0;
+          v[u] = in ? __ldg(A.val + k1 + u * 32) : 0.0;
+        }
+        // no branch among the values: their chains overlap (past a row's end G = 0)
+#pragma unroll
+        for (int u = 0; u < kSliceU; ++u) {
+          v[u] *= Di + Ds[c[u]];
+          offsum += v[u];
+        }
+        bool plain = true;
+#pragma unroll
+        for (int u = 0; u < kSliceU; ++u)
+          if (t + u < len) {
+            val[k1 + u * 32] = v[u];
+            if (F32) {
+              val32[k1 + u * 32] = narrow_fast(v[u]);
+              plain = plain && narrow_ok(v[u]);
+            }
+          }
+        if (F32 && !plain)  // rare: zeros and values outside FP32's normal range
+          for (int u = 0; u < kSliceU && t + u < len; ++u)
+            val32[k1 + u * 32] = (float)val[k1 + u * 32];
+      }
+      // Dirichlet couplings, in place order too: the rows that have any are the
+      // short ones, which the sorting puts side by side
+      double wsum = 0.0, gbs = 0.0;
+      const int64_t h0 = gh_ptr[g * kBlock + row], h1 = gh_ptr[g * kBlock + row + 1];
+      for (int64_t k = h0; k < h1; k += 8) {
+        int32_t j[8];
+        double w[8], Dj[8], Ej[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) j[u] = k + u < h1 ? gh_slot[k + u] : -1;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          w[u] = j[u] >= 0 ? gh_W[k + u] : 0.0;
+          Dj[u] = j[u] >= 0 ? D[j[u]] : 0.0;
+          Ej[u] = j[u] >= 0 ? E[j[u]] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (j[u] >= 0) {
+            const double wk = -w[u] * (Di + Dj[u]);
+            wsum += wk;
+            gbs += wk * Ej[u];
+          }
+      }
+      sums[0][row] = offsum;
+      sums[1][row] = wsum;
+      sums[2][row] = gbs;
+    }
+    __syncthreads();  // also: Ds may be staged again
+    if (i >= A.n) continue;
+    const double offsum = sums[0][threadIdx.x], wsum = sums[1][threadIdx.x];
+    const double d = V[i] * (ph.inv_dt + ph.c * sigma[i] * f[i] + wsum) - offsum;
+    const double inv = 1.0 / d;
+    diag[i] = d;
+    invdiag[i] = inv;
+    if (F32) {
+      diag32[i] = (float)d;
+      invdiag32[i] = (float)inv;
+    }
+    gb[i] = sums[2][threadIdx.x];
+    gmax = fmax(gmax, -offsum * inv);  // off-diagonals are <= 0
+  }
+  __shared__ double sh[32];
+  gmax = block_max(gmax, sh);
+  double part[1] = {gmax}, out[1];
+  const bool mx[1] = {true};
+  if (last_block_combine<1>(part, partials, counter, out, mx) && threadIdx.x == 0)
+    *gersh_out = out[0];
+}
+
 // a7: right-hand side of the diffusion solve (B-scaled), the warm start x = E^l,
 // ||b||^2 of the unscaled rows, and reset of the Krylov scalars.
 __global__ void rhs_kernel(Phys ph, int64_t n_int, const double *V, const double *sigma,
@@ -737,6 +849,24 @@ sph_rt_status launch_properties(sph_rt *s, double dt) {
 
 sph_rt_status launch_assembly(sph_rt *s, double dt, double *gersh_out) {
   Phys ph = make_phys(s, dt);
+  if (s->sl.ptr) {
+    const SlicedView<double> A =
+        sliced_view<double>(s->sl, s->n_int, s->nnz_mat, s->sl_G, nullptr, nullptr);
+    const int grid = sliced_grid(s, s->n_int, 4);
+    const size_t smem = sizeof(double) * (size_t)s->sl.dict_max;
+    if (s->sl_val32)
+      assemble_sliced_kernel<true><<<grid, kBlock, smem, s->stream>>>(
+          ph, A, s->sl_val, s->sl_val32, s->gh_ptr, s->gh_slot, s->gh_W, s->V, s->sigma, s->f,
+          s->D, s->E, s->diag, s->invdiag, s->gb, s->partials, &s->sc->counter, gersh_out,
+          s->diag32, s->invdiag32);
+    else
+      assemble_sliced_kernel<false><<<grid, kBlock, smem, s->stream>>>(
+          ph, A, s->sl_val, nullptr, s->gh_ptr, s->gh_slot, s->gh_W, s->V, s->sigma, s->f, s->D,
+          s->E, s->diag, s->invdiag, s->gb, s->partials, &s->sc->counter, gersh_out, nullptr,
+          nullptr);
+    SPH_LAUNCHED(s);
+    return SPH_RT_OK;
+  }
   RowShape sh = shape_for_mean(s->n_int ? (double)s->nnz_mat / (double)s->n_int : 0.0);
   int gr = row_grid_blocks(s->num_sms, s->n_int, sh.W, kPairMinBlocks);
   // the mixed form gets its FP32 copy of the fine operator in the same pass

@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "sliced.cuh"
 
 namespace sphrt {
 
@@ -200,6 +201,10 @@ void free_all(sph_rt *s) {
   s->gcol = nullptr;
   s->gvx = s->gvy = s->gvz = nullptr;
   s->mat_val32 = nullptr;
+  s->sl = SlicedRowsData{};
+  s->sl_G = s->sl_val = nullptr;
+  s->sl_val32 = nullptr;
+  s->sl_refused = false;
   s->diag32 = s->invdiag32 = nullptr;
   s->amg_gersh = nullptr;
   s->cheb_slots = nullptr;
@@ -814,6 +819,7 @@ static sph_rt_status step_common(sph_rt *s, double dt, const double *Qe_c, const
   tm.end();
 
   SPH_TRACE("step: properties and ghosts queued");
+  if ((rc = sliced_operator(s))) return rc;
   tm.begin(1);
   if ((rc = launch_assembly(s, dt, s->gersh))) return rc;  // a4
   tm.end();
@@ -822,7 +828,7 @@ static sph_rt_status step_common(sph_rt *s, double dt, const double *Qe_c, const
     // coefficients on [1 - g, 1 + g] straight from the device Gershgorin bound
     if ((rc = launch_cheb_slots(s, 0, s->gersh, {0}, {s->cfg.cheb_degree}))) return rc;
   }
-  if (s->cfg.autotune && !s->fine_shape_set) {
+  if (s->cfg.autotune && !s->fine_shape_set && !s->sl.ptr) {
     if ((rc = autotune_fine_shape(s))) return rc;
   }
 
@@ -1208,11 +1214,14 @@ extern "C" sph_rt_status sph_rt_get_operator(sph_rt *s, int64_t *rowptr, int64_t
   if ((rc = d2h(s, s2c, s->slot2caller, s->n))) return rc;
   if ((rc = d2h(s, ptr, s->mat_ptr, s->n_int + 1))) return rc;
   if ((rc = d2h(s, col, s->mat_col, s->nnz_mat))) return rc;
-  if ((rc = d2h(s, val, s->mat_val, s->nnz_mat))) return rc;
+  double *csr = nullptr;
+  if (s->sl.ptr && (rc = sliced_to_csr(s, &csr))) return rc;
+  if ((rc = d2h(s, val, csr ? csr : s->mat_val, s->nnz_mat))) return rc;
   if ((rc = d2h(s, dg, s->diag, s->n_int))) return rc;
   if ((rc = d2h(s, g, s->gb, s->n_int))) return rc;
   if ((rc = d2h(s, V, s->V, s->n_int))) return rc;
   SPH_CUDA(s, cudaStreamSynchronize(s->stream));
+  dfree(s, csr);
   const int64_t n = s->n;
   std::vector<int64_t> cnt((size_t)n, 0);
   for (int64_t slot = 0; slot < s->n_int; ++slot) cnt[s2c[slot]] = ptr[slot + 1] - ptr[slot];
