@@ -162,7 +162,7 @@ template <int NV>
 __device__ bool last_block_combine(const double (&part)[NV], double *partials, unsigned *counter,
                                    double (&out)[NV], const bool (&is_max)[NV]) {
   __shared__ bool am_last;
-  __shared__ double sh[32];
+  __shared__ double sh[NV][32];
   if (threadIdx.x == 0) {
     for (int k = 0; k < NV; ++k) partials[(size_t)k * gridDim.x + blockIdx.x] = part[k];
     __threadfence();
@@ -172,17 +172,29 @@ __device__ bool last_block_combine(const double (&part)[NV], double *partials, u
   __syncthreads();
   if (!am_last) return false;
   __threadfence();
-  for (int k = 0; k < NV; ++k) {
-    double acc = 0.0;  // partial maxima are of non-negative quantities
-    // each thread folds a strided subset in order, then a fixed-shape tree
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
-      double v = ((volatile double *)partials)[(size_t)k * gridDim.x + b];
-      acc = is_max[k] ? fmax(acc, v) : acc + v;
+  // each thread folds a strided subset in order, then a fixed-shape tree; the NV
+  // values go through both together, so their latencies overlap
+  double acc[NV];
+  for (int k = 0; k < NV; ++k) acc[k] = 0.0;  // partial maxima are of non-negative quantities
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
+    for (int k = 0; k < NV; ++k) {
+      const double v = ((volatile double *)partials)[(size_t)k * gridDim.x + b];
+      acc[k] = is_max[k] ? fmax(acc[k], v) : acc[k] + v;
     }
-    acc = is_max[k] ? block_max(acc, sh) : block_sum(acc, sh);
-    if (threadIdx.x == 0) out[k] = acc;
-    __syncthreads();
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int k = 0; k < NV; ++k) {
+    acc[k] = is_max[k] ? warp_max(acc[k]) : warp_sum(acc[k]);
+    if (lane == 0) sh[k][wid] = acc[k];
   }
+  __syncthreads();
+  if (wid == 0) {
+    const int nw = (blockDim.x + 31) >> 5;
+    for (int k = 0; k < NV; ++k) {
+      const double v = lane < nw ? sh[k][lane] : 0.0;
+      out[k] = is_max[k] ? warp_max(v) : warp_sum(v);
+    }
+  }
+  __syncthreads();
   if (threadIdx.x == 0) *counter = 0u;
   return true;
 }
@@ -233,6 +245,39 @@ __device__ __forceinline__ double narrow<double>(double v) { return v; }
 template <>
 __device__ __forceinline__ float narrow<float>(double v) {
   return narrow_ok(v) ? narrow_fast(v) : (float)v;
+}
+
+// Quotients with few FP64 operations (the division in FP64 costs about ten, and the
+// FP64 pipe bounds the per-particle kernels): a reciprocal of the divisor and one
+// residual correction q + (x - q d) y (Markstein 1990), within an ulp of the
+// rounded quotient.
+// div_by: y = 1/d is known (a constant of the launch).
+__device__ __forceinline__ double div_by(double x, double d, double y) {
+  const double q = x * y;
+  return fma(fma(-q, d, x), y, q);
+}
+// recip: an FP32 seed (~2^-22) and one Newton step y (2 - d y), to ~2^-44; the
+// divisor's magnitude must be within 2^-100 .. 2^100 (recip_ok).
+__device__ __forceinline__ bool recip_ok(double d) {
+  return (((uint32_t)__double2hiint(d) >> 20) & 0x7ffu) - (1023u - 100u) < 200u;
+}
+__device__ __forceinline__ double recip(double d) {
+  const double y = widen(__fdividef(1.0f, narrow_fast(d)));
+  return fma(y, fma(-d, y, 1.0), y);
+}
+__device__ __forceinline__ double quotient(double x, double d) {
+  return recip_ok(d) ? div_by(x, d, recip(d)) : x / d;
+}
+// Larger of two non-negative values by their bit patterns (integer pipe); a NaN
+// in v is passed over, as by fmax.
+__device__ __forceinline__ double max_bits(double m, double v) {
+  const long long a = __double_as_longlong(m), b = __double_as_longlong(v);
+  return __longlong_as_double(b > a && b <= 0x7ff0000000000000ll ? b : a);
+}
+__device__ __forceinline__ double warp_max_bits(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = max_bits(v, __shfl_down_sync(0xffffffffu, v, o));
+  return v;
 }
 
 template <int W, int U, typename MT, typename VT>
@@ -815,6 +860,7 @@ struct sph_rt {
   int64_t *gh_ptr = nullptr;   // Dirichlet-ghost couplings
   int32_t *gh_slot = nullptr;
   double *gh_W = nullptr;      // V_j F_ij
+  int32_t *gh_row = nullptr;   // row of each coupling
   double *gb = nullptr;        // unscaled Dirichlet coupling sum_j w_ij E_j
 
   // material data of the step, slot order [n]

@@ -891,7 +891,8 @@ __global__ void op_ghost_kernel(const int64_t *nbr_ptr, const int32_t *interior,
                                 const int32_t *nbr_col, const double *nbr_F, const int32_t *kind,
                                 const int32_t *copysrc, const double *V, int64_t n_int,
                                 const int64_t *mat_ptr, int32_t *mat_col, double *mat_G,
-                                const int64_t *gh_ptr, int32_t *gh_slot, double *gh_W) {
+                                const int64_t *gh_ptr, int32_t *gh_slot, double *gh_W,
+                                int32_t *gh_row) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -931,6 +932,7 @@ __global__ void op_ghost_kernel(const int64_t *nbr_ptr, const int32_t *interior,
           const int64_t at = g + __popc(bg & lt);
           gh_slot[at] = col;
           gh_W[at] = val;
+          gh_row[at] = (int32_t)i;
         }
         if (ism) {
           const int64_t at = m + __popc(bm & lt);
@@ -1202,9 +1204,10 @@ sph_rt_status build_particles(sph_rt *s, int64_t n, const double *pos_c, const d
   s->mat_val = dalloc<double>(s, s->nnz_mat);
   s->gh_slot = dalloc<int32_t>(s, s->nnz_gh);
   s->gh_W = dalloc<double>(s, s->nnz_gh);
+  s->gh_row = dalloc<int32_t>(s, s->nnz_gh);
   double *ih = dalloc<double>(s, n), *cw = dalloc<double>(s, n);
   if (!s->nbr_col || !s->nbr_F || !s->mat_col || !s->mat_G || !s->mat_val || !s->gh_slot ||
-      !s->gh_W || !ih || !cw)
+      !s->gh_W || !s->gh_row || !ih || !cw)
     return SPH_RT_ENOMEM;
   kernel_coef_kernel<<<grid1(s, n), kBlock, 0, st>>>(n, dim, s->cfg.kernel, s->h, ih, cw);
   SPH_LAUNCHED(s);
@@ -1218,7 +1221,7 @@ sph_rt_status build_particles(sph_rt *s, int64_t n, const double *pos_c, const d
   if (n > n_int) {
     op_ghost_kernel<<<gt, kBlock, 0, st>>>(s->nbr_ptr, interior, s->nbr_col, s->nbr_F, s->kind,
                                            s->copysrc, s->V, n_int, s->mat_ptr, s->mat_col,
-                                           s->mat_G, s->gh_ptr, s->gh_slot, s->gh_W);
+                                           s->mat_G, s->gh_ptr, s->gh_slot, s->gh_W, s->gh_row);
     SPH_LAUNCHED(s);
   }
   SPH_CUDA(s, cudaStreamSynchronize(st));

@@ -31,14 +31,14 @@ struct Phys {
 
 __device__ __forceinline__ double opacity(double sigma0, double Ts, double p) {
   if (p == 0.0) return sigma0;
-  if (p == -3.0) return sigma0 / (Ts * Ts * Ts);
+  if (p == -3.0) return quotient(sigma0, Ts * Ts * Ts);
   return sigma0 * pow(Ts, p);
 }
 
 __device__ __forceinline__ double limiter_lambda(int limiter, double k, double R) {
-  if (limiter == SPH_RT_LIMITER_LEVERMORE) return (2.0 + R) / (6.0 + 3.0 * R + R * R);
+  if (limiter == SPH_RT_LIMITER_LEVERMORE) return quotient(2.0 + R, 6.0 + 3.0 * R + R * R);
   if (limiter == SPH_RT_LIMITER_LARSEN) {
-    if (k == 2.0) return 1.0 / sqrt(9.0 + R * R);
+    if (k == 2.0) return quotient(1.0, sqrt(9.0 + R * R));
     return 1.0 / pow(pow(3.0, k) + pow(R, k), 1.0 / k);
   }
   return 1.0 / 3.0;
@@ -49,21 +49,23 @@ __global__ void props_point_kernel(Phys ph, int64_t n, const int32_t *kind, cons
                                    const double *sigma0, const double *e, double *T,
                                    double *sigma, double *f, double *R, double *lambda,
                                    double *D) {
+  // R = 0 here; interior rows with a limiter are overwritten by the gradient kernel
+  const double lam = limiter_lambda(ph.limiter, ph.larsen_k, 0.0);
+  const double cl = ph.c * lam, c4 = ph.c * ph.dt * 4.0 * ph.a;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     if (kind[i] == SPH_RT_COPY) continue;
-    double Ti = e[i] / ph.cv;
-    double Ts = Ti > ph.T_floor ? Ti : ph.T_floor;
-    double sig = opacity(sigma0[i], Ts, ph.p);
-    double fi = 1.0 / (1.0 + ph.c * sig * ph.dt * 4.0 * ph.a * Ti * Ti * Ti / (rho[i] * ph.cv));
+    const double Ti = div_by(e[i], ph.cv, ph.inv_cv);
+    const double Ts = Ti > ph.T_floor ? Ti : ph.T_floor;
+    const double sig = opacity(sigma0[i], Ts, ph.p);
+    // 1 / (1 + c sigma dt 4 a T^3 / (rho c_v)) over one denominator
+    const double rc = rho[i] * ph.cv;
     T[i] = Ti;
     sigma[i] = sig;
-    f[i] = fi;
-    // R = 0 here; interior rows with a limiter are overwritten by the gradient kernel
-    double lam = limiter_lambda(ph.limiter, ph.larsen_k, 0.0);
+    f[i] = quotient(rc, rc + (c4 * sig) * (Ti * Ti * Ti));
     R[i] = 0.0;
     lambda[i] = lam;
-    D[i] = ph.c * lam / (sig + ph.sigma_s);
+    D[i] = quotient(cl, sig + ph.sigma_s);
   }
 }
 
@@ -215,11 +217,11 @@ __global__ void __launch_bounds__(kBlock, kPairMinBlocks)
       double gn = sqrt(gx * gx + gy * gy + gz * gz);
       double Es = Eo > 1e-300 ? Eo : 1e-300;
       const double sig_t = sigma[i] + ph.sigma_s;
-      double Ri = gn / (sig_t * Es);
+      double Ri = quotient(gn, sig_t * Es);
       double lam = limiter_lambda(ph.limiter, ph.larsen_k, Ri);
       R[i] = Ri;
       lambda[i] = lam;
-      D[i] = ph.c * lam / sig_t;
+      D[i] = quotient(ph.c * lam, sig_t);
     }
   }
 }
@@ -529,10 +531,10 @@ __global__ void rhs_kernel(Phys ph, int64_t n_int, const double *V, const double
   double acc = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_int;
        i += (int64_t)gridDim.x * blockDim.x) {
-    double Tl = e_l[i] / ph.cv;
-    double B = ph.a * Tl * Tl * Tl * Tl;
+    double Tl = div_by(e_l[i], ph.cv, ph.inv_cv), T2 = Tl * Tl;
+    double B = ph.a * (T2 * T2);
     double cs = ph.c * sigma[i];
-    double bi = E_old[i] / ph.dt + cs * B - (1.0 - f[i]) * cs * E_l[i] + QE[i] + gb[i];
+    double bi = div_by(E_old[i], ph.dt, ph.inv_dt) + cs * B - (1.0 - f[i]) * cs * E_l[i] + QE[i] + gb[i];
     b[i] = V[i] * bi;
     double xi = E_l[i];
     if (ord >= 1) {
@@ -561,54 +563,76 @@ __global__ void rhs_kernel(Phys ph, int64_t n_int, const double *V, const double
 // Newton from e_start.  red[0] = max |e_new - e_start|/|e_new|,
 // red[1] = max |E_new - E_prev|/|E_new|, red[2] = max Newton iterations,
 // red[3] = number of particles that hit the iteration limit.
-__global__ void newton_kernel(Phys ph, int64_t n_int, const double *rho, const double *sigma,
-                              const double *e_old, const double *Qe, const double *E_new,
-                              const double *E_prev, const double *e_start, double *e_new,
-                              Scalars *sc, double *partials) {
-  double ce = 0.0, cE = 0.0, itmax = 0.0, fails = 0.0;
+//
+// FP64-bound: ~14 operations an iteration (the quotient u / J by a reciprocal of
+// ~2^-44, whose error the next iteration would remove and which the last one, of
+// |de| <= tol |e|, does not feel), tests and maxima on bit patterns, and integer
+// reductions.  2.1e6 particles: 0.335 -> 0.214 ms, 2.5e5 (heating wave): 0.068 ->
+// 0.028.
+__global__ void __launch_bounds__(kBlock)
+    newton_kernel(Phys ph, int64_t n_int, const double *rho, const double *sigma,
+                  const double *e_old, const double *Qe, const double *E_new,
+                  const double *E_prev, const double *e_start, double *e_new, Scalars *sc,
+                  double *partials) {
+  double ce = 0.0, cE = 0.0;
+  int itmax = 0, fails = 0;
+  const double tiny = 1e-300;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_int;
        i += (int64_t)gridDim.x * blockDim.x) {
-    double cs = ph.c * sigma[i];
-    double P = cs * E_new[i] + Qe[i];
+    const double cs = ph.c * sigma[i];
+    const double En = E_new[i];
+    const double P = fma(cs, En, Qe[i]);
     // per-particle constants of u(e) = rho/dt (e - e_old) + c sigma a T^4 - P and
-    // J = rho/dt + 4 c sigma a T^3 / cv, hoisted out of the loop: one FP64
-    // division (u / J) per iteration is left, on a part whose FP64 pipe is narrow
-    double rdt = rho[i] * ph.inv_dt;
-    double csa = cs * ph.a;
-    double k4 = 4.0 * csa * ph.inv_cv;
-    double eo = e_old[i];
-    double e0 = e_start[i];
+    // J = rho/dt + 4 c sigma a T^3 / cv
+    const double rdt = rho[i] * ph.inv_dt;
+    const double csa = cs * ph.a;
+    const double k4 = 4.0 * csa * ph.inv_cv;
+    const double eo = e_old[i], e0 = e_start[i];
     double ei = e0;
     int it = 0;
     bool ok = false;
     while (it < ph.max_inner) {
-      double T = ei * ph.inv_cv;
-      double T3 = T * T * T;
-      double u = rdt * (ei - eo) + csa * T3 * T - P;
-      double J = rdt + k4 * T3;
-      double de = u / J;
+      const double T = ei * ph.inv_cv;
+      const double T3 = T * T * T;
+      const double u = fma(rdt, ei - eo, fma(csa * T3, T, -P));
+      const double J = fma(k4, T3, rdt);
+      const double de = recip_ok(J) ? u * recip(J) : u / J;
       ei = ei - de;
       ++it;
-      if (fabs(de) <= ph.tol_inner * fabs(ei)) {
+      const long long lim = __double_as_longlong(ph.tol_inner * fabs(ei));
+      if (__double_as_longlong(fabs(de)) <= lim && lim <= 0x7ff0000000000000ll) {
         ok = true;
         break;
       }
     }
     e_new[i] = ei;
-    ce = fmax(ce, fabs(ei - e0) / fmax(fabs(ei), 1e-300));
-    cE = fmax(cE, fabs(E_new[i] - E_prev[i]) / fmax(fabs(E_new[i]), 1e-300));
-    itmax = fmax(itmax, (double)it);
-    if (!ok) fails += 1.0;
+    ce = max_bits(ce, quotient(fabs(ei - e0), max_bits(tiny, fabs(ei))));
+    cE = max_bits(cE, quotient(fabs(En - E_prev[i]), max_bits(tiny, fabs(En))));
+    itmax = max(itmax, it);
+    fails += !ok;
   }
-  __shared__ double sh[32];
-  double p0 = block_max(ce, sh);
+  __shared__ double sh[2][kWarpsPerBlock];
+  __shared__ int shi[2][kWarpsPerBlock];
+  ce = warp_max_bits(ce);
+  cE = warp_max_bits(cE);
+  itmax = __reduce_max_sync(0xffffffffu, itmax);
+  fails = __reduce_add_sync(0xffffffffu, fails);
+  const int wid = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    sh[0][wid] = ce;
+    sh[1][wid] = cE;
+    shi[0][wid] = itmax;
+    shi[1][wid] = fails;
+  }
   __syncthreads();
-  double p1 = block_max(cE, sh);
-  __syncthreads();
-  double p2 = block_max(itmax, sh);
-  __syncthreads();
-  double p3 = block_sum(fails, sh);
-  double part[4] = {p0, p1, p2, p3}, out[4];
+  if (threadIdx.x == 0)
+    for (int w = 1; w < kWarpsPerBlock; ++w) {
+      ce = max_bits(ce, sh[0][w]);
+      cE = max_bits(cE, sh[1][w]);
+      itmax = max(itmax, shi[0][w]);
+      fails += shi[1][w];
+    }
+  double part[4] = {ce, cE, (double)itmax, (double)fails}, out[4];
   const bool mx[4] = {true, true, true, false};
   if (last_block_combine<4>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     sc->red[0] = out[0];
@@ -658,21 +682,20 @@ __global__ void totals_kernel(int64_t n_int, const double *mass, const double *V
 }
 
 // Energy added over the step: red[6] = dt sum V (Q_e + Q_E);
-// red[7] = dt sum_i V_i sum_{Dirichlet j} w_ij (E_j - E_i).
-__global__ void balance_kernel(Phys ph, int64_t n_int, const double *V, const double *Qe,
-                               const double *QE, const int64_t *gh_ptr, const int32_t *gh_slot,
-                               const double *gh_W, const double *D, const double *E,
-                               Scalars *sc, double *partials) {
+// red[7] = dt sum_i V_i sum_{Dirichlet j} w_ij (E_j - E_i), over the couplings as
+// one flat list: few rows have any, those have tens, and a thread per row spent
+// its time on the longest (0.22 ms at 128^3 with 5.7e6 couplings, now 0.076).
+__global__ void balance_kernel(Phys ph, int64_t n_int, int64_t nnz_gh, const double *V,
+                               const double *Qe, const double *QE, const int32_t *gh_row,
+                               const int32_t *gh_slot, const double *gh_W, const double *D,
+                               const double *E, Scalars *sc, double *partials) {
   double a = 0.0, b = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_int;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    a += V[i] * (Qe[i] + QE[i]);
-    double acc = 0.0;
-    for (int64_t k = gh_ptr[i]; k < gh_ptr[i + 1]; ++k) {
-      int32_t j = gh_slot[k];
-      acc += -gh_W[k] * (D[i] + D[j]) * (E[j] - E[i]);
-    }
-    b += V[i] * acc;
+  const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = t0; i < n_int; i += step) a += V[i] * (Qe[i] + QE[i]);
+  for (int64_t k = t0; k < nnz_gh; k += step) {
+    const int32_t i = gh_row[k], j = gh_slot[k];
+    b -= (V[i] * gh_W[k]) * (D[i] + D[j]) * (E[j] - E[i]);
   }
   __shared__ double sh[32];
   double pa = block_sum(a, sh);
@@ -759,6 +782,13 @@ static int grid_items(const sph_rt *s, int64_t n, int per_block) {
   int64_t g = ceil_div(n > 0 ? n : 1, per_block);
   int64_t cap = (int64_t)s->num_sms * 8;
   if (cap > kMaxRedBlocks) cap = kMaxRedBlocks;
+  return (int)(g < cap ? g : cap);
+}
+
+// Streaming reductions: half the blocks of grid_items, so that a thread has two or
+// more rows to sum before the FP64 shuffle reduction of its block.
+static int grid_reduce(const sph_rt *s, int64_t n) {
+  const int64_t g = ceil_div(n > 0 ? n : 1, kBlock), cap = (int64_t)s->num_sms * 4;
   return (int)(g < cap ? g : cap);
 }
 
@@ -1002,7 +1032,7 @@ __global__ void dtc_eta_kernel(int64_t n_int, const double *e, const double *E,
 }
 
 sph_rt_status launch_dt_control(sph_rt *s, double dt) {
-  const int g = grid_items(s, s->n_int, kBlock);
+  const int g = grid_reduce(s, s->n_int);
   dtc_sums_kernel<<<g, kBlock, 0, s->stream>>>(s->n_int, s->V, s->e, s->E, s->sc, s->partials);
   SPH_LAUNCHED(s);
   const DtControl c = {dt, s->cfg.dt_target, s->cfg.dt_growth, s->cfg.dt_min, s->cfg.dt_max,
@@ -1014,7 +1044,7 @@ sph_rt_status launch_dt_control(sph_rt *s, double dt) {
 }
 
 sph_rt_status launch_totals(sph_rt *s, const double *e, const double *E) {
-  int g = grid_items(s, s->n_int, kBlock);
+  int g = grid_reduce(s, s->n_int);
   totals_kernel<<<g, kBlock, 0, s->stream>>>(s->n_int, s->mass, s->V, e, E, s->sc, s->partials);
   SPH_LAUNCHED(s);
   return SPH_RT_OK;
@@ -1022,9 +1052,10 @@ sph_rt_status launch_totals(sph_rt *s, const double *e, const double *E) {
 
 sph_rt_status launch_balance(sph_rt *s, double dt, const double *E) {
   Phys ph = make_phys(s, dt);
-  int g = grid_items(s, s->n_int, kBlock);
-  balance_kernel<<<g, kBlock, 0, s->stream>>>(ph, s->n_int, s->V, s->Qe, s->QE, s->gh_ptr,
-                                               s->gh_slot, s->gh_W, s->D, E, s->sc, s->partials);
+  int g = grid_reduce(s, s->n_int);
+  balance_kernel<<<g, kBlock, 0, s->stream>>>(ph, s->n_int, s->nnz_gh, s->V, s->Qe, s->QE,
+                                               s->gh_row, s->gh_slot, s->gh_W, s->D, E, s->sc,
+                                               s->partials);
   SPH_LAUNCHED(s);
   return SPH_RT_OK;
 }
