@@ -71,7 +71,7 @@ struct BatchView {
 };
 
 struct BatchPhys {
-  double a, c, cv, inv_cv, p, T_floor, larsen_k, dt, tol_inner, tol_outer_e, tol_outer_E,
+  double a, c, cv, inv_cv, inv_dt, p, T_floor, larsen_k, dt, tol_inner, tol_outer_e, tol_outer_E,
       tol_krylov;
   int limiter, max_inner, max_outer, max_krylov, cheb_degree, dim;
   int krylov_start;  // p > 0: first solve from the extrapolation in time of order <= p
@@ -79,13 +79,13 @@ struct BatchPhys {
 
 __device__ __forceinline__ double b_opacity(double sigma0, double Ts, double p) {
   if (p == 0.0) return sigma0;
-  if (p == -3.0) return sigma0 / (Ts * Ts * Ts);
+  if (p == -3.0) return quotient(sigma0, Ts * Ts * Ts);
   return sigma0 * pow(Ts, p);
 }
 __device__ __forceinline__ double b_lambda(int limiter, double k, double R) {
-  if (limiter == SPH_RT_LIMITER_LEVERMORE) return (2.0 + R) / (6.0 + 3.0 * R + R * R);
+  if (limiter == SPH_RT_LIMITER_LEVERMORE) return quotient(2.0 + R, 6.0 + 3.0 * R + R * R);
   if (limiter == SPH_RT_LIMITER_LARSEN) {
-    if (k == 2.0) return 1.0 / sqrt(9.0 + R * R);
+    if (k == 2.0) return quotient(1.0, sqrt(9.0 + R * R));
     return 1.0 / pow(pow(3.0, k) + pow(R, k), 1.0 / k);
   }
   return 1.0 / 3.0;
@@ -200,15 +200,54 @@ __device__ __forceinline__ double bdiv(double num, double den, double *bc, int &
   return out;
 }
 
+// Row tiles (see common.cuh) over this CTA's rows: tile k of 32 rows goes to warp
+// k mod nw; in a tile's W rounds each W-lane group sums one row, and the transposed
+// reduction leaves every lane the sum of one row, so that the row epilogues (the
+// limiter's root and quotients, diagonal terms, inner products) run on 32 rows a
+// warp instruction.  On GB300's FP64 pipe, which bounds this kernel, an epilogue on
+// one lane per group cost W times as much (20 steps of 96 problems of 1k-20k
+// particles, with the short quotients of common.cuh: 2-D 51.1 -> 34.5 ms, 3-D
+// 102.5 -> 83.0).  f(i, s): every row with its sum;
+// round(rb, re, Xi, sub, nmax): the lane's partial of row [rb, re) of a group, Xi
+// being x_own of that row.
+template <int W, typename R, typename X, typename ROUND, typename F>
+__device__ __forceinline__ void b_tiles(const Part &P, const int64_t *ptr, const X &x_own,
+                                        const ROUND &round, const F &f) {
+  const int lane = threadIdx.x & 31, sub = lane % W, own = tile_own_row<W>(lane);
+  const int64_t wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int64_t base = P.q0 + wid * 32; base < P.q1; base += nw * 32) {
+    const int rows = (int)(P.q1 - base < 32 ? P.q1 - base : 32);
+    const bool active = own < rows;
+    const int64_t i = base + own;
+    int64_t b = 0, e = 0;
+    double xo = 0.0;
+    if (active) {
+      b = ptr[i];
+      e = ptr[i + 1];
+      xo = x_own(i);
+    }
+    const R s = tile_tree<W, 1, R>(0, rows, sub, [&](int t) -> R {
+      const int64_t rb = __shfl_sync(0xffffffffu, b, t, W);
+      const int64_t re = __shfl_sync(0xffffffffu, e, t, W);
+      const double Xi = __shfl_sync(0xffffffffu, xo, t, W);
+      // the group's row, for lists beside ptr
+      return round(base + t * (32 / W) + lane / W, rb, re, Xi, sub, tile_nmax<W>(rb, re, sub));
+    });
+    if (active) f(i, s);
+  }
+}
+
 // Row dot product of the batched kernel: the values and x are written earlier
 // in the same launch by other threads, so they are read with plain (coherent)
 // loads, not through the read-only path; the columns are read-only.  Same
-// order of operations as row_dot.
+// order of operations as row_dot_n (nmax: warp-uniform trip count).
 template <int W, int U>
 __device__ __forceinline__ double b_row_dot(int64_t beg, int64_t end, const int32_t *col,
-                                            const double *val, const double *x, int sub) {
+                                            const double *val, const double *x, int sub,
+                                            int nmax) {
   double s = 0.0;
-  for (int64_t k = beg + sub; k < end; k += (int64_t)W * U) {
+  int64_t k = beg + sub;
+  for (int j = 0; j < nmax; j += U, k += (int64_t)W * U) {
     int32_t c[U];
     double a[U];
 #pragma unroll
@@ -229,32 +268,32 @@ __device__ __forceinline__ double b_row_dot(int64_t beg, int64_t end, const int3
 // MODE 1: y = rhs - B xin and bx = B xin, returns its part of ||y / V||^2.
 // No barrier at the end: the reduction that follows is the barrier before y
 // is read.
+template <int W, int U>
+__device__ __forceinline__ auto b_dot_round(const BatchView &v, const double *xin) {
+  return [&v, xin](int64_t, int64_t rb, int64_t re, double, int sub, int nmax) {
+    return b_row_dot<W, U>(rb, re, v.mat_col, v.mat_val, xin, sub, nmax);
+  };
+}
+struct NoOwn {
+  __device__ __forceinline__ double operator()(int64_t) const { return 0.0; }
+};
 template <int W, int U, int MODE>
 __device__ __forceinline__ double b_spmv(const BatchView &v, const Part &P, const double *xin,
                                          const double *rhs, double *y, double *bxout = nullptr) {
-  const int sub = threadIdx.x % W;
-  const int grp = threadIdx.x / W, ngrp = blockDim.x / W;
   double part = 0.0;
-  for (int64_t wb = P.q0 + warp_first_group<W>(grp); wb < P.q1; wb += ngrp) {
-    const int64_t i = wb + group_in_warp<W>(grp);
-    const bool active = i < P.q1;
-    double s = active ? b_row_dot<W, U>(v.mat_ptr[i], v.mat_ptr[i + 1], v.mat_col, v.mat_val, xin, sub)
-                      : 0.0;
-    s = row_reduce<W>(s);
-    if (active && sub == 0) {
-      const double bx = v.diag[i] * xin[i] + s;
-      if (MODE == 0) {
-        y[i] = bx;
-        part += xin[i] * bx;
-      } else {
-        const double yi = rhs[i] - bx;
-        y[i] = yi;
-        bxout[i] = bx;
-        const double yu = yi * v.invV[i];
-        part += yu * yu;
-      }
+  b_tiles<W, double>(P, v.mat_ptr, NoOwn{}, b_dot_round<W, U>(v, xin), [&](int64_t i, double s) {
+    const double xi = xin[i], bx = v.diag[i] * xi + s;
+    if (MODE == 0) {
+      y[i] = bx;
+      part += xi * bx;
+    } else {
+      const double yi = rhs[i] - bx;
+      y[i] = yi;
+      bxout[i] = bx;
+      const double yu = yi * v.invV[i];
+      part += yu * yu;
     }
-  }
+  });
   return part;
 }
 
@@ -275,30 +314,22 @@ __device__ double b_cheb(const BatchView &v, const Part &P, const double *r, dou
     buf[at][i] = di;
     if (degree == 1) rz += r[i] * di;
   }
-  const int sub = threadIdx.x % W;
-  const int grp = threadIdx.x / W, ngrp = blockDim.x / W;
   for (int k = 1; k < degree; ++k) {
     csync();  // the previous iterate, all rows of the problem
     const double c1 = cf.c1[k], c2 = cf.c2[k];
     const double *zin = buf[at];
     double *zout = buf[at ^ 1];
     const bool last = k == degree - 1;
-    for (int64_t wb = P.q0 + warp_first_group<W>(grp); wb < P.q1; wb += ngrp) {
-      const int64_t i = wb + group_in_warp<W>(grp);
-      const bool active = i < P.q1;
-      double s = active ? b_row_dot<W, U>(v.mat_ptr[i], v.mat_ptr[i + 1], v.mat_col, v.mat_val,
-                                          zin, sub)
-                        : 0.0;
-      s = row_reduce<W>(s);
-      if (active && sub == 0) {
-        const double res = r[i] - (v.diag[i] * zin[i] + s);
-        const double di = c1 * v.d[i] + c2 * v.invdiag[i] * res;
-        v.d[i] = di;
-        const double zi = zin[i] + di;
-        zout[i] = zi;
-        if (last) rz += r[i] * zi;
-      }
-    }
+    b_tiles<W, double>(P, v.mat_ptr, NoOwn{}, b_dot_round<W, U>(v, zin),
+                       [&](int64_t i, double s) {
+                         const double zo = zin[i];
+                         const double res = r[i] - (v.diag[i] * zo + s);
+                         const double di = c1 * v.d[i] + c2 * v.invdiag[i] * res;
+                         v.d[i] = di;
+                         const double zi = zo + di;
+                         zout[i] = zi;
+                         if (last) rz += r[i] * zi;
+                       });
     at ^= 1;
   }
   return rz;
@@ -324,28 +355,28 @@ __global__ void __launch_bounds__(512, MINB) batch_step_kernel(BatchView v, Batc
   CRed R{wred, cred_slots, 0};
   int bpar = 0;
   const Part P = make_part(v.slot_off[k], v.slot_off[k + 1], v.n_int[k], (int)cl.block_rank(), C);
-  const int sub = threadIdx.x % W;
-  const int grp = threadIdx.x / W, ngrp = blockDim.x / W;
 
   // a3: material data from the state at the start of the step (every slot but
   // copy ghosts), energy before; Eg = E at each slot's value source (a copy
   // ghost's interior particle)
   double ea = 0.0;
+  const double l0 = b_lambda(ph.limiter, ph.larsen_k, 0.0);
   for (int64_t i = P.s0 + P.ct; i < P.s1; i += P.cn) {
     const bool copy = v.kind[i] == SPH_RT_COPY;
     v.t[i] = v.E[copy ? v.copysrc[i] : i];
     if (copy) continue;
     if (i < P.r1) ea += v.rho[i] * v.V[i] * v.e[i] + v.V[i] * v.E[i];
-    double Ti = v.e[i] * ph.inv_cv;
-    double Ts = Ti > ph.T_floor ? Ti : ph.T_floor;
-    double sig = b_opacity(v.sigma0[i], Ts, ph.p);
+    const double Ti = v.e[i] * ph.inv_cv;
+    const double Ts = Ti > ph.T_floor ? Ti : ph.T_floor;
+    const double sig = b_opacity(v.sigma0[i], Ts, ph.p);
+    // 1 / (1 + c sigma dt 4 a T^3 / (rho c_v)) over one denominator
+    const double rc = v.rho[i] * ph.cv;
     v.T[i] = Ti;
     v.sigma[i] = sig;
-    v.f[i] = 1.0 / (1.0 + ph.c * sig * ph.dt * 4.0 * ph.a * Ti * Ti * Ti / (v.rho[i] * ph.cv));
-    double l0 = b_lambda(ph.limiter, ph.larsen_k, 0.0);
+    v.f[i] = quotient(rc, rc + (ph.c * ph.dt * 4.0 * ph.a * sig) * (Ti * Ti * Ti));
     v.R[i] = 0.0;
     v.lam[i] = l0;
-    v.D[i] = ph.c * l0 / sig;
+    v.D[i] = quotient(ph.c * l0, sig);
   }
   const double energy_before = csum(R, P, ea);  // also the barrier after a3
   if (ph.limiter != SPH_RT_LIMITER_NONE) {
@@ -356,47 +387,44 @@ __global__ void __launch_bounds__(512, MINB) batch_step_kernel(BatchView v, Batc
     const double *Eg = v.t;
     const bool d3 = ph.dim == 3;
     const int64_t na = v.nnz_nbr;
-    for (int64_t wb = P.q0 + warp_first_group<W>(grp); wb < P.q1; wb += ngrp) {
-      const int64_t i = wb + group_in_warp<W>(grp);
-      const bool active = i < P.q1;
-      const int64_t ia = active ? i : P.r0;
-      const double Ei = v.E[ia];
-      double gx = 0.0, gy = 0.0, gz = 0.0;
-      const int64_t kb = active ? v.nbr_ptr[i] : 0, ke = active ? v.nbr_ptr[i + 1] : 0;
-      for (int64_t kk = kb + sub; kk < ke; kk += (int64_t)W * UL) {
-        int32_t jj[UL];
-        double ax[UL], ay[UL], az[UL];
+    b_tiles<W, Sum3>(
+        P, v.nbr_ptr, [&](int64_t i) { return v.E[i]; },
+        [&](int64_t, int64_t rb, int64_t re, double Ei, int sub, int nmax) -> Sum3 {
+          double gx = 0.0, gy = 0.0, gz = 0.0;
+          int64_t kk = rb + sub;
+          for (int j0 = 0; j0 < nmax; j0 += UL, kk += (int64_t)W * UL) {
+            int32_t jj[UL];
+            double ax[UL], ay[UL], az[UL];
 #pragma unroll
-        for (int u = 0; u < UL; ++u) {
-          const int64_t q = kk + (int64_t)u * W;
-          const bool in = q < ke;
-          jj[u] = in ? __ldg(v.nbr_col + q) : -1;
-          ax[u] = in ? __ldg(v.nbr_A + q) : 0.0;
-          ay[u] = in ? __ldg(v.nbr_A + na + q) : 0.0;
-          az[u] = in && d3 ? __ldg(v.nbr_A + 2 * na + q) : 0.0;
-        }
+            for (int u = 0; u < UL; ++u) {
+              const int64_t q = kk + (int64_t)u * W;
+              const bool in = q < re;
+              jj[u] = in ? __ldg(v.nbr_col + q) : -1;
+              ax[u] = in ? __ldg(v.nbr_A + q) : 0.0;
+              ay[u] = in ? __ldg(v.nbr_A + na + q) : 0.0;
+              az[u] = in && d3 ? __ldg(v.nbr_A + 2 * na + q) : 0.0;
+            }
 #pragma unroll
-        for (int u = 0; u < UL; ++u) {
-          if (jj[u] < 0) continue;
-          const double d = Eg[jj[u]] - Ei;
-          gx = fma(ax[u], d, gx);
-          gy = fma(ay[u], d, gy);
-          if (d3) gz = fma(az[u], d, gz);  // 2-D: no z weights
-        }
-      }
-      gx = row_reduce<W>(gx);
-      gy = row_reduce<W>(gy);
-      gz = row_reduce<W>(gz);
-      if (active && sub == 0) {
-        double gn = sqrt(gx * gx + gy * gy + gz * gz);
-        double Es = Ei > 1e-300 ? Ei : 1e-300;
-        double Ri = gn / (v.sigma[i] * Es);
-        double l = b_lambda(ph.limiter, ph.larsen_k, Ri);
-        v.R[i] = Ri;
-        v.lam[i] = l;
-        v.D[i] = ph.c * l / v.sigma[i];
-      }
-    }
+            for (int u = 0; u < UL; ++u) {
+              if (jj[u] < 0) continue;
+              const double d = Eg[jj[u]] - Ei;
+              gx = fma(ax[u], d, gx);
+              gy = fma(ay[u], d, gy);
+              if (d3) gz = fma(az[u], d, gz);  // 2-D: no z weights
+            }
+          }
+          return {gx, gy, gz};
+        },
+        [&](int64_t i, const Sum3 &g) {
+          const double Ei = v.E[i], sig = v.sigma[i];
+          const double gn = sqrt(g.a * g.a + g.b * g.b + g.c * g.c);
+          const double Es = Ei > 1e-300 ? Ei : 1e-300;
+          const double Ri = quotient(gn, sig * Es);
+          const double l = b_lambda(ph.limiter, ph.larsen_k, Ri);
+          v.R[i] = Ri;
+          v.lam[i] = l;
+          v.D[i] = quotient(ph.c * l, sig);
+        });
     csync();  // the copy ghosts read their sources' D
   }
   for (int64_t i = P.r1 + P.ct; i < P.s1; i += P.cn) {
@@ -413,49 +441,49 @@ __global__ void __launch_bounds__(512, MINB) batch_step_kernel(BatchView v, Batc
 
   // a4: operator values, diagonal, Dirichlet coupling, Gershgorin bound
   double gmax = 0.0;
-  for (int64_t wb = P.q0 + warp_first_group<W>(grp); wb < P.q1; wb += ngrp) {
-    const int64_t i = wb + group_in_warp<W>(grp);
-    const bool active = i < P.q1;
-    const double Di = active ? v.D[i] : 0.0;
-    double off = 0.0;
-    const int64_t mb = active ? v.mat_ptr[i] : 0, me = active ? v.mat_ptr[i + 1] : 0;
-    for (int64_t kk = mb + sub; kk < me; kk += (int64_t)W * U) {
-      int32_t jj[U];
-      double G[U];
+  b_tiles<W, Sum3>(
+      P, v.mat_ptr, [&](int64_t i) { return v.D[i]; },
+      [&](int64_t row, int64_t rb, int64_t re, double Di, int sub, int nmax) -> Sum3 {
+        double off = 0.0;
+        int64_t kk = rb + sub;
+        for (int j0 = 0; j0 < nmax; j0 += U, kk += (int64_t)W * U) {
+          int32_t jj[U];
+          double G[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int64_t q = kk + (int64_t)u * W;
-        jj[u] = q < me ? __ldg(v.mat_col + q) : -1;
-        G[u] = q < me ? __ldg(v.mat_G + q) : 0.0;
-      }
+          for (int u = 0; u < U; ++u) {
+            const int64_t q = kk + (int64_t)u * W;
+            jj[u] = q < re ? __ldg(v.mat_col + q) : -1;
+            G[u] = q < re ? __ldg(v.mat_G + q) : 0.0;
+          }
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (jj[u] < 0) continue;
-        const double val = G[u] * (Di + v.D[jj[u]]);
-        v.mat_val[kk + (int64_t)u * W] = val;
-        off += val;
-      }
-    }
-    double wsum = 0.0, gbs = 0.0;
-    const int64_t hb = active ? v.gh_ptr[i] : 0, he = active ? v.gh_ptr[i + 1] : 0;
-    for (int64_t kk = hb + sub; kk < he; kk += W) {
-      int32_t j = v.gh_slot[kk];
-      double wk = -v.gh_W[kk] * (Di + v.D[j]);
-      wsum += wk;
-      gbs += wk * v.E[j];
-    }
-    off = row_reduce<W>(off);
-    wsum = row_reduce<W>(wsum);
-    gbs = row_reduce<W>(gbs);
-    if (active && sub == 0) {
-      double dd = v.V[i] * (1.0 / ph.dt + ph.c * v.sigma[i] * v.f[i] + wsum) - off;
-      const double inv = 1.0 / dd;
-      v.diag[i] = dd;
-      v.invdiag[i] = inv;
-      v.gb[i] = gbs;
-      gmax = fmax(gmax, -off * inv);
-    }
-  }
+          for (int u = 0; u < U; ++u) {
+            if (jj[u] < 0) continue;
+            const double val = G[u] * (Di + v.D[jj[u]]);
+            v.mat_val[kk + (int64_t)u * W] = val;
+            off += val;
+          }
+        }
+        // Dirichlet couplings (few rows have any)
+        double wsum = 0.0, gbs = 0.0;
+        const bool in = row < P.q1;
+        const int64_t he = in ? v.gh_ptr[row + 1] : 0;
+        for (int64_t q = (in ? v.gh_ptr[row] : 0) + sub; q < he; q += W) {
+          const int32_t j = v.gh_slot[q];
+          const double wk = -v.gh_W[q] * (Di + v.D[j]);
+          wsum += wk;
+          gbs += wk * v.E[j];
+        }
+        __syncwarp();
+        return {off, wsum, gbs};
+      },
+      [&](int64_t i, const Sum3 &t) {
+        const double dd = v.V[i] * (ph.inv_dt + ph.c * v.sigma[i] * v.f[i] + t.b) - t.a;
+        const double inv = quotient(1.0, dd);
+        v.diag[i] = dd;
+        v.invdiag[i] = inv;
+        v.gb[i] = t.c;
+        gmax = fmax(gmax, -t.a * inv);
+      });
   // Alg. 1: e^{n,0} = e^{n-1}, E^{n,0} = E^{n-1}.  The first Krylov solve starts
   // from the extrapolation in time of order min(p, converged steps behind)
   // through E^{n-1} and E^{n-2} (E_old, still the last step's start here),
@@ -492,24 +520,26 @@ __global__ void __launch_bounds__(512, MINB) batch_step_kernel(BatchView v, Batc
                     double *e_out, double &ce, double &cE) {
     double mc[2] = {0.0, 0.0};
     for (int64_t i = P.q0 + threadIdx.x; i < P.q1; i += blockDim.x) {
-      const double cs = ph.c * v.sigma[i];
-      const double Pw = cs * E_new[i] + v.Qe[i];
-      const double rdt = v.rho[i] / ph.dt, eo = v.e_old[i], e0 = e_start[i];
-      // one FP64 division an iteration: T = e / c_v as a product, the
-      // Jacobian's factor 4 c sigma a / c_v hoisted out of the loop
+      const double cs = ph.c * v.sigma[i], En = E_new[i];
+      const double Pw = cs * En + v.Qe[i];
+      const double rdt = v.rho[i] * ph.inv_dt, eo = v.e_old[i], e0 = e_start[i];
+      // as in newton_kernel: T = e / c_v as a product, the Jacobian's factor
+      // 4 c sigma a / c_v hoisted, u / J by a reciprocal, tests on bit patterns
       const double ca = cs * ph.a, k1 = 4.0 * ca * ph.inv_cv;
       double ei = e0;
       for (int it = 0; it < ph.max_inner; ++it) {
         const double T = ei * ph.inv_cv, T3 = T * T * T;
-        const double u = rdt * (ei - eo) + ca * T3 * T - Pw;
-        const double J = rdt + k1 * T3;
-        const double de = u / J;
+        const double u = fma(rdt, ei - eo, fma(ca * T3, T, -Pw));
+        const double J = fma(k1, T3, rdt);
+        const double de = recip_ok(J) ? u * recip(J) : u / J;
         ei -= de;
-        if (fabs(de) <= ph.tol_inner * fabs(ei)) break;
+        const long long lim = __double_as_longlong(ph.tol_inner * fabs(ei));
+        if (__double_as_longlong(fabs(de)) <= lim && lim <= 0x7ff0000000000000ll) break;
       }
       e_out[i] = ei;
-      mc[0] = fmax(mc[0], fabs(ei - e0) / fmax(fabs(ei), 1e-300));
-      mc[1] = fmax(mc[1], fabs(E_new[i] - E_prev[i]) / fmax(fabs(E_new[i]), 1e-300));
+      const double tiny = 1e-300;
+      mc[0] = max_bits(mc[0], quotient(fabs(ei - e0), max_bits(tiny, fabs(ei))));
+      mc[1] = max_bits(mc[1], quotient(fabs(En - E_prev[i]), max_bits(tiny, fabs(En))));
     }
     const bool mx[2] = {true, true};
     cred<2>(R, P, mc, mx);
@@ -524,9 +554,9 @@ __global__ void __launch_bounds__(512, MINB) batch_step_kernel(BatchView v, Batc
     // a7: right-hand side (B-scaled), warm start, ||b||
     double bb = 0.0;
     for (int64_t i = P.q0 + threadIdx.x; i < P.q1; i += blockDim.x) {
-      double Tl = v.e_l[i] * ph.inv_cv;
-      double cs = ph.c * v.sigma[i];
-      double bi = v.E_old[i] / ph.dt + cs * ph.a * Tl * Tl * Tl * Tl - (1.0 - v.f[i]) * cs * v.E_l[i] +
+      const double Tl = v.e_l[i] * ph.inv_cv, T2 = Tl * Tl;
+      const double cs = ph.c * v.sigma[i];
+      const double bi = div_by(v.E_old[i], ph.dt, ph.inv_dt) + (cs * ph.a) * (T2 * T2) - (1.0 - v.f[i]) * cs * v.E_l[i] +
                   v.QE[i] + v.gb[i];
       v.b[i] = v.V[i] * bi;
       if (outer > 0 || ord == 0) v.x[i] = v.E_l[i];  // else the extrapolated start
@@ -1060,6 +1090,7 @@ static BatchPhys batch_phys(const sph_rt_batch *B, double dt) {
   ph.c = c.c;
   ph.cv = c.cv;
   ph.inv_cv = 1.0 / c.cv;
+  ph.inv_dt = 1.0 / dt;
   ph.p = c.opacity_exp;
   ph.T_floor = c.T_floor;
   ph.larsen_k = c.larsen_k;
