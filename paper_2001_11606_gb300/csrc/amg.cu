@@ -397,7 +397,8 @@ __global__ void u32_to_i64_kernel(int64_t n, const unsigned *in, int64_t *out) {
 
 // ---------------------------------------------------------------------------
 // coarse sparsity: one block per coarse row, shared-memory hash of the coarse
-// columns reached from the members' rows, then sorted.
+// columns reached from the members' rows, then sorted.  agg == nullptr: the rows'
+// columns are coarse already (the rows of A P) and no targets are wanted.
 // ---------------------------------------------------------------------------
 template <bool FILL>
 __global__ void coarse_struct_kernel(int64_t nc, const int64_t *agg_ptr, const int32_t *agg_mem,
@@ -417,7 +418,7 @@ __global__ void coarse_struct_kernel(int64_t nc, const int64_t *agg_ptr, const i
     for (int64_t m = m0; m < m1; ++m) {
       int32_t i = agg_mem[m];
       for (int64_t k = ptr[i] + threadIdx.x; k < ptr[i + 1]; k += blockDim.x) {
-        int32_t J = agg[col[k]];
+        const int32_t J = agg ? agg[col[k]] : col[k];
         if (J < 0 || J == (int32_t)I) continue;
         uint32_t hsh = hash_u32((uint32_t)J) & (kHash - 1);
         for (int probe = 0; probe < kHash; ++probe) {
@@ -472,7 +473,7 @@ __global__ void coarse_struct_kernel(int64_t nc, const int64_t *agg_ptr, const i
     } else {
       const int64_t base = cptr[I];
       for (int t = threadIdx.x; t < cnt; t += blockDim.x) ccol[base + t] = keys[t];
-      for (int64_t m = m0; m < m1; ++m) {
+      for (int64_t m = m0; m < m1 && tgt; ++m) {
         int32_t i = agg_mem[m];
         if (threadIdx.x == 0) tgt_diag[i] = (int32_t)(nnz_c + I);
         for (int64_t k = ptr[i] + threadIdx.x; k < ptr[i + 1]; k += blockDim.x) {
@@ -495,6 +496,121 @@ __global__ void coarse_struct_kernel(int64_t nc, const int64_t *agg_ptr, const i
     }
     __syncthreads();
   }
+}
+
+// The same from the rows of A P with a warp per coarse row: an aggregate of ~6
+// rows has ~190 A P entries and ~50 distinct columns, too few for a block and its
+// 4096-slot table.  The members' entries are walked 32 at a time into a small hash
+// table, and the distinct columns sorted by the warp and written at off[I] (room
+// for all the members' entries); they are compacted once the counts are known, so
+// the rows are hashed once.  *wide: a row has more than kWarpCols columns; the
+// block kernels above then do the level.  (Both passes of the block kernels, over
+// the operator's own entries, took 3.5 ms for the levels of 97 x 96 x 91 particles;
+// this takes 0.28.)
+constexpr int kWarpTable = 1024, kWarpCols = 512;
+__global__ void member_bound_kernel(int64_t nc, const int64_t *agg_ptr, const int32_t *agg_mem,
+                                    const int64_t *ap_ptr, int64_t *bound) {
+  for (int64_t I = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; I < nc;
+       I += (int64_t)gridDim.x * blockDim.x) {
+    int64_t b = 0;
+    for (int64_t m = agg_ptr[I]; m < agg_ptr[I + 1]; ++m) {
+      const int32_t i = agg_mem[m];
+      b += ap_ptr[i + 1] - ap_ptr[i];
+    }
+    bound[I] = b;
+  }
+}
+constexpr int kCoarseRowWarps = 4;
+__global__ void __launch_bounds__(32 * kCoarseRowWarps)
+    coarse_rows_kernel(int64_t nc, const int64_t *agg_ptr, const int32_t *agg_mem,
+                       const int64_t *ap_ptr, const int32_t *ap_col, const int64_t *off,
+                       int32_t *cols, int64_t *ccount, int *wide) {
+  __shared__ int32_t table_sh[kCoarseRowWarps][kWarpTable];
+  __shared__ int32_t keys_sh[kCoarseRowWarps][kWarpCols];
+  constexpr int32_t kFree = 0x7fffffff;
+  int32_t *table = table_sh[threadIdx.x >> 5], *keys = keys_sh[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int t = lane; t < kWarpTable; t += 32) table[t] = kFree;
+  __syncwarp();
+  for (int64_t I = warp; I < nc; I += nwarps) {
+    int cnt = 0;  // distinct columns so far (warp-uniform)
+    for (int64_t m = agg_ptr[I]; m < agg_ptr[I + 1] && cnt <= kWarpCols; ++m) {
+      const int32_t i = agg_mem[m];
+      const int64_t e = ap_ptr[i + 1];
+      for (int64_t k0 = ap_ptr[i]; k0 < e && cnt <= kWarpCols; k0 += 32) {
+        const int64_t k = k0 + lane;
+        const int32_t J = k < e ? ap_col[k] : (int32_t)I;
+        bool fresh = false;
+        if (J != (int32_t)I) {
+          // at most kWarpCols + 32 of the kWarpTable slots are ever used
+          uint32_t h = hash_u32((uint32_t)J) & (kWarpTable - 1);
+          for (int probe = 0; probe < kWarpTable; ++probe) {
+            const int32_t prev = atomicCAS(&table[h], kFree, J);
+            fresh = prev == kFree;
+            if (fresh || prev == J) break;
+            h = (h + 1) & (kWarpTable - 1);
+          }
+        }
+        const unsigned mask = __ballot_sync(0xffffffffu, fresh);
+        const int at = cnt + __popc(mask & lt);
+        if (fresh && at < kWarpCols) keys[at] = J;
+        cnt += __popc(mask);
+      }
+    }
+    __syncwarp();
+    if (cnt > kWarpCols) {
+      if (lane == 0) {
+        *wide = 1;
+        ccount[I] = 0;
+      }
+      for (int t = lane; t < kWarpTable; t += 32) table[t] = kFree;
+      __syncwarp();
+      continue;
+    }
+    int P2 = 32;
+    while (P2 < cnt) P2 <<= 1;
+    for (int t = cnt + lane; t < P2; t += 32) keys[t] = kFree;
+    __syncwarp();
+    for (int k = 2; k <= P2; k <<= 1)
+      for (int j = k >> 1; j > 0; j >>= 1) {
+        for (int t = lane; t < P2; t += 32) {
+          const int u = t ^ j;
+          if (u > t) {
+            const int32_t a = keys[t], b = keys[u];
+            if ((a > b) == ((t & k) == 0)) {
+              keys[t] = b;
+              keys[u] = a;
+            }
+          }
+        }
+        __syncwarp();
+      }
+    for (int t = lane; t < cnt; t += 32) cols[off[I] + t] = keys[t];
+    if (lane == 0) ccount[I] = cnt;
+    // clear the table for the next row
+    for (int t = lane; t < kWarpTable; t += 32) table[t] = kFree;
+    __syncwarp();
+  }
+}
+// rows of `cnt` entries at in[off[i]] to out[ptr[i]], a warp per row
+__global__ void compact_rows_kernel(int64_t n, const int64_t *off, const int32_t *in,
+                                    const int64_t *ptr, int32_t *out) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t i = warp; i < n; i += nwarps) {
+    const int64_t b = ptr[i], c = ptr[i + 1] - b, o = off[i];
+    for (int64_t t = lane; t < c; t += 32) out[b + t] = in[o + t];
+  }
+}
+// where ap_structure wrote row i's aggregates
+__global__ void ap_offset_kernel(int64_t n, const int64_t *ptr, int64_t *off) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x)
+    off[i] = ptr[i] + i;
 }
 
 // targets of the fine diagonal entries of unaggregated rows stay -1
@@ -893,18 +1009,19 @@ __global__ void ap_structure_warp_kernel(int64_t n, const int64_t *ptr, const in
     __syncwarp();
   }
 }
-// pass 2: compact the keys and make the positions absolute
-__global__ void ap_compact_kernel(int64_t n, const int64_t *ptr, const int32_t *tmp,
-                                  const int64_t *ap_ptr, int32_t *ap_col, int32_t *ap_map,
-                                  int32_t *ap_dmap) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = ap_ptr[i];
-    const int32_t *keys = tmp + ptr[i] + i;
-    for (int64_t q = 0; q < ap_ptr[i + 1] - b; ++q) ap_col[b + q] = keys[q];
-    if (ap_dmap[i] >= 0) ap_dmap[i] = (int32_t)b + ap_dmap[i];
-    for (int64_t k = ptr[i]; k < ptr[i + 1]; ++k)
-      if (ap_map[k] >= 0) ap_map[k] = (int32_t)b + ap_map[k];
+// pass 2 (CSR rows only: the sources of each A P entry are then sorted by it):
+// make the positions absolute, a warp per row
+__global__ void ap_absolute_kernel(int64_t n, const int64_t *ptr, const int64_t *ap_ptr,
+                                   int32_t *ap_map, int32_t *ap_dmap) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t i = warp; i < n; i += nwarps) {
+    const int32_t b = (int32_t)ap_ptr[i];
+    if (lane == 0 && ap_dmap[i] >= 0) ap_dmap[i] += b;
+    const int64_t e = ptr[i + 1];
+    for (int64_t k = ptr[i] + lane; k < e; k += 32)
+      if (ap_map[k] >= 0) ap_map[k] += b;
   }
 }
 // The values (every step) are fixed-order sums of each entry's sources, the
@@ -1456,8 +1573,232 @@ static sph_rt_status launch_galerkin(sph_rt *s, int64_t nnz_c, int64_t nc, const
   return SPH_RT_OK;
 }
 
+__global__ void max_len_kernel(int64_t n, const int32_t *len, int *most) {
+  int m = 0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x)
+    m = max(m, len[i]);
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(most, m);
+}
+
+// Slices of the finest level's A P from its CSR rows.  *again: they have no
+// dictionary within the caps, and the fine operator is back in CSR rows; A P is
+// then to be built like a coarser level's.
+static void *take_level(sph_rt *s, void *L, size_t bytes) {
+  return lvl_alloc(s, static_cast<SphLevel *>(L), bytes);
+}
+static sph_rt_status build_ap_slices(sph_rt *s, SphLevel *L, bool *again) {
+  bool ok = false;
+  sph_rt_status rc = sliced_build(s, L->n, L->ap_ptr, L->ap_col, nullptr, take_level, L, &L->ap_sl,
+                                  nullptr, &ok);
+  if (rc) return rc;
+  int *most = scratch<int>(s, 1);
+  if (!most) return SPH_RT_ENOMEM;
+  SPH_CUDA(s, cudaMemsetAsync(most, 0, sizeof(int), s->stream));
+  if (ok) {
+    max_len_kernel<<<gcap(s, L->n, kBlock), kBlock, 0, s->stream>>>(L->n, L->ap_sl.len, most);
+    SPH_LAUNCHED(s);
+  }
+  SPH_CUDA(s, cudaMemcpyAsync(&L->ap_most, most, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+  SPH_CUDA(s, cudaStreamSynchronize(s->stream));
+  dfree(s, most);
+  if (!ok || L->ap_most >= kNoPlace) {
+    L->ap_sl = SlicedRowsData{};
+    L->ap_pos = nullptr;
+    *again = true;
+    return sliced_undo(s);
+  }
+  const size_t size = (size_t)L->ap_sl.padded + 1;
+  if (s->cfg.precision == SPH_RT_MIXED)
+    L->ap_val32 = lalloc<float>(s, L, size);
+  else
+    L->ap_val = lalloc<double>(s, L, size);
+  return L->ap_val || L->ap_val32 ? SPH_RT_OK : SPH_RT_ENOMEM;
+}
+
+// structure of A P of the last level so far (see ap_structure_kernel)
+static sph_rt_status build_ap(sph_rt *s) {
+  const size_t l = s->levels.size() - 1;
+  SphLevel *L = s->levels[l];
+  const int64_t n = L->n;
+  int32_t *tmp = scratch<int32_t>(s, (size_t)(L->nnz + n));
+  int64_t *cnt = scratch<int64_t>(s, (size_t)n + 1);
+  // target A P entry of each source: off-diagonal entries, then the diagonals
+  int32_t *map = scratch<int32_t>(s, (size_t)(L->nnz + n));
+  L->ap_ptr = lalloc<int64_t>(s, L, n + 1);
+  if (!tmp || !cnt || !map || !L->ap_ptr) return SPH_RT_ENOMEM;
+  int32_t *dmap = map + L->nnz;
+  int *ovf = scratch<int>(s, 1);
+  if (!ovf) return SPH_RT_ENOMEM;
+  SPH_CUDA(s, cudaMemsetAsync(ovf, 0, sizeof(int), s->stream));
+  ap_structure_warp_kernel<<<gcap(s, n, kWarpsPerBlock), kBlock, 0, s->stream>>>(
+      n, L->ptr, L->col, L->agg, tmp, cnt, map, dmap, ovf);
+  SPH_LAUNCHED(s);
+  int h_ovf = 0;
+  SPH_CUDA(s, cudaMemcpyAsync(&h_ovf, ovf, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+  SPH_CUDA(s, cudaStreamSynchronize(s->stream));
+  dfree(s, ovf);
+  if (h_ovf) {  // a row with more distinct aggregates than the warp keeps: one thread a row
+    ap_structure_kernel<<<gcap(s, n, kBlock), kBlock, 0, s->stream>>>(n, L->ptr, L->col, L->agg,
+                                                                      tmp, cnt, map, dmap);
+    SPH_LAUNCHED(s);
+  }
+  sph_rt_status rc;
+  const bool sliced = l == 0 && s->sl.ptr != nullptr;
+  if (sliced) {  // the relative places, before they are made absolute
+    L->ap_pos = lalloc<uint16_t>(s, L, (size_t)s->sl.padded + 1);
+    if (!L->ap_pos) return SPH_RT_ENOMEM;
+    if ((rc = sliced_places(s, map, L->ap_pos))) return rc;
+  }
+  if ((rc = exclusive_scan(s, cnt, n, L->ap_ptr))) return rc;
+  int64_t total = 0;
+  SPH_CUDA(s, cudaMemcpyAsync(&total, L->ap_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost,
+                              s->stream));
+  SPH_CUDA(s, cudaStreamSynchronize(s->stream));
+  if (total >= ((int64_t)1 << 31)) return set_error(s, SPH_RT_EINVAL, "A P too large");
+  L->nnz_ap = total;
+  L->ap_col = lalloc<int32_t>(s, L, (size_t)total);
+  if (!L->ap_col) return SPH_RT_ENOMEM;
+  const int gw = gcap(s, n, kWarpsPerBlock);  // a warp per row
+  ap_offset_kernel<<<gcap(s, n, kBlock), kBlock, 0, s->stream>>>(n, L->ptr, cnt);
+  SPH_LAUNCHED(s);
+  compact_rows_kernel<<<gw, kBlock, 0, s->stream>>>(n, cnt, tmp, L->ap_ptr, L->ap_col);
+  SPH_LAUNCHED(s);
+  bool again = false;
+  if (sliced && (rc = build_ap_slices(s, L, &again))) return rc;
+  if (!sliced || again) {
+    L->ap_val = lalloc<double>(s, L, (size_t)total);
+    if (!L->ap_val) return SPH_RT_ENOMEM;
+    if (s->cfg.precision == SPH_RT_MIXED && !(L->ap_val32 = lalloc<float>(s, L, (size_t)total)))
+      return SPH_RT_ENOMEM;
+    ap_absolute_kernel<<<gw, kBlock, 0, s->stream>>>(n, L->ptr, L->ap_ptr, map, dmap);
+    SPH_LAUNCHED(s);
+    // sources of each A P entry in increasing source order
+    if ((rc = source_sort(s, L, L->nnz + n, map, total, &L->ap_seg_ptr, &L->ap_seg_src)))
+      return rc;
+  }
+  SPH_CUDA(s, cudaStreamSynchronize(s->stream));
+  dfree(s, tmp);
+  dfree(s, cnt);
+  dfree(s, map);
+  return SPH_RT_OK;
+}
+
+// The next level's sparsity from the rows of A P.  *overflow: a coarse row is too
+// wide for the block kernel's table too (the level is then not built).
+static sph_rt_status coarse_from_ap(sph_rt *s, SphLevel *L, SphLevel *C, int64_t *ccount,
+                                    int *overflow) {
+  const int64_t nc = C->n;
+  cudaStream_t st = s->stream;
+  int64_t *bound = scratch<int64_t>(s, nc), *off = scratch<int64_t>(s, nc + 1);
+  int32_t *cols = scratch<int32_t>(s, (size_t)L->nnz_ap + 1);
+  int *flags = scratch<int>(s, 2);  // wide, overflow
+  if (!bound || !off || !cols || !flags) return SPH_RT_ENOMEM;
+  SPH_CUDA(s, cudaMemsetAsync(flags, 0, 2 * sizeof(int), st));
+  member_bound_kernel<<<gcap(s, nc, kBlock), kBlock, 0, st>>>(nc, L->agg_ptr, L->agg_mem,
+                                                             L->ap_ptr, bound);
+  SPH_LAUNCHED(s);
+  sph_rt_status rc = exclusive_scan(s, bound, nc, off);
+  if (rc) return rc;
+  coarse_rows_kernel<<<(int)std::min<int64_t>(ceil_div(nc, kCoarseRowWarps), s->num_sms * 9),
+                       32 * kCoarseRowWarps, 0, st>>>(nc, L->agg_ptr, L->agg_mem, L->ap_ptr,
+                                                      L->ap_col, off, cols, ccount, flags);
+  SPH_LAUNCHED(s);
+  int hf[2] = {0, 0};
+  SPH_CUDA(s, cudaMemcpyAsync(hf, flags, sizeof hf, cudaMemcpyDeviceToHost, st));
+  SPH_CUDA(s, cudaStreamSynchronize(st));
+  const int gb = (int)std::min<int64_t>(nc, (int64_t)s->num_sms * 16);
+  if (hf[0]) {
+    coarse_struct_kernel<false><<<gb, kBlock, 0, st>>>(nc, L->agg_ptr, L->agg_mem, L->ap_ptr,
+                                                       L->ap_col, nullptr, ccount, nullptr, nullptr,
+                                                       nullptr, 0, nullptr, flags + 1);
+    SPH_LAUNCHED(s);
+    SPH_CUDA(s, cudaMemcpyAsync(hf, flags, sizeof hf, cudaMemcpyDeviceToHost, st));
+    SPH_CUDA(s, cudaStreamSynchronize(st));
+  }
+  *overflow = hf[1];
+  if (!hf[1]) {
+    if ((rc = exclusive_scan(s, ccount, nc, C->ptr))) return rc;
+    SPH_CUDA(s, cudaMemcpyAsync(&C->nnz, C->ptr + nc, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    SPH_CUDA(s, cudaStreamSynchronize(st));
+    C->col = lalloc<int32_t>(s, C, C->nnz);
+    if (!C->col) return SPH_RT_ENOMEM;
+    if (hf[0])
+      coarse_struct_kernel<true><<<gb, kBlock, 0, st>>>(nc, L->agg_ptr, L->agg_mem, L->ap_ptr,
+                                                        L->ap_col, nullptr, nullptr, C->ptr, C->col,
+                                                        nullptr, C->nnz, nullptr, flags + 1);
+    else
+      compact_rows_kernel<<<gcap(s, nc, kWarpsPerBlock), kBlock, 0, st>>>(nc, off, cols, C->ptr,
+                                                                          C->col);
+    SPH_LAUNCHED(s);
+  }
+  SPH_CUDA(s, cudaStreamSynchronize(st));
+  dfree(s, bound);
+  dfree(s, off);
+  dfree(s, cols);
+  dfree(s, flags);
+  return SPH_RT_OK;
+}
+
+// values and vectors of a coarse level
+static sph_rt_status coarse_storage(sph_rt *s, SphLevel *C) {
+  const int64_t nc = C->n;
+  C->val = lalloc<double>(s, C, C->nnz);
+  C->diag = lalloc<double>(s, C, nc);
+  C->invdiag = lalloc<double>(s, C, nc);
+  C->r = lalloc<double>(s, C, nc);
+  C->z = lalloc<double>(s, C, nc);
+  C->res = lalloc<double>(s, C, nc);
+  C->d = lalloc<double>(s, C, nc);
+  C->t = lalloc<double>(s, C, nc);
+  if (!C->val || !C->diag || !C->invdiag || !C->r || !C->z || !C->res || !C->d || !C->t)
+    return SPH_RT_ENOMEM;
+  {
+    RowShape sh = shape_for_mean(nc ? (double)C->nnz / (double)nc : 0.0);
+    C->W = sh.W;
+    C->U = sh.U;
+  }
+  return SPH_RT_OK;
+}
+
+// Lists of the next level's sums over A P entries.
+static sph_rt_status build_apg(sph_rt *s, SphLevel *L, SphLevel *C) {
+  const int64_t n = L->n, total = L->nnz_ap;
+  sph_rt_status rc;
+  // next level's Galerkin sources: the A P entries of its members' rows, numbered
+  // as they are stored
+  const int64_t stored = L->ap_sl.ptr ? L->ap_sl.padded : total;
+  int32_t *tgt = scratch<int32_t>(s, (size_t)stored + 1);
+  int *missing = scratch<int>(s, 1);
+  if (!tgt || !missing) return SPH_RT_ENOMEM;
+  SPH_CUDA(s, cudaMemsetAsync(missing, 0, sizeof(int), s->stream));
+  if (L->ap_sl.ptr) {
+    fill_i32_kernel<<<gcap(s, stored, kBlock), kBlock, 0, s->stream>>>(stored, -1, tgt);
+    SPH_LAUNCHED(s);
+    ap_sliced_target_kernel<<<gcap(s, n, kBlock), kBlock, 0, s->stream>>>(
+        n, L->ap_ptr, L->ap_col, L->ap_sl, L->agg, C->nnz, C->ptr, C->col, tgt, missing);
+  } else {
+    ap_galerkin_target_kernel<<<gcap(s, n, kBlock), kBlock, 0, s->stream>>>(
+        n, L->ap_ptr, L->ap_col, L->agg, C->nnz, C->ptr, C->col, tgt, missing);
+  }
+  SPH_LAUNCHED(s);
+  if ((rc = bucket_sort<int32_t>(s, L, stored, tgt, C->nnz + C->n, &L->apg_ptr, &L->apg_src,
+                                 nullptr)))
+    return rc;
+  int miss = 0;
+  SPH_CUDA(s, cudaMemcpyAsync(&miss, missing, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+  SPH_CUDA(s, cudaStreamSynchronize(s->stream));
+  dfree(s, tgt);
+  dfree(s, missing);
+  if (miss) return set_error(s, SPH_RT_EDEVICE, "A P entry outside the coarse sparsity");
+  return SPH_RT_OK;
+}
+
 // Aggregate level L and build the next level's sparsity plus the Galerkin
-// contribution lists.  Returns the new level in *next (nullptr: stop).
+// contribution lists: through A P on the levels above kTailMaxNnz entries (~a
+// third of the sources, and no list over the operator's own entries), else from
+// the level's entries.  Returns the new level in *next (nullptr: stop).
 static sph_rt_status coarsen(sph_rt *s, SphLevel *L, SphLevel **next) {
   *next = nullptr;
   const int64_t n = L->n, nnz = L->nnz;
@@ -1526,8 +1867,24 @@ static sph_rt_status coarsen(sph_rt *s, SphLevel *L, SphLevel **next) {
   // coarse sparsity: count, scan, fill (+ Galerkin targets of every fine entry)
   int64_t *ccount = lalloc<int64_t>(s, C, nc);
   C->ptr = lalloc<int64_t>(s, C, nc + 1);
+  if (!ccount || !C->ptr) return SPH_RT_ENOMEM;
+  auto drop = [&]() {  // stop coarsening here
+    for (void *p : C->owned) dfree(s, p);
+    delete C;
+    return SPH_RT_OK;
+  };
+  if (nnz > kTailMaxNnz) {
+    if ((rc = build_ap(s))) return rc;
+    int ovf = 0;
+    if ((rc = coarse_from_ap(s, L, C, ccount, &ovf))) return rc;
+    if (ovf) return drop();
+    if ((rc = build_apg(s, L, C))) return rc;
+    if ((rc = coarse_storage(s, C))) return rc;
+    *next = C;
+    return SPH_RT_OK;
+  }
   int *overflow = scratch<int>(s, 1);
-  if (!ccount || !C->ptr || !overflow) return SPH_RT_ENOMEM;
+  if (!overflow) return SPH_RT_ENOMEM;
   SPH_CUDA(s, cudaMemsetAsync(overflow, 0, sizeof(int), st));
   int gb = (int)std::min<int64_t>(nc, (int64_t)s->num_sms * 16);
   coarse_struct_kernel<false><<<gb, kBlock, 0, st>>>(nc, L->agg_ptr, L->agg_mem, L->ptr, L->col,
@@ -1539,9 +1896,7 @@ static sph_rt_status coarsen(sph_rt *s, SphLevel *L, SphLevel **next) {
   SPH_CUDA(s, cudaStreamSynchronize(st));
   if (ovf) {
     dfree(s, overflow);
-    for (void *p : C->owned) dfree(s, p);
-    delete C;
-    return SPH_RT_OK;  // stop coarsening here
+    return drop();
   }
   if ((rc = exclusive_scan(s, ccount, nc, C->ptr))) return rc;
   SPH_CUDA(s, cudaMemcpyAsync(&C->nnz, C->ptr + nc, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
@@ -1561,22 +1916,7 @@ static sph_rt_status coarsen(sph_rt *s, SphLevel *L, SphLevel **next) {
   dfree(s, tgt);
   dfree(s, overflow);
   if (rc) return rc;
-  // coarse values and vectors
-  C->val = lalloc<double>(s, C, C->nnz);
-  C->diag = lalloc<double>(s, C, nc);
-  C->invdiag = lalloc<double>(s, C, nc);
-  C->r = lalloc<double>(s, C, nc);
-  C->z = lalloc<double>(s, C, nc);
-  C->res = lalloc<double>(s, C, nc);
-  C->d = lalloc<double>(s, C, nc);
-  C->t = lalloc<double>(s, C, nc);
-  if (!C->val || !C->diag || !C->invdiag || !C->r || !C->z || !C->res || !C->d || !C->t)
-    return SPH_RT_ENOMEM;
-  {
-    RowShape sh = shape_for_mean(nc ? (double)C->nnz / (double)nc : 0.0);
-    C->W = sh.W;
-    C->U = sh.U;
-  }
+  if ((rc = coarse_storage(s, C))) return rc;
   *next = C;
   return SPH_RT_OK;
 }
@@ -1587,140 +1927,6 @@ static sph_rt_status level_vectors_fine(sph_rt *s, SphLevel *L) {
   L->t = lalloc<double>(s, L, L->n);
   if (!L->res || !L->d || !L->t) return SPH_RT_ENOMEM;
   (void)s;
-  return SPH_RT_OK;
-}
-
-__global__ void max_len_kernel(int64_t n, const int32_t *len, int *most) {
-  int m = 0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    m = max(m, len[i]);
-  m = __reduce_max_sync(0xffffffffu, m);
-  if ((threadIdx.x & 31) == 0) atomicMax(most, m);
-}
-
-// Slices of the finest level's A P from its CSR rows.  *again: they have no
-// dictionary within the caps, and the fine operator is back in CSR rows; A P is
-// then to be built like a coarser level's.
-static void *take_level(sph_rt *s, void *L, size_t bytes) {
-  return lvl_alloc(s, static_cast<SphLevel *>(L), bytes);
-}
-static sph_rt_status build_ap_slices(sph_rt *s, SphLevel *L, bool *again) {
-  bool ok = false;
-  sph_rt_status rc = sliced_build(s, L->n, L->ap_ptr, L->ap_col, nullptr, take_level, L, &L->ap_sl,
-                                  nullptr, &ok);
-  if (rc) return rc;
-  int *most = scratch<int>(s, 1);
-  if (!most) return SPH_RT_ENOMEM;
-  SPH_CUDA(s, cudaMemsetAsync(most, 0, sizeof(int), s->stream));
-  if (ok) {
-    max_len_kernel<<<gcap(s, L->n, kBlock), kBlock, 0, s->stream>>>(L->n, L->ap_sl.len, most);
-    SPH_LAUNCHED(s);
-  }
-  SPH_CUDA(s, cudaMemcpyAsync(&L->ap_most, most, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
-  SPH_CUDA(s, cudaStreamSynchronize(s->stream));
-  dfree(s, most);
-  if (!ok || L->ap_most >= kNoPlace) {
-    L->ap_sl = SlicedRowsData{};
-    L->ap_pos = nullptr;
-    *again = true;
-    return sliced_undo(s);
-  }
-  const size_t size = (size_t)L->ap_sl.padded + 1;
-  if (s->cfg.precision == SPH_RT_MIXED)
-    L->ap_val32 = lalloc<float>(s, L, size);
-  else
-    L->ap_val = lalloc<double>(s, L, size);
-  return L->ap_val || L->ap_val32 ? SPH_RT_OK : SPH_RT_ENOMEM;
-}
-
-// structure of A P on the finest level (see ap_structure_kernel)
-static sph_rt_status build_ap(sph_rt *s, size_t l) {
-  SphLevel *L = s->levels[l];
-  const int64_t n = L->n;
-  int32_t *tmp = scratch<int32_t>(s, (size_t)(L->nnz + n));
-  int64_t *cnt = scratch<int64_t>(s, (size_t)n + 1);
-  // target A P entry of each source: off-diagonal entries, then the diagonals
-  int32_t *map = scratch<int32_t>(s, (size_t)(L->nnz + n));
-  L->ap_ptr = lalloc<int64_t>(s, L, n + 1);
-  if (!tmp || !cnt || !map || !L->ap_ptr) return SPH_RT_ENOMEM;
-  int32_t *dmap = map + L->nnz;
-  int *ovf = scratch<int>(s, 1);
-  if (!ovf) return SPH_RT_ENOMEM;
-  SPH_CUDA(s, cudaMemsetAsync(ovf, 0, sizeof(int), s->stream));
-  ap_structure_warp_kernel<<<gcap(s, n, kWarpsPerBlock), kBlock, 0, s->stream>>>(
-      n, L->ptr, L->col, L->agg, tmp, cnt, map, dmap, ovf);
-  SPH_LAUNCHED(s);
-  int h_ovf = 0;
-  SPH_CUDA(s, cudaMemcpyAsync(&h_ovf, ovf, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
-  SPH_CUDA(s, cudaStreamSynchronize(s->stream));
-  dfree(s, ovf);
-  if (h_ovf) {  // a row with more distinct aggregates than the warp keeps: one thread a row
-    ap_structure_kernel<<<gcap(s, n, kBlock), kBlock, 0, s->stream>>>(n, L->ptr, L->col, L->agg,
-                                                                      tmp, cnt, map, dmap);
-    SPH_LAUNCHED(s);
-  }
-  sph_rt_status rc;
-  const bool sliced = l == 0 && s->sl.ptr != nullptr;
-  if (sliced) {  // the relative places, before they are made absolute
-    L->ap_pos = lalloc<uint16_t>(s, L, (size_t)s->sl.padded + 1);
-    if (!L->ap_pos) return SPH_RT_ENOMEM;
-    if ((rc = sliced_places(s, map, L->ap_pos))) return rc;
-  }
-  if ((rc = exclusive_scan(s, cnt, n, L->ap_ptr))) return rc;
-  int64_t total = 0;
-  SPH_CUDA(s, cudaMemcpyAsync(&total, L->ap_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost,
-                              s->stream));
-  SPH_CUDA(s, cudaStreamSynchronize(s->stream));
-  if (total >= ((int64_t)1 << 31)) return set_error(s, SPH_RT_EINVAL, "A P too large");
-  L->nnz_ap = total;
-  L->ap_col = lalloc<int32_t>(s, L, (size_t)total);
-  if (!L->ap_col) return SPH_RT_ENOMEM;
-  ap_compact_kernel<<<gcap(s, n, kBlock), kBlock, 0, s->stream>>>(n, L->ptr, tmp, L->ap_ptr,
-                                                                  L->ap_col, map, dmap);
-  SPH_LAUNCHED(s);
-  bool again = false;
-  if (sliced && (rc = build_ap_slices(s, L, &again))) return rc;
-  if (!sliced || again) {
-    L->ap_val = lalloc<double>(s, L, (size_t)total);
-    if (!L->ap_val) return SPH_RT_ENOMEM;
-    if (s->cfg.precision == SPH_RT_MIXED && !(L->ap_val32 = lalloc<float>(s, L, (size_t)total)))
-      return SPH_RT_ENOMEM;
-    // sources of each A P entry in increasing source order
-    if ((rc = source_sort(s, L, L->nnz + n, map, total, &L->ap_seg_ptr, &L->ap_seg_src)))
-      return rc;
-  }
-  // next level's Galerkin sources: the A P entries of its members' rows, numbered
-  // as they are stored
-  SphLevel *C = s->levels[l + 1];
-  const int64_t stored = L->ap_sl.ptr ? L->ap_sl.padded : total;
-  int32_t *tgt = scratch<int32_t>(s, (size_t)stored + 1);
-  int *missing = scratch<int>(s, 1);
-  if (!tgt || !missing) return SPH_RT_ENOMEM;
-  SPH_CUDA(s, cudaMemsetAsync(missing, 0, sizeof(int), s->stream));
-  if (L->ap_sl.ptr) {
-    fill_i32_kernel<<<gcap(s, stored, kBlock), kBlock, 0, s->stream>>>(stored, -1, tgt);
-    SPH_LAUNCHED(s);
-    ap_sliced_target_kernel<<<gcap(s, n, kBlock), kBlock, 0, s->stream>>>(
-        n, L->ap_ptr, L->ap_col, L->ap_sl, L->agg, C->nnz, C->ptr, C->col, tgt, missing);
-  } else {
-    ap_galerkin_target_kernel<<<gcap(s, n, kBlock), kBlock, 0, s->stream>>>(
-        n, L->ap_ptr, L->ap_col, L->agg, C->nnz, C->ptr, C->col, tgt, missing);
-  }
-  SPH_LAUNCHED(s);
-  if ((rc = bucket_sort<int32_t>(s, L, stored, tgt, C->nnz + C->n, &L->apg_ptr, &L->apg_src,
-                                 nullptr)))
-    return rc;
-  int miss = 0;
-  SPH_CUDA(s, cudaMemcpyAsync(&miss, missing, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
-  SPH_CUDA(s, cudaStreamSynchronize(s->stream));
-  dfree(s, tgt);
-  dfree(s, missing);
-  if (miss) return set_error(s, SPH_RT_EDEVICE, "A P entry outside the coarse sparsity");
-  SPH_CUDA(s, cudaStreamSynchronize(s->stream));
-  dfree(s, tmp);
-  dfree(s, cnt);
-  dfree(s, map);
   return SPH_RT_OK;
 }
 
@@ -1751,9 +1957,27 @@ static sph_rt_status build_structure(sph_rt *s, double *csr) {
     if (!C) break;
     s->levels.push_back(C);
     // numeric Galerkin product for C so that the next strength test can run
-    if ((rc = launch_galerkin<double>(s, C->nnz, C->n, L->seg_ptr, L->seg_src, L->nnz, L->val,
-                                      L->diag, C->val, C->diag, C->invdiag)))
+    if (L->apg_ptr) {
+      // A P in FP64 (scratch where the mixed form keeps it in FP32 only), then P^T (A P)
+      const int64_t stored = L->ap_sl.ptr ? L->ap_sl.padded : L->nnz_ap;
+      double *ap = L->ap_val ? L->ap_val : scratch<double>(s, (size_t)stored + 1);
+      if (!ap) return SPH_RT_ENOMEM;
+      rc = L->ap_sl.ptr ? sliced_ap_values<double>(s, L->ap_pos, L->agg, L->ap_sl, L->ap_most,
+                                                   s->sl_val, L->diag, ap)
+                        : launch_galerkin<double>(s, L->nnz_ap, 0, L->ap_seg_ptr, L->ap_seg_src,
+                                                  L->nnz, L->val, L->diag, ap, nullptr, nullptr);
+      if (rc) return rc;
+      if ((rc = launch_galerkin<double>(s, C->nnz, C->n, L->apg_ptr, SrcList{L->apg_src, nullptr},
+                                        stored, ap, nullptr, C->val, C->diag, C->invdiag)))
+        return rc;
+      if (!L->ap_val) {
+        SPH_CUDA(s, cudaStreamSynchronize(s->stream));
+        dfree(s, ap);
+      }
+    } else if ((rc = launch_galerkin<double>(s, C->nnz, C->n, L->seg_ptr, L->seg_src, L->nnz,
+                                             L->val, L->diag, C->val, C->diag, C->invdiag))) {
       return rc;
+    }
     L = C;
   }
   s->amg_ready = true;
@@ -1946,11 +2170,6 @@ sph_rt_status amg_setup(sph_rt *s) {
       tail_setup<float>(s);
     else
       tail_setup<double>(s);
-    // A P of the levels larger than the tail threshold: the smaller ones
-    // post-smooth the same way with or without the cluster tail, so both give
-    // bitwise the same V-cycle
-    for (size_t l = 0; l + 1 < s->levels.size() && s->levels[l]->nnz > kTailMaxNnz; ++l)
-      if ((rc = build_ap(s, l))) return rc;
     if (csr) {
       SPH_CUDA(s, cudaStreamSynchronize(s->stream));
       dfree(s, csr);
