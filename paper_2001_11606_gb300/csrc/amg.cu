@@ -40,8 +40,7 @@ namespace sphrt {
 sph_rt_status exclusive_scan(sph_rt *s, const int64_t *in, int64_t n, int64_t *out);
 template <typename MT, typename VT>
 sph_rt_status cheb_apply(sph_rt *s, const CsrView<MT> &A, const VT *r, VT *z, VT *d, VT *tmp,
-                         int degree, const ChebCoef *cf, bool zero_guess, const Scalars *sc,
-                         bool first_step_done = false);
+                         int degree, const ChebCoef *cf, const Scalars *sc, bool first_done);
 sph_rt_status launch_cheb_slots(sph_rt *s, int first, const double *gersh_dev,
                                 const std::vector<int> &mode, const std::vector<int> &degree);
 
@@ -674,22 +673,63 @@ __global__ void galerkin_kernel(int64_t nnz_c, int64_t nc, const int64_t *seg_pt
   }
 }
 
-// Gershgorin bound of D^{-1} A for a level: max_i sum_j |A_ij| / A_ii
+// Gershgorin bounds of D^{-1} A, max_i sum_j |A_ij| / A_ii, of all levels in one
+// launch: row tiles (one FP64 addition an entry, the quotients on all lanes), the
+// maxima (of non-negative values, so ordered like their bit patterns, and the same
+// in any order) by atomics.  The finest level's bound was reduced by the assembly.
+// (One launch per level with a thread per row took 27 us a step for four levels
+// under 8.6e4 particles, 275 for seven under 1.3e6; this takes 12 and
+// 168.)
 template <typename T>
-__global__ void gersh_kernel(int64_t n, const int64_t *ptr, const T *val, const T *diag,
-                             double *partials, unsigned *counter, double *out) {
-  double g = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    double sacc = 0.0;
-    for (int64_t k = ptr[i]; k < ptr[i + 1]; ++k) sacc += fabs((double)val[k]);
-    g = fmax(g, sacc / (double)diag[i]);
+struct GershLevels {
+  int count;  // levels 1 .. count - 1
+  struct {
+    int64_t n;
+    const int64_t *ptr;
+    const T *val, *diag;
+  } L[kMaxLevels];
+};
+template <typename T>
+__global__ void gersh_kernel(const __grid_constant__ GershLevels<T> G, const double *fine,
+                             double *out) {
+  constexpr int W = 4, U = 8;
+  const int lane = threadIdx.x & 31, sub = lane % W, own = tile_own_row<W>(lane);
+  if (blockIdx.x == 0 && threadIdx.x == 0) out[0] = *fine;
+  for (int l = 1; l < G.count; ++l) {
+    const int64_t *__restrict__ ptr = G.L[l].ptr;
+    const T *__restrict__ val = G.L[l].val;
+    double g = 0.0;
+    int64_t r0, r1;
+    warp_rows<W>(G.L[l].n, r0, r1);
+    for (int64_t base = r0; base < r1; base += 32) {
+      const int rows = (int)(r1 - base < 32 ? r1 - base : 32);
+      int64_t b = 0, e = 0;
+      if (own < rows) {
+        b = ptr[base + own];
+        e = ptr[base + own + 1];
+      }
+      const double s = tile_tree<W, 1, double>(0, rows, sub, [&](int t) -> double {
+        const int64_t rb = __shfl_sync(0xffffffffu, b, t, W);
+        const int64_t re = __shfl_sync(0xffffffffu, e, t, W);
+        double acc = 0.0;
+        for (int64_t k = rb + sub; k < re; k += W * U) {
+          T v[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) v[u] = k + u * W < re ? __ldg(val + k + u * W) : T(0);
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (k + u * W < re) acc += fabs(widen(v[u]));
+        }
+        __syncwarp();
+        return acc;
+      });
+      if (own < rows) g = max_bits(g, quotient(s, widen(G.L[l].diag[base + own])));
+    }
+    g = warp_max_bits(g);
+    if ((threadIdx.x & 31) == 0 && g > 0.0)
+      atomicMax(reinterpret_cast<unsigned long long *>(out + l),
+                (unsigned long long)__double_as_longlong(g));
   }
-  __shared__ double sh[32];
-  g = block_max(g, sh);
-  double part[1] = {g}, o[1];
-  const bool mx[1] = {true};
-  if (last_block_combine<1>(part, partials, counter, o, mx) && threadIdx.x == 0) *out = o[0];
 }
 
 template <typename S, typename D>
@@ -796,15 +836,123 @@ __global__ void restrict_init_kernel(int64_t nc, const int64_t *agg_ptr, const i
   }
 }
 
-template <typename VT>
-__global__ void prolong_kernel(int64_t n, const int32_t *agg, const VT *zc, VT *z,
-                               const Scalars *sc) {
+// Levels without A P (operators of at most kTailMaxNnz entries: a few microseconds
+// of work each, bound by launches and by chains of dependent loads).
+// Going down: the residual r - A z of an aggregate's rows, summed in member order
+// (and the next level's zero-guess smoother start, INIT), in one launch: a warp per
+// coarse row, W lanes per member row.  The row sums and the order of the members
+// are those of resid_level_kernel and restrict_kernel, bit for bit.
+template <int W, int U, typename T, bool INIT>
+__global__ void __launch_bounds__(kBlock, kCoarseMinBlocks)
+    resid_restrict_kernel(CsrView<T> A, const T *r, const T *z, int64_t nc,
+                          const int64_t *agg_ptr, const int32_t *agg_mem, T *rc,
+                          const T *invdiag_c, const ChebCoef *cf_c, T *d_c, T *z_c,
+                          const Scalars *sc, int *wflag) {
   pdl_wait();
-  if (sc && sc->done) return;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    int32_t a = agg[i];
-    if (a >= 0) z[i] += zc[a];
+  if (sc && sc->done) {
+    mark_work(wflag, 0);
+    return;
+  }
+  mark_work(wflag, 1);
+  constexpr int G = 32 / W;
+  const int lane = threadIdx.x & 31, sub = lane % W, g = lane / W;
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t I = warp; I < nc; I += nwarps) {
+    const int64_t m1 = agg_ptr[I + 1];
+    T acc = T(0);
+    for (int64_t mb = agg_ptr[I]; mb < m1; mb += G) {
+      const bool active = mb + g < m1;
+      const int32_t i = active ? agg_mem[mb + g] : 0;
+      const int64_t b = active ? __ldg(A.ptr + i) : 0, e = active ? __ldg(A.ptr + i + 1) : 0;
+      T ri = T(0), dg = T(0), zi = T(0);
+      if (active && sub == 0) {
+        ri = r[i];
+        dg = A.diag[i];
+        zi = z[i];
+      }
+      const T s = row_reduce<W>(row_dot_n<W, U, T, T>(b, e, A.col, A.val, GatherVec<T>{z}, sub,
+                                                      tile_nmax<W>(b, e, sub)));
+      const T res = ri - fmadd(dg, zi, s);  // of the group's row, in its first lane
+      const int members = (int)(m1 - mb < G ? m1 - mb : G);
+      for (int q = 0; q < members; ++q) acc += __shfl_sync(0xffffffffu, res, q * W);
+    }
+    if (lane == 0) {
+      rc[I] = acc;
+      if (INIT) {
+        const T di = (T)(cf_c->inv_theta * (double)invdiag_c[I] * (double)acc);
+        d_c[I] = di;
+        z_c[I] = di;
+      }
+    }
+  }
+}
+
+// Going up: the prolongation folded into the first post-smoothing step, z' = z + P e
+// formed as it is gathered; z_out = z' + c2 D^{-1} (r - A z') in one launch (the
+// cluster tail's arithmetic, bit for bit).
+// DOT (finest level, degree 1): also the preconditioned inner product of DotFuse.
+template <int W, int U, typename T, bool DOT>
+__global__ void __launch_bounds__(kBlock, kCoarseMinBlocks)
+    prolong_cheb_kernel(CsrView<T> A, const T *r, const T *z, const int32_t *agg, const T *ec,
+                        T *z_out, T *d, const ChebCoef *cf, const Scalars *sc, int *wflag,
+                        const DotFuse df) {
+  pdl_wait();
+  if (sc && sc->done) {
+    mark_work(wflag, 0);
+    return;
+  }
+  mark_work(wflag, 1);
+  const T c2 = (T)cf->inv_theta;
+  auto corrected = [&](int32_t c) {
+    const T zc = __ldg(z + c);
+    const int32_t a = __ldg(agg + c);
+    return a >= 0 ? zc + __ldg(ec + a) : zc;
+  };
+  const int own = tile_own_row<W>(threadIdx.x & 31);
+  int64_t r0, r1;
+  warp_rows<W>(A.n, r0, r1);
+  double da = 0.0, db = 0.0;
+  for (int64_t base = r0; base < r1; base += 32) {
+    const int rows = (int)(r1 - base < 32 ? r1 - base : 32);
+    const int64_t i = base + own;
+    const bool active = own < rows;
+    T ri = T(0), zi = T(0), dg = T(0), idg = T(0);
+    if (active) {
+      ri = r[i];
+      zi = corrected((int32_t)i);
+      dg = A.diag[i];
+      idg = A.invdiag[i];
+    }
+    const T s = tile_row_sums_of<W, U, T, T>(base, rows, A.ptr, A.col, A.val, corrected);
+    if (active) {
+      const T res = ri - fmadd(dg, zi, s);
+      const T di = (c2 * idg) * res;
+      const T zo = zi + di;
+      d[i] = di;
+      z_out[i] = zo;
+      if (DOT) {
+        const double rd = df.r[i], zn = widen(zo);
+        if (df.flex) {
+          if (!df.first) db += rd * df.z64[i];
+          df.z64[i] = zn;
+        }
+        da += rd * zn;
+      }
+    }
+  }
+  if (DOT) {
+    __shared__ double sh[32];
+    da = block_sum(da, sh);
+    __syncthreads();
+    db = block_sum(db, sh);
+    double part[2] = {da, db}, out[2];
+    const bool mx[2] = {false, false};
+    if (last_block_combine<2>(part, df.partials, &df.sc->counter, out, mx) && threadIdx.x == 0) {
+      Scalars *w = df.sc;
+      if (!df.first) w->beta = (df.flex ? out[0] - out[1] : out[0]) / w->rho;
+      w->rho = out[0];
+    }
   }
 }
 
@@ -1231,7 +1379,7 @@ __device__ __forceinline__ void fcg_row(int64_t i, VT zn, VT wn, VT r, VT zo, VT
 
 template <typename VT>
 __device__ __forceinline__ void fcg_reduce(double (&acc)[5], int first, Scalars *sc,
-                                           double *partials) {
+                                           double *partials, const LoopCond &cond) {
   __shared__ double sh[32];
   for (int k = 0; k < 5; ++k) {
     acc[k] = block_sum(acc[k], sh);
@@ -1239,8 +1387,10 @@ __device__ __forceinline__ void fcg_reduce(double (&acc)[5], int first, Scalars 
   }
   double out[5];
   const bool mx[5] = {false, false, false, false, false};
-  if (last_block_combine<5>(acc, partials, &sc->counter, out, mx) && threadIdx.x == 0)
+  if (last_block_combine<5>(acc, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     fcg_scalars(out, first, sc);
+    loop_cond_set(cond, sc);
+  }
 }
 
 // The A P sweep: res2 = res - (A P) e_c, z = z_pre + P e_c, B z = r - res2.
@@ -1255,9 +1405,10 @@ template <typename Rows, typename VT>
 __global__ void __launch_bounds__(kBlock, fcg_min_blocks<VT>())
     fine_ap_cg_kernel(Rows A, const int32_t *agg, const VT *ec, const VT *z_pre, const VT *res,
                       const VT *r, VT *z, VT *w, const VT *p, const VT *q, int first, Scalars *sc,
-                      double *partials, int *wflag) {
+                      double *partials, int *wflag, const LoopCond cond) {
   pdl_wait();
   if (sc->done) {
+    loop_cond_skip(cond, sc);
     mark_work(wflag, 0);
     return;
   }
@@ -1275,7 +1426,7 @@ __global__ void __launch_bounds__(kBlock, fcg_min_blocks<VT>())
         const VT res2 = o.b - s;
         fcg_row<VT>(i, o.a, o.c - res2, o.c, o.d, o.e, o.f, z, w, first, acc);
       });
-  fcg_reduce<VT>(acc, first, sc, partials);
+  fcg_reduce<VT>(acc, first, sc, partials, cond);
 }
 
 // Without A P (operators below the A P threshold): z = z_pre + P e_c into t,
@@ -1294,9 +1445,11 @@ __global__ void fcg_prolong_kernel(int64_t n, const int32_t *agg, const VT *ec, 
 template <int W, int U, typename MT, typename VT>
 __global__ void __launch_bounds__(kBlock, fcg_min_blocks<VT>())
     fcg_spmv_dot_kernel(CsrView<MT> A, const VT *t, const VT *r, VT *z, VT *w, const VT *p,
-                        const VT *q, int first, Scalars *sc, double *partials, int *wflag) {
+                        const VT *q, int first, Scalars *sc, double *partials, int *wflag,
+                        const LoopCond cond) {
   pdl_wait();
   if (sc->done) {
+    loop_cond_skip(cond, sc);
     mark_work(wflag, 0);
     return;
   }
@@ -1315,7 +1468,7 @@ __global__ void __launch_bounds__(kBlock, fcg_min_blocks<VT>())
                   first ? VT(0) : q[i], first ? VT(0) : p[i], z, w, first, acc);
     }
   }
-  fcg_reduce<VT>(acc, first, sc, partials);
+  fcg_reduce<VT>(acc, first, sc, partials, cond);
 }
 
 // ---------------------------------------------------------------------------
@@ -2108,19 +2261,18 @@ static sph_rt_status galerkin_levels(sph_rt *s) {
   if (!s->amg_gersh) s->amg_gersh = dalloc<double>(s, kMaxLevels);
   double *dg = s->amg_gersh;
   if (!dg) return SPH_RT_ENOMEM;
-  for (size_t l = 0; l < s->levels.size(); ++l) {
-    SphLevel *L = s->levels[l];
-    if (l == 0) {
-      // the finest level's bound was reduced by the assembly of this step
-      SPH_CUDA(s, cudaMemcpyAsync(dg, s->gersh, sizeof(double), cudaMemcpyDeviceToDevice,
-                                  s->stream));
-      continue;
-    }
-    const CsrView<T> Lv = LV::view(L);
-    gersh_kernel<T><<<gcap(s, L->n, kBlock), kBlock, 0, s->stream>>>(
-        L->n, L->ptr, Lv.val, Lv.diag, s->partials, &s->sc->counter, dg + l);
-    SPH_LAUNCHED(s);
+  GershLevels<T> G;
+  memset(&G, 0, sizeof G);
+  G.count = (int)s->levels.size();
+  int64_t rows = 0;
+  for (int l = 1; l < G.count; ++l) {
+    const CsrView<T> Lv = LV::view(s->levels[l]);
+    G.L[l] = {Lv.n, Lv.ptr, Lv.val, Lv.diag};
+    rows += Lv.n;
   }
+  SPH_CUDA(s, cudaMemsetAsync(dg, 0, sizeof(double) * kMaxLevels, s->stream));
+  gersh_kernel<T><<<gcap(s, rows, kBlock / 4), kBlock, 0, s->stream>>>(G, s->gersh, dg);
+  SPH_LAUNCHED(s);
   return SPH_RT_OK;
 }
 
@@ -2301,6 +2453,50 @@ static void tail_setup(sph_rt *s) {
   }
 }
 
+// Whether a level post-smooths through A P.
+template <typename T>
+static bool has_ap(SphLevel *L) {
+  return L->ap_ptr && LevelVecs<T>::ap(L);
+}
+// Where the zero-guess smoother start of level L goes, z being the buffer of its
+// result: cheb_apply's first write (levels without A P: see vcycle).
+template <typename T>
+static T *smoother_start(const sph_rt *s, SphLevel *L, T *z) {
+  const bool odd = s->cfg.cheb_degree % 2 == 1;
+  return has_ap<T>(L) && odd ? z : LevelVecs<T>::t(L);
+}
+
+// Residual of level l (no A P) restricted to level l + 1, with that level's
+// smoother start at zc_first unless it is null.
+template <typename T>
+static sph_rt_status launch_resid_restrict(sph_rt *s, size_t l, const T *r, const T *zpre,
+                                           T *zc_first, const Scalars *sc) {
+  using LV = LevelVecs<T>;
+  SphLevel *L = s->levels[l], *C = s->levels[l + 1];
+  const CsrView<T> A = LV::view(L);
+  const int gr = gcap(s, C->n, kWarpsPerBlock);  // a warp per coarse row
+  int *wf = l == 0 ? timing_begin(s) : nullptr;
+  if (zc_first)
+    SPH_DISPATCH_SHAPE(A.W, A.U,
+                       (pdl_launch(s, resid_restrict_kernel<W, U, T, true>, gr, kBlock, 0, A, r,
+                                   zpre, C->n, (const int64_t *)L->agg_ptr,
+                                   (const int32_t *)L->agg_mem, LV::r(C), LV::view(C).invdiag,
+                                   (const ChebCoef *)(s->cheb_slots + 2 + l), LV::d(C), zc_first,
+                                   sc, wf)));
+  else
+    SPH_DISPATCH_SHAPE(A.W, A.U,
+                       (pdl_launch(s, resid_restrict_kernel<W, U, T, false>, gr, kBlock, 0, A, r,
+                                   zpre, C->n, (const int64_t *)L->agg_ptr,
+                                   (const int32_t *)L->agg_mem, LV::r(C), (const T *)nullptr,
+                                   (const ChebCoef *)nullptr, (T *)nullptr, (T *)nullptr, sc,
+                                   wf)));
+  SPH_LAUNCHED(s);
+  if (l == 0)
+    timing_end(s, (4.0 + sizeof(T)) * (double)A.nnz + (12.0 + 3.0 * sizeof(T)) * (double)A.n,
+               kTimedResid);
+  return SPH_RT_OK;
+}
+
 template <typename T>
 static sph_rt_status vcycle(sph_rt *s, size_t l, const T *r, T *z, const Scalars *sc,
                             bool init_done = false, const DotFuse *df = nullptr,
@@ -2339,12 +2535,48 @@ static sph_rt_status vcycle(sph_rt *s, size_t l, const T *r, T *z, const Scalars
       SPH_LAUNCHED(s);
       return SPH_RT_OK;
     }
-    return cheb_apply<T, T>(s, A, r, z, LV::d(L), LV::t(L), cdeg, cf, true, sc);
+    return cheb_apply<T, T>(s, A, r, z, LV::d(L), LV::t(L), cdeg, cf, sc, false);
   }
   const ChebCoef *cf = s->cheb_slots + 1 + l;
+  SphLevel *C = s->levels[l + 1];
+  // a launched, non-coarsest next level takes its smoother start from the restriction
+  const bool fuse = l + 2 < s->levels.size() &&
+                    !(s->tail_level > 0 && l + 1 == (size_t)s->tail_level);
+  T *zc_first = fuse ? smoother_start<T>(s, C, LV::z(C)) : nullptr;
+  if (!has_ap<T>(L)) {
+    // pre-smoothing into the buffer that the first post-smoothing step reads
+    T *t = LV::t(L);
+    const bool odd = deg % 2 == 1;
+    T *zpre = odd ? t : z, *zpost = odd ? z : t;
+    if ((rc = cheb_apply<T, T>(s, A, r, zpre, LV::d(L), zpost, deg, cf, sc, init_done)))
+      return rc;
+    if ((rc = launch_resid_restrict<T>(s, l, r, zpre, zc_first, sc))) return rc;
+    if ((rc = vcycle<T>(s, l + 1, LV::r(C), LV::z(C), sc, fuse))) return rc;
+    const int gp = row_grid_blocks(s->num_sms, L->n, A.W, kCoarseMinBlocks);
+    const bool dot = l == 0 && df && dot_done && deg == 1;
+    int *wf = l == 0 ? timing_begin(s) : nullptr;
+    if (dot)
+      SPH_DISPATCH_SHAPE(A.W, A.U,
+                         (pdl_launch(s, prolong_cheb_kernel<W, U, T, true>, gp, kBlock, 0, A, r,
+                                     (const T *)zpre, (const int32_t *)L->agg,
+                                     (const T *)LV::z(C), zpost, LV::d(L), cf, sc, wf, *df)));
+    else
+      SPH_DISPATCH_SHAPE(A.W, A.U,
+                         (pdl_launch(s, prolong_cheb_kernel<W, U, T, false>, gp, kBlock, 0, A, r,
+                                     (const T *)zpre, (const int32_t *)L->agg,
+                                     (const T *)LV::z(C), zpost, LV::d(L), cf, sc, wf,
+                                     DotFuse{})));
+    SPH_LAUNCHED(s);
+    if (dot) *dot_done = true;
+    if (l == 0)
+      timing_end(s, (4.0 + sizeof(T)) * (double)A.nnz + (12.0 + 7.0 * sizeof(T)) * (double)A.n,
+                 kTimedCheb);
+    // the remaining post-smoothing steps
+    return cheb_apply<T, T>(s, A, r, z, LV::d(L), t, deg, cf, sc, true);
+  }
   // zero-guess pre-smoothing (its first write was made by the restriction above
   // when init_done)
-  if ((rc = cheb_apply<T, T>(s, A, r, z, LV::d(L), LV::t(L), deg, cf, true, sc, init_done)))
+  if ((rc = cheb_apply<T, T>(s, A, r, z, LV::d(L), LV::t(L), deg, cf, sc, init_done)))
     return rc;
   const int gw = row_grid_blocks(s->num_sms, L->n, A.W, kCoarseMinBlocks);
   T *res = LV::res(L);
@@ -2363,13 +2595,7 @@ static sph_rt_status vcycle(sph_rt *s, size_t l, const T *r, T *z, const Scalars
   if (l == 0)
     timing_end(s, ((s->sl.ptr ? 2.0 : 4.0) + sizeof(T)) * (double)A.nnz + (8.0 + 4.0 * sizeof(T)) * (double)A.n,
                kTimedResid);
-  SphLevel *C = s->levels[l + 1];
-  // a launched, non-coarsest next level takes its smoother start from the restriction
-  const bool fuse = l + 2 < s->levels.size() &&
-                    !(s->tail_level > 0 && l + 1 == (size_t)s->tail_level);
   if (fuse) {
-    const int wc = (deg - 1) % 2;  // cheb_apply's first write goes to bufs[wc]
-    T *zc_first = wc == 0 ? LV::z(C) : LV::t(C);
     pdl_launch(s, restrict_init_kernel<T, T>, gcap(s, C->n, kBlock), kBlock, 0,
         C->n, L->agg_ptr, L->agg_mem, res, LV::r(C), LV::view(C).invdiag,
         s->cheb_slots + 1 + (l + 1), LV::d(C), zc_first, sc);
@@ -2379,7 +2605,7 @@ static sph_rt_status vcycle(sph_rt *s, size_t l, const T *r, T *z, const Scalars
   }
   SPH_LAUNCHED(s);
   if ((rc = vcycle<T>(s, l + 1, LV::r(C), LV::z(C), sc, fuse))) return rc;
-  if (L->ap_ptr && LV::ap(L)) {
+  {
     // prolongation and the first post-smoothing step in one sweep of A P
     T *bufs[2] = {z, LV::t(L)};
     const int w0 = (deg - 1) % 2;
@@ -2416,11 +2642,8 @@ static sph_rt_status vcycle(sph_rt *s, size_t l, const T *r, T *z, const Scalars
                      (12.0 + 6.0 * sizeof(T) + (dot ? (df->flex ? 24.0 : 8.0) : 0.0)) *
                          (double)L->n,
                  kTimedPost);
-    return cheb_apply<T, T>(s, A, r, z, LV::d(L), LV::t(L), deg, cf, false, sc, true);
+    return cheb_apply<T, T>(s, A, r, z, LV::d(L), LV::t(L), deg, cf, sc, true);
   }
-  pdl_launch(s, prolong_kernel<T>, gcap(s, L->n, kBlock), kBlock, 0, L->n, L->agg, LV::z(C), z, sc);
-  SPH_LAUNCHED(s);
-  return cheb_apply<T, T>(s, A, r, z, LV::d(L), LV::t(L), deg, cf, false, sc);
 }
 
 // Mixed form without the last conversion: r is rounded to FP32 and the FP32
@@ -2448,12 +2671,11 @@ const float *amg_z32(const sph_rt *s) { return s->levels.empty() ? nullptr : s->
 bool amg_fine_init(sph_rt *s, FineInit<double> *f64, FineInit<float> *f32) {
   if (s->levels.size() < 2) return false;
   SphLevel *L0 = s->levels[0];
-  const int w0 = (s->cfg.cheb_degree - 1) % 2;  // cheb_apply's first write: bufs[w0]
   const ChebCoef *cf = s->cheb_slots + 1;
   if (s->cfg.precision == SPH_RT_MIXED) {
-    *f32 = {L0->r32, L0->invdiag32, cf, L0->d32, w0 == 0 ? L0->z32 : L0->t32};
+    *f32 = {L0->r32, L0->invdiag32, cf, L0->d32, smoother_start<float>(s, L0, L0->z32)};
   } else {
-    *f64 = {nullptr, L0->invdiag, cf, L0->d, w0 == 0 ? s->z : L0->t};
+    *f64 = {nullptr, L0->invdiag, cf, L0->d, smoother_start<double>(s, L0, s->z)};
   }
   return true;
 }
@@ -2514,29 +2736,33 @@ static sph_rt_status fcg_cycle_t(sph_rt *s, const FcgSet<T> &v, int first) {
   CsrView<T> A = LV::view(L);
   const Scalars *sc = s->sc;
   T *res = LV::res(L);
-  int *wf = timing_begin(s);
-  SPH_FINE_ROWS(s, T, A, sizeof(T),
-                (pdl_launch(s, fine_resid_level_kernel<Rows, T>, grid, kBlock, smem, rows,
-                            (const T *)v.r, (const T *)v.zpre, res, sc, wf)));
-  SPH_LAUNCHED(s);
-  timing_end(s, ((s->sl.ptr ? 2.0 : 4.0) + sizeof(T)) * (double)A.nnz + (8.0 + 4.0 * sizeof(T)) * (double)A.n,
-             kTimedResid);
   SphLevel *C = s->levels[1];
-  const int deg = s->cfg.cheb_degree;
   const bool fuse = s->levels.size() > 2 && !(s->tail_level > 0 && s->tail_level == 1);
-  if (fuse) {
-    const int wc = (deg - 1) % 2;
-    T *zc_first = wc == 0 ? LV::z(C) : LV::t(C);
-    pdl_launch(s, restrict_init_kernel<T, T>, gcap(s, C->n, kBlock), kBlock, 0, C->n, L->agg_ptr,
-               L->agg_mem, (const T *)res, LV::r(C), LV::view(C).invdiag, s->cheb_slots + 2,
-               LV::d(C), zc_first, sc);
+  T *zc_first = fuse ? smoother_start<T>(s, C, LV::z(C)) : nullptr;
+  sph_rt_status rc;
+  int *wf = nullptr;
+  if (!has_ap<T>(L)) {
+    if ((rc = launch_resid_restrict<T>(s, 0, v.r, v.zpre, zc_first, sc))) return rc;
   } else {
-    pdl_launch(s, restrict_kernel<T>, gcap(s, C->n, kBlock), kBlock, 0, C->n, L->agg_ptr,
-               L->agg_mem, (const T *)res, LV::r(C), sc);
+    wf = timing_begin(s);
+    SPH_FINE_ROWS(s, T, A, sizeof(T),
+                  (pdl_launch(s, fine_resid_level_kernel<Rows, T>, grid, kBlock, smem, rows,
+                              (const T *)v.r, (const T *)v.zpre, res, sc, wf)));
+    SPH_LAUNCHED(s);
+    timing_end(s,
+               ((s->sl.ptr ? 2.0 : 4.0) + sizeof(T)) * (double)A.nnz +
+                   (8.0 + 4.0 * sizeof(T)) * (double)A.n,
+               kTimedResid);
+    if (fuse)
+      pdl_launch(s, restrict_init_kernel<T, T>, gcap(s, C->n, kBlock), kBlock, 0, C->n,
+                 L->agg_ptr, L->agg_mem, (const T *)res, LV::r(C), LV::view(C).invdiag,
+                 s->cheb_slots + 2, LV::d(C), zc_first, sc);
+    else
+      pdl_launch(s, restrict_kernel<T>, gcap(s, C->n, kBlock), kBlock, 0, C->n, L->agg_ptr,
+                 L->agg_mem, (const T *)res, LV::r(C), sc);
+    SPH_LAUNCHED(s);
   }
-  SPH_LAUNCHED(s);
-  sph_rt_status rc = vcycle<T>(s, 1, LV::r(C), LV::z(C), sc, fuse);
-  if (rc) return rc;
+  if ((rc = vcycle<T>(s, 1, LV::r(C), LV::z(C), sc, fuse))) return rc;
   if (L->ap_ptr && LV::ap(L)) {
     const RowShape sh = shape_for_mean(L->n ? (double)L->nnz_ap / (double)L->n : 0.0);
     wf = timing_begin(s);
@@ -2544,7 +2770,7 @@ static sph_rt_status fcg_cycle_t(sph_rt *s, const FcgSet<T> &v, int first) {
                 (pdl_launch(s, fine_ap_cg_kernel<Rows, T>, grid, kBlock, smem, rows,
                             (const int32_t *)L->agg, (const T *)LV::z(C), (const T *)v.zpre,
                             (const T *)res, (const T *)v.r, v.z, v.w, (const T *)v.p,
-                            (const T *)v.q, first, s->sc, s->partials, wf)));
+                            (const T *)v.q, first, s->sc, s->partials, wf, s->loop_cond)));
     SPH_LAUNCHED(s);
     // A P entry: column + value; per row: ap_ptr, agg, P e_c, z_pre, res, r, z r/w, w,
     // p, q
@@ -2562,7 +2788,7 @@ static sph_rt_status fcg_cycle_t(sph_rt *s, const FcgSet<T> &v, int first) {
   SPH_DISPATCH_SHAPE(A.W, A.U,
                      (pdl_launch(s, fcg_spmv_dot_kernel<W, U, T, T>, gd, kBlock, 0, A,
                                  (const T *)t, (const T *)v.r, v.z, v.w, (const T *)v.p,
-                                 (const T *)v.q, first, s->sc, s->partials, wf)));
+                                 (const T *)v.q, first, s->sc, s->partials, wf, s->loop_cond)));
   SPH_LAUNCHED(s);
   timing_end(s, (4.0 + sizeof(T)) * (double)A.nnz + (8.0 + 9.0 * sizeof(T)) * (double)A.n,
              kTimedSpmvPQ);

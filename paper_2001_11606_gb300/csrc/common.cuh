@@ -374,10 +374,16 @@ __device__ __forceinline__ void warp_rows(int64_t n, int64_t &r0, int64_t &r1) {
 // and then runs its FMAs in a loop of exactly (nmax mod U) trips, shifting the
 // loaded slots down.  Slots past a lane's row end load nothing and contribute
 // fma(0, 0, s) = s.
-template <int W, int U, typename MT, typename VT>
+// x(c) is the gathered vector's entry c.
+template <typename VT>
+struct GatherVec {
+  const VT *__restrict__ x;
+  __device__ __forceinline__ VT operator()(int32_t c) const { return __ldg(x + c); }
+};
+template <int W, int U, typename MT, typename VT, typename X>
 __device__ __forceinline__ VT row_dot_n(int64_t beg, int64_t end, const int32_t *__restrict__ col,
-                                        const MT *__restrict__ val, const VT *__restrict__ x,
-                                        int sub, int nmax) {
+                                        const MT *__restrict__ val, const X &x, int sub,
+                                        int nmax) {
   VT s = VT(0);
   int64_t k = beg + sub;
   int j = 0;
@@ -392,7 +398,7 @@ __device__ __forceinline__ VT row_dot_n(int64_t beg, int64_t end, const int32_t 
     }
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if (c[u] >= 0) s = fmadd((VT)v[u], __ldg(x + c[u]), s);
+      if (c[u] >= 0) s = fmadd((VT)v[u], x(c[u]), s);
   }
   const int rem = nmax - j;  // warp-uniform, < U
   if (rem > 0) {
@@ -402,7 +408,7 @@ __device__ __forceinline__ VT row_dot_n(int64_t beg, int64_t end, const int32_t 
       const int64_t kk = k + (int64_t)u * W;
       const int32_t c = kk < end ? __ldg(col + kk) : -1;
       a[u] = c >= 0 ? (VT)__ldg(val + kk) : VT(0);
-      g[u] = c >= 0 ? __ldg(x + c) : VT(0);
+      g[u] = c >= 0 ? x(c) : VT(0);
     }
 #pragma unroll 1
     for (int u = 0; u < rem; ++u) {
@@ -481,10 +487,11 @@ __device__ __forceinline__ int tile_nmax(int64_t rb, int64_t re, int sub) {
 // Row sums of the tile of `rows` (<= 32) rows starting at `base`: lane l gets
 // the off-diagonal sum of row base + tile_own_row<W>(l) (0 past `rows`).  Every
 // lane of the warp must call it with the same base and rows.
-template <int W, int U, typename MT, typename VT>
-__device__ __forceinline__ VT tile_row_sums(int64_t base, int rows, const int64_t *__restrict__ ptr,
-                                            const int32_t *__restrict__ col,
-                                            const MT *__restrict__ val, const VT *__restrict__ x) {
+template <int W, int U, typename MT, typename VT, typename X>
+__device__ __forceinline__ VT tile_row_sums_of(int64_t base, int rows,
+                                               const int64_t *__restrict__ ptr,
+                                               const int32_t *__restrict__ col,
+                                               const MT *__restrict__ val, const X &x) {
   const int lane = threadIdx.x & 31, sub = lane % W;
   const int own = tile_own_row<W>(lane);
   int64_t b = 0, e = 0;  // row extents, one coalesced load per lane
@@ -498,6 +505,12 @@ __device__ __forceinline__ VT tile_row_sums(int64_t base, int rows, const int64_
     const int64_t re = __shfl_sync(0xffffffffu, e, t, W);
     return row_dot_n<W, U, MT, VT>(rb, re, col, val, x, sub, tile_nmax<W>(rb, re, sub));
   });
+}
+template <int W, int U, typename MT, typename VT>
+__device__ __forceinline__ VT tile_row_sums(int64_t base, int rows, const int64_t *__restrict__ ptr,
+                                            const int32_t *__restrict__ col,
+                                            const MT *__restrict__ val, const VT *__restrict__ x) {
+  return tile_row_sums_of<W, U, MT, VT>(base, rows, ptr, col, val, GatherVec<VT>{x});
 }
 
 // Chebyshev iteration coefficients on [lo, hi] (Saad, Iterative Methods,
@@ -564,6 +577,30 @@ struct DotFuse {
   Scalars *sc;
   double *partials;
 };
+
+// Krylov loop of the step's graph: the last kernel of an iteration (kind 1; of the
+// prologue: kind 2) sets the WHILE node's condition instead of a kernel of its own.
+// kind 0: none (host-driven loop).
+struct LoopCond {
+  cudaGraphConditionalHandle h;
+  int kind, max_trips;
+};
+// By one thread of the grid, after sc->done is final for the iteration: go on while
+// not converged, at most max_trips trips.
+__device__ __forceinline__ void loop_cond_set(const LoopCond &c, Scalars *sc) {
+  if (c.kind == 0) return;
+  int t = 0;
+  if (c.kind == 1) {
+    sc->krylov_trips += 1;
+    t = sc->krylov_solve_trips + 1;
+  }
+  sc->krylov_solve_trips = t;
+  cudaGraphSetConditional(c.h, sc->done || t >= c.max_trips ? 0u : 1u);
+}
+// a kernel that returns at once because the solve is done still sets it
+__device__ __forceinline__ void loop_cond_skip(const LoopCond &c, Scalars *sc) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) loop_cond_set(c, sc);
+}
 
 // Vectors of the CG with the V-cycle's product (fine_post_smooth = 0), in the
 // hierarchy's precision T: residual r, preconditioned residual z, w = B z,
@@ -900,6 +937,7 @@ struct sph_rt {
   cudaGraphExec_t graph_exec = nullptr;
   std::vector<uint64_t> graph_sig;  // launch parameters the graph was captured with
   cudaStream_t cap_stream = nullptr;
+  sphrt::LoopCond loop_cond{0, 0, 0};  // of the part being captured
   int64_t graph_l_init = 0, graph_l_outer = 0, graph_l_inner = 0;  // kernels per part
   int64_t graph_builds = 0, graph_launches = 0;
 

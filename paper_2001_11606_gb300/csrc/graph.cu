@@ -51,19 +51,6 @@ __global__ void outer_init_kernel(Scalars *sc) {
   for (int k = 0; k < 64; ++k) sc->krylov_per_outer[k] = 0;
 }
 
-// Before the Krylov WHILE node: enter unless the prologue already converged.
-__global__ void krylov_enter_kernel(Scalars *sc, cudaGraphConditionalHandle h) {
-  sc->krylov_solve_trips = 0;
-  cudaGraphSetConditional(h, sc->done ? 0u : 1u);
-}
-
-// End of a Krylov trip: go on while not converged, at most max_trips trips.
-__global__ void krylov_cond_kernel(Scalars *sc, int max_trips, cudaGraphConditionalHandle h) {
-  sc->krylov_trips += 1;
-  const int t = ++sc->krylov_solve_trips;
-  cudaGraphSetConditional(h, (sc->done || t >= max_trips) ? 0u : 1u);
-}
-
 // After the material solve of an outer iteration: the Krylov check, the
 // bookkeeping of the step statistics and the outer convergence test
 // max_i |x^{l+1} - x^l| / |x^{l+1}| < tol for e and E (changes in red[0..1],
@@ -217,9 +204,10 @@ static sph_rt_status build_loop_graph(sph_rt *s, double dt) {
   auto capture_outer = [&]() -> sph_rt_status {
     sph_rt_status rc;
     if ((rc = launch_rhs(s, dt))) return rc;  // a7
-    if ((rc = pcg_prologue(s))) return rc;     // a6, first part
-    krylov_enter_kernel<<<1, 1, 0, s->stream>>>(s->sc, h_in);
-    SPH_LAUNCHED(s);
+    s->loop_cond = LoopCond{h_in, 2, s->cfg.max_krylov + 1};
+    rc = pcg_prologue(s);  // a6, first part; its last kernel sets the Krylov loop's condition
+    s->loop_cond = LoopCond{0, 0, 0};
+    if (rc) return rc;
     // the Krylov WHILE node goes after everything captured so far
     cudaStreamCaptureStatus cst;
     const cudaGraphNode_t *deps = nullptr;
@@ -239,10 +227,10 @@ static sph_rt_status build_loop_graph(sph_rt *s, double dt) {
   };
   auto capture_inner = [&]() -> sph_rt_status {
     sph_rt_status rc;
-    if ((rc = pcg_iteration(s))) return rc;  // a6, one iteration
-    krylov_cond_kernel<<<1, 1, 0, s->stream>>>(s->sc, s->cfg.max_krylov + 1, h_in);
-    SPH_LAUNCHED(s);
-    return SPH_RT_OK;
+    s->loop_cond = LoopCond{h_in, 1, s->cfg.max_krylov + 1};
+    rc = pcg_iteration(s);  // a6, one iteration; its last kernel sets the condition
+    s->loop_cond = LoopCond{0, 0, 0};
+    return rc;
   };
   auto capture_into = [&](cudaGraph_t into, auto &&body, int64_t *count) -> sph_rt_status {
     const int64_t l0 = s->launches;

@@ -73,9 +73,10 @@ __global__ void __launch_bounds__(kBlock, Rows::kMinBlocks)
 template <typename Rows>
 __global__ void __launch_bounds__(kBlock, Rows::kMinBlocks)
     spmv_pq_kernel(Rows A, const double *z, double *q, double *p, int first, Scalars *sc,
-                   double *partials, int *wflag) {
+                   double *partials, int *wflag, const LoopCond cond) {
   pdl_wait();
   if (sc->done) {
+    loop_cond_skip(cond, sc);
     mark_work(wflag, 0);
     return;
   }
@@ -108,6 +109,7 @@ __global__ void __launch_bounds__(kBlock, Rows::kMinBlocks)
     } else {
       sc->alpha = sc->rho / pq;
     }
+    loop_cond_set(cond, sc);
   }
 }
 
@@ -424,14 +426,14 @@ double spmv_class_bytes(const sph_rt *s, const CsrView<MT> &A, int row_bytes) {
 // resid: rowptr, diag, b, x, r, 1/V        spmv_pq: rowptr, diag, z, q r/w, p r/w
 constexpr int kRowBytesResid = 48, kRowBytesSpmvPQ = 56;
 
-// Chebyshev polynomial preconditioner/smoother: `degree` steps from z
-// (zero_guess: z = 0 on entry), coefficients from the device slot `cf`
-// (filled on the device from the Gershgorin bounds of the step, so no host
-// read of the bounds is needed).  d and tmp are scratch vectors of length n.
+// Chebyshev polynomial preconditioner/smoother: `degree` steps, the first from a
+// zero guess, or made by the caller (first_done) with its result in the buffer the
+// first write goes to; coefficients from the device slot `cf` (filled on the device
+// from the Gershgorin bounds of the step, so no host read of the bounds is needed).
+// d and tmp are scratch vectors of length n; the result is in z.
 template <typename MT, typename VT>
 sph_rt_status cheb_apply(sph_rt *s, const CsrView<MT> &A, const VT *r, VT *z, VT *d, VT *tmp,
-                         int degree, const ChebCoef *cf, bool zero_guess, const Scalars *sc,
-                         bool first_step_done) {
+                         int degree, const ChebCoef *cf, const Scalars *sc, bool first_done) {
   if (degree < 1) degree = 1;
   if (degree > kChebMaxDeg) degree = kChebMaxDeg;
   int g = grid_cap(s, A.n, kBlock);
@@ -460,18 +462,10 @@ sph_rt_status cheb_apply(sph_rt *s, const CsrView<MT> &A, const VT *r, VT *z, VT
   // first goes to bufs[w0], each later one flips buffers, the last hits bufs[0].
   int w0 = (degree - 1) % 2;
   sph_rt_status rc;
-  if (first_step_done) {
-    // the caller has made step 0 from a nonzero guess, result in bufs[w0]
-  } else if (zero_guess) {
+  if (!first_done) {
     pdl_launch(s, cheb_init_zero_kernel<MT, VT>, g, kBlock, 0, A.n, r, A.invdiag, cf, d,
                                                                  bufs[w0], sc);
     SPH_LAUNCHED(s);
-  } else {
-    // the guess is read from bufs[w0 ^ 1]
-    if (w0 == 0) {
-      SPH_CUDA(s, cudaMemcpyAsync(tmp, z, sizeof(VT) * A.n, cudaMemcpyDeviceToDevice, s->stream));
-    }
-    if ((rc = step(bufs[w0 ^ 1], bufs[w0], 0))) return rc;
   }
   int at = w0;
   for (int k = 1; k < degree; ++k) {
@@ -483,10 +477,10 @@ sph_rt_status cheb_apply(sph_rt *s, const CsrView<MT> &A, const VT *r, VT *z, VT
 
 template sph_rt_status cheb_apply<double, double>(sph_rt *, const CsrView<double> &, const double *,
                                                   double *, double *, double *, int,
-                                                  const ChebCoef *, bool, const Scalars *, bool);
+                                                  const ChebCoef *, const Scalars *, bool);
 template sph_rt_status cheb_apply<float, float>(sph_rt *, const CsrView<float> &, const float *,
                                                 float *, float *, float *, int, const ChebCoef *,
-                                                bool, const Scalars *, bool);
+                                                const Scalars *, bool);
 
 // Preconditioner hooks implemented by the AMG translation unit.  init_done:
 // the finest level's smoother start was written by the CG update (amg_fine_init);
@@ -519,7 +513,7 @@ static sph_rt_status precondition(sph_rt *s, const CsrView<double> &A, int first
       return SPH_RT_OK;
     case SPH_RT_PRECOND_CHEBYSHEV:
       rc = cheb_apply<double, double>(s, A, s->r, s->z, s->w, s->tmp_n2, s->cfg.cheb_degree,
-                                      s->cheb_slots, true, s->sc, false);
+                                      s->cheb_slots, s->sc, false);
       if (rc) return rc;
       break;
     default: {
@@ -854,7 +848,7 @@ sph_rt_status pcg_prologue(sph_rt *s) {
   wf = timing_begin(s);
   SPH_FINE_ROWS(s, double, A, sizeof(double),
                 (pdl_launch(s, spmv_pq_kernel<Rows>, grid, kBlock, smem, rows, s->z, s->q, s->p, 1,
-                            s->sc, s->partials, wf)));
+                            s->sc, s->partials, wf, s->loop_cond)));
   SPH_LAUNCHED(s);
   timing_end(s, spmv_class_bytes(s, A, kRowBytesSpmvPQ), kTimedSpmvPQ);
   return SPH_RT_OK;
@@ -895,7 +889,7 @@ sph_rt_status pcg_iteration(sph_rt *s) {
   int *wf = timing_begin(s);
   SPH_FINE_ROWS(s, double, A, sizeof(double),
                 (pdl_launch(s, spmv_pq_kernel<Rows>, grid, kBlock, smem, rows, s->z, s->q, s->p, 0,
-                            s->sc, s->partials, wf)));
+                            s->sc, s->partials, wf, s->loop_cond)));
   SPH_LAUNCHED(s);
   timing_end(s, spmv_class_bytes(s, A, kRowBytesSpmvPQ), kTimedSpmvPQ);
   return SPH_RT_OK;
