@@ -602,6 +602,18 @@ __device__ __forceinline__ void loop_cond_skip(const LoopCond &c, Scalars *sc) {
   if (blockIdx.x == 0 && threadIdx.x == 0) loop_cond_set(c, sc);
 }
 
+// What the material solve's last block does beside the reductions.
+//   kOuterNone   nothing
+//   kOuterInit   the initial solve of a step: resets the outer loop's state
+//   kOuterTail   the solve of an outer iteration: the Krylov check, the statistics and
+//                the outer convergence test (outer_check), and the loop condition
+enum OuterMode { kOuterNone = 0, kOuterInit = 1, kOuterTail = 2 };
+struct OuterTail {
+  int mode, max_outer, in_graph;
+  double tol_e, tol_E;
+  cudaGraphConditionalHandle h;
+};
+
 // Vectors of the CG with the V-cycle's product (fine_post_smooth = 0), in the
 // hierarchy's precision T: residual r, preconditioned residual z, w = B z,
 // direction p and q = B p, the finest level's smoother start zpre, and the
@@ -906,7 +918,6 @@ struct sph_rt {
 
   // step vectors (interior)
   double *e_old = nullptr, *E_old = nullptr, *e_l = nullptr, *E_l = nullptr;
-  double *e_new = nullptr;
   double *Qe = nullptr, *QE = nullptr;  // slot order [n]
   double *b = nullptr, *x = nullptr, *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr,
          *w = nullptr;

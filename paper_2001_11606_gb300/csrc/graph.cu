@@ -27,88 +27,21 @@
 namespace sphrt {
 
 sph_rt_status launch_rhs(sph_rt *s, double dt);
-sph_rt_status launch_newton(sph_rt *s, double dt, const double *E_new, const double *E_prev,
-                            const double *e_start, double *e_out);
+sph_rt_status launch_newton(sph_rt *s, double dt, const double *E_new, double *E_prev,
+                            const double *e_start, double *e_out, const OuterTail &tail);
 sph_rt_status pcg_prologue(sph_rt *s);
 sph_rt_status pcg_iteration(sph_rt *s);
 sph_rt_status pcg_solve(sph_rt *s, int *iters, bool *converged);
 void amg_signature(const sph_rt *s, std::vector<uint64_t> &sig);
 CsrView<double> fine_view(const sph_rt *s);
 
-// outer-loop state at the start of a step; newton_max starts from the initial
-// material solve of Alg. 1 (its iteration count is in red[2])
-__global__ void outer_init_kernel(Scalars *sc) {
-  sc->outer_iters = 0;
-  sc->outer_status = 0;
-  sc->outer_trips = 0;
-  sc->krylov_total = 0;
-  sc->krylov_trips = 0;
-  sc->krylov_solve_trips = 0;
-  sc->newton_max = (int)sc->red[2];
-  sc->yvalid = 0;  // a new step has a new operator
-  sc->last_change_e = 0.0;
-  sc->last_change_E = 0.0;
-  for (int k = 0; k < 64; ++k) sc->krylov_per_outer[k] = 0;
-}
-
-// After the material solve of an outer iteration: the Krylov check, the
-// bookkeeping of the step statistics and the outer convergence test
-// max_i |x^{l+1} - x^l| / |x^{l+1}| < tol for e and E (changes in red[0..1],
-// Newton iterations in red[2]).  In the graph it also sets the loop condition.
-__global__ void outer_check_kernel(Scalars *sc, double tol_e, double tol_E, int max_outer,
-                                   cudaGraphConditionalHandle h, int in_graph) {
-  int status = 0;
-  sc->outer_trips += 1;
-  const bool kconv = !sc->breakdown && !(sc->rnorm2 > sc->thresh2);
-  if (!kconv) {
-    status = 2;
-  } else {
-    const int o = sc->outer_iters;
-    if (o < 64) sc->krylov_per_outer[o] = sc->iters;
-    sc->krylov_total += sc->iters;
-    sc->outer_iters = o + 1;
-    const double ce = sc->red[0], cE = sc->red[1];
-    sc->newton_max = max(sc->newton_max, (int)sc->red[2]);
-    sc->last_change_e = ce;
-    sc->last_change_E = cE;
-    if (ce < tol_e && cE < tol_E)
-      status = 1;
-    else if (sc->outer_iters >= max_outer)
-      status = 3;
-  }
-  if (status == 0 && sc->outer_trips > max_outer) status = 3;
-  sc->outer_status = status;
-  if (in_graph) cudaGraphSetConditional(h, status == 0 ? 1u : 0u);
-}
-
-// The new iterate becomes the current one: e^l <- e^{l+1}, E^l <- E^{l+1} (= x).
-__global__ void iterate_copy_kernel(int64_t n, const double *e_new, double *e_l,
-                                    const double *x, double *E_l) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    e_l[i] = e_new[i];
-    E_l[i] = x[i];
-  }
-}
-
-static int copy_grid(const sph_rt *s, int64_t n) {
-  int64_t g = ceil_div(n > 0 ? n : 1, kBlock), cap = (int64_t)s->num_sms * 8;
-  return (int)(g < cap ? g : cap);
-}
-
 static sph_rt_status launch_outer_tail(sph_rt *s, double dt, cudaGraphConditionalHandle h,
                                        int in_graph) {
-  sph_rt_status rc;
-  // a8: material solve with E^{l+1} = x, from e^l
-  if ((rc = launch_newton(s, dt, s->x, s->E_l, s->e_l, s->e_new))) return rc;
-  // a9: convergence test and statistics
-  outer_check_kernel<<<1, 1, 0, s->stream>>>(s->sc, s->cfg.tol_outer_e, s->cfg.tol_outer_E,
-                                              s->cfg.max_outer, h, in_graph);
-  SPH_LAUNCHED(s);
-  iterate_copy_kernel<<<copy_grid(s, s->n_int), kBlock, 0, s->stream>>>(
-      s->n_int, s->e_new, s->e_l, s->x, s->E_l);
-  SPH_LAUNCHED(s);
-  return SPH_RT_OK;
+  // a8: material solve with E^{l+1} = x, from e^l; the new iterate becomes the
+  // current one, e^l <- e^{l+1}, E^l <- x; a9: convergence test and statistics
+  const OuterTail tail = {kOuterTail, s->cfg.max_outer, in_graph, s->cfg.tol_outer_e,
+                          s->cfg.tol_outer_E, h};
+  return launch_newton(s, dt, s->x, s->E_l, s->e_l, s->e_l, tail);
 }
 
 // ---------------------------------------------------------------------------
@@ -116,8 +49,6 @@ static sph_rt_status launch_outer_tail(sph_rt *s, double dt, cudaGraphConditiona
 // ---------------------------------------------------------------------------
 static sph_rt_status outer_loop_host(sph_rt *s, double dt) {
   sph_rt_status rc;
-  outer_init_kernel<<<1, 1, 0, s->stream>>>(s->sc);
-  SPH_LAUNCHED(s);
   for (;;) {
     if ((rc = launch_rhs(s, dt))) return rc;  // a7 (also x = E^l)
     int kit = 0;
@@ -157,7 +88,7 @@ static std::vector<uint64_t> loop_signature(const sph_rt *s, double dt) {
   const int64_t sizes[4] = {s->n, s->n_int, s->nnz_mat, (int64_t)s->num_sms};
   sig_u64(v, sizes, sizeof sizes);
   const void *bufs[] = {s->b,     s->x,     s->r,    s->z,     s->z_old, s->p,      s->q,
-                        s->w,     s->tmp_n2, s->invV, s->sc,   s->partials, s->e_l, s->e_new,
+                        s->w,     s->tmp_n2, s->invV, s->sc,   s->partials, s->e_l,
                         s->E_l,   s->E_old, s->e_old, s->rho, s->sigma, s->f,       s->Qe,
                         s->QE,    s->gb,    s->V,     s->cheb_slots, s->sl.ptr, s->sl.idx,
                         s->sl.len, s->sl.order, s->sl.dptr, s->sl.dict, s->sl_val, s->sl_val32, s->diag,
@@ -268,8 +199,6 @@ static sph_rt_status outer_loop_graph(sph_rt *s, double dt) {
   if (!s->graph_exec || s->graph_sig != loop_signature(s, dt)) {
     if ((rc = build_loop_graph(s, dt))) return rc;
   }
-  outer_init_kernel<<<1, 1, 0, s->stream>>>(s->sc);
-  SPH_LAUNCHED(s);
   SPH_CUDA(s, cudaGraphLaunch(s->graph_exec, s->stream));
   s->graph_launches++;
   return SPH_RT_OK;

@@ -252,19 +252,28 @@ __global__ void grad_geom_kernel(int64_t n_int, const int64_t *nbr_ptr, const in
   }
 }
 
-// copy ghosts take every property of the particle they copy
-__global__ void props_copy_kernel(int64_t n_int, int64_t n, const int32_t *copysrc, double *T,
-                                  double *sigma, double *f, double *R, double *lambda, double *D) {
+// Ghosts, after the gradient: copy ghosts take every property of the particle they
+// copy, Dirichlet ghosts their values at t^n (caller order; null: kept).
+__global__ void ghost_kernel(int64_t n_int, int64_t n, const int32_t *kind,
+                             const int32_t *copysrc, const int64_t *slot2caller,
+                             const double *ge_c, const double *gE_c, double *T, double *sigma,
+                             double *f, double *R, double *lambda, double *D, double *e,
+                             double *E) {
   for (int64_t i = n_int + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    int32_t s = copysrc[i];
-    if (s < 0) continue;
-    T[i] = T[s];
-    sigma[i] = sigma[s];
-    f[i] = f[s];
-    R[i] = R[s];
-    lambda[i] = lambda[s];
-    D[i] = D[s];
+    const int32_t s = copysrc[i];
+    if (s >= 0) {
+      T[i] = T[s];
+      sigma[i] = sigma[s];
+      f[i] = f[s];
+      R[i] = R[s];
+      lambda[i] = lambda[s];
+      D[i] = D[s];
+    } else if (kind[i] == SPH_RT_DIRICHLET && (ge_c || gE_c)) {
+      const int64_t c = slot2caller[i];
+      if (ge_c) e[i] = ge_c[c];
+      if (gE_c) E[i] = gE_c[c];
+    }
   }
 }
 
@@ -558,6 +567,51 @@ __global__ void rhs_kernel(Phys ph, int64_t n_int, const double *V, const double
   }
 }
 
+// outer-loop state at the start of a step; newton_max starts from the initial
+// material solve of Alg. 1 (its iteration count is in red[2])
+__device__ void outer_init(Scalars *sc) {
+  sc->outer_iters = 0;
+  sc->outer_status = 0;
+  sc->outer_trips = 0;
+  sc->krylov_total = 0;
+  sc->krylov_trips = 0;
+  sc->krylov_solve_trips = 0;
+  sc->newton_max = (int)sc->red[2];
+  sc->yvalid = 0;  // a new step has a new operator
+  sc->last_change_e = 0.0;
+  sc->last_change_E = 0.0;
+  for (int k = 0; k < 64; ++k) sc->krylov_per_outer[k] = 0;
+}
+
+// After the material solve of an outer iteration: the Krylov check, the
+// bookkeeping of the step statistics and the outer convergence test
+// max_i |x^{l+1} - x^l| / |x^{l+1}| < tol for e and E (changes in red[0..1],
+// Newton iterations in red[2]).  In the graph it also sets the loop condition.
+__device__ void outer_check(Scalars *sc, const OuterTail &t) {
+  int status = 0;
+  sc->outer_trips += 1;
+  const bool kconv = !sc->breakdown && !(sc->rnorm2 > sc->thresh2);
+  if (!kconv) {
+    status = 2;
+  } else {
+    const int o = sc->outer_iters;
+    if (o < 64) sc->krylov_per_outer[o] = sc->iters;
+    sc->krylov_total += sc->iters;
+    sc->outer_iters = o + 1;
+    const double ce = sc->red[0], cE = sc->red[1];
+    sc->newton_max = max(sc->newton_max, (int)sc->red[2]);
+    sc->last_change_e = ce;
+    sc->last_change_E = cE;
+    if (ce < t.tol_e && cE < t.tol_E)
+      status = 1;
+    else if (sc->outer_iters >= t.max_outer)
+      status = 3;
+  }
+  if (status == 0 && sc->outer_trips > t.max_outer) status = 3;
+  sc->outer_status = status;
+  if (t.in_graph) cudaGraphSetConditional(t.h, status == 0 ? 1u : 0u);
+}
+
 // a8 + a9: material solve with the new radiation energy and the outer
 // convergence measures.  P_i = c sigma_i E_i + Q_e,i (Eq. material-energy-solve);
 // Newton from e_start.  red[0] = max |e_new - e_start|/|e_new|,
@@ -571,9 +625,9 @@ __global__ void rhs_kernel(Phys ph, int64_t n_int, const double *V, const double
 // 0.028.
 __global__ void __launch_bounds__(kBlock)
     newton_kernel(Phys ph, int64_t n_int, const double *rho, const double *sigma,
-                  const double *e_old, const double *Qe, const double *E_new,
-                  const double *E_prev, const double *e_start, double *e_new, Scalars *sc,
-                  double *partials) {
+                  const double *e_old, const double *Qe, const double *E_new, double *E_prev,
+                  const double *e_start, double *e_new, Scalars *sc, double *partials,
+                  const OuterTail tail) {
   double ce = 0.0, cE = 0.0;
   int itmax = 0, fails = 0;
   const double tiny = 1e-300;
@@ -608,6 +662,7 @@ __global__ void __launch_bounds__(kBlock)
     e_new[i] = ei;
     ce = max_bits(ce, quotient(fabs(ei - e0), max_bits(tiny, fabs(ei))));
     cE = max_bits(cE, quotient(fabs(En - E_prev[i]), max_bits(tiny, fabs(En))));
+    if (tail.mode == kOuterTail) E_prev[i] = En;  // the new iterate becomes the current one
     itmax = max(itmax, it);
     fails += !ok;
   }
@@ -639,25 +694,78 @@ __global__ void __launch_bounds__(kBlock)
     sc->red[1] = out[1];
     sc->red[2] = out[2];
     sc->red[3] = out[3];
+    if (tail.mode == kOuterInit) outer_init(sc);
+    if (tail.mode == kOuterTail) outer_check(sc, tail);
   }
 }
 
-// Step inputs must be finite: sources of interior particles, ghost values of
-// Dirichlet ghosts (caller order).  Sets sc->bad_input.
-__global__ void check_inputs_kernel(int64_t n, const int64_t *caller2slot, const int32_t *kind,
-                                    const double *Qe, const double *QE, const double *ge,
-                                    const double *gE, Scalars *sc) {
+// Start of a step, in one pass over the slots: the snapshot of the state, the
+// sources gathered to slot order (null: 0), the check that the step's inputs are
+// finite (sources of interior particles, values of Dirichlet ghosts; caller order)
+// and the energy before the step.
+__global__ void step_begin_kernel(int64_t n_int, int64_t n, const int64_t *slot2caller,
+                                  const int32_t *kind, const double *Qe_c, const double *QE_c,
+                                  const double *ge, const double *gE, const double *mass,
+                                  const double *V, const double *e, const double *E,
+                                  double *e_bak, double *E_bak, double *Qe, double *QE,
+                                  Scalars *sc, double *partials) {
+  double a = 0.0, b = 0.0;
   int bad = 0;
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n;
-       c += (int64_t)gridDim.x * blockDim.x) {
-    const int k = kind[caller2slot[c]];
-    if (k == SPH_RT_INTERIOR) {
-      if ((Qe && !isfinite(Qe[c])) || (QE && !isfinite(QE[c]))) bad = 1;
-    } else if (k == SPH_RT_DIRICHLET) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const double ei = e[i], Ei = E[i];
+    e_bak[i] = ei;
+    E_bak[i] = Ei;
+    const int64_t c = slot2caller[i];
+    if (i < n_int) {
+      const double qe = Qe_c ? Qe_c[c] : 0.0, qE = QE_c ? QE_c[c] : 0.0;
+      Qe[i] = qe;
+      QE[i] = qE;
+      if (!isfinite(qe) || !isfinite(qE)) bad = 1;
+      a += mass[i] * ei;
+      b += V[i] * Ei;
+    } else if (kind[i] == SPH_RT_DIRICHLET) {
       if ((ge && !isfinite(ge[c])) || (gE && !isfinite(gE[c]))) bad = 1;
     }
   }
-  if (bad) atomicExch(&sc->bad_input, 1);
+  __shared__ double sh[32];
+  bad = __syncthreads_or(bad);
+  const double pa = block_sum(a, sh);
+  __syncthreads();
+  const double pb = block_sum(b, sh);
+  double part[3] = {pa, pb, bad ? 1.0 : 0.0}, out[3];
+  const bool mx[3] = {false, false, true};
+  if (last_block_combine<3>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
+    sc->energy_before_e = out[0];
+    sc->energy_before_E = out[1];
+    sc->bad_input = out[2] != 0.0;
+  }
+}
+
+// Before the initial material solve: the history of the extrapolated Krylov start
+// moves down one place (H2 <- H1 <- H0 <- E_old, as far as `depth` reaches), and
+// e_old, E_old and E^{n,0} take the state.
+__global__ void step_start_kernel(int64_t n_int, int depth, const double *e, const double *E,
+                                  double *e_old, double *E_old, double *E_l, double *H0,
+                                  double *H1, double *H2, Scalars *sc, int order, double w0,
+                                  double w1, double w2, double w3) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    sc->guess_order = order;
+    sc->guess_w[0] = w0;
+    sc->guess_w[1] = w1;
+    sc->guess_w[2] = w2;
+    sc->guess_w[3] = w3;
+  }
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_int;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    if (depth >= 3) H2[i] = H1[i];
+    if (depth >= 2) H1[i] = H0[i];
+    if (depth >= 1) H0[i] = E_old[i];
+    const double Ei = E[i];
+    e_old[i] = e[i];
+    E_old[i] = Ei;
+    E_l[i] = Ei;
+  }
 }
 
 // Totals over interior particles: red[4] = sum m e, red[5] = sum V E.
@@ -681,55 +789,68 @@ __global__ void totals_kernel(int64_t n_int, const double *mass, const double *V
   }
 }
 
-// Energy added over the step: red[6] = dt sum V (Q_e + Q_E);
-// red[7] = dt sum_i V_i sum_{Dirichlet j} w_ij (E_j - E_i), over the couplings as
-// one flat list: few rows have any, those have tens, and a thread per row spent
-// its time on the longest (0.22 ms at 128^3 with 5.7e6 couplings, now 0.076).
-__global__ void balance_kernel(Phys ph, int64_t n_int, int64_t nnz_gh, const double *V,
-                               const double *Qe, const double *QE, const int32_t *gh_row,
-                               const int32_t *gh_slot, const double *gh_W, const double *D,
-                               const double *E, Scalars *sc, double *partials) {
-  double a = 0.0, b = 0.0;
+// End of a step, in one pass.  A converged step with valid inputs commits its
+// interior state (copy ghosts take their particle's); any other step restores the
+// snapshot taken at its start (ghost entries included), so a failed step leaves the
+// state unchanged.  Of a committed step also the energies (meaningless otherwise):
+//   red[4], red[5]  totals sum m e, sum V E
+//   red[6]          added by the sources, dt sum V (Q_e + Q_E)
+//   red[7]          added through the boundary, dt sum_i V_i sum_{Dirichlet j} w_ij
+//                   (E_j - E_i), over the couplings as one flat list: few rows have
+//                   any, those have tens, and a thread per row spent its time on the
+//                   longest (0.22 ms at 128^3 with 5.7e6 couplings, now 0.076 alone)
+__global__ void step_end_kernel(Phys ph, int64_t n_int, int64_t n, int64_t nnz_gh,
+                                const int32_t *copysrc, const double *e_new,
+                                const double *E_new, const double *e_bak, const double *E_bak,
+                                const double *mass, const double *V, const double *Qe,
+                                const double *QE, const int32_t *gh_row, const int32_t *gh_slot,
+                                const double *gh_W, const double *D, double *e, double *E,
+                                Scalars *sc, double *partials) {
+  const bool commit = sc->outer_status == 1 && !sc->bad_input;
+  double te = 0.0, tE = 0.0, a = 0.0, b = 0.0;
   const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = t0; i < n_int; i += step) a += V[i] * (Qe[i] + QE[i]);
-  for (int64_t k = t0; k < nnz_gh; k += step) {
-    const int32_t i = gh_row[k], j = gh_slot[k];
-    b -= (V[i] * gh_W[k]) * (D[i] + D[j]) * (E[j] - E[i]);
+  for (int64_t i = t0; i < n; i += step) {
+    if (i < n_int) {
+      const double ei = commit ? e_new[i] : e_bak[i], Ei = commit ? E_new[i] : E_bak[i];
+      e[i] = ei;
+      E[i] = Ei;
+      const double Vi = V[i];
+      te += mass[i] * ei;
+      tE += Vi * Ei;
+      a += Vi * (Qe[i] + QE[i]);
+    } else {
+      const int32_t c = copysrc[i];
+      if (c >= 0) {
+        e[i] = commit ? e_new[c] : e_bak[c];
+        E[i] = commit ? E_new[c] : E_bak[c];
+      } else if (!commit) {
+        e[i] = e_bak[i];
+        E[i] = E_bak[i];
+      }
+    }
   }
+  if (commit)
+    for (int64_t k = t0; k < nnz_gh; k += step) {
+      const int32_t i = gh_row[k], j = gh_slot[k];  // j: a ghost, not written above
+      b -= (V[i] * gh_W[k]) * (D[i] + D[j]) * (E[j] - E_new[i]);
+    }
   __shared__ double sh[32];
-  double pa = block_sum(a, sh);
+  double part[4];
+  part[0] = block_sum(te, sh);
   __syncthreads();
-  double pb = block_sum(b, sh);
-  double part[2] = {pa, pb}, out[2];
-  const bool mx[2] = {false, false};
-  if (last_block_combine<2>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
-    sc->red[6] = ph.dt * out[0];
-    sc->red[7] = ph.dt * out[1];
-  }
-}
-
-// Install Dirichlet ghost values (slot order) from caller-order arrays.
-__global__ void ghost_install_kernel(int64_t n_int, int64_t n, const int32_t *kind,
-                                     const int64_t *slot2caller, const double *ge_c,
-                                     const double *gE_c, double *e, double *E) {
-  for (int64_t s = n_int + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n;
-       s += (int64_t)gridDim.x * blockDim.x) {
-    if (kind[s] != SPH_RT_DIRICHLET) continue;
-    int64_t c = slot2caller[s];
-    if (ge_c) e[s] = ge_c[c];
-    if (gE_c) E[s] = gE_c[c];
-  }
-}
-
-__global__ void copy_ghost_sync_kernel(int64_t n_int, int64_t n, const int32_t *copysrc,
-                                       double *e, double *E) {
-  for (int64_t s = n_int + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n;
-       s += (int64_t)gridDim.x * blockDim.x) {
-    int32_t c = copysrc[s];
-    if (c < 0) continue;
-    e[s] = e[c];
-    E[s] = E[c];
+  part[1] = block_sum(tE, sh);
+  __syncthreads();
+  part[2] = block_sum(a, sh);
+  __syncthreads();
+  part[3] = block_sum(b, sh);
+  double out[4];
+  const bool mx[4] = {false, false, false, false};
+  if (last_block_combine<4>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
+    sc->red[4] = out[0];
+    sc->red[5] = out[1];
+    sc->red[6] = ph.dt * out[2];
+    sc->red[7] = ph.dt * out[3];
   }
 }
 
@@ -746,33 +867,6 @@ __global__ void scatter_caller_kernel(const double *in_s, const int64_t *slot2ca
   for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n;
        s += (int64_t)gridDim.x * blockDim.x)
     out_c[slot2caller[s]] = in_s[s];
-}
-
-// End of a step: a converged step with valid inputs commits its interior
-// state; any other step restores the snapshot taken at its start (ghost
-// entries included), so a failed step leaves the state unchanged.
-__global__ void finish_kernel(int64_t n_int, int64_t n, const double *e_new, const double *E_new,
-                              const double *e_bak, const double *E_bak, double *e, double *E,
-                              const Scalars *sc) {
-  const bool commit = sc->outer_status == 1 && !sc->bad_input;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    if (commit) {
-      if (i < n_int) {
-        e[i] = e_new[i];
-        E[i] = E_new[i];
-      }
-    } else {
-      e[i] = e_bak[i];
-      E[i] = E_bak[i];
-    }
-  }
-}
-
-// the totals just reduced (red[4], red[5]) are the energy before the step
-__global__ void save_before_kernel(Scalars *sc) {
-  sc->energy_before_e = sc->red[4];
-  sc->energy_before_E = sc->red[5];
 }
 
 // ---------------------------------------------------------------------------
@@ -826,7 +920,7 @@ int row_width(int64_t nnz, int64_t rows) {
     SPH_LAUNCHED(s);                                                          \
   } while (0)
 
-sph_rt_status launch_properties(sph_rt *s, double dt) {
+sph_rt_status launch_properties(sph_rt *s, double dt, const double *ge_c, const double *gE_c) {
   Phys ph = make_phys(s, dt);
   int g = grid_items(s, s->n, kBlock);
   props_point_kernel<<<g, kBlock, 0, s->stream>>>(ph, s->n, s->kind, s->rho, s->sigma0, s->e,
@@ -870,8 +964,9 @@ sph_rt_status launch_properties(sph_rt *s, double dt) {
     }
   }
   if (s->n > s->n_int) {
-    props_copy_kernel<<<grid_items(s, s->n - s->n_int, kBlock), kBlock, 0, s->stream>>>(
-        s->n_int, s->n, s->copysrc, s->T, s->sigma, s->f, s->R, s->lambda, s->D);
+    ghost_kernel<<<grid_items(s, s->n - s->n_int, kBlock), kBlock, 0, s->stream>>>(
+        s->n_int, s->n, s->kind, s->copysrc, s->slot2caller, ge_c, gE_c, s->T, s->sigma, s->f,
+        s->R, s->lambda, s->D, s->e, s->E);
     SPH_LAUNCHED(s);
   }
   return SPH_RT_OK;
@@ -929,38 +1024,39 @@ sph_rt_status launch_rhs(sph_rt *s, double dt) {
   return SPH_RT_OK;
 }
 
-__global__ void set_guess_kernel(Scalars *sc, int order, double w0, double w1, double w2,
-                                 double w3) {
-  sc->guess_order = order;
-  sc->guess_w[0] = w0;
-  sc->guess_w[1] = w1;
-  sc->guess_w[2] = w2;
-  sc->guess_w[3] = w3;
-}
-
 // order and weights of the extrapolated start of the step's first solve (order 0: E^l)
-sph_rt_status launch_set_guess(sph_rt *s, int order, const double *w) {
-  set_guess_kernel<<<1, 1, 0, s->stream>>>(s->sc, order, w[0], w[1], w[2], w[3]);
+sph_rt_status launch_step_start(sph_rt *s, int depth, int order, const double *w) {
+  step_start_kernel<<<grid_items(s, s->n_int, kBlock), kBlock, 0, s->stream>>>(
+      s->n_int, depth, s->e, s->E, s->e_old, s->E_old, s->E_l, s->E_hist[0], s->E_hist[1],
+      s->E_hist[2], s->sc, order, w[0], w[1], w[2], w[3]);
   SPH_LAUNCHED(s);
   return SPH_RT_OK;
 }
 
-sph_rt_status launch_newton(sph_rt *s, double dt, const double *E_new, const double *E_prev,
-                            const double *e_start, double *e_out) {
+sph_rt_status launch_newton(sph_rt *s, double dt, const double *E_new, double *E_prev,
+                            const double *e_start, double *e_out, const OuterTail &tail) {
   Phys ph = make_phys(s, dt);
   int g = grid_items(s, s->n_int, kBlock);
   newton_kernel<<<g, kBlock, 0, s->stream>>>(ph, s->n_int, s->rho, s->sigma, s->e_old, s->Qe,
-                                              E_new, E_prev, e_start, e_out, s->sc, s->partials);
+                                              E_new, E_prev, e_start, e_out, s->sc, s->partials, tail);
   SPH_LAUNCHED(s);
   return SPH_RT_OK;
 }
 
-sph_rt_status launch_check_inputs(sph_rt *s, const double *Qe, const double *QE,
-                                  const double *ge, const double *gE) {
-  SPH_CUDA(s, cudaMemsetAsync(&s->sc->bad_input, 0, sizeof(int), s->stream));
-  if (!Qe && !QE && !ge && !gE) return SPH_RT_OK;
-  check_inputs_kernel<<<grid_items(s, s->n, kBlock), kBlock, 0, s->stream>>>(
-      s->n, s->caller2slot, s->kind, Qe, QE, ge, gE, s->sc);
+sph_rt_status launch_step_begin(sph_rt *s, const double *Qe, const double *QE, const double *ge,
+                                const double *gE) {
+  step_begin_kernel<<<grid_reduce(s, s->n), kBlock, 0, s->stream>>>(
+      s->n_int, s->n, s->slot2caller, s->kind, Qe, QE, ge, gE, s->mass, s->V, s->e, s->E,
+      s->e_bak, s->E_bak, s->Qe, s->QE, s->sc, s->partials);
+  SPH_LAUNCHED(s);
+  return SPH_RT_OK;
+}
+
+sph_rt_status launch_step_end(sph_rt *s, double dt, const double *e_new, const double *E_new) {
+  step_end_kernel<<<grid_reduce(s, s->n), kBlock, 0, s->stream>>>(
+      make_phys(s, dt), s->n_int, s->n, s->nnz_gh, s->copysrc, e_new, E_new, s->e_bak, s->E_bak,
+      s->mass, s->V, s->Qe, s->QE, s->gh_row, s->gh_slot, s->gh_W, s->D, s->e, s->E, s->sc,
+      s->partials);
   SPH_LAUNCHED(s);
   return SPH_RT_OK;
 }
@@ -1050,33 +1146,6 @@ sph_rt_status launch_totals(sph_rt *s, const double *e, const double *E) {
   return SPH_RT_OK;
 }
 
-sph_rt_status launch_balance(sph_rt *s, double dt, const double *E) {
-  Phys ph = make_phys(s, dt);
-  int g = grid_reduce(s, s->n_int);
-  balance_kernel<<<g, kBlock, 0, s->stream>>>(ph, s->n_int, s->nnz_gh, s->V, s->Qe, s->QE,
-                                               s->gh_row, s->gh_slot, s->gh_W, s->D, E, s->sc,
-                                               s->partials);
-  SPH_LAUNCHED(s);
-  return SPH_RT_OK;
-}
-
-sph_rt_status launch_ghost_install(sph_rt *s, const double *ge_c, const double *gE_c) {
-  if (s->n == s->n_int || (!ge_c && !gE_c)) return SPH_RT_OK;
-  int g = grid_items(s, s->n - s->n_int, kBlock);
-  ghost_install_kernel<<<g, kBlock, 0, s->stream>>>(s->n_int, s->n, s->kind, s->slot2caller,
-                                                     ge_c, gE_c, s->e, s->E);
-  SPH_LAUNCHED(s);
-  return SPH_RT_OK;
-}
-
-sph_rt_status launch_copy_sync(sph_rt *s) {
-  if (s->n == s->n_int) return SPH_RT_OK;
-  int g = grid_items(s, s->n - s->n_int, kBlock);
-  copy_ghost_sync_kernel<<<g, kBlock, 0, s->stream>>>(s->n_int, s->n, s->copysrc, s->e, s->E);
-  SPH_LAUNCHED(s);
-  return SPH_RT_OK;
-}
-
 sph_rt_status launch_gather_interior(sph_rt *s, const double *in_c, double *out) {
   int g = grid_items(s, s->n_int, kBlock);
   gather_interior_kernel<<<g, kBlock, 0, s->stream>>>(in_c, s->slot2caller, s->n_int, out);
@@ -1087,20 +1156,6 @@ sph_rt_status launch_gather_interior(sph_rt *s, const double *in_c, double *out)
 sph_rt_status launch_scatter_caller(sph_rt *s, const double *in_s, int64_t count, double *out_c) {
   int g = grid_items(s, count, kBlock);
   scatter_caller_kernel<<<g, kBlock, 0, s->stream>>>(in_s, s->slot2caller, count, out_c);
-  SPH_LAUNCHED(s);
-  return SPH_RT_OK;
-}
-
-sph_rt_status launch_finish(sph_rt *s, const double *e_new, const double *E_new) {
-  int g = grid_items(s, s->n, kBlock);
-  finish_kernel<<<g, kBlock, 0, s->stream>>>(s->n_int, s->n, e_new, E_new, s->e_bak, s->E_bak,
-                                             s->e, s->E, s->sc);
-  SPH_LAUNCHED(s);
-  return SPH_RT_OK;
-}
-
-sph_rt_status launch_save_before(sph_rt *s) {
-  save_before_kernel<<<1, 1, 0, s->stream>>>(s->sc);
   SPH_LAUNCHED(s);
   return SPH_RT_OK;
 }

@@ -23,22 +23,18 @@ sph_rt_status build_particles(sph_rt *s, int64_t n, const double *pos_c, const d
                               const double *rho_c, const double *h_c, const double *sig0_c,
                               const int32_t *kind_c, const int64_t *copy_of_c, const double *e0_c,
                               const double *E0_c, int64_t n_int);
-sph_rt_status launch_properties(sph_rt *s, double dt);
+sph_rt_status launch_properties(sph_rt *s, double dt, const double *ge_c, const double *gE_c);
 sph_rt_status launch_assembly(sph_rt *s, double dt, double *gersh_out);
 sph_rt_status launch_rhs(sph_rt *s, double dt);
-sph_rt_status launch_set_guess(sph_rt *s, int order, const double *w);
-sph_rt_status launch_newton(sph_rt *s, double dt, const double *E_new, const double *E_prev,
-                            const double *e_start, double *e_out);
+sph_rt_status launch_step_start(sph_rt *s, int depth, int order, const double *w);
+sph_rt_status launch_newton(sph_rt *s, double dt, const double *E_new, double *E_prev,
+                            const double *e_start, double *e_out, const OuterTail &tail);
 sph_rt_status launch_totals(sph_rt *s, const double *e, const double *E);
-sph_rt_status launch_check_inputs(sph_rt *s, const double *Qe, const double *QE,
-                                  const double *ge, const double *gE);
-sph_rt_status launch_balance(sph_rt *s, double dt, const double *E);
-sph_rt_status launch_ghost_install(sph_rt *s, const double *ge_c, const double *gE_c);
-sph_rt_status launch_copy_sync(sph_rt *s);
+sph_rt_status launch_step_begin(sph_rt *s, const double *Qe, const double *QE, const double *ge,
+                                const double *gE);
+sph_rt_status launch_step_end(sph_rt *s, double dt, const double *e_new, const double *E_new);
 sph_rt_status launch_gather_interior(sph_rt *s, const double *in_c, double *out);
 sph_rt_status launch_scatter_caller(sph_rt *s, const double *in_s, int64_t count, double *out_c);
-sph_rt_status launch_finish(sph_rt *s, const double *e_new, const double *E_new);
-sph_rt_status launch_save_before(sph_rt *s);
 sph_rt_status launch_dt_control(sph_rt *s, double dt);
 sph_rt_status pcg_solve(sph_rt *s, int *iters, bool *converged);
 sph_rt_status autotune_fine_shape(sph_rt *s);
@@ -481,7 +477,7 @@ static sph_rt_status alloc_step_vectors(sph_rt *s) {
                      &s->tmp_n3, &s->e_bak, &s->E_bak, &s->stage_ge, &s->stage_gE};
   for (double **p : full)
     if (!(*p = dalloc<double>(s, n))) return SPH_RT_ENOMEM;
-  double **inner[] = {&s->e_old, &s->E_old, &s->e_l, &s->E_l, &s->e_new, &s->Qe, &s->QE, &s->b,
+  double **inner[] = {&s->e_old, &s->E_old, &s->e_l, &s->E_l, &s->Qe, &s->QE, &s->b,
                       &s->x, &s->r, &s->z, &s->p, &s->q, &s->w, &s->diag, &s->invdiag, &s->gb,
                       &s->z_old, &s->E_hist[0], &s->E_hist[1], &s->E_hist[2]};
   for (double **p : inner)
@@ -788,17 +784,14 @@ static sph_rt_status step_common(sph_rt *s, double dt, const double *Qe_c, const
   sph_rt_stats st;
   memset(&st, 0, sizeof st);
   const int64_t ni = s->n_int;
-  const size_t nb = sizeof(double) * ni;
-
   SPH_TRACE("step: begin n=%lld n_int=%lld nnz=%lld dt=%g", (long long)s->n, (long long)s->n_int,
             (long long)s->nnz_mat, dt);
-  // input check and energy before the step.  They are read with the step's
-  // results at the end (one host round trip per step); a step that will build
-  // the AMG structure reads them first, so that the kept hierarchy never comes
-  // from a rejected input.
-  if ((rc = launch_check_inputs(s, Qe_c, QE_c, ge_c, gE_c))) return rc;
-  if ((rc = launch_totals(s, s->e, s->E))) return rc;
-  if ((rc = launch_save_before(s))) return rc;
+  // snapshot of the state (restored if the step does not converge), sources in slot
+  // order, input check and energy before the step.  The check is read with the
+  // step's results at the end (one host round trip per step); a step that will build
+  // the AMG structure reads it first, so that the kept hierarchy never comes from a
+  // rejected input.
+  if ((rc = launch_step_begin(s, Qe_c, QE_c, ge_c, gE_c))) return rc;
   if (s->cfg.precond == SPH_RT_PRECOND_AMG && (!s->amg_ready || s->cfg.amg_rebuild)) {
     if ((rc = read_scalars(s))) return rc;
     if (s->sc_host->bad_input)
@@ -806,16 +799,9 @@ static sph_rt_status step_common(sph_rt *s, double dt, const double *Qe_c, const
   }
 
   tm.begin(0);
-  // snapshot of the state (restored if the step does not converge)
-  SPH_CUDA(s, cudaMemcpyAsync(s->e_bak, s->e, sizeof(double) * s->n, cudaMemcpyDeviceToDevice, s->stream));
-  SPH_CUDA(s, cudaMemcpyAsync(s->E_bak, s->E, sizeof(double) * s->n, cudaMemcpyDeviceToDevice, s->stream));
-  // sources (interior, slot order)
-  if ((rc = launch_gather_interior(s, Qe_c, s->Qe))) return rc;
-  if ((rc = launch_gather_interior(s, QE_c, s->QE))) return rc;
-  // material data from the state at the start of the step (a3)
-  if ((rc = launch_properties(s, dt))) return rc;
-  // Dirichlet ghost values at t^n
-  if ((rc = launch_ghost_install(s, ge_c, gE_c))) return rc;
+  // material data from the state at the start of the step (a3), then the Dirichlet
+  // ghost values at t^n
+  if ((rc = launch_properties(s, dt, ge_c, gE_c))) return rc;
   tm.end();
 
   SPH_TRACE("step: properties and ghosts queued");
@@ -846,22 +832,15 @@ static sph_rt_status step_common(sph_rt *s, double dt, const double *Qe_c, const
   // (E^{n-2}, the last step's start, before E_old is overwritten).
   const int K = s->cfg.krylov_start;
   const int order = std::min(K, s->hist);
-  if (K >= 1) {
-    for (int j = K - 1; j >= 1; --j)
-      SPH_CUDA(s, cudaMemcpyAsync(s->E_hist[j], s->E_hist[j - 1], nb, cudaMemcpyDeviceToDevice,
-                                  s->stream));
-    SPH_CUDA(s, cudaMemcpyAsync(s->E_hist[0], s->E_old, nb, cudaMemcpyDeviceToDevice, s->stream));
-  }
   double gw[4] = {1.0, 0.0, 0.0, 0.0};
   if (order >= 1) extrap_weights(order, dt, s->dt_hist, gw);
-  if ((rc = launch_set_guess(s, order, gw))) return rc;
+  if ((rc = launch_step_start(s, K, order, gw))) return rc;
   const int hist0 = s->hist;
   s->hist = 0;  // until this step has converged
-  SPH_CUDA(s, cudaMemcpyAsync(s->e_old, s->e, nb, cudaMemcpyDeviceToDevice, s->stream));
-  SPH_CUDA(s, cudaMemcpyAsync(s->E_old, s->E, nb, cudaMemcpyDeviceToDevice, s->stream));
-  SPH_CUDA(s, cudaMemcpyAsync(s->E_l, s->E, nb, cudaMemcpyDeviceToDevice, s->stream));
   tm.begin(4);
-  if ((rc = launch_newton(s, dt, s->E_l, s->E_l, s->e_old, s->e_l))) return rc;  // a8
+  if ((rc = launch_newton(s, dt, s->E_l, s->E_l, s->e_old, s->e_l,
+                          OuterTail{kOuterInit, 0, 0, 0.0, 0.0, 0})))  // a8
+    return rc;
   tm.end();
 
   // Alg. 1 outer loop: rhs (a7), Krylov solve (a6), material solve (a8) and the
@@ -871,10 +850,7 @@ static sph_rt_status step_common(sph_rt *s, double dt, const double *Qe_c, const
   tm.end();
   // commit (converged, valid input) or restore the snapshot, ghost copies,
   // energy balance and totals; then the one host read of the step
-  if ((rc = launch_finish(s, s->e_l, s->E_l))) return rc;
-  if ((rc = launch_copy_sync(s))) return rc;
-  if ((rc = launch_balance(s, dt, s->E))) return rc;
-  if ((rc = launch_totals(s, s->e, s->E))) return rc;
+  if ((rc = launch_step_end(s, dt, s->e_l, s->E_l))) return rc;
   // time step choice (Sec. 3.3) from the committed state; a step that did not
   // converge restored the snapshot, so its proposal is not reported
   if (s->cfg.dt_target > 0.0 && (rc = launch_dt_control(s, dt))) return rc;
