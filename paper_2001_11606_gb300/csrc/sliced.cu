@@ -14,8 +14,9 @@ sph_rt_status exclusive_scan(sph_rt *s, const int64_t *in, int64_t n, int64_t *o
 // keys, at most kWordCap of them used.
 constexpr int kWordTable = 2048;
 constexpr int kWordCap = 1024;
-// largest dictionary: its FP64 staging stays within 48 KB of shared memory
-constexpr int kDictCap = 5632;
+// largest dictionary: a block stages it in FP64 beside its own shared memory (up to
+// 7.2 KB: the assembly), and the two stay within the 48 KB of any launch
+constexpr int kDictCap = 5120;
 
 static int blocks_for(const sph_rt *s, int64_t n, int per_block, int per_sm) {
   const int64_t g = ceil_div(n > 0 ? n : 1, per_block), cap = (int64_t)s->num_sms * per_sm;
