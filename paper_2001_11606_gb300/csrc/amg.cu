@@ -942,11 +942,8 @@ __global__ void __launch_bounds__(kBlock, kCoarseMinBlocks)
     }
   }
   if (DOT) {
-    __shared__ double sh[32];
-    da = block_sum(da, sh);
-    __syncthreads();
-    db = block_sum(db, sh);
     double part[2] = {da, db}, out[2];
+    block_sums(part);
     const bool mx[2] = {false, false};
     if (last_block_combine<2>(part, df.partials, &df.sc->counter, out, mx) && threadIdx.x == 0) {
       Scalars *w = df.sc;
@@ -1276,11 +1273,8 @@ __global__ void __launch_bounds__(kBlock, Rows::kMinBlocks)
         }
       });
   if (DOT) {
-    __shared__ double sh[32];
-    da = block_sum(da, sh);
-    __syncthreads();
-    db = block_sum(db, sh);
     double part[2] = {da, db}, out[2];
+    block_sums(part);
     const bool mx[2] = {false, false};
     if (last_block_combine<2>(part, df.partials, &df.sc->counter, out, mx) && threadIdx.x == 0) {
       Scalars *w = df.sc;
@@ -1380,12 +1374,8 @@ __device__ __forceinline__ void fcg_row(int64_t i, VT zn, VT wn, VT r, VT zo, VT
 template <typename VT>
 __device__ __forceinline__ void fcg_reduce(double (&acc)[5], int first, Scalars *sc,
                                            double *partials, const LoopCond &cond) {
-  __shared__ double sh[32];
-  for (int k = 0; k < 5; ++k) {
-    acc[k] = block_sum(acc[k], sh);
-    __syncthreads();
-  }
   double out[5];
+  block_sums(acc);
   const bool mx[5] = {false, false, false, false, false};
   if (last_block_combine<5>(acc, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     fcg_scalars(out, first, sc);

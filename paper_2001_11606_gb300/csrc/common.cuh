@@ -124,77 +124,95 @@ __device__ __forceinline__ double group_sum(double v) {
   return v;
 }
 
-// Sum of v over the block; result valid in thread 0.  `sh` holds >= 32 doubles.
-__device__ __forceinline__ double block_sum(double v, double *sh) {
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  v = warp_sum(v);
-  __syncthreads();
-  if (lane == 0) sh[wid] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (wid == 0) {
-    int nw = (blockDim.x + 31) >> 5;
-    s = lane < nw ? sh[lane] : 0.0;
-    s = warp_sum(s);
+// Reduction of NV values over a block of kBlock threads, valid in thread 0: sums, or
+// maxima (of non-negative quantities) where is_max[k].  Every thread calls it, twice in
+// a kernel only with a barrier between.
+//
+// An FP64 operation costs a warp 16 cycles of its SM whatever its active lanes, so a
+// shuffle tree in each of the 8 warps is 8 x 5 of them per value.  Here the warps
+// shuffle once (twice with several values: shared memory is what the sliced rows'
+// dictionaries leave) and ONE warp per value adds what they left, in a fixed order:
+// 8 + 3 + 5 operations per value (16 + 1 + 5).
+template <int NV>
+__device__ __forceinline__ void block_reduce(double (&v)[NV], const bool (&is_max)[NV]) {
+  static_assert(NV <= kWarpsPerBlock, "one warp per value");
+  constexpr int R = NV == 1 ? 1 : 2;                 // shuffles before shared memory
+  constexpr int N = kBlock >> R;                     // values left, of each
+  __shared__ double sh[NV][N];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+#pragma unroll
+    for (int o = 16; o > (16 >> R); o >>= 1) {
+      const double u = __shfl_xor_sync(0xffffffffu, v[k], o);
+      v[k] = is_max[k] ? fmax(v[k], u) : v[k] + u;
+    }
+    if (lane < (32 >> R)) sh[k][wid * (32 >> R) + lane] = v[k];
   }
-  return s;
+  __syncthreads();
+  if (wid < NV) {
+    const double *p = sh[wid] + lane;
+    bool mx = false;
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+      if (wid == k) mx = is_max[k];
+    double x = p[0], y = p[32];
+#pragma unroll
+    for (int w = 64; w < N; w += 64) {
+      x = mx ? fmax(x, p[w]) : x + p[w];
+      y = mx ? fmax(y, p[w + 32]) : y + p[w + 32];
+    }
+    x = mx ? warp_max(fmax(x, y)) : warp_sum(x + y);
+    if (NV == 1)
+      v[0] = x;
+    else if (lane == 0)
+      sh[wid][0] = x;
+  }
+  if (NV > 1) {
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] = sh[k][0];
+  }
 }
-__device__ __forceinline__ double block_max(double v, double *sh) {
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  v = warp_max(v);
-  __syncthreads();
-  if (lane == 0) sh[wid] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (wid == 0) {
-    int nw = (blockDim.x + 31) >> 5;
-    s = lane < nw ? sh[lane] : 0.0;
-    s = warp_max(s);
-  }
-  return s;
+
+template <int NV>
+__device__ __forceinline__ void block_sums(double (&v)[NV]) {
+  const bool mx[NV] = {};
+  block_reduce<NV>(v, mx);
 }
 
 // Last-block reduction: every block stores its NV partial values, the block
 // that arrives last combines all partials in block order (so the result does
 // not depend on scheduling) and returns true in all its threads; `out` then
 // holds the NV totals in thread 0 (sums, or maxima where is_max[k]).
+//
+// The ticket is taken with acquire-release order: it publishes the partials of
+// thread 0 and, in the last block, makes all of them visible behind the barrier.  (A
+// __threadfence before it and one per thread after it are sequentially consistent
+// fences, of ~1 us each on the critical path of every reduction.)
 template <int NV>
 __device__ bool last_block_combine(const double (&part)[NV], double *partials, unsigned *counter,
                                    double (&out)[NV], const bool (&is_max)[NV]) {
   __shared__ bool am_last;
-  __shared__ double sh[NV][32];
   if (threadIdx.x == 0) {
     for (int k = 0; k < NV; ++k) partials[(size_t)k * gridDim.x + blockIdx.x] = part[k];
-    __threadfence();
-    unsigned ticket = atomicAdd(counter, 1u);
+    unsigned ticket;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;"
+                 : "=r"(ticket)
+                 : "l"(__cvta_generic_to_global(counter))
+                 : "memory");
     am_last = (ticket == gridDim.x - 1);
   }
   __syncthreads();
   if (!am_last) return false;
-  __threadfence();
-  // each thread folds a strided subset in order, then a fixed-shape tree; the NV
-  // values go through both together, so their latencies overlap
-  double acc[NV];
-  for (int k = 0; k < NV; ++k) acc[k] = 0.0;  // partial maxima are of non-negative quantities
+  // each thread folds a strided subset in order, then the block's reduction
+  for (int k = 0; k < NV; ++k) out[k] = 0.0;  // partial maxima are of non-negative quantities
   for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
     for (int k = 0; k < NV; ++k) {
       const double v = ((volatile double *)partials)[(size_t)k * gridDim.x + b];
-      acc[k] = is_max[k] ? fmax(acc[k], v) : acc[k] + v;
+      out[k] = is_max[k] ? fmax(out[k], v) : out[k] + v;
     }
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int k = 0; k < NV; ++k) {
-    acc[k] = is_max[k] ? warp_max(acc[k]) : warp_sum(acc[k]);
-    if (lane == 0) sh[k][wid] = acc[k];
-  }
-  __syncthreads();
-  if (wid == 0) {
-    const int nw = (blockDim.x + 31) >> 5;
-    for (int k = 0; k < NV; ++k) {
-      const double v = lane < nw ? sh[k][lane] : 0.0;
-      out[k] = is_max[k] ? warp_max(v) : warp_sum(v);
-    }
-  }
-  __syncthreads();
+  block_reduce<NV>(out, is_max);
   if (threadIdx.x == 0) *counter = 0u;
   return true;
 }

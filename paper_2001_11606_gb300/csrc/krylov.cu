@@ -54,9 +54,8 @@ __global__ void __launch_bounds__(kBlock, Rows::kMinBlocks)
         const double ru = ri * o.d;
         acc += ru * ru;
       });
-  __shared__ double sh[32];
-  acc = block_sum(acc, sh);
   double part[1] = {acc}, out[1];
+  block_sums(part);
   const bool mx[1] = {false};
   if (last_block_combine<1>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     sc->rnorm2 = out[0];
@@ -96,9 +95,8 @@ __global__ void __launch_bounds__(kBlock, Rows::kMinBlocks)
         p[i] = pi;
         acc += pi * qi;
       });
-  __shared__ double sh[32];
-  acc = block_sum(acc, sh);
   double part[1] = {acc}, out[1];
+  block_sums(part);
   const bool mx[1] = {false};
   if (last_block_combine<1>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     double pq = out[0];
@@ -141,9 +139,8 @@ __global__ void update_kernel(int64_t n, double *x, double *r, const double *p, 
       fi.z[i] = di;
     }
   }
-  __shared__ double sh[32];
-  acc = block_sum(acc, sh);
   double part[1] = {acc}, out[1];
+  block_sums(part);
   const bool mx[1] = {false};
   if (last_block_combine<1>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     sc->rnorm2 = out[0];
@@ -165,9 +162,8 @@ __global__ void jacobi_dot_kernel(int64_t n, const double *r, const double *invd
     z[i] = zi;
     acc += r[i] * zi;
   }
-  __shared__ double sh[32];
-  acc = block_sum(acc, sh);
   double part[1] = {acc}, out[1];
+  block_sums(part);
   const bool mx[1] = {false};
   if (last_block_combine<1>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     if (!first) sc->beta = out[0] / sc->rho;
@@ -185,9 +181,8 @@ __global__ void dot_rz_kernel(int64_t n, const double *r, const VT *z, int first
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     acc += r[i] * (double)z[i];
-  __shared__ double sh[32];
-  acc = block_sum(acc, sh);
   double part[1] = {acc}, out[1];
+  block_sums(part);
   const bool mx[1] = {false};
   if (last_block_combine<1>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     if (!first) sc->beta = out[0] / sc->rho;
@@ -210,11 +205,8 @@ __global__ void dot_rz_flex_kernel(int64_t n, const double *r, const double *z,
     a += ri * z[i];
     if (!first) b += ri * z_old[i];
   }
-  __shared__ double sh[32];
-  a = block_sum(a, sh);
-  __syncthreads();
-  b = block_sum(b, sh);
   double part[2] = {a, b}, out[2];
+  block_sums(part);
   const bool mx[2] = {false, false};
   if (last_block_combine<2>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     if (!first) sc->beta = (out[0] - out[1]) / sc->rho;
@@ -240,11 +232,8 @@ __global__ void dot_rz_flex32_kernel(int64_t n, const double *r, const float *z3
     a += ri * zn;
     z[i] = zn;
   }
-  __shared__ double sh[32];
-  a = block_sum(a, sh);
-  __syncthreads();
-  b = block_sum(b, sh);
   double part[2] = {a, b}, out[2];
+  block_sums(part);
   const bool mx[2] = {false, false};
   if (last_block_combine<2>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     if (!first) sc->beta = (out[0] - out[1]) / sc->rho;
@@ -662,9 +651,8 @@ __global__ void __launch_bounds__(kBlock, Rows::kMinBlocks)
         const double ru = ri * o.d;
         acc += ru * ru;
       });
-  __shared__ double sh[32];
-  acc = block_sum(acc, sh);
   double part[1] = {acc}, out[1];
+  block_sums(part);
   const bool mx[1] = {false};
   if (last_block_combine<1>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     sc->rnorm2 = out[0];
@@ -697,9 +685,8 @@ __global__ void fcg_start_y_kernel(int64_t n, const double *b, const double *y, 
     const double ru = ri * invV[i];
     acc += ru * ru;
   }
-  __shared__ double sh[32];
-  acc = block_sum(acc, sh);
   double part[1] = {acc}, out[1];
+  block_sums(part);
   const bool mx[1] = {false};
   if (last_block_combine<1>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     sc->rnorm2 = out[0];
@@ -743,9 +730,8 @@ __global__ void fcg_update_kernel(int64_t n, double *x, T *r, T *p, T *q, const 
     const double ru = rd * invV[i];
     acc += ru * ru;
   }
-  __shared__ double sh[32];
-  acc = block_sum(acc, sh);
   double part[1] = {acc}, out[1];
+  block_sums(part);
   const bool mx[1] = {false};
   if (last_block_combine<1>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     const double rn = out[0];

@@ -45,12 +45,9 @@ __global__ void totals_noalloc_kernel(int64_t n, const int32_t *kind, const doub
       b += mass[i] / rho[i] * E[i];
     }
   }
-  __shared__ double sh[32];
-  a = sphrt::block_sum(a, sh);
-  __syncthreads();
-  b = sphrt::block_sum(b, sh);
   unsigned *counter = reinterpret_cast<unsigned *>(scratch + kNaCounterSlot);
   double part[2] = {a, b}, res[2];
+  sphrt::block_sums(part);
   const bool mx[2] = {false, false};
   // the last block to arrive combines the partials in block order and resets
   // the counter, so the array is ready for the next call

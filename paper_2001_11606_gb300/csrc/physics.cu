@@ -406,10 +406,9 @@ __global__ void __launch_bounds__(kBlock, kPairMinBlocks)
       gmax = fmax(gmax, -offsum / d);  // off-diagonals are <= 0
     }
   }
-  __shared__ double sh[32];
-  gmax = block_max(gmax, sh);
   double part[1] = {gmax}, out[1];
   const bool mx[1] = {true};
+  block_reduce(part, mx);
   if (last_block_combine<1>(part, partials, counter, out, mx) && threadIdx.x == 0)
     *gersh_out = out[0];
 }
@@ -517,10 +516,9 @@ __global__ void __launch_bounds__(kBlock, 4)
     gb[i] = sums[2][threadIdx.x];
     gmax = fmax(gmax, -offsum * inv);  // off-diagonals are <= 0
   }
-  __shared__ double sh[32];
-  gmax = block_max(gmax, sh);
   double part[1] = {gmax}, out[1];
   const bool mx[1] = {true};
+  block_reduce(part, mx);
   if (last_block_combine<1>(part, partials, counter, out, mx) && threadIdx.x == 0)
     *gersh_out = out[0];
 }
@@ -554,9 +552,8 @@ __global__ void rhs_kernel(Phys ph, int64_t n_int, const double *V, const double
     x[i] = xi;
     acc += bi * bi;
   }
-  __shared__ double sh[32];
-  double bs = block_sum(acc, sh);
-  double part[1] = {bs}, out[1];
+  double part[1] = {acc}, out[1];
+  block_sums(part);
   const bool mx[1] = {false};
   if (last_block_combine<1>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     sc->bnorm2 = out[0];
@@ -728,13 +725,9 @@ __global__ void step_begin_kernel(int64_t n_int, int64_t n, const int64_t *slot2
       if ((ge && !isfinite(ge[c])) || (gE && !isfinite(gE[c]))) bad = 1;
     }
   }
-  __shared__ double sh[32];
-  bad = __syncthreads_or(bad);
-  const double pa = block_sum(a, sh);
-  __syncthreads();
-  const double pb = block_sum(b, sh);
-  double part[3] = {pa, pb, bad ? 1.0 : 0.0}, out[3];
+  double part[3] = {a, b, bad ? 1.0 : 0.0}, out[3];
   const bool mx[3] = {false, false, true};
+  block_reduce(part, mx);
   if (last_block_combine<3>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     sc->energy_before_e = out[0];
     sc->energy_before_E = out[1];
@@ -777,11 +770,8 @@ __global__ void totals_kernel(int64_t n_int, const double *mass, const double *V
     a += mass[i] * e[i];
     b += V[i] * E[i];
   }
-  __shared__ double sh[32];
-  double pa = block_sum(a, sh);
-  __syncthreads();
-  double pb = block_sum(b, sh);
-  double part[2] = {pa, pb}, out[2];
+  double part[2] = {a, b}, out[2];
+  block_sums(part);
   const bool mx[2] = {false, false};
   if (last_block_combine<2>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     sc->red[4] = out[0];
@@ -835,16 +825,8 @@ __global__ void step_end_kernel(Phys ph, int64_t n_int, int64_t n, int64_t nnz_g
       const int32_t i = gh_row[k], j = gh_slot[k];  // j: a ghost, not written above
       b -= (V[i] * gh_W[k]) * (D[i] + D[j]) * (E[j] - E_new[i]);
     }
-  __shared__ double sh[32];
-  double part[4];
-  part[0] = block_sum(te, sh);
-  __syncthreads();
-  part[1] = block_sum(tE, sh);
-  __syncthreads();
-  part[2] = block_sum(a, sh);
-  __syncthreads();
-  part[3] = block_sum(b, sh);
-  double out[4];
+  double part[4] = {te, tE, a, b}, out[4];
+  block_sums(part);
   const bool mx[4] = {false, false, false, false};
   if (last_block_combine<4>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     sc->red[4] = out[0];
@@ -1080,14 +1062,8 @@ __global__ void dtc_sums_kernel(int64_t n_int, const double *V, const double *e,
     b += E[i] * Vi;
     v += Vi;
   }
-  __shared__ double sh[32];
-  double part[3];
-  part[0] = block_sum(a, sh);
-  __syncthreads();
-  part[1] = block_sum(b, sh);
-  __syncthreads();
-  part[2] = block_sum(v, sh);
-  double out[3];
+  double part[3] = {a, b, v}, out[3];
+  block_sums(part);
   const bool mx[3] = {false, false, false};
   if (last_block_combine<3>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     sc->dtc_ebar = out[0] / out[2];
@@ -1110,13 +1086,9 @@ __global__ void dtc_eta_kernel(int64_t n_int, const double *e, const double *E,
     me = fmax(me, fabs(en - e_old[i]) / (en + de));
     mE = fmax(mE, fabs(En - E_old[i]) / (En + dE));
   }
-  __shared__ double sh[32];
-  double part[2];
-  part[0] = block_max(me, sh);
-  __syncthreads();
-  part[1] = block_max(mE, sh);
-  double out[2];
+  double part[2] = {me, mE}, out[2];
   const bool mx[2] = {true, true};
+  block_reduce(part, mx);
   if (last_block_combine<2>(part, partials, &sc->counter, out, mx) && threadIdx.x == 0) {
     double next = fmin(c.growth * c.dt, c.dt_max);
     if (out[0] > 0.0) next = fmin(next, c.dt * sqrt(c.target / out[0]));
