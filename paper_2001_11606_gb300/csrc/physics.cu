@@ -584,6 +584,8 @@ __device__ void outer_init(Scalars *sc) {
 // bookkeeping of the step statistics and the outer convergence test
 // max_i |x^{l+1} - x^l| / |x^{l+1}| < tol for e and E (changes in red[0..1],
 // Newton iterations in red[2]).  In the graph it also sets the loop condition.
+// (As kernels of their own, this, the copy of the iterate and outer_init took 2-4 us
+// each of a step that is 430 us at 1,024 particles.)
 __device__ void outer_check(Scalars *sc, const OuterTail &t) {
   int status = 0;
   sc->outer_trips += 1;
@@ -699,7 +701,9 @@ __global__ void __launch_bounds__(kBlock)
 // Start of a step, in one pass over the slots: the snapshot of the state, the
 // sources gathered to slot order (null: 0), the check that the step's inputs are
 // finite (sources of interior particles, values of Dirichlet ghosts; caller order)
-// and the energy before the step.
+// and the energy before the step.  Latency at small sizes (5.2 us at 1,024 particles),
+// HBM at large ones (10.4 us at 2.5e5), in place of nine launches and copies of 2-4 us
+// each.
 __global__ void step_begin_kernel(int64_t n_int, int64_t n, const int64_t *slot2caller,
                                   const int32_t *kind, const double *Qe_c, const double *QE_c,
                                   const double *ge, const double *gE, const double *mass,
@@ -788,7 +792,8 @@ __global__ void totals_kernel(int64_t n_int, const double *mass, const double *V
 //   red[7]          added through the boundary, dt sum_i V_i sum_{Dirichlet j} w_ij
 //                   (E_j - E_i), over the couplings as one flat list: few rows have
 //                   any, those have tens, and a thread per row spent its time on the
-//                   longest (0.22 ms at 128^3 with 5.7e6 couplings, now 0.076 alone)
+//                   longest (0.22 ms at 128^3 with 5.7e6 couplings, 0.076 flat)
+// One launch, 7.1 us at 1,024 particles and 12 us at 2.5e5, in place of four.
 __global__ void step_end_kernel(Phys ph, int64_t n_int, int64_t n, int64_t nnz_gh,
                                 const int32_t *copysrc, const double *e_new,
                                 const double *E_new, const double *e_bak, const double *E_bak,
