@@ -885,6 +885,7 @@ struct sph_rt {
   std::vector<void *> allocs;  // device allocations of the current particle set
   std::unordered_map<void *, size_t> alloc_size;
   std::multimap<size_t, void *> pool;  // released buffers kept for reuse
+  int64_t test_fail_after = -1;  // sph_rt_test_hook: allocations until one fails (-1: none)
 
   // sizes
   bool have_particles = false;
@@ -925,7 +926,7 @@ struct sph_rt {
   SlicedRowsData sl;
   double *sl_G = nullptr, *sl_val = nullptr;
   float *sl_val32 = nullptr;
-  bool sl_refused = false;  // a group's dictionary was too large for this particle set
+  bool sl_decided = false;  // the layout of this particle set is chosen (sliced_operator)
   int64_t *gh_ptr = nullptr;   // Dirichlet-ghost couplings
   int32_t *gh_slot = nullptr;
   double *gh_W = nullptr;      // V_j F_ij

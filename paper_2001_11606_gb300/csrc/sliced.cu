@@ -28,18 +28,19 @@ static int blocks_for(const sph_rt *s, int64_t n, int per_block, int per_sm) {
 // level must be one that has A P.  Measured: at 1.6 groups per SM (64,000 rows of
 // 256 entries) a job took 31.0 ms sliced and 29.4 in row tiles, at 2.2 (86,387 rows
 // of 26) 25.5 against 27.2, at 54 (2.1e6 rows of 104, mixed) 382 against 457.
-// The slices take ~19 bytes per entry beside the CSR rows while they are built;
-// where that could crowd out the AMG set-up of a set that fills the device, the
-// CSR rows stay.
-bool sliced_wanted(const sph_rt *s) {
-  if (s->n_int < (int64_t)kSliceMinGroups * s->num_sms * kBlock || s->nnz_mat <= kTailMaxNnz || s->sl_refused) return false;
-  if (s->nnz_mat > (int64_t)500000000) {
-    size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
-    for (auto &kv : s->pool) free_b += kv.first;
-    if ((double)free_b < 80.0 * (double)s->nnz_mat) return false;
-  }
-  return true;
+// A set holds ~36 bytes per entry in CSR rows; building the slices takes ~19 more and
+// the AMG set-up its lists: a set that has less than kSliceBytes of the device per
+// entry stays in CSR rows.  Sizes alone decide, never the memory that happens to be
+// free: the two layouts add a row in different orders, and the same set is to give the
+// same bits in every run.
+static bool sliced_wanted(const sph_rt *s) {
+  constexpr double kSliceBytes = 125.0;
+  if (s->n_int < (int64_t)kSliceMinGroups * s->num_sms * kBlock || s->nnz_mat <= kTailMaxNnz)
+    return false;
+  if (s->nnz_mat <= (int64_t)500000000) return true;  // 63 GB, of the 284 of a GB300
+  size_t free_b = 0, total_b = 0;
+  return cudaMemGetInfo(&free_b, &total_b) == cudaSuccess &&
+         kSliceBytes * (double)s->nnz_mat <= (double)total_b;
 }
 
 // ---------------------------------------------------------------------------
@@ -403,11 +404,15 @@ static void release_slices(sph_rt *s) {
   s->sl_val32 = nullptr;
 }
 
-// The fine operator's slices, once per particle set (before its first
-// assembly): geometry moved from mat_G, which is released with the CSR values.
-// Without room for them, or with too large a dictionary, the CSR rows stay.
+// The fine operator's slices, before the particle set's first assembly: geometry
+// moved from mat_G, which is released with the CSR values.  Tried once per particle
+// set: buffers of the kept AMG hierarchy and of the captured step graph refer to the
+// layout, so a set never changes to slices later.  Without room for them, or with too
+// large a dictionary, the CSR rows stay.
 sph_rt_status sliced_operator(sph_rt *s) {
-  if (s->sl.ptr || !sliced_wanted(s)) return SPH_RT_OK;
+  if (s->sl_decided) return SPH_RT_OK;
+  s->sl_decided = true;
+  if (!sliced_wanted(s)) return SPH_RT_OK;
   bool ok = false;
   sph_rt_status rc = sliced_build(s, s->n_int, s->mat_ptr, s->mat_col, s->mat_G, take_handle,
                                   nullptr, &s->sl, &s->sl_G, &ok);
@@ -420,7 +425,6 @@ sph_rt_status sliced_operator(sph_rt *s) {
   if (rc != SPH_RT_OK && rc != SPH_RT_ENOMEM) return rc;
   if (rc != SPH_RT_OK || !ok) {
     release_slices(s);
-    s->sl_refused = true;
     s->err.clear();
     return SPH_RT_OK;
   }
@@ -460,7 +464,6 @@ sph_rt_status sliced_undo(sph_rt *s) {
   }
   SPH_CUDA(s, cudaStreamSynchronize(s->stream));
   release_slices(s);
-  s->sl_refused = true;
   return SPH_RT_OK;
 }
 

@@ -15,7 +15,6 @@ constexpr int kSliceMinGroups = 2;
 constexpr int kNoPlace = 0xffff;            // sliced A P: column without an aggregate
 constexpr int kApSmemMax = 200 * 1024;
 
-bool sliced_wanted(const sph_rt *s);
 sph_rt_status sliced_operator(sph_rt *s);
 sph_rt_status sliced_to_csr(sph_rt *s, double **csr);
 sph_rt_status sliced_undo(sph_rt *s);

@@ -134,6 +134,10 @@ static void pool_release(sph_rt *s) {
 
 void *dalloc_bytes(sph_rt *s, size_t bytes) {
   bytes = (bytes + 255) & ~(size_t)255;
+  if (s->test_fail_after >= 0 && s->test_fail_after-- == 0) {
+    s->err = "device allocation refused by sph_rt_test_hook";
+    return nullptr;
+  }
   auto it = s->pool.lower_bound(bytes);
   if (it != s->pool.end() && it->first <= 2 * bytes) {
     void *p = it->second;
@@ -200,7 +204,7 @@ void free_all(sph_rt *s) {
   s->sl = SlicedRowsData{};
   s->sl_G = s->sl_val = nullptr;
   s->sl_val32 = nullptr;
-  s->sl_refused = false;
+  s->sl_decided = false;
   s->diag32 = s->invdiag32 = nullptr;
   s->amg_gersh = nullptr;
   s->cheb_slots = nullptr;
@@ -396,6 +400,14 @@ extern "C" sph_rt_status sph_rt_release_cached_memory(int32_t device) {
   if (device < 0) return SPH_RT_EINVAL;
   cache_trim(device);
   return SPH_RT_OK;
+}
+
+// For the tests of the fall-backs, not part of the interface: makes one device
+// allocation of the handle fail, after `fail_after` more that succeed (-1: none).
+// Returns the number of buffers in use.
+extern "C" int64_t sph_rt_test_hook(sph_rt *s, int64_t fail_after) {
+  s->test_fail_after = fail_after;
+  return (int64_t)s->allocs.size();
 }
 
 extern "C" const char *sph_rt_last_error(const sph_rt *s) {

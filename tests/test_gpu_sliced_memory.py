@@ -1,0 +1,90 @@
+"""The sliced layout where memory is short: whichever allocation of the first step
+fails, the set falls back to CSR rows and stays there; results are those of that layout,
+bit for bit."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+from paper_2001_11606_gb300 import inputs as I
+from paper_2001_11606_gb300 import sphrt
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _workload():
+    # the sliced layout starts at 512 rows per SM
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = int(np.ceil(np.sqrt(512 * sms)))
+    P = I.make_lattice(2, (n, n), 1.0 / n, 4)
+    m = I.Manufactured(dim=2)
+    e0, E0 = m.fields(P.pos, 0.0)
+    return I.Workload("mms", P, dict(dim=2, tol_krylov=1e-13), 1e-3, 3, mms=m, e0=e0, E0=E0)
+
+
+def _hook(S, fail_after=-1):
+    fn = sphrt.load().sph_rt_test_hook
+    fn.restype, fn.argtypes = C.c_int64, [C.c_void_p, C.c_int64]
+    return fn(S._h, fail_after)
+
+
+def _column_bytes(S, w):
+    """Bytes per stored column of the CG's product sweep: 2 in slices, 4 in CSR rows."""
+    launches, _, by = S.kernel_stats_by_kind()["spmv_pq"]
+    if launches == 0:  # the CG takes its product from the V-cycle
+        return None
+    n_int, _, nnz = S.sizes()
+    return round((by / launches - 56.0 * n_int) / nnz - 8.0)
+
+
+@pytest.fixture(scope="module")
+def case():
+    w = _workload()
+    return w, [w.step_inputs(k) for k in (1, 2, 3)]
+
+
+def _run(case, fail_after=-1, steps=3, **over):
+    w, ins = case
+    S = sphrt.solver_for(w, kernel_timing=1, **over)
+    before = _hook(S, fail_after)
+    out, held = [], []
+    for k in range(steps):
+        S.step(w.dt, *ins[k])
+        out.append(_column_bytes(S, w))
+        # the hook's own call ends the countdown: what it did not reach stays alive
+        held.append(_hook(S, -1) - before)
+    e, E, _ = S.get_energies()
+    S.close()
+    return out, held, e, E
+
+
+def _same(a, b):
+    return np.array_equal(a[2], b[2]) and np.array_equal(a[3], b[3])
+
+
+@pytest.mark.parametrize("over", [dict(precond=0), dict(precond=0, precision=1)])
+def test_any_failed_allocation_falls_back(case, over):
+    sliced = _run(case, **over)
+    csr = _run(case, fail_after=0, **over)
+    assert sliced[0] == [2, 2, 2] and csr[0] == [4, 4, 4]
+    seen = set()
+    for k in range(24):  # past the layout's
+        got = _run(case, fail_after=k, **over)
+        seen.add(got[0][0])
+        assert len(set(got[0])) == 1  # the layout of the first step is kept
+        assert _same(got, csr if got[0][0] == 4 else sliced)
+    assert 4 in seen and seen <= {2, 4}
+
+
+def test_a_new_set_chooses_again(case):
+    w, ins = case
+    S = sphrt.solver_for(w, precond=0, kernel_timing=1)
+    _hook(S, 0)
+    S.step(w.dt, *ins[0])
+    assert _column_bytes(S, w) == 4
+    S.move_particles(w.particles.pos)
+    S.kernel_stats(reset=True)
+    S.step(w.dt, *ins[1])
+    assert _column_bytes(S, w) == 2
+    S.close()
