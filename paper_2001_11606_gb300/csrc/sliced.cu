@@ -3,6 +3,8 @@
 // moving arrays between the two orders, and the values of A P.
 #include <cuda_runtime.h>
 
+#include <vector>
+
 #include "common.cuh"
 #include "sliced.cuh"
 
@@ -328,8 +330,9 @@ static sph_rt_status slice_move(sph_rt *s, int64_t n, const int64_t *ptr, const 
 }
 
 // Slices and dictionaries of the CSR rows (ptr, col); with `val`, those values in
-// slice order too.  *ok = false (nothing kept): a group's columns exceed the caps.
-// Buffers come from `take` (the caller owns them).
+// slice order too.  *ok = false: a group's columns exceed the caps.  Buffers come
+// from `take`; *out and *out_val hold those taken so far whatever the outcome, and
+// the caller releases them where the slices are not kept.
 sph_rt_status sliced_build(sph_rt *s, int64_t n, const int64_t *ptr, const int32_t *col,
                            const double *val, void *(*take)(sph_rt *, void *, size_t), void *owner,
                            SlicedRowsData *out, double **out_val, bool *ok) {
@@ -339,17 +342,25 @@ sph_rt_status sliced_build(sph_rt *s, int64_t n, const int64_t *ptr, const int32
   cudaStream_t st = s->stream;
   const int64_t slices = ceil_div(n, 32), groups = ceil_div(n, kBlock);
   SlicedRowsData &D = *out;  // filled in as it is allocated
-  int32_t *key = dalloc<int32_t>(s, groups * kWordCap), *nw = dalloc<int32_t>(s, groups);
-  uint32_t *mask = dalloc<uint32_t>(s, groups * kWordCap);
-  int64_t *nc = dalloc<int64_t>(s, groups), *w32 = dalloc<int64_t>(s, slices);
-  int *flags = dalloc<int>(s, 2);  // largest dictionary, refused
+  struct Scratch {           // back to the free list on every return
+    sph_rt *s;
+    std::vector<void *> held;
+    ~Scratch() {
+      cudaStreamSynchronize(s->stream);
+      for (void *p : held) dfree(s, p);
+    }
+    void *take(size_t bytes) {
+      held.push_back(dalloc_bytes(s, bytes));
+      return held.back();
+    }
+  } tmp{s, {}};
+  int32_t *key = (int32_t *)tmp.take(sizeof(int32_t) * groups * kWordCap);
+  uint32_t *mask = (uint32_t *)tmp.take(sizeof(uint32_t) * groups * kWordCap);
+  int32_t *nw = (int32_t *)tmp.take(sizeof(int32_t) * groups);
+  int64_t *nc = (int64_t *)tmp.take(sizeof(int64_t) * groups);
+  int64_t *w32 = (int64_t *)tmp.take(sizeof(int64_t) * slices);
+  int *flags = (int *)tmp.take(sizeof(int) * 2);  // largest dictionary, refused
   if (!key || !nw || !mask || !nc || !w32 || !flags) return SPH_RT_ENOMEM;
-  auto done = [&](sph_rt_status rc) {
-    cudaStreamSynchronize(st);
-    void *scratch[] = {key, nw, mask, nc, w32, flags};
-    for (void *p : scratch) dfree(s, p);
-    return rc;
-  };
   SPH_CUDA(s, cudaMemsetAsync(flags, 0, 2 * sizeof(int), st));
   dict_words_kernel<<<blocks_for(s, groups, 1, 6), kBlock, 0, st>>>(n, ptr, col, key, mask, nw, nc,
                                                                     flags, flags + 1);
@@ -357,21 +368,21 @@ sph_rt_status sliced_build(sph_rt *s, int64_t n, const int64_t *ptr, const int32
   int hf[2] = {0, 0};
   SPH_CUDA(s, cudaMemcpyAsync(hf, flags, sizeof hf, cudaMemcpyDeviceToHost, st));
   SPH_CUDA(s, cudaStreamSynchronize(st));
-  if (hf[1]) return done(SPH_RT_OK);
+  if (hf[1]) return SPH_RT_OK;
   D.dict_max = hf[0];
   D.len = (int32_t *)take(s, owner, sizeof(int32_t) * n);
   D.ptr = (int64_t *)take(s, owner, sizeof(int64_t) * (slices + 1));
   D.dptr = (int64_t *)take(s, owner, sizeof(int64_t) * (groups + 1));
   D.order = (uint8_t *)take(s, owner, n);
   D.place = (uint8_t *)take(s, owner, n);
-  if (!D.len || !D.ptr || !D.dptr || !D.order || !D.place) return done(SPH_RT_ENOMEM);
+  if (!D.len || !D.ptr || !D.dptr || !D.order || !D.place) return SPH_RT_ENOMEM;
   static_assert(kBlock == 256, "a place within a group is a byte");
   slice_order_kernel<<<blocks_for(s, groups, 1, 8), kBlock, 0, st>>>(n, ptr, D.order, D.place,
                                                                     D.len, w32);
   SPH_LAUNCHED(s);
   sph_rt_status rc;
-  if ((rc = exclusive_scan(s, w32, slices, D.ptr))) return done(rc);
-  if ((rc = exclusive_scan(s, nc, groups, D.dptr))) return done(rc);
+  if ((rc = exclusive_scan(s, w32, slices, D.ptr))) return rc;
+  if ((rc = exclusive_scan(s, nc, groups, D.dptr))) return rc;
   int64_t total[2];
   SPH_CUDA(s, cudaMemcpyAsync(&total[0], D.ptr + slices, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
   SPH_CUDA(s, cudaMemcpyAsync(&total[1], D.dptr + groups, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
@@ -381,7 +392,7 @@ sph_rt_status sliced_build(sph_rt *s, int64_t n, const int64_t *ptr, const int32
   D.dict = (int32_t *)take(s, owner, sizeof(int32_t) * (total[1] + 1));
   double *v = val ? (double *)take(s, owner, sizeof(double) * (D.padded + 1)) : nullptr;
   if (out_val) *out_val = v;
-  if (!D.idx || !D.dict || (val && !v)) return done(SPH_RT_ENOMEM);
+  if (!D.idx || !D.dict || (val && !v)) return SPH_RT_ENOMEM;
   const int smem = (int)(sizeof(SliceTile) * kWarpsPerBlock + 12 * kWordCap);
   SPH_CUDA(s, cudaFuncSetAttribute(slice_fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    smem));
@@ -390,18 +401,14 @@ sph_rt_status sliced_build(sph_rt *s, int64_t n, const int64_t *ptr, const int32
       v);
   SPH_LAUNCHED(s);
   *ok = true;
-  return done(SPH_RT_OK);
+  return SPH_RT_OK;
 }
 
 static void *take_handle(sph_rt *s, void *, size_t bytes) { return dalloc_bytes(s, bytes); }
-static void release_slices(sph_rt *s) {
-  void *bufs[] = {s->sl.ptr, s->sl.dptr, s->sl.idx, s->sl.len, s->sl.dict, s->sl.order,
-                  s->sl.place, s->sl_G, s->sl_val,
-                  s->sl_val32};
+static void release_slices(sph_rt *s, const SlicedRowsData &d, double *G, double *val,
+                           float *val32) {
+  void *bufs[] = {d.ptr, d.dptr, d.idx, d.len, d.dict, d.order, d.place, G, val, val32};
   for (void *p : bufs) dfree(s, p);
-  s->sl = SlicedRowsData{};
-  s->sl_G = s->sl_val = nullptr;
-  s->sl_val32 = nullptr;
 }
 
 // The fine operator's slices, before the particle set's first assembly: geometry
@@ -414,20 +421,26 @@ sph_rt_status sliced_operator(sph_rt *s) {
   s->sl_decided = true;
   if (!sliced_wanted(s)) return SPH_RT_OK;
   bool ok = false;
+  SlicedRowsData d;
+  double *G = nullptr, *val = nullptr;
+  float *val32 = nullptr;
   sph_rt_status rc = sliced_build(s, s->n_int, s->mat_ptr, s->mat_col, s->mat_G, take_handle,
-                                  nullptr, &s->sl, &s->sl_G, &ok);
+                                  nullptr, &d, &G, &ok);
   if (rc == SPH_RT_OK && ok) {
-    // + 1: never of size 0
-    s->sl_val = dalloc<double>(s, s->sl.padded + 1);
-    if (s->cfg.precision == SPH_RT_MIXED) s->sl_val32 = dalloc<float>(s, s->sl.padded + 1);
-    ok = s->sl_val && (s->cfg.precision != SPH_RT_MIXED || s->sl_val32);
+    val = dalloc<double>(s, d.padded + 1);  // + 1: never of size 0
+    if (s->cfg.precision == SPH_RT_MIXED) val32 = dalloc<float>(s, d.padded + 1);
+    if (!val || (s->cfg.precision == SPH_RT_MIXED && !val32)) rc = SPH_RT_ENOMEM;
   }
-  if (rc != SPH_RT_OK && rc != SPH_RT_ENOMEM) return rc;
   if (rc != SPH_RT_OK || !ok) {
-    release_slices(s);
+    release_slices(s, d, G, val, val32);
+    if (rc != SPH_RT_OK && rc != SPH_RT_ENOMEM) return rc;
     s->err.clear();
     return SPH_RT_OK;
   }
+  s->sl = d;
+  s->sl_G = G;
+  s->sl_val = val;
+  s->sl_val32 = val32;
   dfree(s, s->mat_G);
   dfree(s, s->mat_val);
   dfree(s, s->mat_val32);
@@ -463,7 +476,10 @@ sph_rt_status sliced_undo(sph_rt *s) {
       return rc;
   }
   SPH_CUDA(s, cudaStreamSynchronize(s->stream));
-  release_slices(s);
+  release_slices(s, s->sl, s->sl_G, s->sl_val, s->sl_val32);
+  s->sl = SlicedRowsData{};
+  s->sl_G = s->sl_val = nullptr;
+  s->sl_val32 = nullptr;
   return SPH_RT_OK;
 }
 

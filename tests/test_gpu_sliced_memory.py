@@ -1,6 +1,6 @@
 """The sliced layout where memory is short: whichever allocation of the first step
-fails, the set falls back to CSR rows and stays there; results are those of that layout,
-bit for bit."""
+fails, the step falls back to CSR rows, holds nothing more than a set that was in CSR
+rows from the start, and stays there; results are those of that layout, bit for bit."""
 import ctypes as C
 
 import numpy as np
@@ -74,6 +74,7 @@ def test_any_failed_allocation_falls_back(case, over):
         seen.add(got[0][0])
         assert len(set(got[0])) == 1  # the layout of the first step is kept
         assert _same(got, csr if got[0][0] == 4 else sliced)
+        assert got[1] == (csr if got[0][0] == 4 else sliced)[1], k
     assert 4 in seen and seen <= {2, 4}
 
 
