@@ -1645,6 +1645,7 @@ __global__ void __launch_bounds__(1024, 1) vcycle_tail_kernel(const __grid_const
 // host: structure
 // ---------------------------------------------------------------------------
 CsrView<double> fine_view(const sph_rt *s);
+sph_rt_status launch_assembly(sph_rt *s, double dt, double *gersh_out);
 
 
 // bucket sort of ids by bucket[i] into (start, out); nb buckets
@@ -1725,13 +1726,13 @@ __global__ void max_len_kernel(int64_t n, const int32_t *len, int *most) {
   if ((threadIdx.x & 31) == 0) atomicMax(most, m);
 }
 
-// Slices of the finest level's A P from its CSR rows.  *again: they have no
-// dictionary within the caps, and the fine operator is back in CSR rows; A P is
-// then to be built like a coarser level's.
+// Slices of the finest level's A P from its CSR rows.  Where they have no dictionary
+// within the caps, the set-up fails as it does without memory for them, and amg_setup
+// starts again from CSR rows.
 static void *take_level(sph_rt *s, void *L, size_t bytes) {
   return lvl_alloc(s, static_cast<SphLevel *>(L), bytes);
 }
-static sph_rt_status build_ap_slices(sph_rt *s, SphLevel *L, bool *again) {
+static sph_rt_status build_ap_slices(sph_rt *s, SphLevel *L) {
   bool ok = false;
   sph_rt_status rc = sliced_build(s, L->n, L->ap_ptr, L->ap_col, nullptr, take_level, L, &L->ap_sl,
                                   nullptr, &ok);
@@ -1746,12 +1747,8 @@ static sph_rt_status build_ap_slices(sph_rt *s, SphLevel *L, bool *again) {
   SPH_CUDA(s, cudaMemcpyAsync(&L->ap_most, most, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
   SPH_CUDA(s, cudaStreamSynchronize(s->stream));
   dfree(s, most);
-  if (!ok || L->ap_most >= kNoPlace) {
-    L->ap_sl = SlicedRowsData{};
-    L->ap_pos = nullptr;
-    *again = true;
-    return sliced_undo(s);
-  }
+  if (!ok || L->ap_most >= kNoPlace || s->test_refuse_ap)
+    return set_error(s, SPH_RT_ENOMEM, "A P does not fit the sliced layout");
   const size_t size = (size_t)L->ap_sl.padded + 1;
   if (s->cfg.precision == SPH_RT_MIXED)
     L->ap_val32 = lalloc<float>(s, L, size);
@@ -1808,9 +1805,9 @@ static sph_rt_status build_ap(sph_rt *s) {
   SPH_LAUNCHED(s);
   compact_rows_kernel<<<gw, kBlock, 0, s->stream>>>(n, cnt, tmp, L->ap_ptr, L->ap_col);
   SPH_LAUNCHED(s);
-  bool again = false;
-  if (sliced && (rc = build_ap_slices(s, L, &again))) return rc;
-  if (!sliced || again) {
+  if (sliced) {
+    if ((rc = build_ap_slices(s, L))) return rc;
+  } else {
     L->ap_val = lalloc<double>(s, L, (size_t)total);
     if (!L->ap_val) return SPH_RT_ENOMEM;
     if (s->cfg.precision == SPH_RT_MIXED && !(L->ap_val32 = lalloc<float>(s, L, (size_t)total)))
@@ -2301,7 +2298,7 @@ static sph_rt_status numeric(sph_rt *s) {
 template <typename T>
 static void tail_setup(sph_rt *s);
 
-sph_rt_status amg_setup(sph_rt *s) {
+static sph_rt_status setup_levels(sph_rt *s) {
   sph_rt_status rc;
   if (!s->amg_ready || s->cfg.amg_rebuild) {
     // the set-up reads the finest level's values in CSR order
@@ -2315,10 +2312,34 @@ sph_rt_status amg_setup(sph_rt *s) {
     if (csr) {
       SPH_CUDA(s, cudaStreamSynchronize(s->stream));
       dfree(s, csr);
-      s->levels[0]->val = s->mat_val;  // none, unless A P took the slices back
+      s->levels[0]->val = nullptr;
     }
   }
   return numeric(s);
+}
+
+sph_rt_status amg_setup(sph_rt *s, double dt) {
+  if (!s->sl.ptr || (s->amg_ready && !s->cfg.amg_rebuild)) return setup_levels(s);
+  // beside the slices the device may be too small for a set-up that has room beside
+  // CSR rows: what it took goes back, and it starts again from those, assembled anew
+  // (a diagonal's sum runs in the order of its row's entries there)
+  amg_release(s);
+  std::vector<void *> held = s->allocs;
+  std::sort(held.begin(), held.end());
+  sph_rt_status rc = setup_levels(s);
+  if (rc != SPH_RT_ENOMEM) return rc;
+  cudaStreamSynchronize(s->stream);
+  amg_release(s);
+  const std::vector<void *> now = s->allocs;
+  for (void *p : now)
+    if (!std::binary_search(held.begin(), held.end(), p)) {
+      if (p == s->amg_gersh) s->amg_gersh = nullptr;
+      dfree(s, p);
+    }
+  if ((rc = sliced_undo(s))) return rc;
+  s->err.clear();
+  if ((rc = launch_assembly(s, dt, s->gersh))) return rc;
+  return setup_levels(s);
 }
 
 // ---------------------------------------------------------------------------

@@ -885,7 +885,9 @@ struct sph_rt {
   std::vector<void *> allocs;  // device allocations of the current particle set
   std::unordered_map<void *, size_t> alloc_size;
   std::multimap<size_t, void *> pool;  // released buffers kept for reuse
-  int64_t test_fail_after = -1;  // sph_rt_test_hook: allocations until one fails (-1: none)
+  // sph_rt_test_hook: allocations until one fails (-1: none), A P's slices refused
+  int64_t test_fail_after = -1;
+  bool test_refuse_ap = false;
 
   // sizes
   bool have_particles = false;

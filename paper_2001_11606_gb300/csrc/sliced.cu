@@ -457,29 +457,25 @@ sph_rt_status sliced_to_csr(sph_rt *s, double **csr) {
   return slice_move<double, double, false>(s, s->n_int, s->mat_ptr, s->sl, s->sl_val, *csr);
 }
 
-// Back to the CSR rows (geometry and the current values): the A P of this set
-// has no dictionary within the caps.
+// Back to the CSR rows, whose values the next assembly writes.  Without room for them
+// the slices stay.
 sph_rt_status sliced_undo(sph_rt *s) {
-  s->mat_G = dalloc<double>(s, s->nnz_mat);
-  s->mat_val = dalloc<double>(s, s->nnz_mat);
-  if (!s->mat_G || !s->mat_val) return SPH_RT_ENOMEM;
-  sph_rt_status rc;
-  if ((rc = slice_move<double, double, false>(s, s->n_int, s->mat_ptr, s->sl, s->sl_G, s->mat_G)))
+  double *G = dalloc<double>(s, s->nnz_mat), *val = dalloc<double>(s, s->nnz_mat);
+  float *val32 = s->sl_val32 ? dalloc<float>(s, s->nnz_mat) : nullptr;
+  sph_rt_status rc = G && val && (val32 || !s->sl_val32) ? SPH_RT_OK : SPH_RT_ENOMEM;
+  if (!rc) rc = slice_move<double, double, false>(s, s->n_int, s->mat_ptr, s->sl, s->sl_G, G);
+  cudaStreamSynchronize(s->stream);
+  if (rc) {
+    release_slices(s, SlicedRowsData{}, G, val, val32);
     return rc;
-  if ((rc = slice_move<double, double, false>(s, s->n_int, s->mat_ptr, s->sl, s->sl_val,
-                                              s->mat_val)))
-    return rc;
-  if (s->sl_val32) {
-    if (!(s->mat_val32 = dalloc<float>(s, s->nnz_mat))) return SPH_RT_ENOMEM;
-    if ((rc = slice_move<float, float, false>(s, s->n_int, s->mat_ptr, s->sl, s->sl_val32,
-                                              s->mat_val32)))
-      return rc;
   }
-  SPH_CUDA(s, cudaStreamSynchronize(s->stream));
   release_slices(s, s->sl, s->sl_G, s->sl_val, s->sl_val32);
   s->sl = SlicedRowsData{};
   s->sl_G = s->sl_val = nullptr;
   s->sl_val32 = nullptr;
+  s->mat_G = G;
+  s->mat_val = val;
+  s->mat_val32 = val32;
   return SPH_RT_OK;
 }
 

@@ -43,7 +43,7 @@ void outer_loop_account(sph_rt *s, const Scalars &h);
 void loop_graph_release(sph_rt *s);
 sph_rt_status launch_cheb_slots(sph_rt *s, int first, const double *gersh_dev,
                                 const std::vector<int> &mode, const std::vector<int> &degree);
-sph_rt_status amg_setup(sph_rt *s);
+sph_rt_status amg_setup(sph_rt *s, double dt);
 void amg_release(sph_rt *s);
 sph_rt_status validate_device_particles(sph_rt *s, int64_t n, const double *pos,
                                         const double *mass, const double *rho, const double *h,
@@ -403,10 +403,11 @@ extern "C" sph_rt_status sph_rt_release_cached_memory(int32_t device) {
 }
 
 // For the tests of the fall-backs, not part of the interface: makes one device
-// allocation of the handle fail, after `fail_after` more that succeed (-1: none).
-// Returns the number of buffers in use.
-extern "C" int64_t sph_rt_test_hook(sph_rt *s, int64_t fail_after) {
+// allocation of the handle fail, after `fail_after` more that succeed (-1: none), and
+// refuses the slices of A P (refuse_ap).  Returns the number of buffers in use.
+extern "C" int64_t sph_rt_test_hook(sph_rt *s, int64_t fail_after, int32_t refuse_ap) {
   s->test_fail_after = fail_after;
+  s->test_refuse_ap = refuse_ap != 0;
   return (int64_t)s->allocs.size();
 }
 
@@ -832,7 +833,7 @@ static sph_rt_status step_common(sph_rt *s, double dt, const double *Qe_c, const
 
   if (s->cfg.precond == SPH_RT_PRECOND_AMG) {  // a5
     tm.begin(2);
-    if ((rc = amg_setup(s))) return rc;
+    if ((rc = amg_setup(s, dt))) return rc;
     tm.end();
   }
 
