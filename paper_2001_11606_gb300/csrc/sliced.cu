@@ -450,7 +450,7 @@ sph_rt_status sliced_operator(sph_rt *s) {
 }
 
 // The current values in CSR order (a scratch buffer of nnz_mat doubles; the
-// caller releases it): for the AMG set-up and the operator read-back.
+// caller releases it), for the AMG set-up.
 sph_rt_status sliced_to_csr(sph_rt *s, double **csr) {
   *csr = dalloc<double>(s, s->nnz_mat);
   if (!*csr) return SPH_RT_ENOMEM;

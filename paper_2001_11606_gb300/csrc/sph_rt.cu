@@ -1203,14 +1203,19 @@ extern "C" sph_rt_status sph_rt_get_operator(sph_rt *s, int64_t *rowptr, int64_t
   if ((rc = d2h(s, s2c, s->slot2caller, s->n))) return rc;
   if ((rc = d2h(s, ptr, s->mat_ptr, s->n_int + 1))) return rc;
   if ((rc = d2h(s, col, s->mat_col, s->nnz_mat))) return rc;
-  double *csr = nullptr;
-  if (s->sl.ptr && (rc = sliced_to_csr(s, &csr))) return rc;
-  if ((rc = d2h(s, val, csr ? csr : s->mat_val, s->nnz_mat))) return rc;
+  // values in slices are read as they stand: entry t of a row at first + t * stride
+  std::vector<int64_t> sptr;
+  std::vector<uint8_t> place;
+  const bool sliced = s->sl.ptr != nullptr;
+  if ((rc = sliced ? d2h(s, val, s->sl_val, s->sl.padded) : d2h(s, val, s->mat_val, s->nnz_mat)))
+    return rc;
+  if (sliced && ((rc = d2h(s, sptr, s->sl.ptr, ceil_div(s->n_int, 32) + 1)) ||
+                 (rc = d2h(s, place, s->sl.place, s->n_int))))
+    return rc;
   if ((rc = d2h(s, dg, s->diag, s->n_int))) return rc;
   if ((rc = d2h(s, g, s->gb, s->n_int))) return rc;
   if ((rc = d2h(s, V, s->V, s->n_int))) return rc;
   SPH_CUDA(s, cudaStreamSynchronize(s->stream));
-  dfree(s, csr);
   const int64_t n = s->n;
   std::vector<int64_t> cnt((size_t)n, 0);
   for (int64_t slot = 0; slot < s->n_int; ++slot) cnt[s2c[slot]] = ptr[slot + 1] - ptr[slot];
@@ -1224,10 +1229,15 @@ extern "C" sph_rt_status sph_rt_get_operator(sph_rt *s, int64_t *rowptr, int64_t
   for (int64_t slot = 0; slot < s->n_int; ++slot) {
     int64_t c = s2c[slot];
     double invVi = 1.0 / V[slot];
+    int64_t first = ptr[slot], stride = 1;
+    if (sliced) {
+      first = sptr[slot / kBlock * kWarpsPerBlock + place[slot] / 32] + place[slot] % 32;
+      stride = 32;
+    }
     for (int64_t k = ptr[slot]; k < ptr[slot + 1]; ++k) {
-      int64_t at = rp[c] + (k - ptr[slot]);
+      const int64_t t = k - ptr[slot], at = rp[c] + t;
       if (cols) cols[at] = s2c[col[k]];
-      if (vals) vals[at] = val[k] * invVi;
+      if (vals) vals[at] = val[first + t * stride] * invVi;
     }
     if (diag) diag[c] = dg[slot] * invVi;
     if (gb) gb[c] = g[slot];

@@ -88,6 +88,17 @@ def test_refused_slices_of_ap_take_the_operator_back(case, over):
     assert got[0] == csr[0] and _same(got, csr)
 
 
+def test_operator_read_back_needs_no_device_memory(case):
+    w, ins = case
+    S = sphrt.solver_for(w, precond=0)
+    S.step(w.dt, *ins[0])
+    want = S.get_operator()
+    _hook(S, 0)
+    got = S.get_operator()
+    assert all(np.array_equal(a, b) for a, b in zip(want, got))
+    S.close()
+
+
 def test_a_new_set_chooses_again(case):
     w, ins = case
     S = sphrt.solver_for(w, precond=0, kernel_timing=1)
