@@ -2811,8 +2811,11 @@ sph_rt_status fcg_cycle(sph_rt *s, const FcgVecs &v, int first) {
   return fcg_cycle_t<double>(s, v.f64, first);
 }
 
-// Launch-relevant layout of the hierarchy (sizes, shapes and every buffer the
-// V-cycle touches), appended to the signature of a captured loop graph.
+// Launch-relevant layout of the hierarchy, appended to the signature of a captured loop
+// graph: sizes, shapes, the finest level's own buffers and EVERY buffer that belongs to a
+// level, in the order of allocation, which gives each its role.  (Rebuilt hierarchies
+// take their buffers from a free list keyed by size: buffers of one size can change
+// places while all others stay.)
 void amg_signature(const sph_rt *s, std::vector<uint64_t> &sig) {
   sig.push_back(s->levels.size());
   sig.push_back((uint64_t)s->tail_level);
@@ -2820,8 +2823,11 @@ void amg_signature(const sph_rt *s, std::vector<uint64_t> &sig) {
   for (const SphLevel *L : s->levels) {
     const uint64_t v[] = {(uint64_t)L->n,
                           (uint64_t)L->nnz,
+                          (uint64_t)L->nnz_ap,
                           (uint64_t)L->W,
                           (uint64_t)L->U,
+                          (uint64_t)L->ap_sl.dict_max,
+                          (uint64_t)L->ap_sl.padded,
                           (uint64_t)(uintptr_t)L->ptr,
                           (uint64_t)(uintptr_t)L->col,
                           (uint64_t)(uintptr_t)L->val,
@@ -2830,30 +2836,9 @@ void amg_signature(const sph_rt *s, std::vector<uint64_t> &sig) {
                           (uint64_t)(uintptr_t)L->val32,
                           (uint64_t)(uintptr_t)L->diag32,
                           (uint64_t)(uintptr_t)L->invdiag32,
-                          (uint64_t)(uintptr_t)L->agg,
-                          (uint64_t)(uintptr_t)L->agg_ptr,
-                          (uint64_t)(uintptr_t)L->agg_mem,
-                          (uint64_t)(uintptr_t)L->r,
-                          (uint64_t)(uintptr_t)L->z,
-                          (uint64_t)(uintptr_t)L->res,
-                          (uint64_t)(uintptr_t)L->d,
-                          (uint64_t)(uintptr_t)L->t,
-                          (uint64_t)(uintptr_t)L->r32,
-                          (uint64_t)(uintptr_t)L->z32,
-                          (uint64_t)(uintptr_t)L->res32,
-                          (uint64_t)(uintptr_t)L->d32,
-                          (uint64_t)(uintptr_t)L->t32,
-                          (uint64_t)(uintptr_t)L->ap_ptr,
-                          (uint64_t)(uintptr_t)L->ap_col,
-                          (uint64_t)(uintptr_t)L->ap_val,
-                          (uint64_t)(uintptr_t)L->ap_val32,
-                          (uint64_t)(uintptr_t)L->ap_sl.ptr,
-                          (uint64_t)(uintptr_t)L->ap_sl.idx,
-                          (uint64_t)(uintptr_t)L->ap_sl.dict,
-                          (uint64_t)(uintptr_t)L->ap_sl.dptr,
-                          (uint64_t)(uintptr_t)L->ap_sl.len,
-                          (uint64_t)L->ap_sl.dict_max};
+                          (uint64_t)L->owned.size()};
     sig.insert(sig.end(), v, v + sizeof v / sizeof v[0]);
+    for (void *p : L->owned) sig.push_back((uint64_t)(uintptr_t)p);
   }
 }
 
