@@ -439,12 +439,13 @@ __global__ void __launch_bounds__(kBlock, 4)
     for (int t = threadIdx.x; t < nd; t += kBlock) Ds[t] = D[A.dict[d0 + t]];
     __syncthreads();
     const int64_t i = g * kBlock + threadIdx.x;  // place in the slices, then row
+    const unsigned lanes = __ballot_sync(0xffffffffu, i < A.n);  // of the last slice: its rows
     if (i < A.n) {
       const int len = A.len[i], row = A.order[i];
       const int64_t k0 = A.ptr[i >> 5] + (threadIdx.x & 31);
       const double Di = D[g * kBlock + row];
       double offsum = 0.0;
-      const int width = __reduce_max_sync(__activemask(), len);  // rows of one warp
+      const int width = __reduce_max_sync(lanes, len);  // rows of one warp
       for (int t = 0; t < width; t += kSliceU) {
         int c[kSliceU];
         double v[kSliceU];
