@@ -865,10 +865,12 @@ __global__ void __launch_bounds__(kBlock)
       const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
       const double ir = rsqrt_fp64(r2), d = r2 * ir;
       const double ihj = ih[j];
-      double F = q.cw * pair_dw(kern, d * q.ih);
-      // equal smoothing lengths (the common case): 0.5 (w + w) = w
+      // each product rounded by itself, with no multiply-add across them: F_ij and F_ji
+      // are the same bits, and B is symmetric to the last
+      double F = __dmul_rn(q.cw, pair_dw(kern, __dmul_rn(d, q.ih)));
+      // equal 1/h, of which cw is a function (the common case): 0.5 (w + w) = w
       if (__double_as_longlong(ihj) != __double_as_longlong(q.ih))
-        F = 0.5 * (F + cw[j] * pair_dw(kern, d * ihj));
+        F = 0.5 * __dadd_rn(F, __dmul_rn(cw[j], pair_dw(kern, __dmul_rn(d, ihj))));
       F *= ir;
       nbr_F[k0 + k] = F;
       if (j < n_int) {
