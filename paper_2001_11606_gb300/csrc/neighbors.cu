@@ -543,8 +543,10 @@ __global__ void rel_kernel(Grid g, const double *px, const double *py, const dou
 // 1 / sqrt(r2) in FP64: FP32 seed y refined by one third-order step,
 // y (1 + d/2 + 3/8 d^2) with d = 1 - r2 y^2, the Taylor series of (1 - d)^(-1/2)
 // (the seed's d ~ 2e-7 leaves d^3 ~ 1e-20, below the FP64 rounding): 5 FP64
-// operations and no division or square root.
+// operations and no division or square root.  An r2 outside FP32's normal range, of
+// which the seed would keep few bits or none, takes those.
 __device__ __forceinline__ double rsqrt_fp64(double r2) {
+  if (!narrow_ok(r2)) return 1.0 / sqrt(r2);
   const double y = (double)rsqrtf((float)r2);
   const double d = fma(-(r2 * y), y, 1.0);
   return fma(y, d * fma(0.375, d, 0.5), y);

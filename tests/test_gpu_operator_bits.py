@@ -1,5 +1,6 @@
-"""The operator's entries bit for bit: B is symmetric to the last bit whatever the
-smoothing lengths."""
+"""The operator's entries bit for bit and at the ends of their range: B is symmetric
+to the last bit whatever the smoothing lengths, and particle sets shrunk by a power of
+two have the shrunk operator, also where r^2 is no normal FP32 number."""
 import numpy as np
 import pytest
 
@@ -49,3 +50,20 @@ def test_operator_is_symmetric_to_the_last_bit(dim, n, box, h, kern):
     t = np.lexsort((rows, cols))  # the transposed entries in the same order
     assert np.array_equal(rows, cols[t]) and np.array_equal(cols, rows[t])
     assert vals.size > n and np.array_equal(vals, vals[t])
+
+
+# lengths of 2^-68 leave r^2 ~ 13 bits as an FP32 number, of 2^-80 none; those of 2^68
+# overflow FP32's range
+@pytest.mark.parametrize("power", [-80, -68, -60, 60, 68])
+@pytest.mark.parametrize("kern", [0, 1])
+def test_scaled_lengths_scale_the_operator(power, kern):
+    P = _cloud(3, 500, 7.0, _spread)
+    want = _entries(P, kern)
+    s = 2.0 ** power
+    Q = I.Particles(dim=3, dx=s, counts=P.counts, pos=P.pos * s, kind=P.kind, copy_of=P.copy_of,
+                    mass=P.mass * s ** 3, rho=P.rho, h=P.h * s, sigma0=P.sigma0)
+    # V_j F ~ s^-2; dt by s^2 keeps the diagonals in step
+    got = _entries(Q, kern, dt=1e-3 * s * s)
+    assert np.array_equal(want[0], got[0]) and np.array_equal(want[1], got[1])
+    # an entry takes ~30 roundings, and a power of two scales exactly
+    assert np.max(np.abs(got[2] * s * s - want[2]) / np.abs(want[2]).max()) <= 60 * 2.0 ** -53
