@@ -269,12 +269,19 @@ __device__ __forceinline__ float narrow<float>(double v) {
 
 // Quotients with few FP64 operations (the division in FP64 costs about ten, and the
 // FP64 pipe bounds the per-particle kernels): a reciprocal of the divisor and one
-// residual correction q + (x - q d) y (Markstein 1990), within an ulp of the
-// rounded quotient.
-// div_by: y = 1/d is known (a constant of the launch).
-__device__ __forceinline__ double div_by(double x, double d, double y) {
+// residual correction q + (x - q d) y (Markstein 1990).  Before its last rounding the
+// result is off by ~2^-88 of itself (~2^-104 with div_by's reciprocal): the rounded
+// quotient, but for about one in 2^35, which rounds to its neighbour.
+// An infinite or overflowing product, of which the residual would make a NaN, takes the
+// division.
+__device__ __forceinline__ double corrected_quotient(double x, double d, double y) {
   const double q = x * y;
   return fma(fma(-q, d, x), y, q);
+}
+// div_by: y = 1/d is known (a constant of the launch).
+__device__ __forceinline__ double div_by(double x, double d, double y) {
+  return ((uint32_t)__double2hiint(x * y) & 0x7ff00000u) != 0x7ff00000u ? corrected_quotient(x, d, y)
+                                                                       : x / d;
 }
 // recip: an FP32 seed (~2^-22) and one Newton step y (2 - d y), to ~2^-44; the
 // divisor's magnitude must be within 2^-100 .. 2^100 (recip_ok).
@@ -286,7 +293,9 @@ __device__ __forceinline__ double recip(double d) {
   return fma(y, fma(-d, y, 1.0), y);
 }
 __device__ __forceinline__ double quotient(double x, double d) {
-  return recip_ok(d) ? div_by(x, d, recip(d)) : x / d;
+  // |x| < 2^900: no product with a reciprocal of up to 2^100 overflows
+  const bool fast = recip_ok(d) && ((uint32_t)__double2hiint(x) & 0x7ff00000u) < (1923u << 20);
+  return fast ? corrected_quotient(x, d, recip(d)) : x / d;
 }
 // Larger of two non-negative values by their bit patterns (integer pipe); a NaN
 // in v is passed over, as by fmax.
