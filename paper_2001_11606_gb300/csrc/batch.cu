@@ -519,22 +519,21 @@ __global__ void __launch_bounds__(512, MINB) batch_step_kernel(BatchView v, Batc
   auto newton = [&](const double *E_new, const double *E_prev, const double *e_start,
                     double *e_out, double &ce, double &cE) {
     double mc[2] = {0.0, 0.0};
+    const bool loose = ph.tol_inner > 0x1p-12;
     for (int64_t i = P.q0 + threadIdx.x; i < P.q1; i += blockDim.x) {
       const double cs = ph.c * v.sigma[i], En = E_new[i];
       const double Pw = cs * En + v.Qe[i];
-      const double rdt = v.rho[i] * ph.inv_dt, eo = v.e_old[i], e0 = e_start[i];
+      const double rdt = corrected_quotient(v.rho[i], ph.dt, ph.inv_dt);
+      const double eo = v.e_old[i], e0 = e_start[i];
       // as in newton_kernel: T = e / c_v as a product, the Jacobian's factor
-      // 4 c sigma a / c_v hoisted, u / J by a reciprocal, tests on bit patterns
+      // 4 c sigma a / c_v hoisted
       const double ca = cs * ph.a, k1 = 4.0 * ca * ph.inv_cv;
       double ei = e0;
-      for (int it = 0; it < ph.max_inner; ++it) {
+      for (int it = 1; it <= ph.max_inner; ++it) {
         const double T = ei * ph.inv_cv, T3 = T * T * T;
         const double u = fma(rdt, ei - eo, fma(ca * T3, T, -Pw));
         const double J = fma(k1, T3, rdt);
-        const double de = recip_ok(J) ? u * recip(J) : u / J;
-        ei -= de;
-        const long long lim = __double_as_longlong(ph.tol_inner * fabs(ei));
-        if (__double_as_longlong(fabs(de)) <= lim && lim <= 0x7ff0000000000000ll) break;
+        if (newton_update(u, J, ei, ph.tol_inner, loose || it == ph.max_inner, ei)) break;
       }
       e_out[i] = ei;
       const double tiny = 1e-300;

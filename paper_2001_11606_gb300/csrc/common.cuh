@@ -297,6 +297,25 @@ __device__ __forceinline__ double quotient(double x, double d) {
   const bool fast = recip_ok(d) && ((uint32_t)__double2hiint(x) & 0x7ff00000u) < (1923u << 20);
   return fast ? corrected_quotient(x, d, recip(d)) : x / d;
 }
+// One update e1 = e - u / J of the material Newton solves; true once |u / J| <= tol |e1|.
+// FP64 operations bound them, so the quotient is a product with a reciprocal of ~2^-44:
+// the next iteration removes its error, and the last one's stays below 2^-56 |e1| where
+// |u / J| <= 2^-12 |e1|.  exact (uniform; a looser tol, or the last iteration allowed)
+// adds the residual correction of the quotients above.  The test reads bit patterns.
+__device__ __forceinline__ bool newton_update(double u, double J, double e, double tol, bool exact,
+                                              double &e1) {
+  double de;
+  if (recip_ok(J)) {
+    const double y = recip(J);
+    de = u * y;
+    if (exact) de = fma(fma(-de, J, u), y, de);
+  } else {
+    de = u / J;
+  }
+  e1 = e - de;
+  const long long lim = __double_as_longlong(tol * fabs(e1));
+  return __double_as_longlong(fabs(de)) <= lim && lim <= 0x7ff0000000000000ll;
+}
 // Larger of two non-negative values by their bit patterns (integer pipe); a NaN
 // in v is passed over, as by fmax.
 __device__ __forceinline__ double max_bits(double m, double v) {

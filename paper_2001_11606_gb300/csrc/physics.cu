@@ -618,11 +618,9 @@ __device__ void outer_check(Scalars *sc, const OuterTail &t) {
 // red[1] = max |E_new - E_prev|/|E_new|, red[2] = max Newton iterations,
 // red[3] = number of particles that hit the iteration limit.
 //
-// FP64-bound: ~14 operations an iteration (the quotient u / J by a reciprocal of
-// ~2^-44, whose error the next iteration would remove and which the last one, of
-// |de| <= tol |e|, does not feel), tests and maxima on bit patterns, and integer
-// reductions.  2.1e6 particles: 0.335 -> 0.214 ms, 2.5e5 (heating wave): 0.068 ->
-// 0.028.
+// FP64-bound: ~14 operations an iteration (newton_update in common.cuh), tests and
+// maxima on bit patterns, and integer reductions.  2.1e6 particles: 0.335 -> 0.214 ms,
+// 2.5e5 (heating wave): 0.068 -> 0.028.
 __global__ void __launch_bounds__(kBlock)
     newton_kernel(Phys ph, int64_t n_int, const double *rho, const double *sigma,
                   const double *e_old, const double *Qe, const double *E_new, double *E_prev,
@@ -631,6 +629,7 @@ __global__ void __launch_bounds__(kBlock)
   double ce = 0.0, cE = 0.0;
   int itmax = 0, fails = 0;
   const double tiny = 1e-300;
+  const bool loose = ph.tol_inner > 0x1p-12;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_int;
        i += (int64_t)gridDim.x * blockDim.x) {
     const double cs = ph.c * sigma[i];
@@ -650,14 +649,9 @@ __global__ void __launch_bounds__(kBlock)
       const double T3 = T * T * T;
       const double u = fma(rdt, ei - eo, fma(csa * T3, T, -P));
       const double J = fma(k4, T3, rdt);
-      const double de = recip_ok(J) ? u * recip(J) : u / J;
-      ei = ei - de;
       ++it;
-      const long long lim = __double_as_longlong(ph.tol_inner * fabs(ei));
-      if (__double_as_longlong(fabs(de)) <= lim && lim <= 0x7ff0000000000000ll) {
-        ok = true;
-        break;
-      }
+      ok = newton_update(u, J, ei, ph.tol_inner, loose || it == ph.max_inner, ei);
+      if (ok) break;
     }
     e_new[i] = ei;
     ce = max_bits(ce, quotient(fabs(ei - e0), max_bits(tiny, fabs(ei))));
