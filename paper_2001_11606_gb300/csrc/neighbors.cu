@@ -18,6 +18,7 @@
 // a hash table from cell key to cell (up to 2^58 cells).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
@@ -257,13 +258,14 @@ __global__ void scatter_kernel(const uint32_t *key, int64_t n, const int64_t *st
 
 // Order each key's slice by caller index.  A warp looks at 32 keys at a time
 // and sorts each slice of two or more in turn: the indices (distinct) are staged
-// in shared memory and each is written at its rank.  Slices beyond kSegStage
-// fall back to one lane's insertion sort.  (One thread per slice sorting in
+// in shared memory and each is written at its rank.  (One thread per slice sorting in
 // global memory took 0.20-0.23 ms for cells of 64-125 particles; this takes
-// 0.10 ms.)
+// 0.10 ms.)  The slices beyond kSegStage, of cells that hold very many, are listed
+// (large[0] of them, keys from large[1] on; the order of arrival changes no result)
+// for a kernel with a block each.
 constexpr int kSegStage = 256;
 __global__ void segment_sort_kernel(const int64_t *start, const unsigned *count, int64_t nkeys,
-                                    int64_t *slot2caller) {
+                                    int64_t *slot2caller, unsigned long long *large) {
   __shared__ int64_t stage[kWarpsPerBlock][kSegStage];
   int64_t *sm = stage[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
@@ -271,27 +273,13 @@ __global__ void segment_sort_kernel(const int64_t *start, const unsigned *count,
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t k0 = warp * 32; k0 < nkeys; k0 += nwarps * 32) {
     const unsigned mine = k0 + lane < nkeys ? count[k0 + lane] : 0u;
-    unsigned todo = __ballot_sync(0xffffffffu, mine >= 2);
+    if (mine > kSegStage) large[1 + atomicAdd(large, 1ull)] = (unsigned long long)(k0 + lane);
+    unsigned todo = __ballot_sync(0xffffffffu, mine >= 2 && mine <= kSegStage);
     while (todo) {
       const int t = __ffs(todo) - 1;
       todo &= todo - 1;
       const unsigned c = __shfl_sync(0xffffffffu, mine, t);
       int64_t *a = slot2caller + start[k0 + t];
-      if (c > kSegStage) {
-        if (lane == 0) {
-          for (unsigned q = 1; q < c; ++q) {
-            const int64_t v = a[q];
-            int64_t u = (int64_t)q - 1;
-            while (u >= 0 && a[u] > v) {
-              a[u + 1] = a[u];
-              --u;
-            }
-            a[u + 1] = v;
-          }
-        }
-        __syncwarp();
-        continue;
-      }
       for (unsigned q = lane; q < c; q += 32) sm[q] = a[q];
       __syncwarp();
       for (unsigned q = lane; q < c; q += 32) {
@@ -301,6 +289,45 @@ __global__ void segment_sort_kernel(const int64_t *start, const unsigned *count,
         a[rank] = v;
       }
       __syncwarp();
+    }
+  }
+}
+// The large slices, in place: a merge network that only ever compares upwards (each
+// merge's first pass mirrors its second half), so that places past the end, standing for
+// infinities, never move.  ~c (log2 c)^2 / 4 exchanges by the whole block, where one
+// lane's insertions were c^2 / 4 dependent steps: the set-up of 46,656 particles in
+// cells of 1,728 took 558 ms with those and takes 12 (81 with a thread for each cell).
+__global__ void __launch_bounds__(kBlock)
+    segment_sort_large_kernel(const int64_t *start, const unsigned *count,
+                              const unsigned long long *large, int64_t *slot2caller) {
+  const unsigned long long n_large = large[0];
+  for (unsigned long long q = blockIdx.x; q < n_large; q += gridDim.x) {
+    const unsigned long long k = large[1 + q];
+    const unsigned c = count[k];  // < 2^31
+    int64_t *a = slot2caller + start[k];
+    auto exchange = [&](unsigned lo, unsigned hi) {
+      if (hi < c && a[lo] > a[hi]) {
+        const int64_t v = a[lo];
+        a[lo] = a[hi];
+        a[hi] = v;
+      }
+    };
+    const unsigned pairs = (c + 1) / 2;
+    for (int lg = 0; (c - 1) >> lg; ++lg) {  // merge runs of 2^lg
+      const unsigned half = 1u << lg, low = half - 1;
+      for (unsigned t = threadIdx.x; t < pairs + half; t += kBlock) {
+        const unsigned b = (t >> lg) << (lg + 1), o = t & low;
+        exchange(b + o, b + 2 * half - 1 - o);
+      }
+      __syncthreads();
+      for (int lj = lg - 1; lj >= 0; --lj) {
+        const unsigned j = 1u << lj;
+        for (unsigned t = threadIdx.x; t < pairs + j; t += kBlock) {
+          const unsigned b = ((t >> lj) << (lj + 1)) + (t & (j - 1));
+          exchange(b, b + j);
+        }
+        __syncthreads();
+      }
     }
   }
 }
@@ -1056,8 +1083,19 @@ sph_rt_status build_particles(sph_rt *s, int64_t n, const double *pos_c, const d
     if ((rc = exclusive_scan(s, cnt64, nkeys, start))) return rc;
     scatter_kernel<<<grid1(s, n), kBlock, 0, st>>>(key, n, start, cur, s->slot2caller);
     SPH_LAUNCHED(s);
-    segment_sort_kernel<<<grid1(s, nkeys), kBlock, 0, st>>>(start, cnt, nkeys, s->slot2caller);
+    const int64_t most_large = n / (kSegStage + 1);
+    auto *large = dalloc<unsigned long long>(s, most_large + 1);
+    if (!large) return SPH_RT_ENOMEM;
+    SPH_CUDA(s, cudaMemsetAsync(large, 0, sizeof(unsigned long long), st));
+    segment_sort_kernel<<<grid1(s, nkeys), kBlock, 0, st>>>(start, cnt, nkeys, s->slot2caller,
+                                                            large);
     SPH_LAUNCHED(s);
+    if (most_large > 0) {
+      segment_sort_large_kernel<<<(int)std::min<int64_t>(most_large, s->num_sms * 4), kBlock, 0,
+                                  st>>>(start, cnt, large, s->slot2caller);
+      SPH_LAUNCHED(s);
+    }
+    dfree(s, large);  // reuse is stream-ordered
   } else {
     const int64_t nb = ceil_div(n, (int64_t)kRadixTile);
     for (int a = 0; a < 2; ++a) {
