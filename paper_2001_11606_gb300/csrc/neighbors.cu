@@ -296,7 +296,7 @@ __global__ void segment_sort_kernel(const int64_t *start, const unsigned *count,
 // merge's first pass mirrors its second half), so that places past the end, standing for
 // infinities, never move.  ~c (log2 c)^2 / 4 exchanges by the whole block, where one
 // lane's insertions were c^2 / 4 dependent steps: the set-up of 46,656 particles in
-// cells of 1,728 took 558 ms with those and takes 12 (81 with a thread for each cell).
+// cells of 1,728 took 558 ms with those and takes 6.7 (81 with a thread for each cell).
 __global__ void __launch_bounds__(kBlock)
     segment_sort_large_kernel(const int64_t *start, const unsigned *count,
                               const unsigned long long *large, int64_t *slot2caller) {
@@ -649,31 +649,37 @@ struct HashCells {  // occupied cells only, open addressing with linear probing
 // 2.24e8 pairs 42.5 -> 16.9 ms with pair_kernel.
 // --------------------------------------------------------------------------
 constexpr int kCellChunk = 16;
+// Small sets take shorter items, so that they fill the chip: no fewer than ~kItemsPerSm
+// an SM.  sph_rt_set_particles in 3-D on 152 SMs with items of 1, 4 and 16: 1,728
+// particles 0.43, 0.43 and 0.50 ms (of ~900 neighbours 1.61, 1.73 and 2.28), 13,824: 0.59,
+// 0.52 and 0.58, 64,000: 1.30, 0.99 and 1.02, 262,144: 4.15, 2.96 and 2.73.
+constexpr int kItemsPerSm = 24;
 
 // Work items: (first slot, particles) of every kCellChunk-piece of the interior
 // cells.  Their order is that of arrival and changes no result.
-__device__ __forceinline__ void add_items(int64_t beg, int64_t cnt, int2 *items, unsigned *nitems) {
-  const unsigned k = (unsigned)((cnt + kCellChunk - 1) / kCellChunk);
+__device__ __forceinline__ void add_items(int64_t beg, int64_t cnt, int chunk, int2 *items,
+                                          unsigned *nitems) {
+  const unsigned k = (unsigned)((cnt + chunk - 1) / chunk);
   const unsigned at = atomicAdd(nitems, k);
   for (unsigned q = 0; q < k; ++q) {
-    const int64_t b = beg + (int64_t)q * kCellChunk;
+    const int64_t b = beg + (int64_t)q * chunk;
     const int64_t left = beg + cnt - b;
-    items[at + q] = make_int2((int)b, (int)(left < kCellChunk ? left : kCellChunk));
+    items[at + q] = make_int2((int)b, (int)(left < chunk ? left : chunk));
   }
 }
 __global__ void dense_items_kernel(const int64_t *start, const unsigned *count, int64_t ninterior,
-                                   int2 *items, unsigned *nitems) {
+                                   int chunk, int2 *items, unsigned *nitems) {
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < ninterior;
        k += (int64_t)gridDim.x * blockDim.x)
-    if (count[k]) add_items(start[k], count[k], items, nitems);
+    if (count[k]) add_items(start[k], count[k], chunk, items, nitems);
 }
 __global__ void sorted_items_kernel(const uint64_t *cell_key, const int64_t *cell_start,
-                                    int64_t ncells, int ghost_shift, int2 *items,
+                                    int64_t ncells, int ghost_shift, int chunk, int2 *items,
                                     unsigned *nitems) {
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < ncells;
        c += (int64_t)gridDim.x * blockDim.x)
     if (!((cell_key[c] >> ghost_shift) & 1ull))
-      add_items(cell_start[c], cell_start[c + 1] - cell_start[c], items, nitems);
+      add_items(cell_start[c], cell_start[c + 1] - cell_start[c], chunk, items, nitems);
 }
 
 struct NbrCounts {  // per interior particle (COUNT)
@@ -1203,12 +1209,14 @@ sph_rt_status build_particles(sph_rt *s, int64_t n, const double *pos_c, const d
   rel_kernel<<<grid1(s, n), kBlock, 0, st>>>(g, s->px, s->py, s->pz, s->h, n, rel);
   SPH_LAUNCHED(s);
   SPH_CUDA(s, cudaMemsetAsync(nitems, 0, sizeof(unsigned), st));
+  const int chunk = (int)std::min<int64_t>(
+      kCellChunk, std::max<int64_t>(1, n_int / ((int64_t)kItemsPerSm * s->num_sms)));
   if (dense)
-    dense_items_kernel<<<grid1(s, nkeys / 2), kBlock, 0, st>>>(start, cnt, nkeys / 2, items,
+    dense_items_kernel<<<grid1(s, nkeys / 2), kBlock, 0, st>>>(start, cnt, nkeys / 2, chunk, items,
                                                                nitems);
   else
     sorted_items_kernel<<<grid1(s, n_cells), kBlock, 0, st>>>(cell_key, cell_start, n_cells,
-                                                              g.ghost_shift, items, nitems);
+                                                              g.ghost_shift, chunk, items, nitems);
   SPH_LAUNCHED(s);
   int gw = (int)ceil_div(n_int, kWarpsPerBlock);
   if (gw > s->num_sms * 8) gw = s->num_sms * 8;

@@ -1,5 +1,7 @@
-"""Cells that hold far more particles than one warp orders in shared memory; neighbour
-lists bit for bit as the oracle's, cell lists alike."""
+"""The neighbour search over its range of work items and cells: sets whose items are of
+one, a few and the most particles (they grow with the particles per SM), and cells that
+hold far more particles than one warp orders in shared memory; lists bit for bit as the
+oracle's, cell lists alike."""
 import numpy as np
 import pytest
 
@@ -35,6 +37,13 @@ def _check(P, cells, sample=None):
     orp, ocols = O.neighbors_of_rows(P.pos, P.h, rows)
     for k, i in enumerate(rows):
         assert np.array_equal(np.sort(cols[rp[i]:rp[i + 1]]), ocols[orp[k]:orp[k + 1]])
+
+
+# 24 items of 16 particles an SM: 152 SMs have the longest items from 58,368 particles on
+@pytest.mark.parametrize("n,box", [(900, 12.0), (9000, 26.0), (20000, 34.0), (90000, 56.0)])
+@pytest.mark.parametrize("cells", [sphrt.CELLS_DENSE, sphrt.CELLS_SORTED])
+def test_items_of_every_length(n, box, cells):
+    _check(_cloud(3, n, box, 1.1, n), cells, 400)
 
 
 # one cell of 255 .. 258 particles, of ~3,000; clumps among small cells
