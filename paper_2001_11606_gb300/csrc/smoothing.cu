@@ -194,10 +194,14 @@ struct HIter {
 // FP32 radius is widened by it.slack, so the list holds every point of the
 // support; a listed point outside adds w = 0.  h^d cancels from the update's
 // h^d S = k_d (1 + sum w(r / h)), which leaves one root and one division per
-// update.  A point with more than kHList listed distances sums over its cells
-// directly.  Sums run in member order, so they are deterministic.
+// update.  A point of which the list cannot hold all distances is scanned in every
+// update, its candidates collected in the same list and summed whenever that is full,
+// so that FP64 work is done for the points of the support alone and on full warps.
+// Sums run in member order, so they are deterministic.
 // sph_rt_adapt_smoothing_lengths on 48,840 points (40 x 37 x 33, Wendland,
-// eta = 4), its rebuild of the particle set (2.5 ms) included: 40.1 -> 6.4 ms.
+// eta = 4), its rebuild of the particle set (2.5 ms) included: 40.1 -> 6.4 ms; on
+// 13,824 points with eta = 5.5, beyond the list, 25.9 (every candidate
+// summed in every update) -> 5.2 ms.
 constexpr int kHList = 448;
 constexpr double kHMargin = 1.08;
 __global__ void __launch_bounds__(kBlock)
@@ -232,56 +236,70 @@ __global__ void __launch_bounds__(kBlock)
     };
     double hi = h[i];
     double hc = 0.0;  // h the list covers (0: no list yet)
-    int cnt = 0;      // listed distances (warp-uniform), > kHList: not listed
+    int listed = -1;  // listed distances (warp-uniform), -1: more than the list holds
     int k = 0;
     bool capped = false;
+    // the points (but i) within radius r of i by the widened FP32 test, as slots in ls in
+    // member order: put(count) takes them whenever the list fills up, and the rest at
+    // the end, and says whether to go on
+    auto scan = [&](double r, const auto &put) {
+      const float rf = (float)(r * g.inv_cell) * 1.00001f + it.slack;
+      const float cut = rf * rf * 1.00001f;
+      int cnt = 0;  // slots in the list (warp-uniform)
+      for (int q = 0; q < nruns; ++q) {
+        int64_t b, e;
+        run(q, b, e);
+        for (int64_t m0 = b; m0 < e; m0 += 32) {
+          const int64_t m = m0 + lane;
+          bool hit = false;
+          int32_t j = -1;
+          if (m < e) {
+            const float4 p = rel[m];
+            const float dx = fx - p.x, dy = fy - p.y, dz = fz - p.z;
+            j = __float_as_int(p.w);
+            hit = dx * dx + dy * dy + dz * dz <= cut && j != (int32_t)i;
+          }
+          const unsigned mask = __ballot_sync(0xffffffffu, hit);
+          if (cnt + __popc(mask) > kHList) {
+            __syncwarp();
+            if (!put(cnt, false)) return;
+            __syncwarp();
+            cnt = 0;
+          }
+          if (hit) ls[cnt + __popc(mask & lt)] = __longlong_as_double((long long)j);
+          cnt += __popc(mask);
+        }
+      }
+      __syncwarp();
+      put(cnt, true);
+      __syncwarp();
+    };
+    // distance of the point whose slot stands at place t of the list
+    auto distance = [&](int t) {
+      const int64_t j = __double_as_longlong(ls[t]);
+      return sqrt(hr2(xi, yi, zi, px[j], py[j], pz[j]));
+    };
     while (k < it.max_iter) {
       if (hi > hc || hi < 0.8 * hc) {
         hc = fmax(fmin(kHMargin * hi, it.cap), hi);
-        const float rf = (float)(it.support * hc * g.inv_cell) * 1.00001f + it.slack;
-        const float cut = rf * rf * 1.00001f;
-        cnt = 0;
-        for (int q = 0; q < nruns; ++q) {
-          int64_t b, e;
-          run(q, b, e);
-          for (int64_t m0 = b; m0 < e; m0 += 32) {
-            const int64_t m = m0 + lane;
-            bool hit = false;
-            int32_t j = -1;
-            if (m < e) {
-              const float4 p = rel[m];
-              const float dx = fx - p.x, dy = fy - p.y, dz = fz - p.z;
-              j = __float_as_int(p.w);
-              hit = dx * dx + dy * dy + dz * dz <= cut && j != (int32_t)i;
-            }
-            const unsigned mask = __ballot_sync(0xffffffffu, hit);
-            const int at = cnt + __popc(mask & lt);
-            cnt += __popc(mask);
-            // the slot for now; its distance follows below, 32 at a time
-            if (hit && at < kHList) ls[at] = __longlong_as_double((long long)j);
-          }
-        }
-        __syncwarp();
-        for (int t = lane; t < cnt && cnt <= kHList; t += 32) {
-          const int64_t j = __double_as_longlong(ls[t]);
-          ls[t] = sqrt(hr2(xi, yi, zi, px[j], py[j], pz[j]));
-        }
+        listed = -1;
+        scan(it.support * hc, [&](int cnt, bool last) {
+          if (!last) return false;  // more than the list holds
+          for (int t = lane; t < cnt; t += 32) ls[t] = distance(t);
+          listed = cnt;
+          return true;
+        });
         __syncwarp();
       }
       const double ih = 1.0 / hi;
       double part = 0.0;
-      if (cnt <= kHList) {
-        for (int t = lane; t < cnt; t += 32) part += kernel_poly(it.kern, ls[t] * ih);
+      if (listed >= 0) {
+        for (int t = lane; t < listed; t += 32) part += kernel_poly(it.kern, ls[t] * ih);
       } else {
-        for (int q = 0; q < nruns; ++q) {
-          int64_t b, e;
-          run(q, b, e);
-          for (int64_t m = b + lane; m < e; m += 32) {
-            const int32_t j = __float_as_int(rel[m].w);
-            if (j == (int32_t)i) continue;
-            part += kernel_poly(it.kern, sqrt(hr2(xi, yi, zi, px[j], py[j], pz[j])) * ih);
-          }
-        }
+        scan(it.support * hi, [&](int cnt, bool) {
+          for (int t = lane; t < cnt; t += 32) part += kernel_poly(it.kern, distance(t) * ih);
+          return true;
+        });
       }
       // lane 0 holds the sum; every lane takes the update from it
       const double S = it.norm * (1.0 + __shfl_sync(0xffffffffu, warp_sum(part), 0));
