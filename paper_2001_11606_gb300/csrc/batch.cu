@@ -200,8 +200,8 @@ __device__ __forceinline__ double bdiv(double num, double den, double *bc, int &
   return out;
 }
 
-// Row tiles (see common.cuh) over this CTA's rows: tile k of 32 rows goes to warp
-// k mod nw; in a tile's W rounds each W-lane group sums one row, and the transposed
+// Row tiles (see common.cuh) over this CTA's rows: tile k of (at most) 32 rows goes to
+// warp k mod nw; in a tile's W rounds each W-lane group sums one row, and the transposed
 // reduction leaves every lane the sum of one row, so that the row epilogues (the
 // limiter's root and quotients, diagonal terms, inner products) run on 32 rows a
 // warp instruction.  On GB300's FP64 pipe, which bounds this kernel, an epilogue on
@@ -215,8 +215,12 @@ __device__ __forceinline__ void b_tiles(const Part &P, const int64_t *ptr, const
                                         const ROUND &round, const F &f) {
   const int lane = threadIdx.x & 31, sub = lane % W, own = tile_own_row<W>(lane);
   const int64_t wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int64_t base = P.q0 + wid * 32; base < P.q1; base += nw * 32) {
-    const int rows = (int)(P.q1 - base < 32 ? P.q1 - base : 32);
+  // a CTA of fewer than 32 rows a warp spreads them over all its warps
+  constexpr int G = 32 / W;
+  const int64_t share = ((P.q1 - P.q0 + nw - 1) / nw + G - 1) / G * G;
+  const int64_t tile = share < 32 ? share : 32;
+  for (int64_t base = P.q0 + wid * tile; base < P.q1; base += nw * tile) {
+    const int rows = (int)(P.q1 - base < tile ? P.q1 - base : tile);
     const bool active = own < rows;
     const int64_t i = base + own;
     int64_t b = 0, e = 0;
