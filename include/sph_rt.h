@@ -97,7 +97,9 @@ typedef struct {
   int32_t autotune;     /* 1: autotune on the first step.  The fine SpMV loads in flight (U = 4
                            or 8; never changes a result bit) on the first step of a particle
                            set (kept for later particle sets within 25 % of its rows and
-                           entries), and once per handle the smoother: one timed trial step (after
+                           entries; a set kept in slices, as most of 512 or more interior
+                           particles per SM are, has no such choice and is not timed for it),
+                           and once per handle the smoother: one timed trial step (after
                            an untimed one that captures its graph) from the same state for
                            each candidate -- with the AMG preconditioner finest-level
                            post-smoothing off (fine_post_smooth = 0, cheb_degree = 1; in the
