@@ -296,7 +296,7 @@ __global__ void segment_sort_kernel(const int64_t *start, const unsigned *count,
 // merge's first pass mirrors its second half), so that places past the end, standing for
 // infinities, never move.  ~c (log2 c)^2 / 4 exchanges by the whole block, where one
 // lane's insertions were c^2 / 4 dependent steps: the set-up of 46,656 particles in
-// cells of 1,728 took 558 ms with those and takes 6.7 (81 with a thread for each cell).
+// cells of 1,728 took 558 ms with those and takes 2.9 (81 with a thread for each cell).
 __global__ void __launch_bounds__(kBlock)
     segment_sort_large_kernel(const int64_t *start, const unsigned *count,
                               const unsigned long long *large, int64_t *slot2caller) {
@@ -835,8 +835,9 @@ __global__ void __launch_bounds__(kBlock)
 // ones, whatever its active lanes): a warp takes kPairRows consecutive rows and
 // walks their entries as one flat range, so that only the last instruction of a
 // range has idle lanes (of 200 entries in 2-D, 850-2,000 in 3-D); the rows' own
-// data sit in shared memory.  Longer ranges left 4e4 rows too few warps.  ~23 FP64 operations
-// a pair: r^2 by fused multiply-adds, the reciprocal root in 5, tests on q and
+// data sit in shared memory.  Longer ranges left 4e4 rows too few warps, and small sets
+// take fewer rows a warp, by the rule of the search's items: the set-up of 512 particles
+// of ~270 neighbours takes 0.43 ms (0.60 with 8 rows a warp).  ~23 FP64 operations a pair: r^2 by fused multiply-adds, the reciprocal root in 5, tests on q and
 // on equal smoothing lengths by bit patterns, and 0.5 (w + w) = w for the
 // latter (two evaluations otherwise).  1.26e7 pairs of unequal h: 1.02 ms.
 // --------------------------------------------------------------------------
@@ -857,7 +858,7 @@ __device__ __forceinline__ double pair_dw(int kern, double q) {
   return __double2hiint(t) < 0 ? 0.0 : a * b;  // 0 beyond the support
 }
 
-constexpr int kPairRows = 8;
+constexpr int kPairRows = 8;  // most rows of a warp's range
 struct PairRow {
   double x, y, z, ih, cw, V;
 };
@@ -866,7 +867,7 @@ __global__ void __launch_bounds__(kBlock)
     pair_kernel(int kern, int64_t n_int, const int64_t *nbr_ptr, const int32_t *nbr_col,
                 const double *px, const double *py, const double *pz, const double *ih,
                 const double *cw, const double *V, const int64_t *mat_ptr, double *nbr_F,
-                int32_t *mat_col, double *mat_G) {
+                int32_t *mat_col, double *mat_G, int tile_rows) {
   __shared__ PairRow rows_sh[kWarpsPerBlock][kPairRows];
   __shared__ int ptr_sh[kWarpsPerBlock][kPairRows + 1];
   __shared__ int64_t mat_sh[kWarpsPerBlock][kPairRows];
@@ -876,10 +877,8 @@ __global__ void __launch_bounds__(kBlock)
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t ntiles = ceil_div(n_int, kPairRows);
-  for (int64_t tile = warp; tile < ntiles; tile += nwarps) {
-    const int64_t r0 = tile * kPairRows;
-    const int rows = (int)(n_int - r0 < kPairRows ? n_int - r0 : kPairRows);
+  for (int64_t r0 = warp * tile_rows; r0 < n_int; r0 += nwarps * tile_rows) {
+    const int rows = (int)(n_int - r0 < tile_rows ? n_int - r0 : tile_rows);
     const int64_t k0 = nbr_ptr[r0];
     __syncwarp();
     if (lane < rows) {
@@ -921,7 +920,7 @@ __global__ void __launch_bounds__(kBlock)
 // Operator entries of ghost neighbours: copy-ghost columns (moved to the copied
 // particle; a copy of the row itself drops out) follow the interior ones in B;
 // Dirichlet ghosts form the boundary-coupling list.  Few rows have any: a warp
-// looks at kPairRows rows at a time and takes those with ghosts in turn, 32
+// looks at tile_rows rows at a time and takes those with ghosts in turn, 32
 // entries at a time (ballots keep the entries in list order).
 // --------------------------------------------------------------------------
 __global__ void op_ghost_kernel(const int64_t *nbr_ptr, const int32_t *interior,
@@ -929,15 +928,15 @@ __global__ void op_ghost_kernel(const int64_t *nbr_ptr, const int32_t *interior,
                                 const int32_t *copysrc, const double *V, int64_t n_int,
                                 const int64_t *mat_ptr, int32_t *mat_col, double *mat_G,
                                 const int64_t *gh_ptr, int32_t *gh_slot, double *gh_W,
-                                int32_t *gh_row) {
+                                int32_t *gh_row, int tile_rows) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t r0 = warp * kPairRows; r0 < n_int; r0 += nwarps * kPairRows) {
+  for (int64_t r0 = warp * tile_rows; r0 < n_int; r0 += nwarps * tile_rows) {
     const int64_t il = r0 + lane;
     unsigned todo = __ballot_sync(0xffffffffu,
-                                  lane < kPairRows && il < n_int &&
+                                  lane < tile_rows && il < n_int &&
                                       nbr_ptr[il + 1] - nbr_ptr[il] > interior[il]);
     while (todo) {
       const int64_t i = r0 + __ffs(todo) - 1;
@@ -1209,8 +1208,9 @@ sph_rt_status build_particles(sph_rt *s, int64_t n, const double *pos_c, const d
   rel_kernel<<<grid1(s, n), kBlock, 0, st>>>(g, s->px, s->py, s->pz, s->h, n, rel);
   SPH_LAUNCHED(s);
   SPH_CUDA(s, cudaMemsetAsync(nitems, 0, sizeof(unsigned), st));
-  const int chunk = (int)std::min<int64_t>(
-      kCellChunk, std::max<int64_t>(1, n_int / ((int64_t)kItemsPerSm * s->num_sms)));
+  const int per_item =
+      (int)std::max<int64_t>(1, n_int / ((int64_t)kItemsPerSm * s->num_sms));
+  const int chunk = std::min(kCellChunk, per_item);
   if (dense)
     dense_items_kernel<<<grid1(s, nkeys / 2), kBlock, 0, st>>>(start, cnt, nkeys / 2, chunk, items,
                                                                nitems);
@@ -1262,16 +1262,19 @@ sph_rt_status build_particles(sph_rt *s, int64_t n, const double *pos_c, const d
   kernel_coef_kernel<<<grid1(s, n), kBlock, 0, st>>>(n, dim, s->cfg.kernel, s->h, ih, cw);
   SPH_LAUNCHED(s);
   if ((rc = search(std::true_type{}, NbrCounts{}, s->nbr_ptr, s->nbr_col))) return rc;
-  int gt = (int)ceil_div(ceil_div(n_int, kPairRows), kWarpsPerBlock);
+  int tile_rows = kPairRows;  // in halves: 7 rows would load some SMs with one block more
+  while (tile_rows > per_item) tile_rows /= 2;
+  int gt = (int)ceil_div(ceil_div(n_int, tile_rows), kWarpsPerBlock);
   if (gt > s->num_sms * 8) gt = s->num_sms * 8;
   pair_kernel<<<gt, kBlock, 0, st>>>(s->cfg.kernel, n_int, s->nbr_ptr, s->nbr_col, s->px, s->py,
                                      s->pz, ih, cw, s->V, s->mat_ptr, s->nbr_F, s->mat_col,
-                                     s->mat_G);
+                                     s->mat_G, tile_rows);
   SPH_LAUNCHED(s);
   if (n > n_int) {
     op_ghost_kernel<<<gt, kBlock, 0, st>>>(s->nbr_ptr, interior, s->nbr_col, s->nbr_F, s->kind,
                                            s->copysrc, s->V, n_int, s->mat_ptr, s->mat_col,
-                                           s->mat_G, s->gh_ptr, s->gh_slot, s->gh_W, s->gh_row);
+                                           s->mat_G, s->gh_ptr, s->gh_slot, s->gh_W, s->gh_row,
+                                           tile_rows);
     SPH_LAUNCHED(s);
   }
   SPH_CUDA(s, cudaStreamSynchronize(st));
