@@ -1203,12 +1203,18 @@ extern "C" sph_rt_status sph_rt_get_operator(sph_rt *s, int64_t *rowptr, int64_t
   if ((rc = d2h(s, s2c, s->slot2caller, s->n))) return rc;
   if ((rc = d2h(s, ptr, s->mat_ptr, s->n_int + 1))) return rc;
   if ((rc = d2h(s, col, s->mat_col, s->nnz_mat))) return rc;
-  // values in slices are read as they stand: entry t of a row at first + t * stride
+  // values of slices: moved to CSR order on the device or, where it has no room for
+  // them, read as they stand: entry t of a row at first + t * stride
   std::vector<int64_t> sptr;
   std::vector<uint8_t> place;
-  const bool sliced = s->sl.ptr != nullptr;
-  if ((rc = sliced ? d2h(s, val, s->sl_val, s->sl.padded) : d2h(s, val, s->mat_val, s->nnz_mat)))
-    return rc;
+  double *csr = nullptr;
+  if (s->sl.ptr && (rc = sliced_to_csr(s, &csr)) && rc != SPH_RT_ENOMEM) return rc;
+  const bool sliced = s->sl.ptr && !csr;
+  if (sliced) s->err.clear();
+  rc = sliced ? d2h(s, val, s->sl_val, s->sl.padded)
+              : d2h(s, val, csr ? csr : s->mat_val, s->nnz_mat);
+  dfree(s, csr);
+  if (rc) return rc;
   if (sliced && ((rc = d2h(s, sptr, s->sl.ptr, ceil_div(s->n_int, 32) + 1)) ||
                  (rc = d2h(s, place, s->sl.place, s->n_int))))
     return rc;
