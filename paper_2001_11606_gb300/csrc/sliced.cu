@@ -491,15 +491,19 @@ sph_rt_status sliced_places(sph_rt *s, const int32_t *map, uint16_t *pos) {
 }
 
 // A thread per row adds its entries, in list order, to the row's A P entries (the
-// diagonal first, into entry 0, the row's own aggregate).  SMEM: the sums are
-// kept in shared memory, entry q of thread t at [q][t] (no bank conflicts); else
-// (rows with more aggregates than fit) in the A P array itself.
+// diagonal first, into entry 0, the row's own aggregate).  The sums are kept in shared
+// memory, entry q of thread t at [q][t] (no bank conflicts).
 // Replaces a gather over 4-byte source lists with one thread per A P entry:
 // 1.0 -> 0.36 ms a step in FP32 at 128^3 (2.18e8 entries), 0.10 ms in FP64 at 64^3.
-template <typename T, bool SMEM>
+// WINDOWS: rows of more A P entries than kApSmemMax holds walk their own entries once per
+// `window` of them, of the half that leaves room for two blocks an SM: 7.0e7 FP64 entries
+// of rows of 223 0.66 ms (summed in the A P array itself 1.07; windows of a third 0.71, of
+// the whole 0.74).  One window is the faster form wherever it fits, even with one block an
+// SM (244 entries a row, < 100 in A P: 0.79 ms against 1.06 in windows).
+template <typename T, bool WINDOWS>
 __global__ void __launch_bounds__(kBlock)
     ap_values_kernel(int64_t n, SlicedRowsData A, const uint16_t *pos, const T *val,
-                     const T *diag, const int32_t *agg, SlicedRowsData ap, T *ap_val) {
+                     const T *diag, const int32_t *agg, SlicedRowsData ap, int window, T *ap_val) {
   extern __shared__ __align__(16) unsigned char ap_smem[];
   T *acc = reinterpret_cast<T *>(ap_smem) + threadIdx.x;
   const int64_t groups = ceil_div(n, kBlock);
@@ -511,26 +515,27 @@ __global__ void __launch_bounds__(kBlock)
     const int m = ap.len[g * kBlock + q0], l = A.len[at];
     const int64_t o0 = ap.ptr[g * kWarpsPerBlock + q0 / 32] + q0 % 32;
     const int64_t k0 = A.ptr[at >> 5] + (threadIdx.x & 31);
-    T *out = SMEM ? acc : ap_val + o0;
-    constexpr int step = SMEM ? kBlock : 32;
-    for (int q = 0; q < m; ++q) out[q * step] = T(0);
-    if (agg[i] >= 0) out[0] = diag[i];
-    constexpr int U = 8;
-    for (int t = 0; t < l; t += U) {
-      int p[U];
-      T v[U];
+    for (int w0 = 0; w0 < m; w0 += WINDOWS ? window : m) {
+      const int mw = WINDOWS && m - w0 > window ? window : m - w0;
+      for (int q = 0; q < mw; ++q) acc[q * kBlock] = T(0);
+      if (w0 == 0 && agg[i] >= 0) acc[0] = diag[i];
+      constexpr int U = 8;
+      for (int t = 0; t < l; t += U) {
+        int p[U];
+        T v[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const bool in = t + u < l;
-        p[u] = in ? (int)__ldg(pos + k0 + (int64_t)(t + u) * 32) : kNoPlace;
-        v[u] = in ? __ldg(val + k0 + (int64_t)(t + u) * 32) : T(0);
+        for (int u = 0; u < U; ++u) {
+          const bool in = t + u < l;
+          p[u] = in ? (int)__ldg(pos + k0 + (int64_t)(t + u) * 32) : kNoPlace;
+          v[u] = in ? __ldg(val + k0 + (int64_t)(t + u) * 32) : T(0);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (WINDOWS ? (unsigned)(p[u] - w0) < (unsigned)mw : p[u] != kNoPlace)
+            acc[(p[u] - w0) * kBlock] += v[u];
       }
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (p[u] != kNoPlace) out[p[u] * step] += v[u];
+      for (int q = 0; q < mw; ++q) ap_val[o0 + (int64_t)(w0 + q) * 32] = acc[q * kBlock];
     }
-    if (SMEM)
-      for (int q = 0; q < m; ++q) ap_val[o0 + (int64_t)q * 32] = acc[q * step];
   }
 }
 
@@ -538,16 +543,20 @@ template <typename T>
 sph_rt_status sliced_ap_values(sph_rt *s, const uint16_t *pos, const int32_t *agg,
                                const SlicedRowsData &ap, int ap_most, const T *val, const T *diag,
                                T *ap_val) {
-  const int smem = ap_most * kBlock * (int)sizeof(T);
-  const int64_t groups = ceil_div(s->n_int, kBlock);
-  if (smem <= kApSmemMax) {
-    SPH_CUDA(s, cudaFuncSetAttribute(ap_values_kernel<T, true>,
+  constexpr int entry = kBlock * (int)sizeof(T);  // of one A P entry of a block's rows
+  const int grid = blocks_for(s, ceil_div(s->n_int, kBlock), 1, 8);
+  if (ap_most * entry <= kApSmemMax) {
+    SPH_CUDA(s, cudaFuncSetAttribute(ap_values_kernel<T, false>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, kApSmemMax));
-    ap_values_kernel<T, true><<<blocks_for(s, groups, 1, 8), kBlock, smem, s->stream>>>(
-        s->n_int, s->sl, pos, val, diag, agg, ap, ap_val);
+    ap_values_kernel<T, false><<<grid, kBlock, ap_most * entry, s->stream>>>(
+        s->n_int, s->sl, pos, val, diag, agg, ap, ap_most, ap_val);
   } else {
-    ap_values_kernel<T, false><<<blocks_for(s, groups, 1, 8), kBlock, 0, s->stream>>>(
-        s->n_int, s->sl, pos, val, diag, agg, ap, ap_val);
+    const int64_t passes = ceil_div(ap_most, kApSmemMax / 2 / entry);
+    const int window = (int)ceil_div(ap_most, passes);
+    SPH_CUDA(s, cudaFuncSetAttribute(ap_values_kernel<T, true>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, kApSmemMax / 2));
+    ap_values_kernel<T, true><<<grid, kBlock, window * entry, s->stream>>>(
+        s->n_int, s->sl, pos, val, diag, agg, ap, window, ap_val);
   }
   SPH_LAUNCHED(s);
   return SPH_RT_OK;

@@ -13,7 +13,7 @@ namespace sphrt {
 constexpr int64_t kTailMaxNnz = 600000;
 constexpr int kSliceMinGroups = 2;
 constexpr int kNoPlace = 0xffff;            // sliced A P: column without an aggregate
-constexpr int kApSmemMax = 200 * 1024;
+constexpr int kApSmemMax = 200 * 1024;      // of a block that sums A P entries
 
 sph_rt_status sliced_operator(sph_rt *s);
 sph_rt_status sliced_to_csr(sph_rt *s, double **csr);

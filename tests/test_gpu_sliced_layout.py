@@ -51,8 +51,8 @@ def test_slices_start_at_512_rows_per_sm():
 
 # Particles in pairs a tenth of a spacing apart, ~430 neighbours each: with a strength
 # threshold between the pairs' coupling and the next one the aggregates are the pairs, and
-# rows of A P have more than the 100 (FP64) and 200 (FP32) entries that are summed in
-# shared memory.
+# rows of A P have more than the 100 (FP64) and 200 (FP32) entries that shared memory holds
+# at once: they are summed in windows.
 def _pairs(n, h=2.34):
     P = I.make_lattice(3, (n,) * 3, 1.0 / n, 4, h_over_dx=h, jitter=0.0)
     odd = np.round(P.pos[:, 0] * n - 0.5).astype(int) % 2
