@@ -770,9 +770,10 @@ struct CsrView {
 // What it buys over the CSR row tiles: 2 instead of 4 bytes of column per entry
 // (6 instead of 8 bytes in FP32, 10 instead of 12 in FP64), one line per warp
 // load instead of 8 sectors, and gathers that do not go through the L1 tags,
-// which bound the FP32 sweeps.  V-cycle residual at 128^3 in FP32: 0.38 -> 0.24 ms
-// (5.9 TB/s of the bytes it must move); FP64 sweeps stay FP64-bound (one
-// multiply-add per entry): 0.21 -> 0.18 ms at 97 x 96 x 91.
+// which bound the FP32 sweeps.  V-cycle residual at 128^3 in FP32, in the
+// jobs: 0.410 -> 0.264 ms (5.16 TB/s of its 6 bytes an entry and 24 a row, 0.76 of the
+// copy bandwidth); FP64 sweeps stay FP64-bound (one multiply-add per entry):
+// 0.21 -> 0.18 ms at 97 x 96 x 91.
 // ---------------------------------------------------------------------------
 template <typename T>
 struct SlicedView {

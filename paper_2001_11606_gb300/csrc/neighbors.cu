@@ -837,9 +837,10 @@ __global__ void __launch_bounds__(kBlock)
 // range has idle lanes (of 200 entries in 2-D, 850-2,000 in 3-D); the rows' own
 // data sit in shared memory.  Longer ranges left 4e4 rows too few warps, and small sets
 // take fewer rows a warp, by the rule of the search's items: the set-up of 512 particles
-// of ~270 neighbours takes 0.43 ms (0.60 with 8 rows a warp).  ~23 FP64 operations a pair: r^2 by fused multiply-adds, the reciprocal root in 5, tests on q and
-// on equal smoothing lengths by bit patterns, and 0.5 (w + w) = w for the
-// latter (two evaluations otherwise).  1.26e7 pairs of unequal h: 1.02 ms.
+// of ~270 neighbours takes 0.43 ms (0.60 with 8 rows a warp).  ~23 FP64 operations a
+// pair: r^2 by fused multiply-adds, the reciprocal root in 5, tests on q and on equal
+// smoothing lengths by bit patterns, and 0.5 (w + w) = w for the latter (two
+// evaluations otherwise).  1.26e7 pairs of unequal h: 1.02 ms.
 // --------------------------------------------------------------------------
 // w'(q) without its normalisation.  Wendland C4 (Sec. 2.4, Eq. wendlandc4): the
 // printed polynomial (1 - q)^5 (8 q^2 + 5 q + 1) on q <= 1 has the derivative

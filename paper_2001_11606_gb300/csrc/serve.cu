@@ -23,7 +23,9 @@
 //            them, all steps in one CUDA-graph launch
 //
 // Each problem's kernels are the library's deterministic kernels on its own
-// data, so a request's result does not depend on what else is resident.
+// data, in the layout that its sizes choose, so a request's result does not depend
+// on what else is resident (short of a device too full for that layout's buffers:
+// sliced_operator).
 #include <cuda_runtime.h>
 #include <string.h>
 

@@ -27,9 +27,13 @@ static int blocks_for(const sph_rt *s, int64_t n, int per_block, int per_sm) {
 
 // Rows worth slicing: a block takes 256 rows, so the layout needs kSliceMinGroups
 // groups per SM to spread them evenly, and A P is formed from it (amg.cu), so the
-// level must be one that has A P.  Measured: at 1.6 groups per SM (64,000 rows of
-// 256 entries) a job took 31.0 ms sliced and 29.4 in row tiles, at 2.2 (86,387 rows
-// of 26) 25.5 against 27.2, at 54 (2.1e6 rows of 104, mixed) 382 against 457.
+// level must be one that has A P.  FP64 steps in ms, row tiles and slices, at 1.2, 2.0,
+// 3.0, 5.0 and 16 groups per SM: 240 entries a row (3-D) 1.05 1.27, 2.14 2.17, 3.08 3.19,
+// 4.49 4.47, 11.2 9.7; 104 entries 1.18 1.20, 1.57 1.58, 1.84 1.77 and, at 26 groups,
+// 10.0 8.7; 25 entries (2-D) 1.32 1.24, 1.72 1.66, 2.00 1.97.  The long rows set the line:
+// below two groups they lose up to a fifth, between two and four up to 7 % (616 groups on
+// 608 resident blocks), from five on nothing.  Mixed steps gain 4-30 % from two groups on.
+// The first step of a set pays 0.1-2 ms for building them.
 // A set holds ~36 bytes per entry in CSR rows; building the slices takes ~19 more and
 // the AMG set-up its lists: a set that has less than kSliceBytes of the device per
 // entry stays in CSR rows.  Sizes alone decide, never the memory that happens to be
